@@ -38,7 +38,7 @@ BULK_MIN, BULK_MAX = 16, 64  # between 16 and 64 window blocks per call
 # figure is reported only while the sources still hash to that.
 NCU_TRAFFIC = {"c2": {"bytes": 84.05e6 + 2.60e6,
                       "sources_sha256": "aafe1f3193d74c1d55e9d1a4309874d6a8a793292f0d4dcb65080bbb7dc7a849"}}
-KERNEL_SOURCES = ("xq_decode_umma.cu", "xq_layout.cuh", "xq_internal.h")
+KERNEL_SOURCES = ("xq_decode_mma.cuh", "xq_mma.cuh", "xq_layout.cuh", "xq_internal.h")
 
 
 def _kernel_sources_hash():

@@ -66,11 +66,11 @@ extern "C" {
 
 #define XQ_KERNEL_AUTO 0    /* tensor-core kernel when the shape allows it, else generic   */
 #define XQ_KERNEL_GENERIC 1 /* scalar kernel: any supported shape, slow, used as cross-check */
-/* Tensor-core kernel (tcgen05, integer operands): head_dim 128, group of <= 8 query
- * heads, layers that hold quantized tokens.  The products q_d * s_d (query times
- * key scale) and p_t * s_t (softmax numerator times value scale) enter the matrix
- * products as 21- and 23-bit fixed point relative to their largest member, the
- * accumulation is exact (32-bit integers), everything else is fp32. */
+/* Tensor-core kernel: group of <= 8 query heads; this value asks for it and wants head_dim
+ * 128 (XQ_KERNEL_AUTO takes it for head_dim 64 too).  The products q_d * s_d (query times
+ * key scale) and p_t * s_t (softmax numerator times value scale) enter the matrix products
+ * as unevaluated sums of two halves (22 significant bits), codes are exact, accumulation
+ * and everything else is fp32. */
 #define XQ_KERNEL_MMA 2
 
 #define XQ_MEM_DEVICE 0

@@ -26,7 +26,7 @@ constexpr int GEN_WARPS = 4;
 constexpr int GEN_HEADS = 8;  // query heads processed per pass
 
 template <int DPL>
-__global__ void __launch_bounds__(GEN_WARPS * 32) decode_generic_kernel(DecodeParams p) {
+__global__ void __launch_bounds__(GEN_WARPS * 32) decode_generic_kernel(const __grid_constant__ DecodeParams p) {
   constexpr int D = DPL * 32;
   __shared__ float sm_acc[GEN_WARPS][GEN_HEADS][D];
   __shared__ float sm_ml[GEN_WARPS][GEN_HEADS][2];
@@ -53,13 +53,13 @@ __global__ void __launch_bounds__(GEN_WARPS * 32) decode_generic_kernel(DecodePa
     t1 = min(t1 * 16, p.r);
   }
 
-  const int bk = p.L.bk, bv = p.L.bv;
-  const uint32_t* kc = p.L.k_codes + (size_t)bh * ((size_t)dm.nq_cap * D * bk / 32);
-  const uint32_t* vc = p.L.v_codes + (size_t)bh * ((size_t)dm.nq_cap * D * bv / 32);
-  const uint16_t* km = p.L.k_meta + (size_t)bh * (dm.nq_cap / g) * 2 * D;
-  const uint16_t* vm = p.L.v_meta + (size_t)bh * dm.nq_cap * 2 * NG;
-  const uint16_t* wk = p.L.win_k + (size_t)bh * dm.R * D;
-  const uint16_t* wv = p.L.win_v + (size_t)bh * dm.R * D;
+  const int bk = p.layer[0].L.bk, bv = p.layer[0].L.bv;
+  const uint32_t* kc = p.layer[0].L.k_codes + (size_t)bh * ((size_t)dm.nq_cap * D * bk / 32);
+  const uint32_t* vc = p.layer[0].L.v_codes + (size_t)bh * ((size_t)dm.nq_cap * D * bv / 32);
+  const uint16_t* km = p.layer[0].L.k_meta + (size_t)bh * (dm.nq_cap / g) * 2 * D;
+  const uint16_t* vm = p.layer[0].L.v_meta + (size_t)bh * dm.nq_cap * 2 * NG;
+  const uint16_t* wk = p.layer[0].L.win_k + (size_t)bh * dm.R * D;
+  const uint16_t* wv = p.layer[0].L.win_v + (size_t)bh * dm.R * D;
   const float scale2 = p.scale * 1.4426950408889634f;
 
   for (int g0 = 0; g0 < dm.G; g0 += GEN_HEADS) {
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(GEN_WARPS * 32) decode_generic_kernel(DecodePa
 #pragma unroll
       for (int j = 0; j < DPL; ++j) {
         acc[a][j] = 0.f;
-        q[a][j] = (a < nh) ? io_bits_f(p.q[((size_t)b * dm.Hq + hk * dm.G + g0 + a) * D + lane + 32 * j], p.f16) : 0.f;
+        q[a][j] = (a < nh) ? io_bits_f(p.layer[0].q[((size_t)b * dm.Hq + hk * dm.G + g0 + a) * D + lane + 32 * j], p.f16) : 0.f;
       }
     }
     for (int t = t0 + warp; t < t1; t += GEN_WARPS) {

@@ -110,7 +110,7 @@ void make_plan(const xq_config* c, Plan& pl) {
   }
   pl.part_acc = take((size_t)dm.B * dm.Hq * XQ_MAX_SPLITS * dm.D * 4);
   pl.part_ml = take((size_t)dm.B * dm.Hq * XQ_MAX_SPLITS * 2 * 4);
-  pl.tickets = take(BH * 4);
+  pl.tickets = take(BH * DECODE_MAX_LAYERS * 4);
   pl.status = take(4);
   pl.delta = take((size_t)c->n_layers * 2 * 4 * 8);  // per layer and cache kind: elements by code difference 0..3
   pl.staging_kv_bytes = (size_t)c->n_layers * BH * dm.D * 2;
@@ -161,7 +161,7 @@ struct xq_cache {
   bool tickets_clean;  // the ticket counters have been zeroed on a stream
   bool delta_clean;    // the code-difference counters have been zeroed on a stream
   std::vector<uint8_t> repacked;  // per layer: codes or parameters it reads were written since its last decode
-  int mma_ctas[2][2];  // resident CTAs per SM of the tensor-core kernel by (key bits - 1, value bits - 1); 0 = not asked yet
+  MmaShape mma_shape[2][2];  // the tensor-core kernel by (key bits - 1, value bits - 1); warps 0 = not asked yet
   // timing
   bool timing;
   std::vector<EventPair> pool;
@@ -194,58 +194,85 @@ void token_bytes(const xq_cache* c, int l, double& q_bytes, double& w_bytes) {
   w_bytes = 4.0 * dm.D;
 }
 
-bool layer_uses_mma(const xq_cache* c, int l) {
-  if (c->cfg.kernel == XQ_KERNEL_GENERIC) return false;
-  return decode_mma_supported(c->plan.dm, layer_bits(l, c->cfg.kq), layer_bits(l, c->cfg.vq));
+bool uses_mma(const xq_cache* c) {
+  const Dims& dm = c->plan.dm;
+  if (c->cfg.kernel == XQ_KERNEL_GENERIC || dm.G > 8) return false;
+  return dm.D == 128 || c->cfg.kernel == XQ_KERNEL_AUTO;  // XQ_KERNEL_MMA names the head_dim 128 kernel
 }
 
-int mma_ctas_per_sm(const xq_cache* c, int l) {
-  int bk = layer_bits(l, c->cfg.kq), bv = layer_bits(l, c->cfg.vq);
-  int& slot = const_cast<xq_cache*>(c)->mma_ctas[bk - 1][bv - 1];
-  if (slot == 0) {
-    slot = decode_mma_ctas_per_sm(c->plan.dm, bk, bv);
-    if (slot <= 0) slot = 2;  // no device to ask
+// FN<D, HP, NT> of the tensor-core kernel that serves these dimensions
+#define XQ_MMA_BY_HEADS(FN, D, ...)                   \
+  (dm.G == 1   ? FN<D, 1, 1>(__VA_ARGS__)             \
+   : dm.G == 2 ? FN<D, 2, 1>(__VA_ARGS__)             \
+   : dm.G <= 4 ? FN<D, 4, 1>(__VA_ARGS__)             \
+               : FN<D, 4, 2>(__VA_ARGS__))
+
+cudaError_t launch_decode_mma(const DecodeParams& p, cudaStream_t st) {
+  const Dims& dm = p.dm;
+  return dm.D == 128 ? XQ_MMA_BY_HEADS(launch_decode_mma_t, 128, p, st) : XQ_MMA_BY_HEADS(launch_decode_mma_t, 64, p, st);
+}
+
+// The tensor-core kernel that serves layer l, prepared for the handle's device on first use.
+MmaShape mma_shape(const xq_cache* c, int l) {
+  const Dims& dm = c->plan.dm;
+  const int bk = layer_bits(l, c->cfg.kq), bv = layer_bits(l, c->cfg.vq);
+  MmaShape& s = const_cast<xq_cache*>(c)->mma_shape[bk - 1][bv - 1];
+  if (s.warps == 0) {
+    s = dm.D == 128 ? XQ_MMA_BY_HEADS(decode_mma_shape_t, 128, dm.g, bk, bv) : XQ_MMA_BY_HEADS(decode_mma_shape_t, 64, dm.g, bk, bv);
+    if (s.ctas_per_sm <= 0) s.ctas_per_sm = 2;  // no device to ask
   }
-  return slot;
+  return s;
 }
 
-// Splits per (sequence, kv head) stream.  Tensor-core kernel (layers with quantized
-// tokens): every split takes whole batches of the packed region and a share of the
-// window (ns_w = 0), sized towards whole waves of resident CTAs.  Generic kernel:
+// Splits per (sequence, kv head) stream.  Tensor-core kernel: every split takes whole
+// batches of the packed region and a share of the window (ns_w = 0), sized towards
+// whole waves of resident CTAs.  Generic kernel:
 // separate splits for the packed region and for the window, in proportion to their bytes.
 // nq packed tokens and r window tokens are visible to the call.
-void plan_splits(const xq_cache* c, int l, int nq, int r, int& ns_q, int& ns_w, int* n_ctas_out = nullptr) {
+void plan_splits(const xq_cache* c, int l, int nq, int r, int& ns_q, int& ns_w, int* n_ctas_out = nullptr, int* deal_out = nullptr) {
   const Dims& dm = c->plan.dm;
   int units = (nq + 31) / 32, tiles = (r + 15) / 16;
   const int streams = dm.B * dm.Hkv;
-  if (layer_uses_mma(c, l) && nq > 0) {
-    // the tensor-core kernel: whole 128-token batches per CTA, every CTA also takes a share of the window
+  if (uses_mma(c)) {
+    // the tensor-core kernel: a CTA takes whole 128-token batches, dealt to its warps, and a share of the window
+    const MmaShape shape = mma_shape(c, l);
     const int batches = (nq + XQ_BATCH - 1) / XQ_BATCH;
+    // Batches are dealt to the CTAs in runs of one per warp where there are plenty (no warp of a CTA then waits for
+    // another's last batch; the CTAs that got fewer runs make room for the next layer), else one by one.
+    const int slot_count = c->sm_count * shape.ctas_per_sm;
+    const int deal = (long long)batches * streams >= 2LL * slot_count * shape.warps ? shape.warps : 1;
+    const int runs = (batches + deal - 1) / deal;
+    const int most = batches > 0 ? runs : tiles;  // no CTA without tokens
     ns_w = 0;
+    if (deal_out) *deal_out = deal;
     if (c->cfg.n_splits > 0) {
-      ns_q = c->cfg.n_splits < batches ? c->cfg.n_splits : batches;
+      ns_q = c->cfg.n_splits < most ? c->cfg.n_splits : most;
       if (n_ctas_out) *n_ctas_out = ns_q * streams;
       return;
     }
-    const long long slot_count = (long long)c->sm_count * mma_ctas_per_sm(c, l);
+    // Time of a launch in units of one batch's time on an SM of which nothing is idle: a wave costs a start and an
+    // end of about 12 units, and as long as its CTAs' batches take: one after the other in the slowest warp (a warp
+    // alone takes about 6 units for a batch), or all of the SM's together.
     int best = 1;
-    double best_score = -1.0;
-    for (int ns = 1; ns <= XQ_MAX_SPLITS && ns <= batches; ++ns) {
-      double ctas = (double)ns * streams;
-      double waves = ceil(ctas / (double)slot_count);
-      double fill = ctas / (waves * (double)slot_count);
-      double bpc = (double)batches / ns;         // batches per CTA
-      double score = fill * bpc / (bpc + 5.0);   // ~5 batches' worth of fixed cost per CTA
-      if (score > best_score) { best_score = score; best = ns; }
+    double best_time = 0.0;
+    for (int ns = 1; ns <= XQ_MAX_SPLITS && ns <= most; ++ns) {
+      const long long ctas = (long long)ns * streams;
+      const double waves = (double)((ctas + slot_count - 1) / slot_count);
+      long long resident = (ctas + c->sm_count - 1) / c->sm_count;
+      if (resident > shape.ctas_per_sm) resident = shape.ctas_per_sm;
+      const int per = (runs + ns - 1) / ns * deal;
+      const double chain = 6.0 * ((per + shape.warps - 1) / shape.warps), together = (double)per * (double)resident;
+      const double time = waves * (12.0 + (chain > together ? chain : together)) + 0.05 * ns;
+      if (ns == 1 || time < best_time) { best_time = time; best = ns; }
     }
     ns_q = best;
     if (n_ctas_out) *n_ctas_out = best * streams;
     // One wave that does not fill every resident slot: give some streams one split more, if the splits are many
     // enough for the CTAs' sizes to stay within a few percent of each other.
     if ((long long)best * streams < slot_count && slot_count < (long long)(best + 1) * streams && best >= 8 &&
-        best + 1 <= batches && best + 1 <= XQ_MAX_SPLITS) {
+        best + 1 <= most && best + 1 <= XQ_MAX_SPLITS) {
       ns_q = best + 1;
-      if (n_ctas_out) *n_ctas_out = (int)slot_count;
+      if (n_ctas_out) *n_ctas_out = slot_count;
     }
     return;
   }
@@ -330,24 +357,22 @@ int prepare_decode(const xq_cache* c, int layer, const void* q, void* out, int o
   for (int o : {k_owner(&c->cfg, layer), v_owner(&c->cfg, layer)}) {
     if (o != layer && c->seq[o] - residual_count(c->seq[o], dm.R) < nq) return XQ_ERR_ORDER;
   }
-  use_mma = layer_uses_mma(c, layer) && nq > 0;
-  if (c->cfg.kernel >= XQ_KERNEL_MMA && !layer_uses_mma(c, layer)) return XQ_ERR_CONFIG;
+  use_mma = uses_mma(c);
+  if (c->cfg.kernel >= XQ_KERNEL_MMA && !use_mma) return XQ_ERR_CONFIG;
   if (K_new && !use_mma) return XQ_ERR_ARG;
   p.dm = dm;
-  p.L = layer_ptrs(c, layer);
-  p.q = (const uint16_t*)q;
+  p.n_layers = 1;
+  p.layer[0] = {layer_ptrs(c, layer), (const uint16_t*)q, out, (const uint16_t*)K_new, (const uint16_t*)V_new};
   p.n_q = nq;
   p.r = r;
   p.n_ctas = 0;
-  plan_splits(c, layer, nq, r, p.ns_q, p.ns_w, &p.n_ctas);
+  p.deal = 1;
+  plan_splits(c, layer, nq, r, p.ns_q, p.ns_w, &p.n_ctas, &p.deal);
   p.scale = c->scale;
-  p.out = out;
   p.out_f32 = out_f32;
   p.early_fetch = 0;
   p.late_wait = 0;
   p.f16 = c->cfg.io_dtype == XQ_F16;
-  p.K_new = (const uint16_t*)K_new;
-  p.V_new = (const uint16_t*)V_new;
   return XQ_OK;
 }
 
@@ -371,7 +396,7 @@ int launch_decode(xq_cache* c, DecodeParams& p, bool use_mma, const Scratch& s, 
   m.f16 = p.f16;
   m.part_acc = p.part_acc;
   m.part_ml = p.part_ml;
-  m.out = p.out;
+  m.out = p.layer[0].out;
   m.out_f32 = p.out_f32;
   {
     Timer t(c, st, 1);
@@ -395,7 +420,7 @@ Scratch workspace_scratch(const xq_cache* c) {
 int ensure_clean_scratch(xq_cache* c, cudaStream_t st) {
   if (c->tickets_clean) return XQ_OK;
   const Dims& dm = c->plan.dm;
-  cudaError_t e = cudaMemsetAsync(c->ws + c->plan.tickets, 0, (size_t)dm.B * dm.Hkv * 4, st);
+  cudaError_t e = cudaMemsetAsync(c->ws + c->plan.tickets, 0, (size_t)dm.B * dm.Hkv * DECODE_MAX_LAYERS * 4, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + c->plan.status, 0, 4, st);
   if (e != cudaSuccess) return fail_cuda(c, e);
   c->tickets_clean = true;
@@ -481,15 +506,14 @@ int pack_layers(xq_cache* c, const int* layers, int n, const void* K, const void
 // chained: the launch before this one in the stream is a tensor-core decode launch of the same call, so nothing this
 // launch reads (q, the new token, the window, the packed streams) can still be written when its CTAs start; it
 // waits for that launch only before it writes.  *was_mma tells the caller whether this launch can head such a chain.
-int decode_impl(xq_cache* c, int layer, const void* q, void* out, int out_f32, cudaStream_t st,
-                const void* K_new = nullptr, const void* V_new = nullptr, int vis = -1, bool chained = false,
-                bool* was_mma = nullptr) {
+int decode_impl(xq_cache* c, int layer, const void* q, void* out, int out_f32, cudaStream_t st, int vis = -1,
+                bool chained = false, bool* was_mma = nullptr) {
   if (was_mma) *was_mma = false;
   if (!c) return XQ_ERR_ARG;
   if (layer < 0 || layer >= c->cfg.n_layers) return XQ_ERR_ARG;
   DecodeParams p;
   bool use_mma = false;
-  int rc = prepare_decode(c, layer, q, out, out_f32, K_new, V_new, c->seq[layer] + (K_new ? 1 : 0), p, use_mma, vis);
+  int rc = prepare_decode(c, layer, q, out, out_f32, nullptr, nullptr, c->seq[layer], p, use_mma, vis);
   if (rc != XQ_OK) return rc;
   if (use_mma) {
     rc = ensure_clean_scratch(c, st);
@@ -505,8 +529,45 @@ int decode_impl(xq_cache* c, int layer, const void* q, void* out, int out_f32, c
     return rc;
   }
   if (use_mma) c->repacked[layer] = 0;
-  if (K_new) c->seq[layer] += 1;
   if (was_mma) *was_mma = use_mma;
+  return XQ_OK;
+}
+
+// Tensor-core decode of the layers order[0 .. n).  Layer l's q and out are slice l of q and out; with K_new / V_new the launch appends slice l
+// of them to layer l (no layer's window is full).  Nothing in a launch reads what another layer of it writes: a layer
+// writes its own window row, its own part of the scratch and its own result.
+int decode_layers(xq_cache* c, const int* order, int n, const uint8_t* q, uint8_t* out, const uint8_t* K_new,
+                  const uint8_t* V_new, cudaStream_t st) {
+  const Dims& dm = c->plan.dm;
+  const size_t kv_layer = (size_t)dm.B * dm.Hkv * dm.D * 2, q_layer = (size_t)dm.B * dm.Hq * dm.D * 2;
+  int rc = ensure_clean_scratch(c, st);
+  if (rc != XQ_OK) return rc;
+  for (int i = 0; i < n;) {
+    DecodeParams p;
+    bool use_mma;
+    const int l0 = order[i], S = c->seq[l0] + (K_new ? 1 : 0);
+    rc = prepare_decode(c, l0, q + l0 * q_layer, out + l0 * q_layer, 0, K_new ? K_new + l0 * kv_layer : nullptr,
+                        V_new ? V_new + l0 * kv_layer : nullptr, S, p, use_mma);
+    if (rc != XQ_OK) return rc;
+    const bool packed = c->repacked[l0] != 0;
+    const int j = i + 1;
+    p.n_layers = j - i;
+    // The packed streams may be fetched ahead of the preceding kernel unless a pack kernel wrote them since the
+    // layers' last decode (then that kernel may be the writer, or only just behind it).  The launches after the first
+    // are chained: nothing they read (q, the new token, the window, the packed streams) can still be written when
+    // their CTAs start; they wait for their predecessor only before they write.
+    p.early_fetch = i > 0 || !packed;
+    p.late_wait = i > 0;
+    rc = launch_decode(c, p, true, workspace_scratch(c), st);
+    if (rc != XQ_OK) {
+      c->tickets_clean = false;
+      return rc;
+    }
+    for (; i < j; ++i) {
+      c->repacked[order[i]] = 0;
+      if (K_new) c->seq[order[i]] += 1;
+    }
+  }
   return XQ_OK;
 }
 
@@ -546,7 +607,7 @@ int xq_create(const xq_config* cfg, void* dev_workspace, size_t bytes, xq_cache*
   c->delta_clean = false;
   c->device = -1;
   c->static_base = nullptr;
-  memset(c->mma_ctas, 0, sizeof(c->mma_ctas));
+  memset(c->mma_shape, 0, sizeof(c->mma_shape));
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) == cudaSuccess &&
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) {
@@ -647,7 +708,7 @@ int chunk_impl(xq_cache* c, int layer, const void* q, void* out, int n, int out_
   for (int j = 0; j < n; ++j) {
     const uint8_t* qj = (const uint8_t*)q + (size_t)j * row * 2;
     uint8_t* oj = (uint8_t*)out + (size_t)j * row * (out_f32 ? 4 : 2);
-    const int rc = decode_impl(c, layer, qj, oj, out_f32, (cudaStream_t)stream, nullptr, nullptr, S - n + 1 + j, chain, &chain);
+    const int rc = decode_impl(c, layer, qj, oj, out_f32, (cudaStream_t)stream, S - n + 1 + j, chain, &chain);
     if (rc != XQ_OK) return rc;
   }
   return XQ_OK;
@@ -721,7 +782,7 @@ int xq_decode_step(xq_cache* c, const void* K_new, const void* V_new, const void
         const int nq = len[l] - residual_count(len[l], dm.R), nqo = len[o] - residual_count(len[o], dm.R);
         if (nqo < nq) return XQ_ERR_ORDER;
       }
-      if (c->cfg.kernel >= XQ_KERNEL_MMA && !layer_uses_mma(c, l)) return XQ_ERR_CONFIG;
+      if (c->cfg.kernel >= XQ_KERNEL_MMA && !uses_mma(c)) return XQ_ERR_CONFIG;
     }
   }
   cudaStream_t st = (cudaStream_t)stream;
@@ -760,28 +821,25 @@ int xq_decode_step(xq_cache* c, const void* K_new, const void* V_new, const void
       appended = true;
     }
   }
-  bool chain = false;  // the launch before the next one is a tensor-core decode launch of this call
-  for (int i = 0; i < L; ++i) {
-    const int l = layer_order ? layer_order[i] : i;
-    if (appended) {
-      const int rc = decode_impl(c, l, dq + l * q_layer, dout + l * q_layer, 0, st, nullptr, nullptr, -1, chain, &chain);
+  std::vector<int> order(L);
+  for (int i = 0; i < L; ++i) order[i] = layer_order ? layer_order[i] : i;
+  for (int i = 0; i < L;) {
+    const int l = order[i];
+    // A token that fills no window block goes into the window inside the tensor-core decode kernel, all such layers
+    // together; every other layer appends with its own kernels first.
+    auto fills = [&](int layer) { return c->seq[layer] > 0 && c->seq[layer] % dm.R == 0; };
+    int n = 1;
+    if (uses_mma(c) && (appended || !fills(l))) {
+      while (i + n < L && (appended || !fills(order[i + n]))) ++n;
+      const int rc = decode_layers(c, &order[i], n, dq, dout, appended ? nullptr : dk, appended ? nullptr : dv, st);
       if (rc != XQ_OK) return rc;
-      continue;
-    }
-    // One token that neither fills a window block nor is the layer's first quantized step goes into the window
-    // inside the tensor-core decode kernel; every other case appends with its own kernels first.
-    const int s_old = c->seq[l];
-    const int nq_old = s_old - residual_count(s_old, dm.R), nq_new = s_old + 1 - residual_count(s_old + 1, dm.R);
-    int rc;
-    if (nq_new == nq_old && nq_old > 0 && layer_uses_mma(c, l)) {
-      rc = decode_impl(c, l, dq + l * q_layer, dout + l * q_layer, 0, st, dk + l * kv_layer, dv + l * kv_layer, -1, chain,
-                       &chain);
     } else {
-      rc = xq_append_kv(c, l, dk + l * kv_layer, dv + l * kv_layer, 1, stream);
+      int rc = appended ? XQ_OK : xq_append_kv(c, l, dk + l * kv_layer, dv + l * kv_layer, 1, stream);
       if (rc != XQ_OK) return rc;
-      rc = decode_impl(c, l, dq + l * q_layer, dout + l * q_layer, 0, st, nullptr, nullptr, -1, false, &chain);
+      rc = decode_impl(c, l, dq + l * q_layer, dout + l * q_layer, 0, st);
+      if (rc != XQ_OK) return rc;
     }
-    if (rc != XQ_OK) return rc;
+    i += n;
   }
   if (mem == XQ_MEM_HOST) {
     cudaError_t e = cudaMemcpyAsync(out, dout, c->plan.staging_q_bytes, cudaMemcpyDeviceToHost, st);

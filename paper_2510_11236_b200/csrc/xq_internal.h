@@ -68,21 +68,34 @@ struct WindowParams {
   int nq_new;  // window slot = absolute token - nq_new
 };
 
-struct DecodeParams {
-  Dims dm;
+// One layer of a decode launch.
+struct DecodeLayer {
   LayerPtrs L;
   const uint16_t* q;  // [B,Hq,D] bf16
+  void* out;          // [B,Hq,D] bf16 or f32
+  // Fused append of one token per stream (tensor-core kernel only; else null): the newest window row, index r - 1, is
+  // not in the window yet but here, [B,Hkv,D] bf16.  The CTA whose share of the window holds that row reads it from
+  // here and stores it into the window.
+  const uint16_t* K_new;
+  const uint16_t* V_new;
+};
+
+constexpr int DECODE_MAX_LAYERS = 32;  // layers one launch can take (of equal lengths and bit-widths)
+
+struct DecodeParams {
+  Dims dm;
+  int n_layers;       // the scalar kernel takes one
   int n_q;            // quantized tokens
   int r;              // window tokens
   int ns_q, ns_w;     // splits over the quantized region (most of any stream) / over the window
-  int n_ctas;         // tensor-core kernel: CTAs over all streams (n_ctas / streams splits per stream, or one more)
+  int n_ctas;         // tensor-core kernel: CTAs of a layer over all streams (n_ctas / streams splits each, or one more)
+  int deal;           // tensor-core kernel: batches of 128 tokens are dealt to the splits in runs of this many
   float scale;
-  float* part_acc;    // [B,Hq,ns,D]
-  float* part_ml;     // [B,Hq,ns,2]  (running max in log2 units, sum)
+  float* part_acc;    // [n_layers,B,Hq,ns,D]
+  float* part_ml;     // [n_layers,B,Hq,ns,2]  (running max in log2 units, sum)
   // used by kernels that merge the partials themselves (last CTA of a stream):
-  void* out;              // [B,Hq,D] bf16 or f32
   int out_f32;
-  unsigned int* tickets;  // [B*Hkv], zero between launches
+  unsigned int* tickets;  // [n_layers,B*Hkv], zero between launches
   // 1: the packed streams were complete before the preceding kernel in the stream started, so their first
   // copies may be issued before this kernel has waited for that kernel (programmatic dependent launch)
   int early_fetch;
@@ -91,13 +104,9 @@ struct DecodeParams {
   // once and waits for that launch only before its first write that the launch could see (partials, tickets,
   // result, status).  Implies early_fetch.
   int late_wait;
-  // Fused append of one token per stream (tensor-core kernel with quantized tokens only; else null): the newest
-  // window row, index r - 1, is not in the window yet but here, [B,Hkv,D] bf16.  The CTA whose share of the
-  // window holds that row reads it from here and stores it into the window.
-  const uint16_t* K_new;
-  const uint16_t* V_new;
   int* status;  // device word the tensor-core kernel sets when one of its bounded waits gave up
   int f16;      // q, the window and the 16-bit output are IEEE half precision (else bfloat16)
+  DecodeLayer layer[DECODE_MAX_LAYERS];
 };
 
 struct MergeParams {
@@ -145,9 +154,16 @@ cudaError_t launch_dependent(void (*kernel)(P), dim3 grid, dim3 block, size_t sm
 cudaError_t launch_pack(const PackParams& p, cudaStream_t st);
 cudaError_t launch_window_append(const WindowParams& p, cudaStream_t st);
 cudaError_t launch_decode_generic(const DecodeParams& p, cudaStream_t st);
-cudaError_t launch_decode_mma(const DecodeParams& p, cudaStream_t st);
-bool decode_mma_supported(const Dims& dm, int bk, int bv);
-int decode_mma_ctas_per_sm(const Dims& dm, int bk, int bv);
+// Tensor-core decode kernels for HP (1, 2, 4) query heads per kv head, or NT = 2 sets of four.  decode_mma_shape_t
+// also prepares the kernel for the current device: it comes before the first launch of a handle.
+struct MmaShape {
+  int ctas_per_sm;  // 0: no device to ask
+  int warps;        // warps of a CTA
+};
+template <int D, int HP, int NT>
+cudaError_t launch_decode_mma_t(const DecodeParams& p, cudaStream_t st);
+template <int D, int HP, int NT>
+MmaShape decode_mma_shape_t(int g, int bk, int bv);
 cudaError_t launch_merge(const MergeParams& p, cudaStream_t st);
 
 }  // namespace xq
