@@ -237,15 +237,16 @@ int xq_decode_attention_static(xq_cache* c, int layer, const void* q, void* out,
  * stream before reading `out` or reusing the host buffers.
  * The result equals xq_append_kv followed by xq_decode_attention per layer, bit
  * for bit; where the tensor-core kernel serves the layer and the token fills no
- * window block, that kernel stores the token into the window itself (one launch
- * per layer); on the step on which every layer's window block fills (all layers
- * of equal length, no merging or difference counting), one quantize-and-pack
- * launch serves all layers before the decode launches.  K_new and V_new must
+ * window block, that kernel stores the token into the window itself; on the step
+ * on which every layer's window block fills (all layers of equal length, no
+ * merging or difference counting), one quantize-and-pack launch serves all layers
+ * before the decode launches.  From three layers on, layers of equal length and
+ * bit-widths share decode launches (up to 32 layers in one).  K_new and V_new must
  * stay unchanged until the step's kernels have run.  The tensor-core decode
  * launches of a step overlap: the first waits for all earlier work in `stream`
  * before it reads anything; each later one starts while its predecessor still
  * runs, reads at once (everything before the first launch is complete by then,
- * and a decode launch writes only its own window row, scratch and result) and
+ * and a decode launch writes only its own window rows, scratch and results) and
  * waits for the predecessor before its own first write to scratch or result.
  * Every layer's capacity, order and kernel are checked before the first copy or
  * launch: a call refused with XQ_ERR_ARG / CAPACITY / ORDER / CONFIG changes

@@ -682,6 +682,34 @@ def test_chained_decode_launches_equal_single_calls():
     a.close(); b.close()
 
 
+@pytest.mark.parametrize("D,Hq,Hkv,S", [(128, 8, 2, 40), (128, 2, 2, 700), (64, 4, 1, 300)])
+def test_decode_step_layers_that_share_launches(D, Hq, Hkv, S):
+    """Six layers of three bit-width combinations and two lengths (the last pair is five tokens ahead): the layers that
+    share a launch are found anew for each step, also while only some of them fill a window block.  Every result of
+    every step equals separate xq_append_kv / xq_decode_attention calls bit for bit."""
+    L, B, R = 6, 2, 32
+    w = dict(n_layers=L, batch=B, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=D, seq=S + 5, residual_len=R, group_size=32,
+             kq=4, vq=2, km=0, vm=0, n_outliers=3, outlier_scale=10.0, seed=23, n_splits=0)
+    cfg = W.make_xq_config(w, max_seq=S + 128)
+    a, b = xq.Cache(cfg, DEV), xq.Cache(cfg, DEV)
+    for cache in (a, b):
+        for pair in range(L // 2):
+            k0, v0, k1, v1 = W.pair_tokens(w, pair, 0, S + (5 if pair == 2 else 0), DEV)
+            cache.append_kv(2 * pair, k0, v0)
+            cache.append_kv(2 * pair + 1, k1, v1)
+    gen = torch.Generator(device="cpu").manual_seed(3)
+    for step in range(36):
+        kn = torch.randn(L, B, Hkv, 1, D, generator=gen).to(torch.bfloat16).to(DEV)
+        vn = torch.randn(L, B, Hkv, 1, D, generator=gen).to(torch.bfloat16).to(DEV)
+        q = torch.randn(L, B, Hq, D, generator=gen).to(torch.bfloat16).to(DEV)
+        out = a.decode_step(kn, vn, q, torch.empty_like(q))
+        for l in range(L):
+            b.append_kv(l, kn[l], vn[l])
+            assert torch.equal(b.decode_attention(l, q[l]), out[l]), (step, l)
+    a.check_device()
+    a.close(); b.close()
+
+
 def test_decode_step_from_host_buffers_at_full_size():
     """xq_decode_step with pinned host buffers (the end-to-end path the benchmark times) on the 32k GQA shape with
     one layer pair: three steps, sampled streams against the oracle."""
