@@ -705,8 +705,80 @@ int xq_decode_attention_f32(xq_cache* c, int layer, const void* q, float* out, v
 }
 
 namespace {
-// Query token j of n sees the cache up to its own position; one decode launch per token (their visible ranges
-// differ), all on the same stream.
+
+// How the query rows of a chunk are cut: 16 wr rows per CTA, ns splits of a row tile's tokens.
+struct ChunkPlanning {
+  int wr, row_tiles, ns;
+};
+ChunkPlanning plan_chunk(const xq_cache* c, int S, int T) {
+  const Dims& dm = c->plan.dm;
+  const long long streams = (long long)dm.B * dm.Hkv;
+  const int rows = T * dm.G;
+  // tiles of 64 tokens that a row tile goes over: the last one, and on average over the causal chunk
+  const double most = S / 64.0 + 1.0, mean = (S - 0.5 * T) / 64.0 + 1.0;
+  ChunkPlanning best{8, 0, 1};
+  double best_time = 0.0;
+  for (int wr : {8, 4, 2}) {
+    const int row_tiles = (rows + 16 * wr - 1) / (16 * wr);
+    // microseconds of a tile: products, or the expansion that does not fit beside them
+    const double tile = wr == 8 ? 3.0 : (wr == 4 ? 1.8 : 1.2);
+    for (int ns = 1; ns <= 32; ++ns) {
+      if (ns > 1 && (row_tiles > DECODE_MAX_LAYERS || ns > most ||
+                     streams * row_tiles * 16 * wr * ns > (long long)dm.B * dm.Hq * XQ_MAX_SPLITS))
+        break;
+      const double waves = ceil((double)(streams * row_tiles * ns) / c->sm_count);
+      const double longest = most / ns > waves * mean / ns ? most / ns : waves * mean / ns;
+      const double time = longest * tile + waves * (ns > 1 ? 6.0 : 4.0);
+      if (best.row_tiles == 0 || time < best_time) {
+        best_time = time;
+        best = {wr, row_tiles, ns};
+      }
+    }
+  }
+  return best;
+}
+
+int launch_chunk(xq_cache* c, int layer, const void* q, void* out, int T, int out_f32, cudaStream_t st) {
+  int rc = ensure_clean_scratch(c, st);
+  if (rc != XQ_OK) return rc;
+  const Dims& dm = c->plan.dm;
+  const int S = c->seq[layer];
+  const Scratch s = workspace_scratch(c);
+  const ChunkPlanning pl = plan_chunk(c, S, T);
+  ChunkParams p;
+  p.dm = dm;
+  p.L = layer_ptrs(c, layer);
+  p.q = (const uint16_t*)q;
+  p.out = out;
+  p.r = residual_count(S, dm.R);
+  p.n_q = S - p.r;
+  p.S = S;
+  p.T = T;
+  p.row_tiles = pl.row_tiles;
+  p.ns = pl.ns;
+  p.scale = c->scale;
+  p.part_acc = s.part_acc;
+  p.part_ml = s.part_ml;
+  p.tickets = s.tickets;
+  p.out_f32 = out_f32;
+  p.f16 = c->cfg.io_dtype == XQ_F16;
+  cudaError_t e;
+  {
+    Timer t(c, st, 0);
+    if (dm.D == 128) e = pl.wr == 8 ? launch_chunk_t<128, 8>(p, st) : pl.wr == 4 ? launch_chunk_t<128, 4>(p, st) : launch_chunk_t<128, 2>(p, st);
+    else e = pl.wr == 8 ? launch_chunk_t<64, 8>(p, st) : pl.wr == 4 ? launch_chunk_t<64, 4>(p, st) : launch_chunk_t<64, 2>(p, st);
+  }
+  c->launches++;
+  if (e != cudaSuccess) {
+    c->tickets_clean = false;
+    return fail_cuda(c, e);
+  }
+  c->repacked[layer] = 0;  // the launch began after everything before it in the stream had completed
+  return XQ_OK;
+}
+
+// Query token j of n sees the cache up to its own position.  The tensor-core kernels: one launch for the chunk;
+// otherwise (the scalar kernel, a single token) one decode launch per token, all on the same stream.
 int chunk_impl(xq_cache* c, int layer, const void* q, void* out, int n, int out_f32, void* stream) {
   if (!c || !q || !out) return XQ_ERR_ARG;
   if (layer < 0 || layer >= c->cfg.n_layers) return XQ_ERR_ARG;
@@ -714,14 +786,15 @@ int chunk_impl(xq_cache* c, int layer, const void* q, void* out, int n, int out_
   if (n < 1 || n > S) return XQ_ERR_ARG;
   if (((uintptr_t)q & 15) || ((uintptr_t)out & 15)) return XQ_ERR_ARG;
   const Dims& dm = c->plan.dm;
+  bool use_mma;
   // everything that can be refused is the same for every token: check the first and the last before any launch
   {
     DecodeParams p;
-    bool use_mma;
     int rc = prepare_decode(c, layer, q, out, out_f32, nullptr, nullptr, S, p, use_mma, S - n + 1);
     if (rc == XQ_OK) rc = prepare_decode(c, layer, q, out, out_f32, nullptr, nullptr, S, p, use_mma, S);
     if (rc != XQ_OK) return rc;
   }
+  if (use_mma && n > 1) return launch_chunk(c, layer, q, out, n, out_f32, (cudaStream_t)stream);
   const size_t row = (size_t)dm.B * dm.Hq * dm.D;  // elements of one token's queries: [batch, heads, head_dim]
   bool chain = false;  // launches after the first read what the first one waited for and write their own rows
   for (int j = 0; j < n; ++j) {

@@ -569,6 +569,42 @@ def test_attention_chunk(T, shape, kernel):
     cache.close()
 
 
+@pytest.mark.parametrize("shape", [
+    # (D, Hq, Hkv, B, g, R, kq, vq, S, T, f16): whole prompts, pieces, ragged rows, one to many row tiles and splits
+    (128, 4, 1, 1, 32, 128, 2, 0, 2, 2, False),         # nothing quantized yet
+    (128, 8, 8, 2, 32, 64, 2, 2, 129, 129, False),      # a whole prompt; 64-token tiles that end in the middle
+    (128, 5, 1, 1, 64, 64, 0, 2, 1500, 77, True),       # groups of five heads, 1-bit keys, groups of 64, fp16
+    (128, 8, 2, 1, 32, 32, 2, 0, 3000, 33, False),      # splits
+    (128, 16, 2, 3, 32, 256, 2, 2, 2200, 300, False),   # 128-row tiles, a window of several tiles
+    (128, 3, 3, 1, 64, 128, 2, 0, 700, 5, True),        # 15 rows
+    (64, 6, 2, 2, 32, 96, 0, 0, 500, 130, False),       # head_dim 64, all 1-bit, a last tile of 32 tokens
+    (64, 8, 1, 1, 64, 64, 2, 2, 1000, 1000, True),
+])
+def test_attention_chunk_tiles(shape):
+    """Chunks over the edges of the chunk kernel's tiles against the scalar kernel on the same cache (which the oracle
+    checks elsewhere), with outlier key channels and small inputs: each side is within the usual bound of the oracle."""
+    D, Hq, Hkv, B, g, R, kq, vq, S, T, f16 = shape
+    w = dict(n_layers=2, batch=B, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=D, seq=S, residual_len=R, group_size=g,
+             kq=kq, vq=vq, km=0, vm=0, n_outliers=3, outlier_scale=10.0, seed=51, n_splits=0)
+    dt = torch.float16 if f16 else torch.bfloat16
+    for scale in (1.0, 2.0 ** -11):
+        outs = []
+        for kernel in (xq.XQ_KERNEL_AUTO, xq.XQ_KERNEL_GENERIC):
+            cache = xq.Cache(W.make_xq_config(w, kernel=kernel, io_dtype=int(f16)), DEV)
+            for l, (K, V) in enumerate(zip(*[iter(W.pair_tokens(w, 0, 0, S, DEV))] * 2)):
+                cache.append_kv(l, (K.float() * scale).to(dt), (V.float() * scale).to(dt))
+            gen = torch.Generator(device="cpu").manual_seed(T)
+            q = (torch.randn(T, B, Hq, D, generator=gen) / scale ** 0.5).to(dt).to(DEV)
+            outs.append([cache.attention_chunk(l, q, f32=True) for l in (0, 1)] + [cache.attention_chunk(1, q)])
+            torch.cuda.synchronize()
+            cache.check_device()
+            cache.close()
+        for a, b in zip(*outs):
+            # 16-bit results: both sides are rounded, each by at most half a bf16 ulp <= 2^-8 |x|: 2^-7 |x| together
+            bound = util.ATTN_TOL * scale + (2.0 ** -7 * b.abs().float() if a.dtype != torch.float32 else 0.0)
+            assert ((a.float() - b.float()).abs() <= bound).all(), (a.float() - b.float()).abs().max().item()
+
+
 @pytest.mark.parametrize("bits", [(2, 2), (2, 0), (0, 0)])
 def test_delta_histogram(bits):
     """The pack kernel's optional statistic (Section 3.3.1): per layer and cache kind the elements by
