@@ -1,20 +1,22 @@
 // Attention of a chunk of query tokens over the packed cache plus the window, causal inside the chunk: the query rows
-// (tokens x heads of a kv head) share one pass over the cache.
+// (tokens x heads of a kv head) share one pass over the cache.  tcgen05 products.
 //
-// A CTA takes M = 16 WR rows and a range of 64-token tiles of one (sequence, kv head).  With M rows per code it pays
-// to dequantize: four warps expand the keys of a tile and four its values, once for all rows, into fp16 pairs
-// hi + lo in shared memory (22 significant bits of c s + z, relative to the group's largest member), and the products
-// are q hi + q lo for the logits and p_hi v_hi + p_hi v_lo + p_lo v_hi for the result, p_hi + p_lo the softmax
-// numerators as fp16 pairs, accumulation in fp32.  The tile after the current one is expanded while the current one
-// is multiplied: of the two warps that share a sub-partition one expands before its products, the other after them.
-// The eight warps are WR row groups of 16 rows times WT = 8 / WR parts of a tile's tokens.  Window tiles are 16-bit
-// already and are multiplied as they are (bf16 or fp16 products, numerators as pairs of that type).
-// Split partials are merged by the last CTA of a row tile, as in the decode kernel.
+// A CTA takes 128 rows and a range of 64-token tiles of one (sequence, kv head).  With that many rows per code it pays
+// to dequantize: eight warps expand a tile's keys and values once for all rows into fp16 pairs hi + lo in shared
+// memory (22 significant bits of c s + z, relative to the largest member of the group), the B operands of
 //
-// What bounds it: the rate of mma.sync (8 cycles per m16n8k16 and sub-partition here), five products for every
-// (row, token, channel) instead of the two that plain fp16 attention takes.  One decode launch per query token before:
-// 16 tokens at 32k context, batch 4 and 8 kv heads 508 -> 451 us per layer, 250 tokens at 8k 1308 -> 501 us, a whole
-// prompt of 1024 tokens, 32 heads 2470 -> 134 us.
+//   S = Q K_hi + Q K_lo                          (A: q as fp16 in tensor memory; S: 64 columns, two buffers)
+//   O += P_hi V_hi + P_hi V_lo + P_lo V_hi       (A: the softmax numerators as fp16 pairs, over the columns of S)
+//
+// accumulated in fp32 in tensor memory.  Two groups of four warps (thread = row = tensor-memory lane) take the softmax
+// of the even and of the odd tiles; the softmax reference of a row goes from one to the other through shared memory
+// and is raised only when a logit exceeds it by more than 8 (log2 units), which rescales O (rare).  One warp issues the products: keys of tile i + 1,
+// then values of tile i.  Tokens of the 16-bit window are expanded into the same pairs (exactly).  Split partials are
+// merged by the last CTA of a row tile, as in the decode kernel.
+//
+// Every wait on an mbarrier is bounded: a thread that gives up sets a flag in shared memory that makes every other
+// wait of the CTA give up too; the CTA then waits for its products in flight, frees its tensor memory, reports through
+// the status word and leaves without a result.
 #pragma once
 #include <type_traits>
 
@@ -24,27 +26,83 @@
 namespace xq {
 namespace {
 
+constexpr int CM = CHUNK_ROWS;     // query rows of a CTA
 constexpr int CT = 64;             // tokens of a tile
 constexpr int C_STAGES = 3;        // raw tiles in flight
-constexpr float C_TAU = 3.f;       // log2 units a logit may exceed the softmax reference before it is raised
-constexpr int C_PEXP = 11;         // numerators are carried times 2^C_PEXP
+constexpr float C_TAU = 8.f;       // log2 units a logit may exceed the softmax reference before it is raised
+constexpr int C_PEXP = 6;          // numerators are carried times 2^C_PEXP (at most 2^14 as fp16)
+constexpr int C_EXPAND = 8;        // expanding warps (8 .. 15): keys 0 .. 3, values 4 .. 7
+constexpr int C_THREADS = (8 + C_EXPAND + 1) * 32;
 
-template <int D, int BK, int BV, int GS, int WR>
+// ---- tensor memory and tcgen05 ----
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
+__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
+      "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};\n" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]),
+      "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
+      "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
+      "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr) : "memory");
+}
+// shared-memory matrix descriptor, K-major, no swizzle: core matrices of 8 rows x 16 bytes;
+// lbo / sbo: byte distance between core matrices along K / along the rows
+__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
+  uint64_t d = 0;
+  d |= (uint64_t)((addr >> 4) & 0x3fff);
+  d |= (uint64_t)((lbo >> 4) & 0x3fff) << 16;
+  d |= (uint64_t)((sbo >> 4) & 0x3fff) << 32;
+  d |= (uint64_t)1 << 46;  // descriptor version of this architecture
+  return d;
+}
+// kind::f16 instruction descriptor: fp16 A and B (both K-major), fp32 accumulate, M = 128
+__host__ __device__ constexpr uint32_t idesc_f16(int n) {
+  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+}
+// D[128 x N] (+)= A[128 x 16] (tensor memory) * B[16 x N] (shared memory); issued by one thread
+__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, bool accumulate) {
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ne.b32 p, %5, 0;\n"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%4,%4,%4,%4}, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(0u), "r"((uint32_t)accumulate) : "memory");
+}
+__device__ __forceinline__ void umma_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t pred;
+  asm volatile("{\n.reg .pred P;\nelect.sync _|P, 0xffffffff;\nselp.u32 %0, 1, 0, P;\n}\n" : "=r"(pred));
+  return pred;
+}
+
+template <int D, int BK, int BV, int GS>
 struct ChunkPlan {
-  static constexpr int M = 16 * WR, WT = 8 / WR, TW = CT / WT;  // rows; token parts; tokens of a warp
   static constexpr int NG = D / GS;
-  static constexpr int QROW = 2 * D + 16;                       // a staged row of q
   static constexpr int KROW = D * BK / 8;                       // packed bytes of a token's keys
   static constexpr int MAT = CT * 2 * D;                        // one matrix of a tile: K hi, K lo, V hi, V lo
   static constexpr int BUF = 4 * MAT;
-  static constexpr int RAW_K = 16 * KROW + 4 * D;               // a key warp's codes and parameters
-  static constexpr int RAW_VC = (D / 4) * 8 * BV, RAW_V = RAW_VC + CT * 4 * NG;
+  static constexpr int K_SBO = 16 * D, V_SBO = 16 * CT;         // eight rows of the keys (tokens) / of the values (channels)
+  static constexpr int RAW_KC = 32 * KROW, RAW_K = RAW_KC + 4 * D;  // a key warp's codes (32 tokens) and parameters
+  static constexpr int RAW_VC = (D / 4) * 8 * BV, RAW_V = RAW_VC + 4 * (64 * NG + 16);
   static constexpr int RAW = RAW_K > RAW_V ? RAW_K : RAW_V;     // of one warp and stage
   static constexpr int OFF_RAW = 2 * BUF;
-  static constexpr int OFF_Q = OFF_RAW + 8 * C_STAGES * RAW;
-  static constexpr int TOTAL = OFF_Q + M * QROW;
-  static constexpr int MS = D + 4;                              // state row: acc[D], m, l
-  static_assert(8 * 16 * MS * 4 <= 2 * BUF, "the warps' states fit the tile buffers");
+  static constexpr int TOTAL = OFF_RAW + C_EXPAND * C_STAGES * RAW;
+  // tensor memory columns: q, S and numerators of even and odd tiles, O
+  static constexpr uint32_t COL_Q = 0, COL_S = 64, COL_O = 192;
   static_assert(TOTAL <= 226 * 1024, "shared memory");
 };
 
@@ -53,6 +111,12 @@ __device__ __forceinline__ void chunk_store(const ChunkParams& p, size_t row, in
   if (p.out_f32) reinterpret_cast<float*>(p.out)[row * D + c] = v;
   else if (p.f16) reinterpret_cast<__half*>(p.out)[row * D + c] = __float2half_rn(v);
   else reinterpret_cast<__nv_bfloat16*>(p.out)[row * D + c] = __float2bfloat16_rn(v);
+}
+
+// hi = RN16(v), lo = RN16(v - hi) of a pair
+__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
+  hi = pack_io2<true>(a, b);
+  lo = pack_io2<true>(a - io2_lo<true>(hi), b - io2_hi<true>(hi));
 }
 
 // 16 codes of a packed word (`w` shifted so that the codes 4 e + j sit at bit BITS * e of byte j) with the parameters
@@ -69,493 +133,523 @@ __device__ __forceinline__ void expand16(uint32_t w, const float (&s)[16], const
       const float c = __uint_as_float(__byte_perm(m, 0x4B000000u, 0x7440 + j)) - 8388608.f;  // 2^23 + code, less 2^23
       v[j] = fmaf(c, s[4 * e + j], z[4 * e + j]);
     }
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const uint32_t h = pack_io2<true>(v[2 * j], v[2 * j + 1]);
-      hi[2 * e + j] = h;
-      lo[2 * e + j] = pack_io2<true>(v[2 * j] - io2_lo<true>(h), v[2 * j + 1] - io2_hi<true>(h));
-    }
+    split2(v[0], v[1], hi[2 * e], lo[2 * e]);
+    split2(v[2], v[3], hi[2 * e + 1], lo[2 * e + 1]);
   }
 }
-
-// x[0 .. 15] *= f
+__device__ __forceinline__ void store16(uint32_t a, uint32_t lbo, uint32_t mat, const uint32_t (&hi)[8], const uint32_t (&lo)[8]) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {  // the two 16-byte pieces of 16 elements, of the hi and of the lo matrix
+    sts128(a + i * lbo, hi[4 * i], hi[4 * i + 1], hi[4 * i + 2], hi[4 * i + 3]);
+    sts128(a + i * lbo + mat, lo[4 * i], lo[4 * i + 1], lo[4 * i + 2], lo[4 * i + 3]);
+  }
+}
 __device__ __forceinline__ void scale16(float (&x)[16], float f) {
 #pragma unroll
   for (int k = 0; k < 16; ++k) x[k] *= f;
 }
 
-template <int D, int BK, int BV, int GS, int WR>
-__global__ void __launch_bounds__(256, 1) chunk_kernel(const __grid_constant__ ChunkParams p) {
-  using Pl = ChunkPlan<D, BK, BV, GS, WR>;
-  constexpr int M = Pl::M, WT = Pl::WT, TW = Pl::TW, NG = Pl::NG, KS = D / 16, NT = TW / 8, NO = D / 8;
-  constexpr int QT = D / 32;  // output tiles of 8 channels in a quarter of the channels
+template <int D, int BK, int BV, int GS>
+__global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_constant__ ChunkParams p) {
+  using Pl = ChunkPlan<D, BK, BV, GS>;
+  constexpr int NG = Pl::NG, DQ = D / 4;
   extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ float k_unit[2][4];  // [buffer][16 tokens]: what a unit of the expanded keys is worth
-  __shared__ int v_exp[2][4];     // [buffer][channel quarter]: the expanded values are times 2^v_exp
+  __shared__ __align__(8) unsigned long long bar_mem[18];
+  __shared__ float k_unit[4][2];            // [tile % 4][32 tokens]: what a unit of the expanded keys is worth
+  __shared__ int v_exp[4][4];               // [tile % 4][channel quarter]: the expanded values are times 2^v_exp
+  __shared__ float cq_sm[CM], m_sm[CM];     // logits from products of the scaled q; softmax reference (-infinity: none)
+  __shared__ float l_sm[2][CM], ml_sm[2][CM];
+  __shared__ uint32_t tmem_base_sm;
   __shared__ int s_flag;
+  __shared__ volatile int dead_sm;
 
   const Dims& dm = p.dm;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
-  const int wr = warp % WR, wt = warp / WR;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int G = dm.G, n_streams = dm.B * dm.Hkv;
   // the row tiles with the most visible tokens first
   const int split = blockIdx.x % p.ns, bh = (blockIdx.x / p.ns) % n_streams, rt = p.row_tiles - 1 - blockIdx.x / p.ns / n_streams;
   const int hk = bh % dm.Hkv, b = bh / dm.Hkv;
-  const int row0 = rt * M, n_rows = min(M, p.T * G - row0);  // row: query token row / G, head row % G
-  const int vis0 = p.S - p.T + 1;                            // tokens that query token 0 sees
-  const int vis_max = vis0 + (row0 + n_rows - 1) / G, vis_min = vis0 + row0 / G;
+  const int row0 = rt * CM, n_rows = min(CM, p.T * G - row0);  // row: query token row / G, head row % G
+  const int vis0 = p.S - p.T + 1;                              // tokens that query token 0 sees
+  const int vis_max = vis0 + (row0 + n_rows - 1) / G;
   const int n_packed = min(p.n_q, vis_max);
   const int pk_tiles = (n_packed + CT - 1) / CT, all_tiles = pk_tiles + (vis_max - n_packed + CT - 1) / CT;
   int t_lo, t_hi;
   share_of(all_tiles, p.ns, split, t_lo, t_hi);
+  const int N = t_hi - t_lo;
 
   const uint32_t sm = (uint32_t)__cvta_generic_to_shared(smem);
-  const uint32_t raw = sm + Pl::OFF_RAW + warp * C_STAGES * Pl::RAW, qs = sm + Pl::OFF_Q;
-  const uint8_t* const g_kc = reinterpret_cast<const uint8_t*>(p.L.k_codes) + (size_t)bh * ((size_t)dm.nq_cap * Pl::KROW);
-  const uint8_t* const g_km = reinterpret_cast<const uint8_t*>(p.L.k_meta) + (size_t)bh * ((size_t)(dm.nq_cap / GS) * 4 * D);
-  const uint8_t* const g_vc = reinterpret_cast<const uint8_t*>(p.L.v_codes) + (size_t)bh * ((size_t)dm.nq_cap * (D * BV / 8));
-  const uint8_t* const g_vm = reinterpret_cast<const uint8_t*>(p.L.v_meta) + (size_t)bh * ((size_t)dm.nq_cap * 4 * NG);
+  const uint32_t bars = (uint32_t)__cvta_generic_to_shared(&bar_mem[0]);
+  const uint32_t bar_kfull = bars;             // [2] a tile is expanded
+  const uint32_t bar_free = bar_kfull + 16;    // [2] its buffer may be written again
+  const uint32_t bar_s = bar_free + 16;        // [2] S is complete
+  const uint32_t bar_p = bar_s + 16;           // [2] the numerators are written
+  const uint32_t bar_o = bar_p + 16;           // the value products of a tile are complete
+  const uint32_t bar_turn = bar_o + 8;         // [4 warps][2] a row's reference for an even / odd tile is there
+  const uint32_t bar_end = bar_turn + 64;      // every product that was issued is complete (after a wait gave up)
 
-  // Raw data of tile `t` that this warp expands, into its own stage; one commit per call (empty beyond the last tile).
-  // Warps 0..3: keys of 16 tokens each; warps 4..7: values of D / 4 channels each.
-  auto fetch = [&](int t) {
-    if (t < min(t_hi, pk_tiles)) {
-      const uint32_t dst = raw + (t % C_STAGES) * Pl::RAW;
-      if (warp < 4) {
-        const int tok = t * CT + 16 * warp;
-        const uint8_t* src = g_kc + (size_t)(tok / 32) * (32 * Pl::KROW);
-        if (lane < Pl::KROW) {  // 16 tokens x KROW bytes in 16-byte pieces
-          if constexpr (Pl::KROW == 32) cp_async16(dst + lane * 16, src + (lane >> 4) * 512 + (tok % 32 + (lane & 15)) * 16);
-          else cp_async16(dst + lane * 16, src + (tok % 32) * Pl::KROW + lane * 16);
-        }
-        if (lane < D / 4) cp_async16(dst + 16 * Pl::KROW + lane * 16, g_km + (size_t)(tok / GS) * (4 * D) + lane * 16);
-      } else {
-        const int c0 = (warp - 4) * (D / 4);
-        const uint8_t* src = g_vc + (size_t)(t / 2) * (D * 16 * BV);
-        if (lane < D / 4) {
-          if constexpr (BV == 2) cp_async16(dst + lane * 16, src + (t & 1) * (D * 16) + (c0 + lane) * 16);
-          else cp_async8(dst + lane * 8, src + (c0 + lane) * 16 + (t & 1) * 8);
-        }
-        for (int i = lane; i < CT * 4 * NG / 16; i += 32)
-          cp_async16(dst + Pl::RAW_VC + i * 16, g_vm + (size_t)t * (CT * 4 * NG) + i * 16);
-      }
+  if (tid == 0) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(bar_kfull + 8 * i, C_EXPAND);
+      mbar_init(bar_free + 8 * i, 1);
+      mbar_init(bar_s + 8 * i, 1);
+      mbar_init(bar_p + 8 * i, 4);
     }
-    cp_async_commit();
-  };
-
-  int ev_mine = 0;        // value warps: exponent in use for this warp's channels
-  bool ev_set = false;
-  // Expands this warp's part of tile `t` into buffer `buf`.  nq % 32 == 0, so 16 tokens exist or do not together.
-  auto expand = [&](int t, int buf) {
-    const uint32_t src = raw + (t % C_STAGES) * Pl::RAW, dst = sm + buf * Pl::BUF;
-    float s[16], z[16];
-    if (warp < 4) {
-      constexpr int NU = D / 16, NS = 32 / NU;  // lanes: NU units of 16 channels, NS tokens
-      const int u = lane % NU, sub = lane / NU;
-      const bool exists = t * CT + 16 * warp < p.n_q;
-      float mx = 0.f;
+    mbar_init(bar_o, 1);
+    mbar_init(bar_end, 1);
 #pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const int d = 16 * u + k, pos = (d % 32) * (D / 32) + d / 32;
-        s[k] = exists ? f16_to_f(lds16(src + 16 * Pl::KROW + 2 * pos)) : 0.f;
-        z[k] = exists ? f16_to_f(lds16(src + 16 * Pl::KROW + 2 * D + 2 * pos)) : 0.f;
-        mx = fmaxf(mx, fmaf((float)((1 << BK) - 1), s[k], fabsf(z[k])));
-      }
-      mx = __uint_as_float(redux_max_u32(__float_as_uint(mx)));
-      const int e = mx > 0.f ? 14 - exponent_of(mx) : 0;  // the largest |k| of the tokens' group below 2^15
-      const float f = pow2i(e);
-      if (lane == 0) k_unit[buf][warp] = pow2i(-e);
-      scale16(s, f);
-      scale16(z, f);
-#pragma unroll
-      for (int k = 0; k < 16 / NS; ++k) {
-        const int tl = sub + NS * k, tok = 16 * warp + tl;
-        uint32_t w;
-        if constexpr (BK == 2) w = lds32(src + (Pl::KROW == 32 ? (u >> 2) * 256 : 0) + tl * 16 + (u & 3) * 4);
-        else w = lds32(src + tl * Pl::KROW + (u >> 1) * 4) >> (4 * (u & 1));
-        uint32_t hi[8], lo[8];
-        expand16<BK>(w, s, z, hi, lo);
-        const uint32_t row = dst + tok * 2 * D;
-        // 16 channels: the 16-byte pieces 2 u and 2 u + 1, the second one first in the upper half of the row (banks)
-        const bool swap = u >= 4;
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const int piece = 2 * u + (swap ? 1 - i : i);
-          const uint32_t a = row + (piece ^ (tok & 7)) * 16;
-          const bool up = swap != (i == 1);
-          sts128(a, up ? hi[4] : hi[0], up ? hi[5] : hi[1], up ? hi[6] : hi[2], up ? hi[7] : hi[3]);
-          sts128(a + Pl::MAT, up ? lo[4] : lo[0], up ? lo[5] : lo[1], up ? lo[6] : lo[2], up ? lo[7] : lo[3]);
-        }
-      }
-    } else {
-      const int u = lane & 3, sub = lane >> 2;  // 16 tokens; channel
-      const int c0 = (warp - 4) * (D / 4), gi = c0 / GS;
-      const bool exists = t * CT + 16 * u < p.n_q;
-      float mx = 0.f;
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const uint32_t a = src + Pl::RAW_VC + (16 * u + k) * 4 * NG + 2 * gi;
-        s[k] = exists ? f16_to_f(lds16(a)) : 0.f;
-        z[k] = exists ? f16_to_f(lds16(a + 2 * NG)) : 0.f;
-        mx = fmaxf(mx, fmaf((float)((1 << BV) - 1), s[k], fabsf(z[k])));
-      }
-      mx = __uint_as_float(redux_max_u32(__float_as_uint(mx)));
-      const int em = mx > 0.f ? exponent_of(mx) : -30;
-      // the largest |v| times 2^ev_mine in [2^6, 2^14): the exponent moves only outside that
-      if (!ev_set || em + ev_mine > 13 || (em + ev_mine < 6 && em > -30)) {
-        ev_mine = 13 - em;
-        ev_set = true;
-      }
-      const float f = pow2i(ev_mine);
-      if (lane == 0) v_exp[buf][warp - 4] = ev_mine;
-      scale16(s, f);
-      scale16(z, f);
-#pragma unroll
-      for (int k = 0; k < D / 32; ++k) {
-        const int cl = sub + 8 * k, c = c0 + cl;
-        uint32_t w;
-        if constexpr (BV == 2) w = lds32(src + cl * 16 + u * 4);
-        else w = lds32(src + cl * 8 + (u >> 1) * 4) >> (4 * (u & 1));
-        uint32_t hi[8], lo[8];
-        expand16<BV>(w, s, z, hi, lo);
-        const uint32_t row = dst + 2 * Pl::MAT + c * (2 * CT);  // [channel][token]
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const uint32_t a = row + ((2 * u + i) ^ (c & 7)) * 16;
-          sts128(a, hi[4 * i], hi[4 * i + 1], hi[4 * i + 2], hi[4 * i + 3]);
-          sts128(a + Pl::MAT, lo[4 * i], lo[4 * i + 1], lo[4 * i + 2], lo[4 * i + 3]);
-        }
-      }
-    }
-  };
-
-  // ---- q: rows as they came (zeros beyond the chunk), then fp16 fragments scaled per row into [1, 2) ----
-  grid_dependency_wait();
-  for (int i = tid; i < M * (D / 8); i += 256) {
-    const int r = i / (D / 8), c = i % (D / 8);
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (r < n_rows) {
-      const int row = row0 + r, j = row / G, h = row - j * G;
-      v = reinterpret_cast<const uint4*>(p.q + (((size_t)j * dm.B + b) * dm.Hq + hk * G + h) * D)[c];
-    }
-    sts128(qs + r * Pl::QROW + c * 16, v.x, v.y, v.z, v.w);
+    for (int i = 0; i < 8; ++i) mbar_init(bar_turn + 8 * i, 1);
+    dead_sm = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  fetch(t_lo);
-  fetch(t_lo + 1);
+  if (warp == 8 + C_EXPAND) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(&tmem_base_sm)), "r"(512u) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+  }
+  tc_fence_before();
   __syncthreads();
-  const float scale2 = p.scale * 1.4426950408889634f;
-  uint32_t qf[KS][4];
-  float cq[2];  // logits of rows gid, gid + 8 from products of the scaled q
-  int vis[2];   // tokens that these rows see
-  {
-    const uint32_t qa = qs + (16 * wr + gid) * Pl::QROW + tig * 4;
-    float am[2] = {0.f, 0.f};
+  tc_fence_after();
+  const uint32_t tbase = tmem_base_sm;
+  const uint32_t row_t = tbase + ((uint32_t)((warp & 3) * 32) << 16);
+  grid_dependency_wait();
+
+  if (warp < 4) {
+    // ---- q: this thread's row as fp16 scaled by a power of two into [1, 2), to tensor memory ----
+    const int row = row0 + tid, j = row / G, h = row - j * G;
+    const bool real = tid < n_rows;
+    const uint4* src = reinterpret_cast<const uint4*>(p.q + (real ? (((size_t)j * dm.B + b) * dm.Hq + hk * G + h) * D : 0));
+    uint32_t w[D / 2];
+    float am = 0.f;
 #pragma unroll
-    for (int ks = 0; ks < KS; ++ks)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {  // a0: row gid, a1: row gid + 8; a2, a3: 8 channels on
-        qf[ks][k] = lds32(qa + (k & 1) * 8 * Pl::QROW + ks * 32 + (k >> 1) * 16);
-        am[k & 1] = fmaxf(am[k & 1], fmaxf(fabsf(io_to_f(qf[ks][k] & 0xffffu, p.f16)), fabsf(io_to_f(qf[ks][k] >> 16, p.f16))));
-      }
-    float f[2];
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      am[r] = fmaxf(am[r], __shfl_xor_sync(0xffffffffu, am[r], 1));
-      am[r] = fmaxf(am[r], __shfl_xor_sync(0xffffffffu, am[r], 2));
-      const int e = am[r] > 0.f ? max(-100, min(100, -exponent_of(am[r]))) : 0;
-      f[r] = pow2i(e);
-      cq[r] = scale2 * pow2i(-e);
-      vis[r] = min(vis0 + (row0 + 16 * wr + gid + 8 * r) / G, vis_max);
+    for (int i = 0; i < D / 8; ++i) {
+      const uint4 v = real ? src[i] : make_uint4(0u, 0u, 0u, 0u);
+      w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
     }
 #pragma unroll
-    for (int ks = 0; ks < KS; ++ks)
+    for (int i = 0; i < D / 2; ++i)
+      am = fmaxf(am, fmaxf(fabsf(io_to_f(w[i] & 0xffffu, p.f16)), fabsf(io_to_f(w[i] >> 16, p.f16))));
+    const int e = am > 0.f ? max(-100, min(100, -exponent_of(am))) : 0;
+    const float f = pow2i(e);
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        qf[ks][k] = pack_io2<true>(io_to_f(qf[ks][k] & 0xffffu, p.f16) * f[k & 1], io_to_f(qf[ks][k] >> 16, p.f16) * f[k & 1]);
+    for (int c = 0; c < D / 64; ++c) {
+      uint32_t r[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i)
+        r[i] = pack_io2<true>(io_to_f(w[32 * c + i] & 0xffffu, p.f16) * f, io_to_f(w[32 * c + i] >> 16, p.f16) * f);
+      tmem_st32(row_t + Pl::COL_Q + 32 * c, r);
+    }
+    tc_wait_st();
+    cq_sm[tid] = p.scale * 1.4426950408889634f * pow2i(-e);
+    m_sm[tid] = -CUDART_INF_F;
   }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
 
-  // softmax state of rows gid, gid + 8: reference (log2 units; 0 and `set` false before the first visible token)
-  float mr[2] = {0.f, 0.f}, l[2] = {0.f, 0.f}, o[NO][4];
-  bool set[2] = {false, false};
-  int ev[4] = {0, 0, 0, 0};  // the result of channel quarter i is held times 2^ev[i]
+  if (warp == 8 + C_EXPAND) {
+    // ================= products: the loop is warp-uniform, one elected lane issues =================
+    constexpr uint32_t IDK = idesc_f16(CT), IDV = idesc_f16(D);
+    for (int i = 0; i <= N; ++i) {
+      bool ok = true;
+      if (i < N) {
+        ok = __all_sync(0xffffffffu, mbar_wait(bar_kfull + 8 * (i & 1), (i >> 1) & 1, &dead_sm));
+        tc_fence_after();
+        if (ok && elect_one()) {
+          const uint32_t base = sm + (i & 1) * Pl::BUF, dS = tbase + Pl::COL_S + (i & 1) * 64;
+          const uint64_t kh = smem_desc(base, 128, Pl::K_SBO), kl = smem_desc(base + Pl::MAT, 128, Pl::K_SBO);
 #pragma unroll
-  for (int n = 0; n < NO; ++n)
+          for (int ks = 0; ks < D / 16; ++ks) {
+            umma_f16(dS, tbase + Pl::COL_Q + 8 * ks, kh + 16 * ks, IDK, ks > 0);
+            umma_f16(dS, tbase + Pl::COL_Q + 8 * ks, kl + 16 * ks, IDK, true);
+          }
+          umma_commit(bar_s + 8 * (i & 1));
+        }
+        __syncwarp();
+      }
+      if (ok && i > 0) {
+        const int j = i - 1;
+        ok = __all_sync(0xffffffffu, mbar_wait(bar_p + 8 * (j & 1), (j >> 1) & 1, &dead_sm));
+        tc_fence_after();
+        if (ok && elect_one()) {
+          const uint32_t base = sm + (j & 1) * Pl::BUF + 2 * Pl::MAT;
+          const uint32_t ph = tbase + Pl::COL_S + (j & 1) * 64, pl = ph + 32, dO = tbase + Pl::COL_O;
+          const uint64_t vh = smem_desc(base, 128, Pl::V_SBO), vl = smem_desc(base + Pl::MAT, 128, Pl::V_SBO);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) o[n][k] = 0.f;
-
-  // Logits s (log2 units) of tokens t0 + 8 n + 2 tig (+ 1), rows gid and gid + 8, into numerators times 2^C_PEXP; tokens
-  // from `end` on do not exist.
-  auto softmax = [&](float (&s)[NT][4], int t0, int end, bool masked) {
-    if (masked) {
-#pragma unroll
-      for (int n = 0; n < NT; ++n)
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (t0 + 8 * n + 2 * tig + (k & 1) >= min(vis[k >> 1], end)) s[n][k] = -CUDART_INF_F;
+          for (int ks = 0; ks < CT / 16; ++ks) {
+            umma_f16(dO, ph + 8 * ks, vh + 16 * ks, IDV, j > 0 || ks > 0);
+            umma_f16(dO, ph + 8 * ks, vl + 16 * ks, IDV, true);
+            umma_f16(dO, pl + 8 * ks, vh + 16 * ks, IDV, true);
+          }
+          umma_commit(bar_o);
+          umma_commit(bar_free + 8 * (j & 1));
+        }
+        __syncwarp();
+      }
+      if (!ok) break;
     }
-    float mx[2] = {-CUDART_INF_F, -CUDART_INF_F};
+    if (__any_sync(0xffffffffu, dead_sm != 0)) {  // products may be in flight: wait for them (bounded) before the memory they use is given up
+      if (elect_one()) {
+        umma_commit(bar_end);
+        for (int k = 0; k < WAIT_LIMIT && !mbar_try_wait(bar_end, 0); ++k) {}
+      }
+      __syncwarp();
+    }
+  } else if (warp < 8) {
+    // ================= softmax: group w takes the tiles i = w, w + 2, ...; thread = row =================
+    const int w = warp >> 2, q = warp & 3, r = tid & 127;
+    const bool idle = 32 * q >= n_rows;  // none of this warp's rows exists: its lanes hold whatever is there
+    const float cq = cq_sm[r];
+    const int vis = min(vis0 + (row0 + r) / G, vis_max);
+    float l = 0.f, ml = -CUDART_INF_F;
+    for (int i = w; i < N; i += 2) {
+      // (the expansion's exponents are there since the first of the two; the second one is the wait)
+      if (!__all_sync(0xffffffffu, mbar_wait(bar_kfull + 8 * (i & 1), (i >> 1) & 1, &dead_sm) &&
+                                       mbar_wait(bar_s + 8 * (i & 1), (i >> 1) & 1, &dead_sm)))
+        break;
+      tc_fence_after();
+      const uint32_t s_t = row_t + Pl::COL_S + (i & 1) * 64;
+      uint32_t s[2][32];
+      float m = -CUDART_INF_F;
+      const float u0 = k_unit[i & 3][0] * cq, u1 = k_unit[i & 3][1] * cq;
+      const int t = t_lo + i;
+      // columns below n_valid are tokens that exist and that this row sees
+      const int n_valid = t < pk_tiles ? min(vis, p.n_q) - t * CT : vis - p.n_q - (t - pk_tiles) * CT;
+      if (!idle) {
+        tmem_ld32(s_t, s[0]);
+        tmem_ld32(s_t + 32, s[1]);
+        tc_wait_ld();
+        const bool masked = __any_sync(0xffffffffu, n_valid < CT);
+        if (masked) {
 #pragma unroll
-    for (int n = 0; n < NT; ++n)
+          for (int k = 0; k < 64; ++k)
+            if (k >= n_valid) s[k / 32][k % 32] = 0xff800000u;
+        }
+        float x0 = -CUDART_INF_F, x1 = -CUDART_INF_F;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) mx[k >> 1] = fmaxf(mx[k >> 1], s[n][k]);
-    bool need = false;
+        for (int k = 0; k < 32; ++k) {
+          x0 = fmaxf(x0, __uint_as_float(s[0][k]));
+          x1 = fmaxf(x1, __uint_as_float(s[1][k]));
+        }
+        const float xm = fmaxf(x0 * u0, x1 * u1);
+        if (i > 0 && !__all_sync(0xffffffffu, mbar_wait(bar_turn + 8 * (2 * q + (i & 1)), ((i - 1) >> 1) & 1, &dead_sm))) break;
+        const float m_old = m_sm[r];
+        m = m_old;
+        if (xm > m_old + C_TAU || (m_old == -CUDART_INF_F && xm > m_old)) m = ceilf(xm);
+        bool change = m != m_old;
+        float ef[4];
 #pragma unroll
-    for (int r = 0; r < 2; ++r) need |= set[r] ? mx[r] > mr[r] + C_TAU : mx[r] > -CUDART_INF_F;
-    if (__any_sync(0xffffffffu, need)) {
+        for (int k = 0; k < 4; ++k) {
+          ef[k] = i > 0 ? pow2i(v_exp[i & 3][k] - v_exp[(i - 1) & 3][k]) : 1.f;
+          change |= ef[k] != 1.f;
+        }
+        if (__any_sync(0xffffffffu, change)) {
+          m_sm[r] = m;
+          if (i > 0) {  // O has to follow: after the products of the tile before, before those of this one
+            if (!__all_sync(0xffffffffu, mbar_wait(bar_o, (i - 1) & 1, &dead_sm))) break;
+            tc_fence_after();
+            const float f = m_old == -CUDART_INF_F ? 0.f : ex2(m_old - m);
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        float v = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
-        v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 2));
-        if (v > -CUDART_INF_F && (!set[r] || v > mr[r] + (C_TAU - 1.f))) {
-          const float mn = ceilf(v), f = set[r] ? ex2(mr[r] - mn) : 0.f;
-          mr[r] = mn;
-          set[r] = true;
-          l[r] *= f;
+            for (int c = 0; c < D; c += 32) {
+              tmem_ld32(row_t + Pl::COL_O + c, s[0]);
+              tc_wait_ld();
 #pragma unroll
-          for (int n = 0; n < NO; ++n) {
-            o[n][2 * r] *= f;
-            o[n][2 * r + 1] *= f;
+              for (int k = 0; k < 32; ++k) s[0][k] = __float_as_uint(__uint_as_float(s[0][k]) * (f * ef[(c + k) / DQ]));
+              tmem_st32(row_t + Pl::COL_O + c, s[0]);
+            }
+            tc_wait_st();
+          }
+          tmem_ld32(s_t, s[0]);
+          tmem_ld32(s_t + 32, s[1]);
+          tc_wait_ld();
+          if (masked) {
+#pragma unroll
+            for (int k = 0; k < 64; ++k)
+              if (k >= n_valid) s[k / 32][k % 32] = 0xff800000u;
           }
         }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_turn + 8 * (2 * q + ((i + 1) & 1)));
+        // numerators
+        const float off = m == -CUDART_INF_F ? 0.f : (float)C_PEXP - m;
+        l *= m == ml ? 1.f : ex2(ml - m);
+        ml = m;
+        float la = 0.f, lb = 0.f;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const float u = c ? u1 : u0;
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            const float a = ex2(fmaf(__uint_as_float(s[c][2 * k]), u, off)), d = ex2(fmaf(__uint_as_float(s[c][2 * k + 1]), u, off));
+            la += a;
+            lb += d;
+            uint32_t hi, lo;
+            split2(a, d, hi, lo);
+            s[c][2 * k] = hi;
+            s[c][2 * k + 1] = lo;
+          }
+        }
+        l += la + lb;
+        uint32_t o[32];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {  // hi, then lo: two tokens per column
+#pragma unroll
+          for (int k = 0; k < 32; ++k) o[k] = s[k / 16][2 * (k % 16) + h];
+          tmem_st32(s_t + 32 * h, o);
+        }
+        tc_wait_st();
       }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_p + 8 * (i & 1));
     }
-    const float off[2] = {(float)C_PEXP - mr[0], (float)C_PEXP - mr[1]};
-#pragma unroll
-    for (int n = 0; n < NT; ++n)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        s[n][k] = ex2(s[n][k] + off[k >> 1]);
-        l[k >> 1] += s[n][k];
-      }
-  };
-
-  const int x4_row = (lane & 7) + 8 * (lane >> 4), x4_piece = (lane >> 3) & 1;  // ldmatrix: this lane's row and 16-byte piece
-  // products of an expanded tile
-  auto multiply = [&](int t, int buf) {
-    const uint32_t base = sm + buf * Pl::BUF;
-    float s[NT][4];
-#pragma unroll
-    for (int n = 0; n < NT; ++n)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) s[n][k] = 0.f;
-    const int tw = wt * TW;
-#pragma unroll
-    for (int ks = 0; ks < KS; ++ks)
-#pragma unroll
-      for (int n = 0; n < NT; n += 2) {
-        const int tok = tw + 8 * n + x4_row;
-        const uint32_t a = base + tok * 2 * D + ((2 * ks + x4_piece) ^ (tok & 7)) * 16;
-        uint32_t b0, b1, b2, b3, c0, c1, c2, c3;
-        ldmatrix_x4(a, b0, b1, b2, b3);
-        ldmatrix_x4(a + Pl::MAT, c0, c1, c2, c3);
-        mma_f16(s[n], qf[ks][0], qf[ks][1], qf[ks][2], qf[ks][3], b0, b1);
-        mma_f16(s[n + 1], qf[ks][0], qf[ks][1], qf[ks][2], qf[ks][3], b2, b3);
-        mma_f16(s[n], qf[ks][0], qf[ks][1], qf[ks][2], qf[ks][3], c0, c1);
-        mma_f16(s[n + 1], qf[ks][0], qf[ks][1], qf[ks][2], qf[ks][3], c2, c3);
-      }
-#pragma unroll
-    for (int n = 0; n < NT; ++n) {
-      const float u = k_unit[buf][(tw + 8 * n) / 16];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) s[n][k] *= cq[k >> 1] * u;
-    }
-    const int t0 = t * CT + tw;
-    softmax(s, t0, p.n_q, t * CT + CT > min(vis_min, p.n_q));
-    // exponents of the values
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int e = v_exp[buf][i];
-      if (e != ev[i]) {
-        const float f = pow2i(e - ev[i]);
-        ev[i] = e;
-#pragma unroll
-        for (int n = i * QT; n < (i + 1) * QT; ++n)
-#pragma unroll
-          for (int k = 0; k < 4; ++k) o[n][k] *= f;
-      }
-    }
-#pragma unroll
-    for (int kk = 0; kk < TW / 16; ++kk) {
-      uint32_t ph[4], pl[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float x = s[2 * kk + (k >> 1)][2 * (k & 1)], y = s[2 * kk + (k >> 1)][2 * (k & 1) + 1];
-        ph[k] = pack_io2<true>(x, y);
-        pl[k] = pack_io2<true>(x - io2_lo<true>(ph[k]), y - io2_hi<true>(ph[k]));
-      }
-#pragma unroll
-      for (int n = 0; n < NO; n += 2) {
-        const int c = 8 * n + x4_row;
-        const uint32_t a = base + 2 * Pl::MAT + c * (2 * CT) + ((wt * (TW / 8) + 2 * kk + x4_piece) ^ (c & 7)) * 16;
-        uint32_t b0, b1, b2, b3, c0, c1, c2, c3;
-        ldmatrix_x4(a, b0, b1, b2, b3);
-        ldmatrix_x4(a + Pl::MAT, c0, c1, c2, c3);
-        mma_f16(o[n], ph[0], ph[1], ph[2], ph[3], b0, b1);
-        mma_f16(o[n + 1], ph[0], ph[1], ph[2], ph[3], b2, b3);
-        mma_f16(o[n], pl[0], pl[1], pl[2], pl[3], b0, b1);
-        mma_f16(o[n + 1], pl[0], pl[1], pl[2], pl[3], b2, b3);
-        mma_f16(o[n], ph[0], ph[1], ph[2], ph[3], c0, c1);
-        mma_f16(o[n + 1], ph[0], ph[1], ph[2], ph[3], c2, c3);
-      }
-    }
-  };
-
-  // ---- packed tiles: tile t is multiplied while tile t + 1 is expanded into the other buffer ----
-  const int t_pk = min(t_hi, pk_tiles);
-  auto expand_next = [&](int t) {
-    cp_async_wait<1>();
-    __syncwarp();
-    fetch(t + 2);
-    expand(t, t & 1);
-  };
-  if (t_lo < t_pk) {
-    expand_next(t_lo);
-    __syncthreads();
-    for (int t = t_lo; t < t_pk; ++t) {
-      if (warp < 4 && t + 1 < t_pk) expand_next(t + 1);
-      multiply(t, t & 1);
-      if (warp >= 4 && t + 1 < t_pk) expand_next(t + 1);
-      __syncthreads();
-    }
-  }
-  cp_async_wait_all();
-
-  // ---- window tiles ----
-  if (max(t_lo, pk_tiles) < t_hi) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float f = pow2i(-ev[i]);
-      ev[i] = 0;
-#pragma unroll
-      for (int n = i * QT; n < (i + 1) * QT; ++n)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) o[n][k] *= f;
-    }
-    const uint8_t* wk = reinterpret_cast<const uint8_t*>(p.L.win_k) + (size_t)bh * dm.R * (2 * D);
-    const uint8_t* wv = reinterpret_cast<const uint8_t*>(p.L.win_v) + (size_t)bh * dm.R * (2 * D);
-    for (int t = max(t_lo, pk_tiles); t < t_hi; ++t) {
-      const int w0 = (t - pk_tiles) * CT;  // first window row of the tile
-      for (int i = tid; i < CT * (D / 8); i += 256) {
-        const int r = i / (D / 8), c = i % (D / 8);
-        const uint32_t dst = sm + r * 2 * D + (c ^ (r & 7)) * 16;
-        if (w0 + r < p.r) {
-          cp_async16(dst, wk + (size_t)(w0 + r) * (2 * D) + c * 16);
-          cp_async16(dst + Pl::MAT, wv + (size_t)(w0 + r) * (2 * D) + c * 16);
+    l_sm[w][r] = l;
+    ml_sm[w][r] = ml;
+  } else {
+    // ================= expansion: keys (warps 8 .. 11: 32 tokens x half of the channels), values (12 .. 15) ==========
+    const int ew = warp - 8;
+    const uint32_t raw = sm + Pl::OFF_RAW + ew * C_STAGES * Pl::RAW;
+    const int n_pk = min(t_hi, pk_tiles);
+    // Raw data of packed tile `t` that this warp expands, into its own stage; one commit per call
+    const int kg = ew >> 1, hc = ew & 1, c0 = (ew & 3) * DQ;
+    const uint8_t* const g_code = ew < 4
+        ? reinterpret_cast<const uint8_t*>(p.L.k_codes) + (size_t)bh * ((size_t)dm.nq_cap * Pl::KROW)
+        : reinterpret_cast<const uint8_t*>(p.L.v_codes) + (size_t)bh * ((size_t)dm.nq_cap * (D * BV / 8));
+    const uint8_t* const g_meta = ew < 4
+        ? reinterpret_cast<const uint8_t*>(p.L.k_meta) + (size_t)bh * ((size_t)(dm.nq_cap / GS) * 4 * D)
+        : reinterpret_cast<const uint8_t*>(p.L.v_meta) + (size_t)bh * ((size_t)dm.nq_cap * 4 * NG);
+    auto fetch = [&](int t) {
+      if (t < n_pk) {
+        const uint32_t dst = raw + (t % C_STAGES) * Pl::RAW;
+        if (ew < 4) {
+          const int tok = t * CT + 32 * kg;
+          if (lane < Pl::RAW_KC / 16)
+            cp_async16(dst + lane * 16, g_code + (size_t)(tok / 32) * (32 * Pl::KROW) + (Pl::KROW == 32 ? hc * 512 : 0) + lane * 16);
+          if (lane < D / 4) cp_async16(dst + Pl::RAW_KC + lane * 16, g_meta + (size_t)(tok / GS) * (4 * D) + lane * 16);
         } else {
-          sts128(dst, 0u, 0u, 0u, 0u);
-          sts128(dst + Pl::MAT, 0u, 0u, 0u, 0u);
+          const uint8_t* src = g_code + (size_t)(t / 2) * (D * 16 * BV);
+          if (lane < DQ) {
+            if constexpr (BV == 2) cp_async16(dst + lane * 16, src + (t & 1) * (D * 16) + (c0 + lane) * 16);
+            else cp_async8(dst + lane * 8, src + (c0 + lane) * 16 + (t & 1) * 8);
+          }
+          for (int i = lane; i < CT * 4 * NG / 16; i += 32)  // 16 bytes more after every 16 tokens (banks)
+            cp_async16(dst + Pl::RAW_VC + i * 16 + i / (4 * NG) * 16, g_meta + (size_t)t * (CT * 4 * NG) + i * 16);
         }
       }
       cp_async_commit();
-      cp_async_wait_all();
-      __syncthreads();
-      auto window = [&](auto f16) {
-        constexpr bool F16 = decltype(f16)::value;
-        float s[NT][4];
+    };
+    constexpr int UPW = D / 32, TP = 32 / UPW;       // keys: 16-channel units of a warp, tokens of a pass
+    const int k_tok = lane % TP, k_u = hc * UPW + lane / TP;
+    const int v_c = lane & 7, v_u = lane >> 3;       // values: channel of a pass, 16 tokens
+    int ev = 0;
+    bool ev_set = false;
+    // exponent of the values in use: the largest |v| times 2^ev in [2^4, 2^14); it moves only outside that
+    auto value_exponent = [&](float mx) {
+      mx = __uint_as_float(redux_max_u32(__float_as_uint(mx)));
+      const int em = mx > 0.f ? exponent_of(mx) : -100;
+      if (em > -100 && (!ev_set || em + ev > 13 || em + ev < 4)) {
+        ev = 9 - em;
+        ev_set = true;
+      }
+    };
+    fetch(t_lo);
+    fetch(t_lo + 1);
+    for (int i = 0; i < N; ++i) {
+      const int t = t_lo + i;
+      cp_async_wait<1>();
+      __syncwarp();
+      fetch(t + 2);
+      if (i >= 2 && !__all_sync(0xffffffffu, mbar_wait(bar_free + 8 * (i & 1), ((i >> 1) - 1) & 1, &dead_sm))) break;
+      const uint32_t src = raw + (t % C_STAGES) * Pl::RAW, dst = sm + (i & 1) * Pl::BUF;
+      if (t < n_pk) {
+        float s[16], z[16];
+        float mx = 0.f;
+        if (ew < 4) {  // n_q % 32 == 0: the 32 tokens exist or do not together
+          const bool exists = t * CT + 32 * kg < p.n_q;
+          // the largest |k| of the group, all channels: this lane looks at channels lane, lane + 32, ...
+          float top = 0.f, low = 0.f;
 #pragma unroll
-        for (int n = 0; n < NT; ++n)
+          for (int k = 0; k < D / 32; ++k) {
+            top = fmaxf(top, f16_to_f(lds16(src + Pl::RAW_KC + 2 * (lane * (D / 32) + k))));
+            low = fmaxf(low, fabsf(f16_to_f(lds16(src + Pl::RAW_KC + 2 * D + 2 * (lane * (D / 32) + k)))));
+          }
+          mx = exists ? fmaf((float)((1 << BK) - 1), top, low) : 0.f;
+          mx = __uint_as_float(redux_max_u32(__float_as_uint(mx)));
+          const int e = mx >= 1.f && mx < 32768.f ? 0 : (mx > 0.f ? 14 - exponent_of(mx) : 0);
+          if (lane == 0) k_unit[i & 3][kg] = pow2i(-e);  // (both halves write the same)
+          const uint32_t meta = src + Pl::RAW_KC + 2 * ((k_u & 1) * 16 * (D / 32) + (k_u >> 1));
 #pragma unroll
-          for (int k = 0; k < 4; ++k) s[n][k] = 0.f;
-        const int tw = wt * TW;
+          for (int k = 0; k < 16; ++k) {
+            s[k] = exists ? f16_to_f(lds16(meta + 2 * k * (D / 32))) : 0.f;
+            z[k] = exists ? f16_to_f(lds16(meta + 2 * D + 2 * k * (D / 32))) : 0.f;
+          }
+          if (e != 0) {
+            scale16(s, pow2i(e));
+            scale16(z, pow2i(e));
+          }
+          constexpr int RS = Pl::KROW < 16 ? Pl::KROW : 16;
 #pragma unroll
-        for (int ks = 0; ks < KS; ++ks) {
-          uint32_t a0, a1, a2, a3;
-          ldmatrix_x4(qs + (16 * wr + (lane & 15)) * Pl::QROW + ks * 32 + (lane >> 4) * 16, a0, a1, a2, a3);
+          for (int k = 0; k < 32 / TP; ++k) {
+            const int tl = k_tok + TP * k, tok = 32 * kg + tl;
+            uint32_t wd;
+            if constexpr (BK == 2) wd = lds32(src + tl * RS + (Pl::KROW == 32 ? (k_u & 3) : k_u) * 4);
+            else wd = lds32(src + tl * RS + (k_u >> 1) * 4) >> (4 * (k_u & 1));
+            uint32_t hi[8], lo[8];
+            expand16<BK>(wd, s, z, hi, lo);
+            store16(dst + (tok >> 3) * Pl::K_SBO + 2 * k_u * 128 + (tok & 7) * 16, 128, Pl::MAT, hi, lo);
+          }
+        } else {
+          const bool exists = t * CT + 16 * v_u < p.n_q;
+          const uint32_t meta = src + Pl::RAW_VC + v_u * (64 * NG + 16) + 2 * (c0 / GS);
 #pragma unroll
-          for (int n = 0; n < NT; n += 2) {
-            const int tok = tw + 8 * n + x4_row;
-            uint32_t b0, b1, b2, b3;
-            ldmatrix_x4(sm + tok * 2 * D + ((2 * ks + x4_piece) ^ (tok & 7)) * 16, b0, b1, b2, b3);
-            mma16816<F16>(s[n], a0, a1, a2, a3, b0, b1);
-            mma16816<F16>(s[n + 1], a0, a1, a2, a3, b2, b3);
+          for (int k = 0; k < 16; ++k) {
+            s[k] = exists ? f16_to_f(lds16(meta + k * 4 * NG)) : 0.f;
+            z[k] = exists ? f16_to_f(lds16(meta + k * 4 * NG + 2 * NG)) : 0.f;
+            mx = fmaxf(mx, fmaf((float)((1 << BV) - 1), s[k], fabsf(z[k])));
+          }
+          value_exponent(mx);
+          if (lane == 0) v_exp[i & 3][ew & 3] = ev;
+          scale16(s, pow2i(ev));
+          scale16(z, pow2i(ev));
+#pragma unroll
+          for (int k = 0; k < D / 32; ++k) {
+            const int cl = v_c + 8 * k, c = c0 + cl;
+            uint32_t wd;
+            if constexpr (BV == 2) wd = lds32(src + cl * 16 + v_u * 4);
+            else wd = lds32(src + cl * 8 + (v_u >> 1) * 4) >> (4 * (v_u & 1));
+            uint32_t hi[8], lo[8];
+            expand16<BV>(wd, s, z, hi, lo);
+            store16(dst + 2 * Pl::MAT + (c >> 3) * Pl::V_SBO + 2 * v_u * 128 + (c & 7) * 16, 128, Pl::MAT, hi, lo);
           }
         }
-#pragma unroll
-        for (int n = 0; n < NT; ++n)
-#pragma unroll
-          for (int k = 0; k < 4; ++k) s[n][k] *= scale2;
-        softmax(s, p.n_q + w0 + tw, p.S, true);
-#pragma unroll
-        for (int kk = 0; kk < TW / 16; ++kk) {
-          uint32_t ph[4], pl[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float x = s[2 * kk + (k >> 1)][2 * (k & 1)], y = s[2 * kk + (k >> 1)][2 * (k & 1) + 1];
-            ph[k] = pack_io2<F16>(x, y);
-            pl[k] = pack_io2<F16>(x - io2_lo<F16>(ph[k]), y - io2_hi<F16>(ph[k]));
+      } else {
+        // a window tile: 16-bit rows as they are, split into pairs (exact for inputs of ordinary magnitude)
+        const int w0 = (t - pk_tiles) * CT;
+        if (ew < 4) {
+          const uint8_t* rows = reinterpret_cast<const uint8_t*>(p.L.win_k) + (size_t)bh * dm.R * (2 * D);
+          float mx = 0.f;
+          for (int k = 0; k < 32; ++k) {  // all channels of the 32 tokens
+            if (w0 + 32 * kg + k < p.r && lane < D / 4) {
+              const uint2 v = reinterpret_cast<const uint2*>(rows + (size_t)(w0 + 32 * kg + k) * (2 * D))[lane];
+              mx = fmaxf(mx, fmaxf(fmaxf(fabsf(io_to_f(v.x & 0xffffu, p.f16)), fabsf(io_to_f(v.x >> 16, p.f16))),
+                                   fmaxf(fabsf(io_to_f(v.y & 0xffffu, p.f16)), fabsf(io_to_f(v.y >> 16, p.f16)))));
+            }
           }
-          const int tok = tw + 16 * kk + (lane & 15);
+          mx = __uint_as_float(redux_max_u32(__float_as_uint(mx)));
+          const int e = mx >= 1.f && mx < 32768.f ? 0 : (mx > 0.f ? 14 - exponent_of(mx) : 0);
+          if (lane == 0) k_unit[i & 3][kg] = pow2i(-e);
+          const float f = pow2i(e);
+          for (int k = 0; k < 32 / TP; ++k) {
+            const int tok = 32 * kg + k_tok + TP * k;
+            uint32_t hi[8], lo[8];
 #pragma unroll
-          for (int n = 0; n < NO; n += 2) {
-            uint32_t b0, b1, b2, b3;
-            ldmatrix_x4_trans(sm + Pl::MAT + tok * 2 * D + ((n + (lane >> 4)) ^ (tok & 7)) * 16, b0, b1, b2, b3);
-            mma16816<F16>(o[n], ph[0], ph[1], ph[2], ph[3], b0, b1);
-            mma16816<F16>(o[n + 1], ph[0], ph[1], ph[2], ph[3], b2, b3);
-            mma16816<F16>(o[n], pl[0], pl[1], pl[2], pl[3], b0, b1);
-            mma16816<F16>(o[n + 1], pl[0], pl[1], pl[2], pl[3], b2, b3);
+            for (int c = 0; c < 2; ++c) {
+              uint4 v = make_uint4(0u, 0u, 0u, 0u);
+              if (w0 + tok < p.r) v = reinterpret_cast<const uint4*>(rows + (size_t)(w0 + tok) * (2 * D))[2 * k_u + c];
+              const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                split2(io_to_f(x[j] & 0xffffu, p.f16) * f, io_to_f(x[j] >> 16, p.f16) * f, hi[4 * c + j], lo[4 * c + j]);
+            }
+            store16(dst + (tok >> 3) * Pl::K_SBO + 2 * k_u * 128 + (tok & 7) * 16, 128, Pl::MAT, hi, lo);
+          }
+        } else {
+          const uint16_t* rows = p.L.win_v + (size_t)bh * dm.R * D;
+          float mx = 0.f;
+          for (int k = 0; k < CT; ++k)
+            if (w0 + k < p.r && lane < DQ) mx = fmaxf(mx, fabsf(io_to_f(rows[(size_t)(w0 + k) * D + c0 + lane], p.f16)));
+          value_exponent(mx);
+          if (lane == 0) v_exp[i & 3][ew & 3] = ev;
+          const float f = pow2i(ev);
+          for (int k = 0; k < D / 32; ++k) {
+            const int c = c0 + v_c + 8 * k;
+            float v[16];
+            uint32_t hi[8], lo[8];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const int tok = w0 + 16 * v_u + j;
+              v[j] = tok < p.r ? io_to_f(rows[(size_t)tok * D + c], p.f16) * f : 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) split2(v[2 * j], v[2 * j + 1], hi[j], lo[j]);
+            store16(dst + 2 * Pl::MAT + (c >> 3) * Pl::V_SBO + 2 * v_u * 128 + (c & 7) * 16, 128, Pl::MAT, hi, lo);
           }
         }
-      };
-      if (p.f16) window(std::true_type{}); else window(std::false_type{});
-      __syncthreads();
+      }
+      proxy_fence();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_kfull + 8 * (i & 1));
     }
+    cp_async_wait_all();
   }
 
-  // ---- state of every warp's 16 rows into shared memory (over the tile buffers; the last tile ended in a barrier) ----
-  {
-    float* ws = reinterpret_cast<float*>(smem) + (size_t)warp * 16 * Pl::MS;
-    float f[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) f[i] = pow2i(-ev[i]);
-#pragma unroll
-    for (int n = 0; n < NO; ++n)
-#pragma unroll
-      for (int r = 0; r < 2; ++r)
-        *reinterpret_cast<float2*>(ws + (gid + 8 * r) * Pl::MS + 8 * n + 2 * tig) =
-            make_float2(o[n][2 * r] * f[n / QT], o[n][2 * r + 1] * f[n / QT]);
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      l[r] += __shfl_xor_sync(0xffffffffu, l[r], 1);
-      l[r] += __shfl_xor_sync(0xffffffffu, l[r], 2);
-      if (tig == 0) {
-        ws[(gid + 8 * r) * Pl::MS + D] = set[r] ? mr[r] : -CUDART_INF_F;
-        ws[(gid + 8 * r) * Pl::MS + D + 1] = l[r];
-      }
-    }
-  }
+  // ---- the row tile's result, or its partial: row r's state in split s at (tile * 128 + r) * ns + s ----
+  tc_fence_before();
   __syncthreads();
-  // ---- the row tile's result, or its partial: row r's state in split s at (tile * M + r) * ns + s ----
-  const size_t part0 = ((size_t)rt * n_streams + bh) * M;
+  const size_t part0 = ((size_t)rt * n_streams + bh) * CM;
   auto out_row = [&](int r) {
     const int row = row0 + r, j = row / G, h = row - j * G;
     return ((size_t)j * dm.B + b) * dm.Hq + hk * G + h;
   };
-  for (int i = tid; i < n_rows * D; i += 256) {
-    const int r = i / D, d = i % D;
-    const float* st = reinterpret_cast<const float*>(smem) + (r / 16 * 16 + r % 16) * Pl::MS;
-    float Mx = -CUDART_INF_F;
+  if (warp < 8) {
+    const bool ok = N == 0 || mbar_wait(bar_o, (N - 1) & 1, &dead_sm);
+    if (__all_sync(0xffffffffu, ok) && dead_sm == 0) {
+      tc_fence_after();
+      const int w = warp >> 2, r = tid & 127;
+      const float M = m_sm[r], M0 = ml_sm[0][r], M1 = ml_sm[1][r];
+      const float L = l_sm[0][r] * (M0 == M ? 1.f : ex2(M0 - M)) + l_sm[1][r] * (M1 == M ? 1.f : ex2(M1 - M));
+      const float inv = p.ns == 1 ? 1.f / L : 1.f;
 #pragma unroll
-    for (int w = 0; w < WT; ++w) Mx = fmaxf(Mx, st[w * M * Pl::MS + D]);
-    float A = 0.f, Ls = 0.f;
+      for (int h = 0; h < D / 64; ++h) {
+        const int cb = w * (D / 2) + 32 * h;
+        uint32_t o[32];
+        if (N > 0) {
+          tmem_ld32(row_t + Pl::COL_O + cb, o);
+          tc_wait_ld();
+        }
+        float f[2];  // of the two channel quarters that 32 channels can span
+        f[0] = (N > 0 ? pow2i(-v_exp[(N - 1) & 3][cb / DQ]) : 0.f) * inv;
+        f[1] = (N > 0 ? pow2i(-v_exp[(N - 1) & 3][(cb + 31) / DQ]) : 0.f) * inv;
+        float v[32];
 #pragma unroll
-    for (int w = 0; w < WT; ++w) {
-      const float mw = st[w * M * Pl::MS + D];
-      const float f = mw == -CUDART_INF_F ? 0.f : ex2(mw - Mx);
-      A = fmaf(st[w * M * Pl::MS + d], f, A);
-      Ls = fmaf(st[w * M * Pl::MS + D + 1], f, Ls);
+        for (int k = 0; k < 32; ++k) v[k] = N > 0 ? __uint_as_float(o[k]) * f[k / 16] : 0.f;
+        if (r < n_rows) {
+          if (p.ns > 1) {
+            float4* dst = reinterpret_cast<float4*>(p.part_acc + ((part0 + r) * p.ns + split) * D + cb);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) dst[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+          } else if (p.out_f32) {
+            float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + out_row(r) * D + cb);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) dst[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+          } else {
+            uint32_t x[16];
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+              x[k] = p.f16 ? pack_io2<true>(v[2 * k], v[2 * k + 1]) : pack_io2<false>(v[2 * k], v[2 * k + 1]);
+            uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(p.out) + out_row(r) * D + cb);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) dst[k] = make_uint4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
+          }
+        }
+      }
+      if (p.ns > 1 && w == 0 && r < n_rows)
+        *reinterpret_cast<float2*>(p.part_ml + ((part0 + r) * p.ns + split) * 2) = make_float2(M, L);
     }
-    if (p.ns == 1) {
-      chunk_store<D>(p, out_row(r), d, A / Ls);
-    } else {
-      const size_t at = (part0 + r) * p.ns + split;
-      p.part_acc[at * D + d] = A;
-      if (d == 0) *reinterpret_cast<float2*>(p.part_ml + at * 2) = make_float2(Mx, Ls);
-    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 8 + C_EXPAND)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tbase), "r"(512u) : "memory");
+  if (dead_sm != 0) {
+    if (tid == 0) atomicExch(p.status, 1);
+    return;
   }
   if (p.ns == 1) return;
   // the last CTA of the row tile merges (ticket as in the decode kernel)
   unsigned* ticket = p.tickets + (size_t)rt * n_streams + bh;
-  __syncthreads();
   if (tid == 0) {
     unsigned t;
     asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;\n" : "=r"(t) : "l"(ticket) : "memory");
@@ -563,7 +657,7 @@ __global__ void __launch_bounds__(256, 1) chunk_kernel(const __grid_constant__ C
   }
   __syncthreads();
   if (!s_flag) return;
-  for (int i = tid; i < n_rows * (D / 2); i += 256) {
+  for (int i = tid; i < n_rows * (D / 2); i += C_THREADS) {
     const int r = i / (D / 2), d = 2 * (i % (D / 2));
     const float* pa = p.part_acc + (part0 + r) * p.ns * D + d;
     const float* ml = p.part_ml + (part0 + r) * p.ns * 2;
@@ -584,28 +678,28 @@ __global__ void __launch_bounds__(256, 1) chunk_kernel(const __grid_constant__ C
   if (tid == 0) *ticket = 0u;
 }
 
-template <int D, int BK, int BV, int GS, int WR>
+template <int D, int BK, int BV, int GS>
 cudaError_t chunk_launch_one(const ChunkParams& p, cudaStream_t st) {
-  using Pl = ChunkPlan<D, BK, BV, GS, WR>;
-  auto kernel = chunk_kernel<D, BK, BV, GS, WR>;
+  using Pl = ChunkPlan<D, BK, BV, GS>;
+  auto kernel = chunk_kernel<D, BK, BV, GS>;
   const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Pl::TOTAL);
   if (e != cudaSuccess) return e;
-  return launch_dependent(kernel, dim3((unsigned)p.row_tiles * p.dm.B * p.dm.Hkv * p.ns), dim3(256), (size_t)Pl::TOTAL, st, p);
+  return launch_dependent(kernel, dim3((unsigned)p.row_tiles * p.dm.B * p.dm.Hkv * p.ns), dim3(C_THREADS), (size_t)Pl::TOTAL, st, p);
 }
 
 }  // namespace
 
-template <int D, int WR>
+template <int D>
 cudaError_t launch_chunk_t(const ChunkParams& p, cudaStream_t st) {
   switch (p.L.bk * 100 + p.L.bv * 10 + (p.dm.g == 64)) {
-    case 220: return chunk_launch_one<D, 2, 2, 32, WR>(p, st);
-    case 221: return chunk_launch_one<D, 2, 2, 64, WR>(p, st);
-    case 210: return chunk_launch_one<D, 2, 1, 32, WR>(p, st);
-    case 211: return chunk_launch_one<D, 2, 1, 64, WR>(p, st);
-    case 120: return chunk_launch_one<D, 1, 2, 32, WR>(p, st);
-    case 121: return chunk_launch_one<D, 1, 2, 64, WR>(p, st);
-    case 110: return chunk_launch_one<D, 1, 1, 32, WR>(p, st);
-    case 111: return chunk_launch_one<D, 1, 1, 64, WR>(p, st);
+    case 220: return chunk_launch_one<D, 2, 2, 32>(p, st);
+    case 221: return chunk_launch_one<D, 2, 2, 64>(p, st);
+    case 210: return chunk_launch_one<D, 2, 1, 32>(p, st);
+    case 211: return chunk_launch_one<D, 2, 1, 64>(p, st);
+    case 120: return chunk_launch_one<D, 1, 2, 32>(p, st);
+    case 121: return chunk_launch_one<D, 1, 2, 64>(p, st);
+    case 110: return chunk_launch_one<D, 1, 1, 32>(p, st);
+    case 111: return chunk_launch_one<D, 1, 1, 64>(p, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -706,33 +706,26 @@ int xq_decode_attention_f32(xq_cache* c, int layer, const void* q, float* out, v
 
 namespace {
 
-// How the query rows of a chunk are cut: 16 wr rows per CTA, ns splits of a row tile's tokens.
-struct ChunkPlanning {
-  int wr, row_tiles, ns;
-};
-ChunkPlanning plan_chunk(const xq_cache* c, int S, int T) {
+// Splits of a row tile's tokens in chunk attention.
+int plan_chunk(const xq_cache* c, int S, int T, int row_tiles) {
   const Dims& dm = c->plan.dm;
   const long long streams = (long long)dm.B * dm.Hkv;
-  const int rows = T * dm.G;
   // tiles of 64 tokens that a row tile goes over: the last one, and on average over the causal chunk
   const double most = S / 64.0 + 1.0, mean = (S - 0.5 * T) / 64.0 + 1.0;
-  ChunkPlanning best{8, 0, 1};
+  int best = 1;
   double best_time = 0.0;
-  for (int wr : {8, 4, 2}) {
-    const int row_tiles = (rows + 16 * wr - 1) / (16 * wr);
-    // microseconds of a tile: products, or the expansion that does not fit beside them
-    const double tile = wr == 8 ? 3.0 : (wr == 4 ? 1.8 : 1.2);
-    for (int ns = 1; ns <= 32; ++ns) {
-      if (ns > 1 && (row_tiles > DECODE_MAX_LAYERS || ns > most ||
-                     streams * row_tiles * 16 * wr * ns > (long long)dm.B * dm.Hq * XQ_MAX_SPLITS))
-        break;
-      const double waves = ceil((double)(streams * row_tiles * ns) / c->sm_count);
-      const double longest = most / ns > waves * mean / ns ? most / ns : waves * mean / ns;
-      const double time = longest * tile + waves * (ns > 1 ? 6.0 : 4.0);
-      if (best.row_tiles == 0 || time < best_time) {
-        best_time = time;
-        best = {wr, row_tiles, ns};
-      }
+  for (int ns = 1; ns <= 32; ++ns) {
+    // scratch: tickets for DECODE_MAX_LAYERS row tiles of a stream, XQ_MAX_SPLITS partials per query head
+    if (ns > 1 && (row_tiles > DECODE_MAX_LAYERS || ns > most ||
+                   streams * row_tiles * CHUNK_ROWS * ns > (long long)dm.B * dm.Hq * XQ_MAX_SPLITS))
+      break;
+    // a tile costs about 1.0 us, the start and the end of a CTA as much as 6 tiles (10 with a merge)
+    const double waves = ceil((double)(streams * row_tiles * ns) / c->sm_count);
+    const double longest = most > waves * mean ? most / ns : waves * mean / ns;
+    const double time = longest + waves * (ns > 1 ? 10.0 : 6.0);
+    if (ns == 1 || time < best_time) {
+      best_time = time;
+      best = ns;
     }
   }
   return best;
@@ -744,7 +737,6 @@ int launch_chunk(xq_cache* c, int layer, const void* q, void* out, int T, int ou
   const Dims& dm = c->plan.dm;
   const int S = c->seq[layer];
   const Scratch s = workspace_scratch(c);
-  const ChunkPlanning pl = plan_chunk(c, S, T);
   ChunkParams p;
   p.dm = dm;
   p.L = layer_ptrs(c, layer);
@@ -754,19 +746,19 @@ int launch_chunk(xq_cache* c, int layer, const void* q, void* out, int T, int ou
   p.n_q = S - p.r;
   p.S = S;
   p.T = T;
-  p.row_tiles = pl.row_tiles;
-  p.ns = pl.ns;
+  p.row_tiles = (T * dm.G + CHUNK_ROWS - 1) / CHUNK_ROWS;
+  p.ns = plan_chunk(c, S, T, p.row_tiles);
   p.scale = c->scale;
   p.part_acc = s.part_acc;
   p.part_ml = s.part_ml;
   p.tickets = s.tickets;
+  p.status = s.status;
   p.out_f32 = out_f32;
   p.f16 = c->cfg.io_dtype == XQ_F16;
   cudaError_t e;
   {
     Timer t(c, st, 0);
-    if (dm.D == 128) e = pl.wr == 8 ? launch_chunk_t<128, 8>(p, st) : pl.wr == 4 ? launch_chunk_t<128, 4>(p, st) : launch_chunk_t<128, 2>(p, st);
-    else e = pl.wr == 8 ? launch_chunk_t<64, 8>(p, st) : pl.wr == 4 ? launch_chunk_t<64, 4>(p, st) : launch_chunk_t<64, 2>(p, st);
+    e = dm.D == 128 ? launch_chunk_t<128>(p, st) : launch_chunk_t<64>(p, st);
   }
   c->launches++;
   if (e != cudaSuccess) {

@@ -109,6 +109,8 @@ struct DecodeParams {
   DecodeLayer layer[DECODE_MAX_LAYERS];
 };
 
+constexpr int CHUNK_ROWS = 128;  // query rows of a chunk CTA
+
 // Attention of a chunk of query tokens (xq_chunk.cuh).
 struct ChunkParams {
   Dims dm;
@@ -117,12 +119,13 @@ struct ChunkParams {
   void* out;          // [T,B,Hq,D] bf16 or f32
   int n_q, r;         // quantized tokens, window tokens
   int S, T;           // tokens of the layer; query token j sees the first S - T + j + 1 of them
-  int row_tiles;      // per (sequence, kv head): T * G rows over the rows of a CTA
+  int row_tiles;      // per (sequence, kv head): T * G rows over CHUNK_ROWS
   int ns;             // splits of a row tile's tokens
   float scale;
   float* part_acc;    // [row_tiles,B*Hkv,rows,ns,D] (ns > 1)
   float* part_ml;     // [row_tiles,B*Hkv,rows,ns,2]
   unsigned int* tickets;  // [row_tiles,B*Hkv], zero between launches
+  int* status;        // device word that is set when a bounded wait gave up
   int out_f32, f16;
 };
 
@@ -181,8 +184,7 @@ template <int D, int HP, int NT>
 cudaError_t launch_decode_mma_t(const DecodeParams& p, cudaStream_t st);
 template <int D, int HP, int NT>
 MmaShape decode_mma_shape_t(int g, int bk, int bv);
-// Chunk attention with 16 WR query rows per CTA (WR 8, 4, 2).
-template <int D, int WR>
+template <int D>
 cudaError_t launch_chunk_t(const ChunkParams& p, cudaStream_t st);
 cudaError_t launch_merge(const MergeParams& p, cudaStream_t st);
 
