@@ -76,9 +76,9 @@ __host__ __device__ constexpr uint32_t idesc_f16(int n) {
 // D[128 x N] (+)= A[128 x 16] (tensor memory) * B[16 x N] (shared memory); issued by one thread
 __device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, bool accumulate) {
   asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %5, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%4,%4,%4,%4}, p;\n}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(0u), "r"((uint32_t)accumulate) : "memory");
+      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate) : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
@@ -94,12 +94,13 @@ struct ChunkPlan {
   static constexpr int NG = D / GS;
   static constexpr int KROW = D * BK / 8;                       // packed bytes of a token's keys
   static constexpr int MAT = CT * 2 * D;                        // one matrix of a tile: K hi, K lo, V hi, V lo
-  static constexpr int BUF = 4 * MAT;
+  static constexpr int KBUFS = 2, VBUFS = 3;                    // expanded tiles of keys, of values
+  static constexpr int OFF_V = KBUFS * 2 * MAT;
   static constexpr int K_SBO = 16 * D, V_SBO = 16 * CT;         // eight rows of the keys (tokens) / of the values (channels)
   static constexpr int RAW_KC = 32 * KROW, RAW_K = RAW_KC + 4 * D;  // a key warp's codes (32 tokens) and parameters
   static constexpr int RAW_VC = (D / 4) * 8 * BV, RAW_V = RAW_VC + 4 * (64 * NG + 16);
   static constexpr int RAW = RAW_K > RAW_V ? RAW_K : RAW_V;     // of one warp and stage
-  static constexpr int OFF_RAW = 2 * BUF;
+  static constexpr int OFF_RAW = OFF_V + VBUFS * 2 * MAT;
   static constexpr int TOTAL = OFF_RAW + C_EXPAND * C_STAGES * RAW;
   // tensor memory columns: q, S and numerators of even and odd tiles, O
   static constexpr uint32_t COL_Q = 0, COL_S = 64, COL_O = 192;
@@ -154,7 +155,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
   using Pl = ChunkPlan<D, BK, BV, GS>;
   constexpr int NG = Pl::NG, DQ = D / 4;
   extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ __align__(8) unsigned long long bar_mem[18];
+  __shared__ __align__(8) unsigned long long bar_mem[24];
   __shared__ float k_unit[4][2];            // [tile % 4][32 tokens]: what a unit of the expanded keys is worth
   __shared__ int v_exp[4][4];               // [tile % 4][channel quarter]: the expanded values are times 2^v_exp
   __shared__ float cq_sm[CM], m_sm[CM];     // logits from products of the scaled q; softmax reference (-infinity: none)
@@ -180,9 +181,11 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
 
   const uint32_t sm = (uint32_t)__cvta_generic_to_shared(smem);
   const uint32_t bars = (uint32_t)__cvta_generic_to_shared(&bar_mem[0]);
-  const uint32_t bar_kfull = bars;             // [2] a tile is expanded
-  const uint32_t bar_free = bar_kfull + 16;    // [2] its buffer may be written again
-  const uint32_t bar_s = bar_free + 16;        // [2] S is complete
+  const uint32_t bar_kfull = bars;             // [2] a tile's keys are expanded
+  const uint32_t bar_kfree = bar_kfull + 16;   // [2] their buffer may be written again
+  const uint32_t bar_vfull = bar_kfree + 16;   // [3] the same of the values
+  const uint32_t bar_vfree = bar_vfull + 24;   // [3]
+  const uint32_t bar_s = bar_vfree + 24;       // [2] S is complete
   const uint32_t bar_p = bar_s + 16;           // [2] the numerators are written
   const uint32_t bar_o = bar_p + 16;           // the value products of a tile are complete
   const uint32_t bar_turn = bar_o + 8;         // [4 warps][2] a row's reference for an even / odd tile is there
@@ -191,10 +194,15 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
   if (tid == 0) {
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      mbar_init(bar_kfull + 8 * i, C_EXPAND);
-      mbar_init(bar_free + 8 * i, 1);
+      mbar_init(bar_kfull + 8 * i, C_EXPAND / 2);
+      mbar_init(bar_kfree + 8 * i, 1);
       mbar_init(bar_s + 8 * i, 1);
       mbar_init(bar_p + 8 * i, 4);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      mbar_init(bar_vfull + 8 * i, C_EXPAND / 2);
+      mbar_init(bar_vfree + 8 * i, 1);
     }
     mbar_init(bar_o, 1);
     mbar_init(bar_end, 1);
@@ -251,30 +259,35 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
   if (warp == 8 + C_EXPAND) {
     // ================= products: the loop is warp-uniform, one elected lane issues =================
     constexpr uint32_t IDK = idesc_f16(CT), IDV = idesc_f16(D);
+    // (uniform values: the issue of a product then takes no moves between register files)
+    const uint32_t tb = __shfl_sync(0xffffffffu, tbase, 0), smu = __shfl_sync(0xffffffffu, sm, 0);
+#pragma unroll 1
     for (int i = 0; i <= N; ++i) {
       bool ok = true;
       if (i < N) {
         ok = __all_sync(0xffffffffu, mbar_wait(bar_kfull + 8 * (i & 1), (i >> 1) & 1, &dead_sm));
         tc_fence_after();
         if (ok && elect_one()) {
-          const uint32_t base = sm + (i & 1) * Pl::BUF, dS = tbase + Pl::COL_S + (i & 1) * 64;
+          const uint32_t base = smu + (i & 1) * 2 * Pl::MAT, dS = tb + Pl::COL_S + (i & 1) * 64;
           const uint64_t kh = smem_desc(base, 128, Pl::K_SBO), kl = smem_desc(base + Pl::MAT, 128, Pl::K_SBO);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks) {
-            umma_f16(dS, tbase + Pl::COL_Q + 8 * ks, kh + 16 * ks, IDK, ks > 0);
-            umma_f16(dS, tbase + Pl::COL_Q + 8 * ks, kl + 16 * ks, IDK, true);
+            umma_f16(dS, tb + Pl::COL_Q + 8 * ks, kh + 16 * ks, IDK, ks > 0);
+            umma_f16(dS, tb + Pl::COL_Q + 8 * ks, kl + 16 * ks, IDK, true);
           }
           umma_commit(bar_s + 8 * (i & 1));
+          umma_commit(bar_kfree + 8 * (i & 1));
         }
         __syncwarp();
       }
       if (ok && i > 0) {
         const int j = i - 1;
-        ok = __all_sync(0xffffffffu, mbar_wait(bar_p + 8 * (j & 1), (j >> 1) & 1, &dead_sm));
+        ok = __all_sync(0xffffffffu, mbar_wait(bar_vfull + 8 * (j % 3), (j / 3) & 1, &dead_sm) &&
+                                         mbar_wait(bar_p + 8 * (j & 1), (j >> 1) & 1, &dead_sm));
         tc_fence_after();
         if (ok && elect_one()) {
-          const uint32_t base = sm + (j & 1) * Pl::BUF + 2 * Pl::MAT;
-          const uint32_t ph = tbase + Pl::COL_S + (j & 1) * 64, pl = ph + 32, dO = tbase + Pl::COL_O;
+          const uint32_t base = smu + Pl::OFF_V + (j % 3) * 2 * Pl::MAT;
+          const uint32_t ph = tb + Pl::COL_S + (j & 1) * 64, pl = ph + 32, dO = tb + Pl::COL_O;
           const uint64_t vh = smem_desc(base, 128, Pl::V_SBO), vl = smem_desc(base + Pl::MAT, 128, Pl::V_SBO);
 #pragma unroll
           for (int ks = 0; ks < CT / 16; ++ks) {
@@ -283,7 +296,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
             umma_f16(dO, pl + 8 * ks, vh + 16 * ks, IDV, true);
           }
           umma_commit(bar_o);
-          umma_commit(bar_free + 8 * (j & 1));
+          umma_commit(bar_vfree + 8 * (j % 3));
         }
         __syncwarp();
       }
@@ -303,9 +316,11 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
     const float cq = cq_sm[r];
     const int vis = min(vis0 + (row0 + r) / G, vis_max);
     float l = 0.f, ml = -CUDART_INF_F;
+#pragma unroll 1
     for (int i = w; i < N; i += 2) {
-      // (the expansion's exponents are there since the first of the two; the second one is the wait)
+      // (the units and exponents of the expanded tile are there since the first two; the third one is the wait)
       if (!__all_sync(0xffffffffu, mbar_wait(bar_kfull + 8 * (i & 1), (i >> 1) & 1, &dead_sm) &&
+                                       mbar_wait(bar_vfull + 8 * (i % 3), (i / 3) & 1, &dead_sm) &&
                                        mbar_wait(bar_s + 8 * (i & 1), (i >> 1) & 1, &dead_sm)))
         break;
       tc_fence_after();
@@ -338,11 +353,9 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         m = m_old;
         if (xm > m_old + C_TAU || (m_old == -CUDART_INF_F && xm > m_old)) m = ceilf(xm);
         bool change = m != m_old;
-        float ef[4];
+        if (i > 0) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          ef[k] = i > 0 ? pow2i(v_exp[i & 3][k] - v_exp[(i - 1) & 3][k]) : 1.f;
-          change |= ef[k] != 1.f;
+          for (int k = 0; k < 4; ++k) change |= v_exp[i & 3][k] != v_exp[(i - 1) & 3][k];
         }
         if (__any_sync(0xffffffffu, change)) {
           m_sm[r] = m;
@@ -350,12 +363,15 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
             if (!__all_sync(0xffffffffu, mbar_wait(bar_o, (i - 1) & 1, &dead_sm))) break;
             tc_fence_after();
             const float f = m_old == -CUDART_INF_F ? 0.f : ex2(m_old - m);
-#pragma unroll
+#pragma unroll 1
             for (int c = 0; c < D; c += 32) {
+              const int qa = c / DQ, qz = (c + 31) / DQ;  // the channel quarters of the columns' halves
+              const float fa = f * pow2i(v_exp[i & 3][qa] - v_exp[(i - 1) & 3][qa]);
+              const float fz = f * pow2i(v_exp[i & 3][qz] - v_exp[(i - 1) & 3][qz]);
               tmem_ld32(row_t + Pl::COL_O + c, s[0]);
               tc_wait_ld();
 #pragma unroll
-              for (int k = 0; k < 32; ++k) s[0][k] = __float_as_uint(__uint_as_float(s[0][k]) * (f * ef[(c + k) / DQ]));
+              for (int k = 0; k < 32; ++k) s[0][k] = __float_as_uint(__uint_as_float(s[0][k]) * (k < 16 ? fa : fz));
               tmem_st32(row_t + Pl::COL_O + c, s[0]);
             }
             tc_wait_st();
@@ -455,13 +471,19 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
     };
     fetch(t_lo);
     fetch(t_lo + 1);
+#pragma unroll 1
     for (int i = 0; i < N; ++i) {
       const int t = t_lo + i;
       cp_async_wait<1>();
       __syncwarp();
       fetch(t + 2);
-      if (i >= 2 && !__all_sync(0xffffffffu, mbar_wait(bar_free + 8 * (i & 1), ((i >> 1) - 1) & 1, &dead_sm))) break;
-      const uint32_t src = raw + (t % C_STAGES) * Pl::RAW, dst = sm + (i & 1) * Pl::BUF;
+      if (ew < 4) {
+        if (i >= 2 && !__all_sync(0xffffffffu, mbar_wait(bar_kfree + 8 * (i & 1), ((i >> 1) - 1) & 1, &dead_sm))) break;
+      } else {
+        if (i >= 3 && !__all_sync(0xffffffffu, mbar_wait(bar_vfree + 8 * (i % 3), (i / 3 - 1) & 1, &dead_sm))) break;
+      }
+      const uint32_t src = raw + (t % C_STAGES) * Pl::RAW;
+      const uint32_t dst = sm + (ew < 4 ? (i & 1) * 2 * Pl::MAT : Pl::OFF_V + (i % 3) * 2 * Pl::MAT);
       if (t < n_pk) {
         float s[16], z[16];
         float mx = 0.f;
@@ -489,7 +511,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
             scale16(z, pow2i(e));
           }
           constexpr int RS = Pl::KROW < 16 ? Pl::KROW : 16;
-#pragma unroll
+#pragma unroll 1
           for (int k = 0; k < 32 / TP; ++k) {
             const int tl = k_tok + TP * k, tok = 32 * kg + tl;
             uint32_t wd;
@@ -512,7 +534,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
           if (lane == 0) v_exp[i & 3][ew & 3] = ev;
           scale16(s, pow2i(ev));
           scale16(z, pow2i(ev));
-#pragma unroll
+#pragma unroll 1
           for (int k = 0; k < D / 32; ++k) {
             const int cl = v_c + 8 * k, c = c0 + cl;
             uint32_t wd;
@@ -520,7 +542,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
             else wd = lds32(src + cl * 8 + (v_u >> 1) * 4) >> (4 * (v_u & 1));
             uint32_t hi[8], lo[8];
             expand16<BV>(wd, s, z, hi, lo);
-            store16(dst + 2 * Pl::MAT + (c >> 3) * Pl::V_SBO + 2 * v_u * 128 + (c & 7) * 16, 128, Pl::MAT, hi, lo);
+            store16(dst + (c >> 3) * Pl::V_SBO + 2 * v_u * 128 + (c & 7) * 16, 128, Pl::MAT, hi, lo);
           }
         }
       } else {
@@ -529,6 +551,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         if (ew < 4) {
           const uint8_t* rows = reinterpret_cast<const uint8_t*>(p.L.win_k) + (size_t)bh * dm.R * (2 * D);
           float mx = 0.f;
+#pragma unroll 4
           for (int k = 0; k < 32; ++k) {  // all channels of the 32 tokens
             if (w0 + 32 * kg + k < p.r && lane < D / 4) {
               const uint2 v = reinterpret_cast<const uint2*>(rows + (size_t)(w0 + 32 * kg + k) * (2 * D))[lane];
@@ -540,6 +563,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
           const int e = mx >= 1.f && mx < 32768.f ? 0 : (mx > 0.f ? 14 - exponent_of(mx) : 0);
           if (lane == 0) k_unit[i & 3][kg] = pow2i(-e);
           const float f = pow2i(e);
+#pragma unroll 1
           for (int k = 0; k < 32 / TP; ++k) {
             const int tok = 32 * kg + k_tok + TP * k;
             uint32_t hi[8], lo[8];
@@ -557,11 +581,13 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         } else {
           const uint16_t* rows = p.L.win_v + (size_t)bh * dm.R * D;
           float mx = 0.f;
+#pragma unroll 4
           for (int k = 0; k < CT; ++k)
             if (w0 + k < p.r && lane < DQ) mx = fmaxf(mx, fabsf(io_to_f(rows[(size_t)(w0 + k) * D + c0 + lane], p.f16)));
           value_exponent(mx);
           if (lane == 0) v_exp[i & 3][ew & 3] = ev;
           const float f = pow2i(ev);
+#pragma unroll 1
           for (int k = 0; k < D / 32; ++k) {
             const int c = c0 + v_c + 8 * k;
             float v[16];
@@ -573,13 +599,13 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
             }
 #pragma unroll
             for (int j = 0; j < 8; ++j) split2(v[2 * j], v[2 * j + 1], hi[j], lo[j]);
-            store16(dst + 2 * Pl::MAT + (c >> 3) * Pl::V_SBO + 2 * v_u * 128 + (c & 7) * 16, 128, Pl::MAT, hi, lo);
+            store16(dst + (c >> 3) * Pl::V_SBO + 2 * v_u * 128 + (c & 7) * 16, 128, Pl::MAT, hi, lo);
           }
         }
       }
       proxy_fence();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar_kfull + 8 * (i & 1));
+      if (lane == 0) mbar_arrive(ew < 4 ? bar_kfull + 8 * (i & 1) : bar_vfull + 8 * (i % 3));
     }
     cp_async_wait_all();
   }
@@ -600,7 +626,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
       const float M = m_sm[r], M0 = ml_sm[0][r], M1 = ml_sm[1][r];
       const float L = l_sm[0][r] * (M0 == M ? 1.f : ex2(M0 - M)) + l_sm[1][r] * (M1 == M ? 1.f : ex2(M1 - M));
       const float inv = p.ns == 1 ? 1.f / L : 1.f;
-#pragma unroll
+#pragma unroll 1
       for (int h = 0; h < D / 64; ++h) {
         const int cb = w * (D / 2) + 32 * h;
         uint32_t o[32];
@@ -662,8 +688,10 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
     const float* pa = p.part_acc + (part0 + r) * p.ns * D + d;
     const float* ml = p.part_ml + (part0 + r) * p.ns * 2;
     float Mx = -CUDART_INF_F;
+#pragma unroll 4
     for (int s = 0; s < p.ns; ++s) Mx = fmaxf(Mx, ld_cg(ml + 2 * s));
     float ax = 0.f, ay = 0.f, Ls = 0.f;
+#pragma unroll 4
     for (int s = 0; s < p.ns; ++s) {
       const float2 x = ld_cg2(ml + 2 * s), v = ld_cg2(pa + (size_t)s * D);
       const float f = x.x == -CUDART_INF_F ? 0.f : ex2(x.x - Mx);
