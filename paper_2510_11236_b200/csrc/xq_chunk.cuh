@@ -59,8 +59,8 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr) : "memory");
 }
-// shared-memory matrix descriptor, K-major, no swizzle: core matrices of 8 rows x 16 bytes;
-// lbo / sbo: byte distance between core matrices along K / along the rows
+// shared-memory matrix descriptor, N-major, no swizzle: core matrices of 8 K-rows x 16 bytes of N;
+// lbo / sbo: byte distance between core matrices along K / along N
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
   uint64_t d = 0;
   d |= (uint64_t)((addr >> 4) & 0x3fff);
@@ -69,9 +69,9 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
   d |= (uint64_t)1 << 46;  // descriptor version of this architecture
   return d;
 }
-// kind::f16 instruction descriptor: fp16 A and B (both K-major), fp32 accumulate, M = 128
+// kind::f16 instruction descriptor: fp16 A (K-major, tensor memory) and B (N-major), fp32 accumulate, M = 128
 __host__ __device__ constexpr uint32_t idesc_f16(int n) {
-  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+  return (1u << 4) | (1u << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
 // D[128 x N] (+)= A[128 x 16] (tensor memory) * B[16 x N] (shared memory); issued by one thread
 __device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, bool accumulate) {
@@ -93,15 +93,19 @@ template <int D, int BK, int BV, int GS>
 struct ChunkPlan {
   static constexpr int NG = D / GS;
   static constexpr int KROW = D * BK / 8;                       // packed bytes of a token's keys
-  static constexpr int MAT = CT * 2 * D;                        // one matrix of a tile: K hi, K lo, V hi, V lo
-  static constexpr int KBUFS = 2, VBUFS = 3;                    // expanded tiles of keys, of values
+  // An expanded matrix: core matrices of 8 x 8 elements (rows: channels of the keys, tokens of the values; a row's 16
+  // bytes: tokens of the keys, channels of the values), CORE bytes apart along the rows (16 more than their size, so
+  // that the four rows which each of eight lanes writes fall into different banks).
+  static constexpr int CORE = 144, K_SBO = D / 8 * CORE, V_SBO = CT / 8 * CORE;
+  static constexpr int MAT = CT / 8 * K_SBO;
+  static constexpr int KBUFS = 2, VBUFS = 3;                    // expanded tiles of keys, of values (hi and lo each)
   static constexpr int OFF_V = KBUFS * 2 * MAT;
-  static constexpr int K_SBO = 16 * D, V_SBO = 16 * CT;         // eight rows of the keys (tokens) / of the values (channels)
-  static constexpr int RAW_KC = 32 * KROW, RAW_K = RAW_KC + 4 * D;  // a key warp's codes (32 tokens) and parameters
-  static constexpr int RAW_VC = (D / 4) * 8 * BV, RAW_V = RAW_VC + 4 * (64 * NG + 16);
-  static constexpr int RAW = RAW_K > RAW_V ? RAW_K : RAW_V;     // of one warp and stage
+  // raw data of a key warp (16 tokens: codes, their group's parameters) and of a value warp (D / 4 channels: codes,
+  // the tile's parameters with 16 bytes more after every four tokens)
+  static constexpr int RAW_KC = 16 * KROW, RAW_K = RAW_KC + 4 * D;
+  static constexpr int RAW_VC = (D / 4) * 8 * BV, V_QUAD = 16 * NG + 16, RAW_V = RAW_VC + CT / 4 * V_QUAD;
   static constexpr int OFF_RAW = OFF_V + VBUFS * 2 * MAT;
-  static constexpr int TOTAL = OFF_RAW + C_EXPAND * C_STAGES * RAW;
+  static constexpr int TOTAL = OFF_RAW + 4 * C_STAGES * (RAW_K + RAW_V);
   // tensor memory columns: q, S and numerators of even and odd tiles, O
   static constexpr uint32_t COL_Q = 0, COL_S = 64, COL_O = 192;
   static_assert(TOTAL <= 226 * 1024, "shared memory");
@@ -120,34 +124,54 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
   lo = pack_io2<true>(a - io2_lo<true>(hi), b - io2_hi<true>(hi));
 }
 
-// 16 codes of a packed word (`w` shifted so that the codes 4 e + j sit at bit BITS * e of byte j) with the parameters
-// s, z of each, as fp16 pairs: element k's hi and lo in hi[k / 2], lo[k / 2].
+// The values that the codes 0 .. 3 of a group stand for, c s + z (s and z in units of the expanded tile), as fp16
+// pairs: hi[c / 2], lo[c / 2].
+struct Table {
+  uint32_t hi[2], lo[2];
+};
+__device__ __forceinline__ Table make_table(float s, float z) {
+  Table t;
+  split2(z, z + s, t.hi[0], t.lo[0]);
+  split2(fmaf(2.f, s, z), fmaf(3.f, s, z), t.hi[1], t.lo[1]);
+  return t;
+}
+// One 4 x 8 block of an expanded matrix: byte j of the words w[k] >> sh holds the code of row j, position k.  Four
+// codes make a selector of two byte permutations (code c selects the bytes 2 c and 2 c + 1 of the table), so an element
+// takes three instructions for its hi and lo.
 template <int BITS>
-__device__ __forceinline__ void expand16(uint32_t w, const float (&s)[16], const float (&z)[16], uint32_t (&hi)[8],
-                                         uint32_t (&lo)[8]) {
+__device__ __forceinline__ void expand_block(const uint32_t (&w)[8], int sh, const Table (&t)[4], uint32_t dst, uint32_t lo_off) {
+  uint32_t c[2][4];  // codes of four positions of row j
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const uint32_t m = (w >> (BITS * e)) & (BITS == 2 ? 0x03030303u : 0x01010101u);
-    float v[4];
+  for (int h = 0; h < 2; ++h) {
+    uint32_t m[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float c = __uint_as_float(__byte_perm(m, 0x4B000000u, 0x7440 + j)) - 8388608.f;  // 2^23 + code, less 2^23
-      v[j] = fmaf(c, s[4 * e + j], z[4 * e + j]);
-    }
-    split2(v[0], v[1], hi[2 * e], lo[2 * e]);
-    split2(v[2], v[3], hi[2 * e + 1], lo[2 * e + 1]);
+    for (int k = 0; k < 4; ++k) m[k] = (w[4 * h + k] >> sh) & (BITS == 2 ? 0x03030303u : 0x01010101u);
+    const uint32_t a0 = __byte_perm(m[0], m[1], 0x5140), a1 = __byte_perm(m[2], m[3], 0x5140);
+    const uint32_t b0 = __byte_perm(m[0], m[1], 0x7362), b1 = __byte_perm(m[2], m[3], 0x7362);
+    c[h][0] = __byte_perm(a0, a1, 0x5410); c[h][1] = __byte_perm(a0, a1, 0x7632);
+    c[h][2] = __byte_perm(b0, b1, 0x5410); c[h][3] = __byte_perm(b0, b1, 0x7632);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t s0 = c[0][j] * 0x22u + 0x10101010u, s1 = c[1][j] * 0x22u + 0x10101010u;
+    const uint32_t u0 = s0 >> 16, u1 = s1 >> 16;
+    sts128(dst + 16 * j, __byte_perm(t[j].hi[0], t[j].hi[1], s0), __byte_perm(t[j].hi[0], t[j].hi[1], u0),
+           __byte_perm(t[j].hi[0], t[j].hi[1], s1), __byte_perm(t[j].hi[0], t[j].hi[1], u1));
+    sts128(dst + lo_off + 16 * j, __byte_perm(t[j].lo[0], t[j].lo[1], s0), __byte_perm(t[j].lo[0], t[j].lo[1], u0),
+           __byte_perm(t[j].lo[0], t[j].lo[1], s1), __byte_perm(t[j].lo[0], t[j].lo[1], u1));
   }
 }
-__device__ __forceinline__ void store16(uint32_t a, uint32_t lbo, uint32_t mat, const uint32_t (&hi)[8], const uint32_t (&lo)[8]) {
+// eight fp32 values as hi and lo rows of 16 bytes
+__device__ __forceinline__ void store_row(const float (&v)[8], uint32_t dst, uint32_t lo_off) {
+  uint32_t hi[4], lo[4];
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {  // the two 16-byte pieces of 16 elements, of the hi and of the lo matrix
-    sts128(a + i * lbo, hi[4 * i], hi[4 * i + 1], hi[4 * i + 2], hi[4 * i + 3]);
-    sts128(a + i * lbo + mat, lo[4 * i], lo[4 * i + 1], lo[4 * i + 2], lo[4 * i + 3]);
-  }
+  for (int k = 0; k < 4; ++k) split2(v[2 * k], v[2 * k + 1], hi[k], lo[k]);
+  sts128(dst, hi[0], hi[1], hi[2], hi[3]);
+  sts128(dst + lo_off, lo[0], lo[1], lo[2], lo[3]);
 }
-__device__ __forceinline__ void scale16(float (&x)[16], float f) {
-#pragma unroll
-  for (int k = 0; k < 16; ++k) x[k] *= f;
+// 2^e that puts mx below 2^15 and, unless it is there already, above 2^14
+__device__ __forceinline__ int key_exponent(float mx) {
+  return mx >= 1.f && mx < 32768.f ? 0 : (mx > 0.f ? 14 - exponent_of(mx) : 0);
 }
 
 template <int D, int BK, int BV, int GS>
@@ -259,6 +283,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
   if (warp == 8 + C_EXPAND) {
     // ================= products: the loop is warp-uniform, one elected lane issues =================
     constexpr uint32_t IDK = idesc_f16(CT), IDV = idesc_f16(D);
+    constexpr uint32_t KSTEP = 2 * Pl::CORE / 16;  // descriptor units per 16 rows of K
     // (uniform values: the issue of a product then takes no moves between register files)
     const uint32_t tb = __shfl_sync(0xffffffffu, tbase, 0), smu = __shfl_sync(0xffffffffu, sm, 0);
 #pragma unroll 1
@@ -269,11 +294,11 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         tc_fence_after();
         if (ok && elect_one()) {
           const uint32_t base = smu + (i & 1) * 2 * Pl::MAT, dS = tb + Pl::COL_S + (i & 1) * 64;
-          const uint64_t kh = smem_desc(base, 128, Pl::K_SBO), kl = smem_desc(base + Pl::MAT, 128, Pl::K_SBO);
+          const uint64_t kh = smem_desc(base, Pl::CORE, Pl::K_SBO), kl = smem_desc(base + Pl::MAT, Pl::CORE, Pl::K_SBO);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks) {
-            umma_f16(dS, tb + Pl::COL_Q + 8 * ks, kh + 16 * ks, IDK, ks > 0);
-            umma_f16(dS, tb + Pl::COL_Q + 8 * ks, kl + 16 * ks, IDK, true);
+            umma_f16(dS, tb + Pl::COL_Q + 8 * ks, kh + KSTEP * ks, IDK, ks > 0);
+            umma_f16(dS, tb + Pl::COL_Q + 8 * ks, kl + KSTEP * ks, IDK, true);
           }
           umma_commit(bar_s + 8 * (i & 1));
           umma_commit(bar_kfree + 8 * (i & 1));
@@ -288,12 +313,12 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         if (ok && elect_one()) {
           const uint32_t base = smu + Pl::OFF_V + (j % 3) * 2 * Pl::MAT;
           const uint32_t ph = tb + Pl::COL_S + (j & 1) * 64, pl = ph + 32, dO = tb + Pl::COL_O;
-          const uint64_t vh = smem_desc(base, 128, Pl::V_SBO), vl = smem_desc(base + Pl::MAT, 128, Pl::V_SBO);
+          const uint64_t vh = smem_desc(base, Pl::CORE, Pl::V_SBO), vl = smem_desc(base + Pl::MAT, Pl::CORE, Pl::V_SBO);
 #pragma unroll
           for (int ks = 0; ks < CT / 16; ++ks) {
-            umma_f16(dO, ph + 8 * ks, vh + 16 * ks, IDV, j > 0 || ks > 0);
-            umma_f16(dO, ph + 8 * ks, vl + 16 * ks, IDV, true);
-            umma_f16(dO, pl + 8 * ks, vh + 16 * ks, IDV, true);
+            umma_f16(dO, ph + 8 * ks, vh + KSTEP * ks, IDV, j > 0 || ks > 0);
+            umma_f16(dO, ph + 8 * ks, vl + KSTEP * ks, IDV, true);
+            umma_f16(dO, pl + 8 * ks, vh + KSTEP * ks, IDV, true);
           }
           umma_commit(bar_o);
           umma_commit(bar_vfree + 8 * (j % 3));
@@ -423,41 +448,51 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
     l_sm[w][r] = l;
     ml_sm[w][r] = ml;
   } else {
-    // ================= expansion: keys (warps 8 .. 11: 32 tokens x half of the channels), values (12 .. 15) ==========
+    // ================= expansion: keys (warps 8 .. 11: 16 tokens each), values (12 .. 15: D / 4 channels each) =========
     const int ew = warp - 8;
-    const uint32_t raw = sm + Pl::OFF_RAW + ew * C_STAGES * Pl::RAW;
+    const bool keys = ew < 4;
+    const uint32_t raw = sm + Pl::OFF_RAW + (keys ? ew * C_STAGES * Pl::RAW_K : C_STAGES * (4 * Pl::RAW_K + (ew - 4) * Pl::RAW_V));
     const int n_pk = min(t_hi, pk_tiles);
-    // Raw data of packed tile `t` that this warp expands, into its own stage; one commit per call
-    const int kg = ew >> 1, hc = ew & 1, c0 = (ew & 3) * DQ;
-    const uint8_t* const g_code = ew < 4
+    const int c0 = (ew & 3) * DQ;  // value warps: first channel
+    const uint8_t* const g_code = keys
         ? reinterpret_cast<const uint8_t*>(p.L.k_codes) + (size_t)bh * ((size_t)dm.nq_cap * Pl::KROW)
         : reinterpret_cast<const uint8_t*>(p.L.v_codes) + (size_t)bh * ((size_t)dm.nq_cap * (D * BV / 8));
-    const uint8_t* const g_meta = ew < 4
+    const uint8_t* const g_meta = keys
         ? reinterpret_cast<const uint8_t*>(p.L.k_meta) + (size_t)bh * ((size_t)(dm.nq_cap / GS) * 4 * D)
         : reinterpret_cast<const uint8_t*>(p.L.v_meta) + (size_t)bh * ((size_t)dm.nq_cap * 4 * NG);
-    auto fetch = [&](int t) {
+    // Raw data of packed tile t_lo + i that this warp expands, into its own stage; one commit per call
+    auto fetch = [&](int i) {
+      const int t = t_lo + i;
       if (t < n_pk) {
-        const uint32_t dst = raw + (t % C_STAGES) * Pl::RAW;
-        if (ew < 4) {
-          const int tok = t * CT + 32 * kg;
-          if (lane < Pl::RAW_KC / 16)
-            cp_async16(dst + lane * 16, g_code + (size_t)(tok / 32) * (32 * Pl::KROW) + (Pl::KROW == 32 ? hc * 512 : 0) + lane * 16);
+        if (keys) {
+          const uint32_t dst = raw + (i % C_STAGES) * Pl::RAW_K;
+          const int tok = t * CT + 16 * ew;
+          const uint8_t* src = g_code + (size_t)(tok / 32) * (32 * Pl::KROW);
+          if (lane < Pl::KROW) {  // 16 tokens x KROW bytes in 16-byte pieces
+            if constexpr (Pl::KROW == 32) cp_async16(dst + lane * 16, src + (lane >> 4) * 512 + (tok % 32 + (lane & 15)) * 16);
+            else cp_async16(dst + lane * 16, src + (tok % 32) * Pl::KROW + lane * 16);
+          }
           if (lane < D / 4) cp_async16(dst + Pl::RAW_KC + lane * 16, g_meta + (size_t)(tok / GS) * (4 * D) + lane * 16);
         } else {
+          const uint32_t dst = raw + (i % C_STAGES) * Pl::RAW_V;
           const uint8_t* src = g_code + (size_t)(t / 2) * (D * 16 * BV);
           if (lane < DQ) {
             if constexpr (BV == 2) cp_async16(dst + lane * 16, src + (t & 1) * (D * 16) + (c0 + lane) * 16);
             else cp_async8(dst + lane * 8, src + (c0 + lane) * 16 + (t & 1) * 8);
           }
-          for (int i = lane; i < CT * 4 * NG / 16; i += 32)  // 16 bytes more after every 16 tokens (banks)
-            cp_async16(dst + Pl::RAW_VC + i * 16 + i / (4 * NG) * 16, g_meta + (size_t)t * (CT * 4 * NG) + i * 16);
+#pragma unroll
+          for (int k = 0; k < (CT * NG / 4 + 31) / 32; ++k) {
+            const int x = lane + 32 * k;
+            if (x < CT * NG / 4) cp_async16(dst + Pl::RAW_VC + x * 16 + x / NG * 16, g_meta + (size_t)t * (CT * 4 * NG) + x * 16);
+          }
         }
       }
       cp_async_commit();
     };
-    constexpr int UPW = D / 32, TP = 32 / UPW;       // keys: 16-channel units of a warp, tokens of a pass
-    const int k_tok = lane % TP, k_u = hc * UPW + lane / TP;
-    const int v_c = lane & 7, v_u = lane >> 3;       // values: channel of a pass, 16 tokens
+    // keys: this lane's four channels 4 k_q .. and its blocks of 8 tokens; values: four tokens 4 v_q .. and 8 channels
+    const int k_q = lane % (D / 4), k_b = lane / (D / 4), v_q = lane & 15, v_h = lane >> 4;
+    constexpr int KB = D / 64;  // blocks of a lane: 2 (D = 128) or 1
+    const uint32_t k_dst = (k_q >> 1) * Pl::CORE + (k_q & 1) * 64, v_dst = (v_q >> 1) * Pl::CORE + (v_q & 1) * 64;
     int ev = 0;
     bool ev_set = false;
     // exponent of the values in use: the largest |v| times 2^ev in [2^4, 2^14); it moves only outside that
@@ -468,144 +503,146 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         ev = 9 - em;
         ev_set = true;
       }
+      return pow2i(ev);
     };
-    fetch(t_lo);
-    fetch(t_lo + 1);
+    fetch(0);
+    fetch(1);
 #pragma unroll 1
     for (int i = 0; i < N; ++i) {
       const int t = t_lo + i;
-      cp_async_wait<1>();
+      fetch(i + 2);
+      cp_async_wait<2>();
       __syncwarp();
-      fetch(t + 2);
-      if (ew < 4) {
+      if (keys) {
         if (i >= 2 && !__all_sync(0xffffffffu, mbar_wait(bar_kfree + 8 * (i & 1), ((i >> 1) - 1) & 1, &dead_sm))) break;
       } else {
         if (i >= 3 && !__all_sync(0xffffffffu, mbar_wait(bar_vfree + 8 * (i % 3), (i / 3 - 1) & 1, &dead_sm))) break;
       }
-      const uint32_t src = raw + (t % C_STAGES) * Pl::RAW;
-      const uint32_t dst = sm + (ew < 4 ? (i & 1) * 2 * Pl::MAT : Pl::OFF_V + (i % 3) * 2 * Pl::MAT);
-      if (t < n_pk) {
-        float s[16], z[16];
-        float mx = 0.f;
-        if (ew < 4) {  // n_q % 32 == 0: the 32 tokens exist or do not together
-          const bool exists = t * CT + 32 * kg < p.n_q;
-          // the largest |k| of the group, all channels: this lane looks at channels lane, lane + 32, ...
-          float top = 0.f, low = 0.f;
+      if (keys) {
+        const uint32_t src = raw + (i % C_STAGES) * Pl::RAW_K, dst = sm + (i & 1) * 2 * Pl::MAT + 2 * ew * Pl::K_SBO + k_dst;
+        if (t < n_pk) {
+          const bool exists = t * CT + 16 * ew < p.n_q;  // n_q % 32 == 0: the 16 tokens exist or do not together
+          float s[4], z[4], mx = 0.f;
 #pragma unroll
-          for (int k = 0; k < D / 32; ++k) {
-            top = fmaxf(top, f16_to_f(lds16(src + Pl::RAW_KC + 2 * (lane * (D / 32) + k))));
-            low = fmaxf(low, fabsf(f16_to_f(lds16(src + Pl::RAW_KC + 2 * D + 2 * (lane * (D / 32) + k)))));
+          for (int j = 0; j < 4; ++j) {
+            const int d = 4 * k_q + j;
+            const uint32_t a = src + Pl::RAW_KC + 2 * ((d % 32) * (D / 32) + d / 32);
+            s[j] = exists ? f16_to_f(lds16(a)) : 0.f;
+            z[j] = exists ? f16_to_f(lds16(a + 2 * D)) : 0.f;
+            mx = fmaxf(mx, fmaf((float)((1 << BK) - 1), s[j], fabsf(z[j])));
           }
-          mx = exists ? fmaf((float)((1 << BK) - 1), top, low) : 0.f;
           mx = __uint_as_float(redux_max_u32(__float_as_uint(mx)));
-          const int e = mx >= 1.f && mx < 32768.f ? 0 : (mx > 0.f ? 14 - exponent_of(mx) : 0);
-          if (lane == 0) k_unit[i & 3][kg] = pow2i(-e);  // (both halves write the same)
-          const uint32_t meta = src + Pl::RAW_KC + 2 * ((k_u & 1) * 16 * (D / 32) + (k_u >> 1));
+          const int e = key_exponent(mx);
+          if (lane == 0) k_unit[i & 3][ew >> 1] = pow2i(-e);  // (two warps of a group write the same)
+          const float f = pow2i(e);
+          Table tab[4];
 #pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            s[k] = exists ? f16_to_f(lds16(meta + 2 * k * (D / 32))) : 0.f;
-            z[k] = exists ? f16_to_f(lds16(meta + 2 * D + 2 * k * (D / 32))) : 0.f;
-          }
-          if (e != 0) {
-            scale16(s, pow2i(e));
-            scale16(z, pow2i(e));
-          }
+          for (int j = 0; j < 4; ++j) tab[j] = make_table(s[j] * f, z[j] * f);
+          constexpr int QW = 8 / BK;  // channel quads of a word
+          const int word = k_q / QW, sh = BK * (k_q % QW);
+          const uint32_t wsrc = src + (Pl::KROW == 32 ? (word >> 2) * 256 + (word & 3) * 4 : word * 4);
           constexpr int RS = Pl::KROW < 16 ? Pl::KROW : 16;
 #pragma unroll 1
-          for (int k = 0; k < 32 / TP; ++k) {
-            const int tl = k_tok + TP * k, tok = 32 * kg + tl;
-            uint32_t wd;
-            if constexpr (BK == 2) wd = lds32(src + tl * RS + (Pl::KROW == 32 ? (k_u & 3) : k_u) * 4);
-            else wd = lds32(src + tl * RS + (k_u >> 1) * 4) >> (4 * (k_u & 1));
-            uint32_t hi[8], lo[8];
-            expand16<BK>(wd, s, z, hi, lo);
-            store16(dst + (tok >> 3) * Pl::K_SBO + 2 * k_u * 128 + (tok & 7) * 16, 128, Pl::MAT, hi, lo);
+          for (int k = 0; k < KB; ++k) {
+            const int blk = KB == 2 ? k : k_b;
+            uint32_t w[8];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) w[x] = lds32(wsrc + (8 * blk + x) * RS);
+            expand_block<BK>(w, sh, tab, dst + blk * Pl::K_SBO, Pl::MAT);
           }
         } else {
-          const bool exists = t * CT + 16 * v_u < p.n_q;
-          const uint32_t meta = src + Pl::RAW_VC + v_u * (64 * NG + 16) + 2 * (c0 / GS);
-#pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            s[k] = exists ? f16_to_f(lds16(meta + k * 4 * NG)) : 0.f;
-            z[k] = exists ? f16_to_f(lds16(meta + k * 4 * NG + 2 * NG)) : 0.f;
-            mx = fmaxf(mx, fmaf((float)((1 << BV) - 1), s[k], fabsf(z[k])));
-          }
-          value_exponent(mx);
-          if (lane == 0) v_exp[i & 3][ew & 3] = ev;
-          scale16(s, pow2i(ev));
-          scale16(z, pow2i(ev));
+          // a window tile: 16-bit rows as they are, split into pairs (exact for inputs of ordinary magnitude)
+          const int w0 = (t - pk_tiles) * CT;
+          const uint2* rows = reinterpret_cast<const uint2*>(p.L.win_k + (size_t)bh * dm.R * D) + k_q;
+          const int r0 = w0 + 32 * (ew >> 1);
+          float mx = 0.f;
 #pragma unroll 1
-          for (int k = 0; k < D / 32; ++k) {
-            const int cl = v_c + 8 * k, c = c0 + cl;
-            uint32_t wd;
-            if constexpr (BV == 2) wd = lds32(src + cl * 16 + v_u * 4);
-            else wd = lds32(src + cl * 8 + (v_u >> 1) * 4) >> (4 * (v_u & 1));
-            uint32_t hi[8], lo[8];
-            expand16<BV>(wd, s, z, hi, lo);
-            store16(dst + (c >> 3) * Pl::V_SBO + 2 * v_u * 128 + (c & 7) * 16, 128, Pl::MAT, hi, lo);
+          for (int x = k_b; x < 32; x += 128 / D) {  // the unit is that of 32 tokens
+            const uint2 v = r0 + x < p.r ? rows[(size_t)(r0 + x) * (D / 4)] : make_uint2(0u, 0u);
+            mx = fmaxf(mx, fmaxf(fmaxf(fabsf(io_to_f(v.x & 0xffffu, p.f16)), fabsf(io_to_f(v.x >> 16, p.f16))),
+                                 fmaxf(fabsf(io_to_f(v.y & 0xffffu, p.f16)), fabsf(io_to_f(v.y >> 16, p.f16)))));
+          }
+          mx = __uint_as_float(redux_max_u32(__float_as_uint(mx)));
+          const int e = key_exponent(mx);
+          if (lane == 0) k_unit[i & 3][ew >> 1] = pow2i(-e);
+          const float f = pow2i(e);
+#pragma unroll 1
+          for (int k = 0; k < KB; ++k) {
+            const int blk = KB == 2 ? k : k_b, r1 = w0 + 16 * ew + 8 * blk;
+            float v[4][8];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) {
+              const uint2 u = r1 + x < p.r ? rows[(size_t)(r1 + x) * (D / 4)] : make_uint2(0u, 0u);
+              v[0][x] = io_to_f(u.x & 0xffffu, p.f16) * f; v[1][x] = io_to_f(u.x >> 16, p.f16) * f;
+              v[2][x] = io_to_f(u.y & 0xffffu, p.f16) * f; v[3][x] = io_to_f(u.y >> 16, p.f16) * f;
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) store_row(v[j], dst + blk * Pl::K_SBO + 16 * j, Pl::MAT);
           }
         }
       } else {
-        // a window tile: 16-bit rows as they are, split into pairs (exact for inputs of ordinary magnitude)
-        const int w0 = (t - pk_tiles) * CT;
-        if (ew < 4) {
-          const uint8_t* rows = reinterpret_cast<const uint8_t*>(p.L.win_k) + (size_t)bh * dm.R * (2 * D);
-          float mx = 0.f;
-#pragma unroll 4
-          for (int k = 0; k < 32; ++k) {  // all channels of the 32 tokens
-            if (w0 + 32 * kg + k < p.r && lane < D / 4) {
-              const uint2 v = reinterpret_cast<const uint2*>(rows + (size_t)(w0 + 32 * kg + k) * (2 * D))[lane];
-              mx = fmaxf(mx, fmaxf(fmaxf(fabsf(io_to_f(v.x & 0xffffu, p.f16)), fabsf(io_to_f(v.x >> 16, p.f16))),
-                                   fmaxf(fabsf(io_to_f(v.y & 0xffffu, p.f16)), fabsf(io_to_f(v.y >> 16, p.f16)))));
-            }
+        const uint32_t src = raw + (i % C_STAGES) * Pl::RAW_V;
+        const uint32_t dst = sm + Pl::OFF_V + (i % 3) * 2 * Pl::MAT + (c0 + v_h * (DQ / 2)) / 8 * Pl::V_SBO + v_dst;
+        if (t < n_pk) {
+          const bool exists = t * CT + 4 * v_q < p.n_q;
+          float s[4], z[4], mx = 0.f;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint32_t a = src + Pl::RAW_VC + v_q * Pl::V_QUAD + j * 4 * NG + 2 * (c0 / GS);
+            s[j] = exists ? f16_to_f(lds16(a)) : 0.f;
+            z[j] = exists ? f16_to_f(lds16(a + 2 * NG)) : 0.f;
+            mx = fmaxf(mx, fmaf((float)((1 << BV) - 1), s[j], fabsf(z[j])));
           }
-          mx = __uint_as_float(redux_max_u32(__float_as_uint(mx)));
-          const int e = mx >= 1.f && mx < 32768.f ? 0 : (mx > 0.f ? 14 - exponent_of(mx) : 0);
-          if (lane == 0) k_unit[i & 3][kg] = pow2i(-e);
-          const float f = pow2i(e);
+          const float f = value_exponent(mx);
+          if (lane == 0) v_exp[i & 3][ew & 3] = ev;
+          Table tab[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) tab[j] = make_table(s[j] * f, z[j] * f);
+          constexpr int QW = 8 / BV, RS = 8 * BV;  // token quads of a word; bytes of a channel
+          const uint32_t wsrc = src + v_h * (DQ / 2) * RS + v_q / QW * 4;
+          const int sh = BV * (v_q % QW);
 #pragma unroll 1
-          for (int k = 0; k < 32 / TP; ++k) {
-            const int tok = 32 * kg + k_tok + TP * k;
-            uint32_t hi[8], lo[8];
+          for (int k = 0; k < KB; ++k) {
+            uint32_t w[8];
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-              uint4 v = make_uint4(0u, 0u, 0u, 0u);
-              if (w0 + tok < p.r) v = reinterpret_cast<const uint4*>(rows + (size_t)(w0 + tok) * (2 * D))[2 * k_u + c];
-              const uint32_t x[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-                split2(io_to_f(x[j] & 0xffffu, p.f16) * f, io_to_f(x[j] >> 16, p.f16) * f, hi[4 * c + j], lo[4 * c + j]);
-            }
-            store16(dst + (tok >> 3) * Pl::K_SBO + 2 * k_u * 128 + (tok & 7) * 16, 128, Pl::MAT, hi, lo);
+            for (int x = 0; x < 8; ++x) w[x] = lds32(wsrc + (8 * k + x) * RS);
+            expand_block<BV>(w, sh, tab, dst + k * Pl::V_SBO, Pl::MAT);
           }
         } else {
-          const uint16_t* rows = p.L.win_v + (size_t)bh * dm.R * D;
+          const int w0 = (t - pk_tiles) * CT;
+          const uint4* rows = reinterpret_cast<const uint4*>(p.L.win_v + (size_t)bh * dm.R * D);
+          auto piece = [&](int tok, int c) {  // 8 channels of a window row
+            return w0 + tok < p.r ? rows[(size_t)(w0 + tok) * (D / 8) + c / 8] : make_uint4(0u, 0u, 0u, 0u);
+          };
           float mx = 0.f;
-#pragma unroll 4
-          for (int k = 0; k < CT; ++k)
-            if (w0 + k < p.r && lane < DQ) mx = fmaxf(mx, fabsf(io_to_f(rows[(size_t)(w0 + k) * D + c0 + lane], p.f16)));
-          value_exponent(mx);
-          if (lane == 0) v_exp[i & 3][ew & 3] = ev;
-          const float f = pow2i(ev);
 #pragma unroll 1
-          for (int k = 0; k < D / 32; ++k) {
-            const int c = c0 + v_c + 8 * k;
-            float v[16];
-            uint32_t hi[8], lo[8];
+          for (int x = 0; x < 4 * KB; ++x) {
+            const uint4 u = piece(4 * v_q + (x & 3), c0 + v_h * (DQ / 2) + 8 * (x >> 2));
+            const uint32_t y[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const int tok = w0 + 16 * v_u + j;
-              v[j] = tok < p.r ? io_to_f(rows[(size_t)tok * D + c], p.f16) * f : 0.f;
+            for (int k = 0; k < 4; ++k)
+              mx = fmaxf(mx, fmaxf(fabsf(io_to_f(y[k] & 0xffffu, p.f16)), fabsf(io_to_f(y[k] >> 16, p.f16))));
+          }
+          const float f = value_exponent(mx);
+          if (lane == 0) v_exp[i & 3][ew & 3] = ev;
+#pragma unroll 1
+          for (int x = 0; x < 4 * KB; ++x) {
+            const int j = x & 3, k = x >> 2;
+            const uint4 u = piece(4 * v_q + j, c0 + v_h * (DQ / 2) + 8 * k);
+            const uint32_t y[4] = {u.x, u.y, u.z, u.w};
+            float v[8];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              v[2 * c] = io_to_f(y[c] & 0xffffu, p.f16) * f;
+              v[2 * c + 1] = io_to_f(y[c] >> 16, p.f16) * f;
             }
-#pragma unroll
-            for (int j = 0; j < 8; ++j) split2(v[2 * j], v[2 * j + 1], hi[j], lo[j]);
-            store16(dst + (c >> 3) * Pl::V_SBO + 2 * v_u * 128 + (c & 7) * 16, 128, Pl::MAT, hi, lo);
+            store_row(v, dst + k * Pl::V_SBO + 16 * j, Pl::MAT);
           }
         }
       }
       proxy_fence();
       __syncwarp();
-      if (lane == 0) mbar_arrive(ew < 4 ? bar_kfull + 8 * (i & 1) : bar_vfull + 8 * (i % 3));
+      if (lane == 0) mbar_arrive(keys ? bar_kfull + 8 * (i & 1) : bar_vfull + 8 * (i % 3));
     }
     cp_async_wait_all();
   }
