@@ -5,12 +5,12 @@
 // to dequantize: eight warps expand a tile's keys and values once for all rows into fp16 pairs hi + lo in shared
 // memory (22 significant bits of c s + z, relative to the largest member of the group), the B operands of
 //
-//   S = Q K_hi + Q K_lo                          (A: q as fp16 in tensor memory; S: 64 columns, two buffers)
+//   S = Q K_hi + Q K_lo                          (A: q as fp16 in tensor memory; S: 64 columns, four buffers)
 //   O += P_hi V_hi + P_hi V_lo + P_lo V_hi       (A: the softmax numerators as fp16 pairs, over the columns of S)
 //
 // accumulated in fp32 in tensor memory.  Two groups of four warps (thread = row = tensor-memory lane) take the softmax
 // of the even and of the odd tiles; the softmax reference of a row goes from one to the other through shared memory
-// and is raised only when a logit exceeds it by more than 8 (log2 units), which rescales O (rare).  One warp issues the products: keys of tile i + 1,
+// and is raised only when a logit exceeds it by more than 8 (log2 units), which rescales O (rare).  One warp issues the products: keys of tile i + 2,
 // then values of tile i.  Tokens of the 16-bit window are expanded into the same pairs (exactly).  Split partials are
 // merged by the last CTA of a row tile, as in the decode kernel.
 //
@@ -106,8 +106,8 @@ struct ChunkPlan {
   static constexpr int RAW_VC = (D / 4) * 8 * BV, V_QUAD = 16 * NG + 16, RAW_V = RAW_VC + CT / 4 * V_QUAD;
   static constexpr int OFF_RAW = OFF_V + VBUFS * 2 * MAT;
   static constexpr int TOTAL = OFF_RAW + 4 * C_STAGES * (RAW_K + RAW_V);
-  // tensor memory columns: q, S and numerators of even and odd tiles, O
-  static constexpr uint32_t COL_Q = 0, COL_S = 64, COL_O = 192;
+  // tensor memory columns: q, S (then numerators) of four tiles, O
+  static constexpr uint32_t COL_Q = 0, COL_S = 64, COL_O = 320;
   static_assert(TOTAL <= 226 * 1024, "shared memory");
 };
 
@@ -179,8 +179,8 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
   using Pl = ChunkPlan<D, BK, BV, GS>;
   constexpr int NG = Pl::NG, DQ = D / 4;
   extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ __align__(8) unsigned long long bar_mem[24];
-  __shared__ float k_unit[4][2];            // [tile % 4][32 tokens]: what a unit of the expanded keys is worth
+  __shared__ __align__(8) unsigned long long bar_mem[39];
+  __shared__ float k_unit[8][2];            // [tile % 8][32 tokens]: what a unit of the expanded keys is worth
   __shared__ int v_exp[4][4];               // [tile % 4][channel quarter]: the expanded values are times 2^v_exp
   __shared__ float cq_sm[CM], m_sm[CM];     // logits from products of the scaled q; softmax reference (-infinity: none)
   __shared__ float l_sm[2][CM], ml_sm[2][CM];
@@ -209,29 +209,36 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
   const uint32_t bar_kfree = bar_kfull + 16;   // [2] their buffer may be written again
   const uint32_t bar_vfull = bar_kfree + 16;   // [3] the same of the values
   const uint32_t bar_vfree = bar_vfull + 24;   // [3]
-  const uint32_t bar_s = bar_vfree + 24;       // [2] S is complete
-  const uint32_t bar_p = bar_s + 16;           // [2] the numerators are written
-  const uint32_t bar_o = bar_p + 16;           // the value products of a tile are complete
-  const uint32_t bar_turn = bar_o + 8;         // [4 warps][2] a row's reference for an even / odd tile is there
-  const uint32_t bar_end = bar_turn + 64;      // every product that was issued is complete (after a wait gave up)
+  const uint32_t bar_s = bar_vfree + 24;       // [4] S is complete
+  const uint32_t bar_p = bar_s + 32;           // [4] the numerators are written
+  const uint32_t bar_o = bar_p + 32;           // [4] the value products of a tile are complete
+  const uint32_t bar_turn = bar_o + 32;        // [4 warps][2] a row's reference for an even / odd tile is there
+  const uint32_t bar_unit = bar_turn + 64;     // [8] the units of a tile's keys are written
+  const uint32_t bar_end = bar_unit + 64;      // every product that was issued is complete (after a wait gave up)
 
   if (tid == 0) {
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar_kfull + 8 * i, C_EXPAND / 2);
       mbar_init(bar_kfree + 8 * i, 1);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
       mbar_init(bar_s + 8 * i, 1);
       mbar_init(bar_p + 8 * i, 4);
+      mbar_init(bar_o + 8 * i, 1);
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       mbar_init(bar_vfull + 8 * i, C_EXPAND / 2);
       mbar_init(bar_vfree + 8 * i, 1);
     }
-    mbar_init(bar_o, 1);
     mbar_init(bar_end, 1);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) mbar_init(bar_turn + 8 * i, 1);
+    for (int i = 0; i < 8; ++i) {
+      mbar_init(bar_turn + 8 * i, 1);
+      mbar_init(bar_unit + 8 * i, C_EXPAND / 2);
+    }
     dead_sm = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
@@ -286,33 +293,34 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
     constexpr uint32_t KSTEP = 2 * Pl::CORE / 16;  // descriptor units per 16 rows of K
     // (uniform values: the issue of a product then takes no moves between register files)
     const uint32_t tb = __shfl_sync(0xffffffffu, tbase, 0), smu = __shfl_sync(0xffffffffu, sm, 0);
+    // keys of tile i + 2 go out before the values of tile i: either softmax group finds its next S complete
 #pragma unroll 1
-    for (int i = 0; i <= N; ++i) {
+    for (int i = 0; i < N + 2; ++i) {
       bool ok = true;
       if (i < N) {
         ok = __all_sync(0xffffffffu, mbar_wait(bar_kfull + 8 * (i & 1), (i >> 1) & 1, &dead_sm));
         tc_fence_after();
         if (ok && elect_one()) {
-          const uint32_t base = smu + (i & 1) * 2 * Pl::MAT, dS = tb + Pl::COL_S + (i & 1) * 64;
+          const uint32_t base = smu + (i & 1) * 2 * Pl::MAT, dS = tb + Pl::COL_S + (i & 3) * 64;
           const uint64_t kh = smem_desc(base, Pl::CORE, Pl::K_SBO), kl = smem_desc(base + Pl::MAT, Pl::CORE, Pl::K_SBO);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks) {
             umma_f16(dS, tb + Pl::COL_Q + 8 * ks, kh + KSTEP * ks, IDK, ks > 0);
             umma_f16(dS, tb + Pl::COL_Q + 8 * ks, kl + KSTEP * ks, IDK, true);
           }
-          umma_commit(bar_s + 8 * (i & 1));
+          umma_commit(bar_s + 8 * (i & 3));
           umma_commit(bar_kfree + 8 * (i & 1));
         }
         __syncwarp();
       }
-      if (ok && i > 0) {
-        const int j = i - 1;
+      if (ok && i >= 2) {
+        const int j = i - 2;
         ok = __all_sync(0xffffffffu, mbar_wait(bar_vfull + 8 * (j % 3), (j / 3) & 1, &dead_sm) &&
-                                         mbar_wait(bar_p + 8 * (j & 1), (j >> 1) & 1, &dead_sm));
+                                         mbar_wait(bar_p + 8 * (j & 3), (j >> 2) & 1, &dead_sm));
         tc_fence_after();
         if (ok && elect_one()) {
           const uint32_t base = smu + Pl::OFF_V + (j % 3) * 2 * Pl::MAT;
-          const uint32_t ph = tb + Pl::COL_S + (j & 1) * 64, pl = ph + 32, dO = tb + Pl::COL_O;
+          const uint32_t ph = tb + Pl::COL_S + (j & 3) * 64, pl = ph + 32, dO = tb + Pl::COL_O;
           const uint64_t vh = smem_desc(base, Pl::CORE, Pl::V_SBO), vl = smem_desc(base + Pl::MAT, Pl::CORE, Pl::V_SBO);
 #pragma unroll
           for (int ks = 0; ks < CT / 16; ++ks) {
@@ -320,7 +328,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
             umma_f16(dO, ph + 8 * ks, vl + KSTEP * ks, IDV, true);
             umma_f16(dO, pl + 8 * ks, vh + KSTEP * ks, IDV, true);
           }
-          umma_commit(bar_o);
+          umma_commit(bar_o + 8 * (j & 3));
           umma_commit(bar_vfree + 8 * (j % 3));
         }
         __syncwarp();
@@ -344,15 +352,18 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
 #pragma unroll 1
     for (int i = w; i < N; i += 2) {
       // (the units and exponents of the expanded tile are there since the first two; the third one is the wait)
-      if (!__all_sync(0xffffffffu, mbar_wait(bar_kfull + 8 * (i & 1), (i >> 1) & 1, &dead_sm) &&
+      // (Phases: the keys run up to four tiles ahead of this one and the values up to two, so that neither the eight
+      // unit barriers nor the three of the values can be a whole round ahead of the parity that is asked for; S of
+      // this tile being complete, so are the value products of the tile three before.)
+      if (!__all_sync(0xffffffffu, mbar_wait(bar_unit + 8 * (i & 7), (i >> 3) & 1, &dead_sm) &&
                                        mbar_wait(bar_vfull + 8 * (i % 3), (i / 3) & 1, &dead_sm) &&
-                                       mbar_wait(bar_s + 8 * (i & 1), (i >> 1) & 1, &dead_sm)))
+                                       mbar_wait(bar_s + 8 * (i & 3), (i >> 2) & 1, &dead_sm)))
         break;
       tc_fence_after();
-      const uint32_t s_t = row_t + Pl::COL_S + (i & 1) * 64;
+      const uint32_t s_t = row_t + Pl::COL_S + (i & 3) * 64;
       uint32_t s[2][32];
       float m = -CUDART_INF_F;
-      const float u0 = k_unit[i & 3][0] * cq, u1 = k_unit[i & 3][1] * cq;
+      const float u0 = k_unit[i & 7][0] * cq, u1 = k_unit[i & 7][1] * cq;
       const int t = t_lo + i;
       // columns below n_valid are tokens that exist and that this row sees
       const int n_valid = t < pk_tiles ? min(vis, p.n_q) - t * CT : vis - p.n_q - (t - pk_tiles) * CT;
@@ -385,7 +396,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         if (__any_sync(0xffffffffu, change)) {
           m_sm[r] = m;
           if (i > 0) {  // O has to follow: after the products of the tile before, before those of this one
-            if (!__all_sync(0xffffffffu, mbar_wait(bar_o, (i - 1) & 1, &dead_sm))) break;
+            if (!__all_sync(0xffffffffu, mbar_wait(bar_o + 8 * ((i - 1) & 3), ((i - 1) >> 2) & 1, &dead_sm))) break;
             tc_fence_after();
             const float f = m_old == -CUDART_INF_F ? 0.f : ex2(m_old - m);
 #pragma unroll 1
@@ -443,7 +454,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar_p + 8 * (i & 1));
+      if (lane == 0) mbar_arrive(bar_p + 8 * (i & 3));
     }
     l_sm[w][r] = l;
     ml_sm[w][r] = ml;
@@ -533,7 +544,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
           }
           mx = __uint_as_float(redux_max_u32(__float_as_uint(mx)));
           const int e = key_exponent(mx);
-          if (lane == 0) k_unit[i & 3][ew >> 1] = pow2i(-e);  // (two warps of a group write the same)
+          if (lane == 0) k_unit[i & 7][ew >> 1] = pow2i(-e);  // (two warps of a group write the same)
           const float f = pow2i(e);
           Table tab[4];
 #pragma unroll
@@ -564,7 +575,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
           }
           mx = __uint_as_float(redux_max_u32(__float_as_uint(mx)));
           const int e = key_exponent(mx);
-          if (lane == 0) k_unit[i & 3][ew >> 1] = pow2i(-e);
+          if (lane == 0) k_unit[i & 7][ew >> 1] = pow2i(-e);
           const float f = pow2i(e);
 #pragma unroll 1
           for (int k = 0; k < KB; ++k) {
@@ -642,7 +653,10 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
       }
       proxy_fence();
       __syncwarp();
-      if (lane == 0) mbar_arrive(keys ? bar_kfull + 8 * (i & 1) : bar_vfull + 8 * (i % 3));
+      if (lane == 0) {
+        mbar_arrive(keys ? bar_kfull + 8 * (i & 1) : bar_vfull + 8 * (i % 3));
+        if (keys) mbar_arrive(bar_unit + 8 * (i & 7));
+      }
     }
     cp_async_wait_all();
   }
@@ -656,7 +670,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
     return ((size_t)j * dm.B + b) * dm.Hq + hk * G + h;
   };
   if (warp < 8) {
-    const bool ok = N == 0 || mbar_wait(bar_o, (N - 1) & 1, &dead_sm);
+    const bool ok = N == 0 || mbar_wait(bar_o + 8 * ((N - 1) & 3), ((N - 1) >> 2) & 1, &dead_sm);
     if (__all_sync(0xffffffffu, ok) && dead_sm == 0) {
       tc_fence_after();
       const int w = warp >> 2, r = tid & 127;

@@ -8,7 +8,7 @@
 
 namespace xq {
 
-constexpr int WAIT_LIMIT = 1 << 20;  // polls of a wait before it gives up
+constexpr int WAIT_LIMIT = 1 << 16;  // polls of a wait before it gives up (a poll is suspended for up to a millisecond or so)
 
 __device__ __forceinline__ float ex2(float x) {
   float y;
