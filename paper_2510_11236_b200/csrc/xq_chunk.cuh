@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) unsigned long long bar_mem[39];
   __shared__ float k_unit[8][2];            // [tile % 8][32 tokens]: what a unit of the expanded keys is worth
-  __shared__ int v_exp[4][4];               // [tile % 4][channel quarter]: the expanded values are times 2^v_exp
+  __shared__ __align__(16) int v_exp[4][4];               // [tile % 4][channel quarter]: the expanded values are times 2^v_exp
   __shared__ float cq_sm[CM], m_sm[CM];     // logits from products of the scaled q; softmax reference (-infinity: none)
   __shared__ float l_sm[2][CM], ml_sm[2][CM];
   __shared__ uint32_t tmem_base_sm;
@@ -320,13 +320,14 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         tc_fence_after();
         if (ok && elect_one()) {
           const uint32_t base = smu + Pl::OFF_V + (j % 3) * 2 * Pl::MAT;
-          const uint32_t ph = tb + Pl::COL_S + (j & 3) * 64, pl = ph + 32, dO = tb + Pl::COL_O;
+          const uint32_t pt = tb + Pl::COL_S + (j & 3) * 64, dO = tb + Pl::COL_O;
           const uint64_t vh = smem_desc(base, Pl::CORE, Pl::V_SBO), vl = smem_desc(base + Pl::MAT, Pl::CORE, Pl::V_SBO);
 #pragma unroll
           for (int ks = 0; ks < CT / 16; ++ks) {
-            umma_f16(dO, ph + 8 * ks, vh + KSTEP * ks, IDV, j > 0 || ks > 0);
-            umma_f16(dO, ph + 8 * ks, vl + KSTEP * ks, IDV, true);
-            umma_f16(dO, pl + 8 * ks, vh + KSTEP * ks, IDV, true);
+            const uint32_t ph = pt + 32 * (ks >> 1) + 8 * (ks & 1), pl = ph + 16;
+            umma_f16(dO, ph, vh + KSTEP * ks, IDV, j > 0 || ks > 0);
+            umma_f16(dO, ph, vl + KSTEP * ks, IDV, true);
+            umma_f16(dO, pl, vh + KSTEP * ks, IDV, true);
           }
           umma_commit(bar_o + 8 * (j & 3));
           umma_commit(bar_vfree + 8 * (j % 3));
@@ -361,37 +362,40 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         break;
       tc_fence_after();
       const uint32_t s_t = row_t + Pl::COL_S + (i & 3) * 64;
-      uint32_t s[2][32];
-      float m = -CUDART_INF_F;
-      const float u0 = k_unit[i & 7][0] * cq, u1 = k_unit[i & 7][1] * cq;
+      const float u[2] = {k_unit[i & 7][0] * cq, k_unit[i & 7][1] * cq};
       const int t = t_lo + i;
       // columns below n_valid are tokens that exist and that this row sees
       const int n_valid = t < pk_tiles ? min(vis, p.n_q) - t * CT : vis - p.n_q - (t - pk_tiles) * CT;
       if (!idle) {
-        tmem_ld32(s_t, s[0]);
-        tmem_ld32(s_t + 32, s[1]);
-        tc_wait_ld();
         const bool masked = __any_sync(0xffffffffu, n_valid < CT);
-        if (masked) {
+        // 32 columns of S at a time, here and below: the loops stay small (the instruction cache bounds this kernel)
+        auto load = [&](int c, uint32_t (&s)[32]) {
+          tmem_ld32(s_t + 32 * c, s);
+          tc_wait_ld();
+          if (masked) {
 #pragma unroll
-          for (int k = 0; k < 64; ++k)
-            if (k >= n_valid) s[k / 32][k % 32] = 0xff800000u;
-        }
-        float x0 = -CUDART_INF_F, x1 = -CUDART_INF_F;
+            for (int k = 0; k < 32; ++k)
+              if (32 * c + k >= n_valid) s[k] = 0xff800000u;
+          }
+        };
+        float xm = -CUDART_INF_F;
+#pragma unroll 1
+        for (int c = 0; c < 2; ++c) {
+          uint32_t s[32];
+          load(c, s);
+          float x = __uint_as_float(s[0]);
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {
-          x0 = fmaxf(x0, __uint_as_float(s[0][k]));
-          x1 = fmaxf(x1, __uint_as_float(s[1][k]));
+          for (int k = 1; k < 32; ++k) x = fmaxf(x, __uint_as_float(s[k]));
+          xm = fmaxf(xm, x * (c ? u[1] : u[0]));
         }
-        const float xm = fmaxf(x0 * u0, x1 * u1);
         if (i > 0 && !__all_sync(0xffffffffu, mbar_wait(bar_turn + 8 * (2 * q + (i & 1)), ((i - 1) >> 1) & 1, &dead_sm))) break;
         const float m_old = m_sm[r];
-        m = m_old;
+        float m = m_old;
         if (xm > m_old + C_TAU || (m_old == -CUDART_INF_F && xm > m_old)) m = ceilf(xm);
         bool change = m != m_old;
         if (i > 0) {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) change |= v_exp[i & 3][k] != v_exp[(i - 1) & 3][k];
+          const int4 e1 = *reinterpret_cast<const int4*>(v_exp[i & 3]), e0 = *reinterpret_cast<const int4*>(v_exp[(i - 1) & 3]);
+          change |= e1.x != e0.x || e1.y != e0.y || e1.z != e0.z || e1.w != e0.w;
         }
         if (__any_sync(0xffffffffu, change)) {
           m_sm[r] = m;
@@ -404,51 +408,37 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
               const int qa = c / DQ, qz = (c + 31) / DQ;  // the channel quarters of the columns' halves
               const float fa = f * pow2i(v_exp[i & 3][qa] - v_exp[(i - 1) & 3][qa]);
               const float fz = f * pow2i(v_exp[i & 3][qz] - v_exp[(i - 1) & 3][qz]);
-              tmem_ld32(row_t + Pl::COL_O + c, s[0]);
+              uint32_t s[32];
+              tmem_ld32(row_t + Pl::COL_O + c, s);
               tc_wait_ld();
 #pragma unroll
-              for (int k = 0; k < 32; ++k) s[0][k] = __float_as_uint(__uint_as_float(s[0][k]) * (k < 16 ? fa : fz));
-              tmem_st32(row_t + Pl::COL_O + c, s[0]);
+              for (int k = 0; k < 32; ++k) s[k] = __float_as_uint(__uint_as_float(s[k]) * (k < 16 ? fa : fz));
+              tmem_st32(row_t + Pl::COL_O + c, s);
             }
             tc_wait_st();
-          }
-          tmem_ld32(s_t, s[0]);
-          tmem_ld32(s_t + 32, s[1]);
-          tc_wait_ld();
-          if (masked) {
-#pragma unroll
-            for (int k = 0; k < 64; ++k)
-              if (k >= n_valid) s[k / 32][k % 32] = 0xff800000u;
           }
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_turn + 8 * (2 * q + ((i + 1) & 1)));
-        // numerators
+        // numerators: the 32 columns of S become 16 of hi and 16 of lo, two tokens in each
         const float off = m == -CUDART_INF_F ? 0.f : (float)C_PEXP - m;
         l *= m == ml ? 1.f : ex2(ml - m);
         ml = m;
-        float la = 0.f, lb = 0.f;
-#pragma unroll
+#pragma unroll 1
         for (int c = 0; c < 2; ++c) {
-          const float u = c ? u1 : u0;
+          uint32_t s[32], o[32];
+          load(c, s);
+          const float uc = c ? u[1] : u[0];
+          float la = 0.f, lb = 0.f;
 #pragma unroll
           for (int k = 0; k < 16; ++k) {
-            const float a = ex2(fmaf(__uint_as_float(s[c][2 * k]), u, off)), d = ex2(fmaf(__uint_as_float(s[c][2 * k + 1]), u, off));
+            const float a = ex2(fmaf(__uint_as_float(s[2 * k]), uc, off)), d = ex2(fmaf(__uint_as_float(s[2 * k + 1]), uc, off));
             la += a;
             lb += d;
-            uint32_t hi, lo;
-            split2(a, d, hi, lo);
-            s[c][2 * k] = hi;
-            s[c][2 * k + 1] = lo;
+            split2(a, d, o[k], o[16 + k]);
           }
-        }
-        l += la + lb;
-        uint32_t o[32];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {  // hi, then lo: two tokens per column
-#pragma unroll
-          for (int k = 0; k < 32; ++k) o[k] = s[k / 16][2 * (k % 16) + h];
-          tmem_st32(s_t + 32 * h, o);
+          l += la + lb;
+          tmem_st32(s_t + 32 * c, o);
         }
         tc_wait_st();
       }
