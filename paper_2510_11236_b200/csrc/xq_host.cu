@@ -453,7 +453,6 @@ int pack_layers(xq_cache* c, const int* layers, int n, const void* K, const void
   p.dm = dm;
   p.n_layers = n;
   p.n_in = n_tokens; p.s_old = s_old; p.nq_old = nq_old; p.n_blocks = (nq_new - nq_old) / dm.R;
-  p.tb = dm.g > 32 ? dm.g : 32;  // tokens per CTA: whole key groups, whole words of either kind
   p.f16 = c->cfg.io_dtype == XQ_F16;
   p.win_count = s_new - nq_new;
   p.nq_new = nq_new;

@@ -45,9 +45,8 @@ struct PackParams {
   int s_old;     // tokens cached before this append
   int nq_old;    // quantized tokens before this append
   int n_blocks;  // R-token blocks to quantize, starting at absolute token nq_old
-  int tb;        // tokens per CTA tile (32 or 64)
   int f16;       // inputs and window are IEEE half precision (else bfloat16)
-  // tokens nq_new .. s_new - 1 of the input go into window rows 0 .. win_count - 1 (the CTAs that staged those rows
+  // tokens nq_new .. s_new - 1 of the input go into window rows 0 .. win_count - 1 (the warps that read those rows
   // of the old window copy them); 0: the caller copies
   int win_count;
   int nq_new;
