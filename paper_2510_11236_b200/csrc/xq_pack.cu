@@ -1,12 +1,14 @@
 // Quantize-and-pack of residual-window blocks (Eq. 1, 2, 12; Algorithm 2) and
-// the window append.  One warp quantizes a tile of one (sequence, kv head) for keys or
-// for values.
+// the window append.  One CTA quantizes a tile of T (32 or 64) tokens x D channels of
+// one (sequence, kv head) for keys or for values.
 //
 // The fp32 arithmetic uses the *_rn intrinsics so that no multiply-add is ever
 // contracted: codes, scales and zero-points are compared bit for bit with a CPU
 // evaluation of the same formulas.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+
+#include <type_traits>
 
 #include "xq_internal.h"
 #include "xq_layout.cuh"
@@ -78,6 +80,7 @@ __device__ __forceinline__ void group_params(float mn, float mx, int bits, float
 }
 
 constexpr int PACK_THREADS = 128;
+constexpr int PACK_ROW_PAD = 16;  // bytes added to each staged row: 8 consecutive rows then fall in 8 different bank groups
 
 // 1/s for the quotient sequence of `quotient`: 0 for a constant group (every code 0), NaN where that sequence is
 // not known to round correctly -- a scale whose significand is all ones, or one so small or large that an
@@ -93,9 +96,8 @@ __device__ __forceinline__ float safe_rcp(float s) {
 // Codes by comparison (Eq. 2).  The code of x in a group, c(x) = clamp(rint(RN(RN(x - z) / s)), 0, 2^B - 1), never
 // decreases with x, and x is a 16-bit float, so the group's codes are fixed by B-bit-many thresholds on the input
 // lattice: X_k = the smallest 16-bit value with c(X_k) >= k, and c(x) = #{k : x >= X_k}.  One thread per group
-// finds the X_k: next to z + (k - 1/2) s, from the rounding bounds of the quotient where they decide, else by
-// evaluating c itself (the quotient exactly as the division gives it, ties of rint to even) at lattice points; the
-// elements are then coded two at a time with packed 16-bit compares.
+// finds the X_k next to z + (k - 1/2) s, where a subtraction and a comparison decide, else by evaluating c itself (the
+// quotient exactly as the division gives it, ties of rint to even) at lattice points; the elements are then coded two at a time with packed 16-bit compares.
 
 // 16-bit float pattern <-> integer that orders like the value (sign-magnitude to two's complement; -0 and +0 -> 0)
 __device__ __forceinline__ int ord16(uint32_t h) {
@@ -122,14 +124,16 @@ __device__ __forceinline__ float quotient(const Quot& g, float x) {
   return __fdiv_rn(a, g.s);
 }
 
-// X_k as a 16-bit pattern for a group with minimum mn and maximum mx.  In real numbers the threshold is
-// tau = z + (k - 1/2) s.  The computed quotient differs from (x - z) / s by less than 2^-23 relative (two
-// roundings), i.e. by less than 3.1 * 2^-23 s in x, and t = RN(tau) from tau by at most 2^-24 |t|: a lattice point
-// at or above t + eps certainly has c >= k, one below t - eps certainly has not, for eps = 2^-22 |t| + 2^-20 s
-// (twice what is needed).  Where the lattice is coarser than eps -- almost always -- no lattice point lies between
-// the bounds and nothing is evaluated; otherwise (a threshold next to zero under a large |z|, an exact tie on the
-// lattice) c itself decides, by bisection between the bounds.  Groups whose scale takes the division (safe_rcp)
-// are bisected from the group's ends (c(mn) = 0, c(mx) = 2^B - 1).
+// X_k as a 16-bit pattern for a group with minimum mn and maximum mx.  With a = RN(x - z), c(x) >= k means
+// RN(a / s) >= k - 1/2 (for odd k: > k - 1/2, rint taking ties to the even neighbour), and that means a >= s m in real
+// numbers, m the midpoint below the first float that counts: 1/2 + 2^-25, 3/2 - 2^-24, 5/2 + 2^-23 for k = 1, 2, 3 (s m
+// is never a float: the odd part of m has 25 bits).  So a >= a* = RU(s m), one fused multiply-add with directed
+// rounding, exactly.  x at or above z + a* satisfies RN(x - z) >= a*; x below it only if it is closer to it than half an
+// ulp of a*.  So X_k is the first lattice point at or above z + a* (1 - 2^-23) if that point passes the test, and else
+// the next one if that one lies above z + a* (the midpoint of minimum and maximum, k = 2, is a lattice point itself
+// more often than not).  Where several lattice points lie between (a threshold next to zero under a large |z|) c
+// itself decides, by bisection.  Groups whose scale takes the division (safe_rcp) are bisected from the
+// group's ends (c(mn) = 0, c(mx) = 2^B - 1).
 template <bool F16>
 __device__ __noinline__ uint32_t bisect16(float z, float sc, float y, int k, int lo, int hi) {
   const Quot g{z, sc, y, y == y};
@@ -142,26 +146,19 @@ __device__ __noinline__ uint32_t bisect16(float z, float sc, float y, int k, int
   }
   return pat16(hi);
 }
-template <bool F16>
-__device__ __forceinline__ uint32_t threshold16(const Quot& g, int k, float mn, float mx) {
-  const float kk = (float)k - 0.5f;
-  int lo, hi;  // ordered integers of lattice points with c(lo) < k <= c(hi)
-  if (g.fast) {
-    const float t = __fmaf_rn(kk, g.s, g.z);
-    const float eps = __fmaf_rn(fabsf(t), 0x1p-22f, __fmul_rn(g.s, 0x1p-20f));
-    // the smallest lattice points at or above t + eps and at or above t - eps: the same point when no lattice
-    // point lies between the two bounds, and then it is X_k (mn lies below t - eps, mx above t + eps: the
-    // thresholds are half a step and more away from both)
-    const uint32_t up = In16<F16>::bits_up(__fadd_ru(t, eps)), up_lo = In16<F16>::bits_up(__fadd_rd(t, -eps));
-    constexpr uint32_t INF16 = F16 ? 0x7c00u : 0x7f80u;
-    if (up == up_lo && up != INF16) return up;
-    hi = up != INF16 ? ord16(up) : ord16(In16<F16>::bits(mx));  // (a bound beyond the largest finite value)
-    lo = ord16(up_lo) - 1;  // below t - eps
-  } else {
-    lo = ord16(In16<F16>::bits(mn));
-    hi = ord16(In16<F16>::bits(mx));
-  }
-  return bisect16<F16>(g.z, g.s, g.y, k, lo, hi);
+template <bool F16, int K>
+__device__ __forceinline__ uint32_t threshold16(const Quot& g, float mn, float mx) {
+  constexpr float KK = (float)K - 0.5f, OFF = K == 1 ? 0x1p-25f : (K == 2 ? -0x1p-24f : 0x1p-23f);
+  const float as = __fmaf_ru(KK, g.s, __fmul_rn(g.s, OFF));
+  const uint32_t up = In16<F16>::bits_up(__fadd_ru(g.z, as));
+  const uint32_t up_lo = In16<F16>::bits_up(__fadd_rd(g.z, __fmul_rd(as, 1.0f - 0x1p-23f)));
+  constexpr uint32_t INF16 = F16 ? 0x7c00u : 0x7f80u;
+  const bool passes = __fsub_rn(In16<F16>::one((uint16_t)up_lo), g.z) >= as;
+  const bool next = up == ((up_lo & 0x8000u) ? up_lo - 1u : up_lo + 1u);
+  if (g.fast && up != INF16 && (passes || next || up == up_lo)) return passes ? up_lo : up;
+  const int lo = g.fast ? ord16(up_lo) - 1 : ord16(In16<F16>::bits(mn));
+  const int hi = g.fast && up != INF16 ? ord16(up) : ord16(In16<F16>::bits(mx));  // (a bound beyond the largest finite value)
+  return bisect16<F16>(g.z, g.s, g.y, K, lo, hi);
 }
 
 // The thresholds X_1 .. X_3 of a group with minimum mn and maximum mx (16-bit values, widened); unused ones (k beyond
@@ -174,10 +171,10 @@ __device__ __forceinline__ void group_thresholds(float mn, float mx, float z, fl
 #pragma unroll
   for (int k = 0; k < 3; ++k) thr[k] = INF16;
   if (sc != 0.0f) {
-#pragma unroll 1
-    for (int k = 1; k < 1 << bits; ++k) {  // (rolled: the code of a threshold is long, and there is one loop for all)
-      const uint32_t x = threshold16<F16>(g, k, mn, mx);
-      if (k == 1) thr[0] = x; else if (k == 2) thr[1] = x; else thr[2] = x;
+    thr[0] = threshold16<F16, 1>(g, mn, mx);
+    if (bits == 2) {
+      thr[1] = threshold16<F16, 2>(g, mn, mx);
+      thr[2] = threshold16<F16, 3>(g, mn, mx);
     }
   }
 }
@@ -213,351 +210,268 @@ __device__ __forceinline__ void delta_count(uint32_t w0, uint32_t w1, uint32_t (
   }
 }
 
-// ---------------------------------------------------------------------------
-// One warp quantizes one tile that it holds in registers: nothing goes through shared memory and no warp waits for
-// another.  Keys: G tokens x C channels; a lane has 16 consecutive channels (a whole code word, or half of a 1-bit one)
-// of every TS-th token; the lanes that share channels reduce minimum and maximum among them so that each ends with
-// its own share of the groups, finds their thresholds and hands them back by shuffles.  Values: 32 tokens x D
-// channels; a lane has D / 16 consecutive channels of 16 consecutive tokens (whole code words of these channels, or
-// halves), and the lanes of a channel group share the tokens' statistics in the same way.
-//
-// What bounds it: HBM on bulk appends.  A tile per CTA in shared memory, the version before, took 19.4 instructions an
-// element, most of them index arithmetic and control of small CTAs.
-// ---------------------------------------------------------------------------
-template <int D, int G>
-struct Tiles {
-  static constexpr int C = 4096 / G < D ? 4096 / G : D;  // channels of a key tile
-  static constexpr int LR = C / 16, TS = 32 / LR;        // lanes of a token's row, tokens of a step
-  static constexpr int STEPS = G / TS;
-  static constexpr int CPL = D / 16;                     // values: channels of a lane
-  static constexpr int LG = G / CPL;                     // values: lanes of a group
-  static constexpr int TPL = 16 / LG;                    // values: groups (tokens) whose thresholds a lane finds
-};
-
-// Of n values a lane keeps half and gives the other half away: out[k] = op(kept, partner's).
-template <int N, typename F>
-__device__ __forceinline__ void scatter_step(uint32_t* v, int mask, bool upper, F op) {
-#pragma unroll
-  for (int k = 0; k < N / 2; ++k) {
-    const uint32_t keep = upper ? v[k + N / 2] : v[k], send = upper ? v[k] : v[k + N / 2];
-    v[k] = op(keep, __shfl_xor_sync(0xffffffffu, send, mask));
-  }
-}
-
-// Stores a lane's words of codes, word k at dst(k); merging and difference counting (own bits 1 and 2) look at the words
-// that are there.
-template <int BITS, int N, typename F>
-__device__ __forceinline__ void put_words(const uint32_t (&w)[N], int n, int own, uint32_t lut, uint32_t (&hist)[4], F dst) {
-  if (own == 1) {
-#pragma unroll
-    for (int k = 0; k < N; ++k)
-      if (k < n) *dst(k) = w[k];
-    return;
-  }
-#pragma unroll 1
-  for (int k = 0; k < n; ++k) {  // rare modes: one copy of the code
-    uint32_t v = w[0];
-#pragma unroll
-    for (int j = 1; j < N; ++j) v = k == j ? w[j] : v;
-    uint32_t* const to = dst(k);
-    const uint32_t o = *to;  // the dominant layer's codes of these positions are in place
-    if (own & 4) delta_count<BITS>(o, v, hist);
-    if (own & 3) *to = merge_words<BITS>(o, v, lut);
-  }
-}
-
-template <int D, int G, bool F16>
-struct Packer {
+// One CTA: T tokens x D channels of one (sequence, kv head), keys (blockIdx.x even) or values (odd).  Staged
+// rows are padded.  Keys: a thread builds whole words of a token's row (four consecutive channels per bit
+// offset), the words are collected in shared memory in stream order and leave in 16-byte vectors.  Values: a
+// thread builds whole words of a channel's row over the tile's tokens and stores them itself.
+// G: group size; T: a multiple of G and of 32; F16: the 16-bit type is IEEE half precision.
+// blockIdx.y is the (sequence, kv head) stream, blockIdx.z the layer of the launch.  With p.win_count > 0 the CTAs of the first block also copy
+// the new window rows that replace the rows they staged.
+template <int D, int G, int T, bool F16>
+__global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __grid_constant__ PackParams p) {
   using I16 = In16<F16>;
   using V2 = typename I16::V2;
-  using Ti = Tiles<D, G>;
-  static __device__ __forceinline__ V2 v2(uint32_t x) { return *reinterpret_cast<V2*>(&x); }
-  static __device__ __forceinline__ uint32_t u32(V2 x) { return *reinterpret_cast<uint32_t*>(&x); }
-  static __device__ __forceinline__ uint32_t min2(uint32_t a, uint32_t b) { return u32(__hmin2(v2(a), v2(b))); }
-  static __device__ __forceinline__ uint32_t max2(uint32_t a, uint32_t b) { return u32(__hmax2(v2(a), v2(b))); }
+  constexpr int ROWB = D * 2 + PACK_ROW_PAD;
+  constexpr int NG = D / G;
+  constexpr int NPAR = (T * NG > (T / G) * D) ? T * NG : (T / G) * D;  // groups of the tile, either kind
+  constexpr int KP = PACK_THREADS / ((T / G) * (D / 2));               // token parts of a key group in the statistics
+  static_assert(KP >= 1 && G % KP == 0, "key statistics: 128 threads over (group, channel pair, token part)");
+  __shared__ __align__(16) uint8_t tile[T * ROWB];
+  // thresholds X_1..X_3 of a group: [k][group]; keys: group = [token group][channel], values: [channel group][token]
+  __shared__ __align__(16) uint16_t thr[3 * NPAR];
+  // packed words (at most T * D * 2 / 32); before that, the key statistics' partial (min, max) pairs, two words per thread
+  constexpr int NWBUF = (T * D * 2 / 32) > 2 * PACK_THREADS ? (T * D * 2 / 32) : 2 * PACK_THREADS;
+  __shared__ __align__(16) uint32_t wbuf[NWBUF];
 
-  // Row pabs (absolute token) of the stream: in the old window while pabs < s_old, else in the input.
-  static __device__ __forceinline__ const uint16_t* row(const PackParams& p, const uint16_t* win, const uint16_t* in, int bh, int pabs) {
-    return pabs < p.s_old ? win + ((size_t)bh * p.dm.R + (pabs - p.nq_old)) * D : in + ((size_t)bh * p.n_in + (pabs - p.s_old)) * D;
-  }
-  // The window rows that a lane has read (rows r of the old window) are free: the tokens that follow the quantized
-  // blocks take them, the same pieces by the same lane.
-  template <int VECS>
-  static __device__ __forceinline__ void refill(const PackParams& p, uint16_t* win, const uint16_t* in, int bh, int r, int c) {
-    if (r < p.win_count) {
-      const uint16_t* src = in + ((size_t)bh * p.n_in + (p.nq_new + r - p.s_old)) * D + c;
-      uint16_t* dst = win + ((size_t)bh * p.dm.R + r) * D + c;
-      if constexpr (VECS > 0) {
-#pragma unroll
-        for (int k = 0; k < VECS; ++k) reinterpret_cast<uint4*>(dst)[k] = reinterpret_cast<const uint4*>(src)[k];
-      } else {
-        *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(src);
-      }
-    }
-  }
+  const Dims& dm = p.dm;
+  const int R = dm.R;
+  const int kind = blockIdx.x & 1;  // 0 keys, 1 values
+  const int tile_idx = blockIdx.x >> 1;
+  const PackLayer pl = p.layer[blockIdx.z];  // by value: its fields are read in every loop below
+  const int bh = blockIdx.y;                  // (sequence, kv head) stream
+  const int tid = threadIdx.x;
+  const int tq0 = p.nq_old + tile_idx * T;  // absolute index of the tile's first token
+  grid_dependency_wait();  // the inputs come from the preceding kernel, and earlier kernels may still read the cache
+  grid_dependents_go();    // the next kernel may get its CTAs placed; it waits for this one before it reads the cache
 
-  template <int BITS>
-  static __device__ __forceinline__ void key_codes(const PackParams& p, const PackLayer& pl, const uint32_t (&x)[Ti::STEPS][8],
-                                                   const uint32_t (&thr)[2][3], int tq0, int d0, int bh, int i, int sub,
-                                                   uint32_t (&hist)[4]) {
-    constexpr int TS = Ti::TS, LR = Ti::LR;
-    uint32_t t1[8], t2[8], t3[8];
+  {
+    const uint16_t* win = kind ? pl.L.win_v : pl.L.win_k;
+    const uint16_t* in = kind ? pl.V_in : pl.K_in;
+    constexpr int VPR = D / 8;
+    // row `pabs` (absolute token) of the stream: in the old window while pabs < s_old, else in the input
+    const uint16_t* const win_rows = win + ((size_t)bh * R - p.nq_old) * D;
+    const uint16_t* const in_rows = in + ((size_t)bh * p.n_in - p.s_old) * D;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {  // pair q was left with the lane whose sub has these bits
-      const int owner = TS == 4 ? ((q >> 2) | ((q & 2))) : ((q >> 2) | (q & 2) | ((q & 1) << 2));
-      const int at = TS == 4 ? q & 1 : 0, src = owner * LR + i;
-      t1[q] = __shfl_sync(0xffffffffu, thr[at][0], src);
-      if constexpr (BITS == 2) {
-        t2[q] = __shfl_sync(0xffffffffu, thr[at][1], src);
-        t3[q] = __shfl_sync(0xffffffffu, thr[at][2], src);
-      } else {
-        t2[q] = t3[q] = 0u;
-      }
+    for (int k = 0; k < T * VPR / PACK_THREADS; ++k) {
+      const int idx = tid + k * PACK_THREADS;
+      const int tl = idx / VPR, c8 = idx % VPR;
+      const int pabs = tq0 + tl;
+      const uint16_t* src = (pabs < p.s_old ? win_rows : in_rows) + (size_t)pabs * D;
+      *reinterpret_cast<uint4*>(tile + tl * ROWB + c8 * 16) = reinterpret_cast<const uint4*>(src)[c8];
     }
-    uint32_t* codes = pl.L.k_codes + (size_t)bh * ((size_t)p.dm.nq_cap * D * BITS / 32);
-    uint32_t w[Ti::STEPS];
-#pragma unroll
-    for (int st = 0; st < Ti::STEPS; ++st) {
-      w[st] = 0u;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const uint32_t lo = code_pair<BITS, V2>(x[st][2 * e], t1[2 * e], t2[2 * e], t3[2 * e]);
-        const uint32_t hi = code_pair<BITS, V2>(x[st][2 * e + 1], t1[2 * e + 1], t2[2 * e + 1], t3[2 * e + 1]);
-        w[st] |= __byte_perm(lo, hi, 0x6420) << (BITS * e);
-      }
-    }
-    const uint32_t lut = p.merge_lut[BITS - 1];
-    if constexpr (BITS == 2) {
-      put_words<2>(w, Ti::STEPS, pl.own_k, lut, hist,
-                   [&](int k) { return codes + k_code_position(tq0 + k * TS + sub, d0, 2, D).word; });
-    } else {  // a word is two lanes' channels: of two tokens each lane completes one
-      const bool upper = (i & 1) != 0;
-#pragma unroll
-      for (int st = 0; st < Ti::STEPS; st += 2) {
-        const uint32_t keep = upper ? w[st + 1] << 4 : w[st], send = upper ? w[st] << 4 : w[st + 1];
-        w[st / 2] = keep | __shfl_xor_sync(0xffffffffu, send, 1);
-      }
-      put_words<1>(w, Ti::STEPS / 2, pl.own_k, lut, hist, [&](int k) {
-        return codes + k_code_position(tq0 + (2 * k + (upper ? 1 : 0)) * TS + sub, d0 & ~31, 1, D).word;
-      });
+  }
+  __syncthreads();
+  // the window rows this CTA staged are free: the tokens that follow the quantized blocks take them
+  if (p.win_count > 0 && tile_idx * T < p.win_count) {
+    uint16_t* win = kind ? pl.L.win_v : pl.L.win_k;
+    const uint16_t* in = kind ? pl.V_in : pl.K_in;
+    constexpr int VPR = D / 8;
+    const int rows = min(T, p.win_count - tile_idx * T);
+    for (int idx = tid; idx < rows * VPR; idx += PACK_THREADS) {
+      const int r = tile_idx * T + idx / VPR, c8 = idx % VPR;
+      const uint4* src = reinterpret_cast<const uint4*>(in + ((size_t)bh * p.n_in + (p.nq_new + r - p.s_old)) * D) + c8;
+      reinterpret_cast<uint4*>(win + ((size_t)bh * R + r) * D)[c8] = *src;
     }
   }
 
-  static __device__ __forceinline__ void keys(const PackParams& p, const PackLayer& pl, int tile, int bh, int lane, uint32_t (&hist)[4]) {
-    constexpr int TS = Ti::TS, LR = Ti::LR, CT = D / Ti::C;
-    const int i = lane % LR, sub = lane / LR, t0 = tile / CT * G, d0 = tile % CT * Ti::C + 16 * i;
-    const int tq0 = p.nq_old + t0;
-    uint32_t x[Ti::STEPS][8];
+  const int bits = kind ? pl.L.bv : pl.L.bk;
+  const float eta = kind ? pl.eta_v : pl.eta_k;
+  const int own = kind ? pl.own_v : pl.own_k;
+
+  if (kind == 0) {
+    // keys: one group per (channel, run of G tokens).  First bf16x2 min / max of a channel pair over a part of the
+    // group's tokens (consecutive threads take consecutive pairs), then one thread per (group, channel).
+    {
+      const int dp = tid % (D / 2), rest = tid / (D / 2);
+      const int gl = rest / KP, part = rest % KP;
+      const uint8_t* col = tile + (gl * G + part * (G / KP)) * ROWB + dp * 4;
+      V2 mn2 = *reinterpret_cast<const V2*>(col), mx2 = mn2;
 #pragma unroll
-    for (int st = 0; st < Ti::STEPS; ++st) {
-      const uint4* src = reinterpret_cast<const uint4*>(row(p, pl.L.win_k, pl.K_in, bh, tq0 + st * TS + sub) + d0);
-      const uint4 a = src[0], b = src[1];
-      x[st][0] = a.x; x[st][1] = a.y; x[st][2] = a.z; x[st][3] = a.w;
-      x[st][4] = b.x; x[st][5] = b.y; x[st][6] = b.z; x[st][7] = b.w;
+      for (int j = 1; j < G / KP; ++j) {
+        const V2 v = *reinterpret_cast<const V2*>(col + j * ROWB);
+        mn2 = __hmin2(mn2, v);
+        mx2 = __hmax2(mx2, v);
+      }
+      wbuf[(rest * (D / 2) + dp) * 2] = *reinterpret_cast<uint32_t*>(&mn2);
+      wbuf[(rest * (D / 2) + dp) * 2 + 1] = *reinterpret_cast<uint32_t*>(&mx2);
     }
-    uint32_t mn[8], mx[8];
+    __syncthreads();
+    __half* meta = reinterpret_cast<__half*>(pl.L.k_meta);
+    const size_t cap_g = (size_t)(dm.nq_cap / G);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      mn[q] = mx[q] = x[0][q];
+    for (int k = 0; k < ((T / G) * D + PACK_THREADS - 1) / PACK_THREADS; ++k) {
+      const int item = tid + k * PACK_THREADS;
+      if (item < (T / G) * D) {
+        const int gl = item / D, d = item % D;
+        float mn = 0.f, mx = 0.f;
 #pragma unroll
-      for (int st = 1; st < Ti::STEPS; ++st) {
-        mn[q] = min2(mn[q], x[st][q]);
-        mx[q] = max2(mx[q], x[st][q]);
+        for (int part = 0; part < KP; ++part) {
+          const uint32_t a2 = wbuf[((gl * KP + part) * (D / 2) + d / 2) * 2], b2 = wbuf[((gl * KP + part) * (D / 2) + d / 2) * 2 + 1];
+          const float lo = (d & 1) ? I16::hi(a2) : I16::lo(a2);
+          const float hi = (d & 1) ? I16::hi(b2) : I16::lo(b2);
+          mn = part == 0 ? lo : fminf(mn, lo);
+          mx = part == 0 ? hi : fmaxf(mx, hi);
+        }
+        float z, sc;
+        __half zh, sh;
+        group_params(mn, mx, bits, eta, z, sc, zh, sh);
+        if (own) {
+          uint32_t x[3];
+          group_thresholds<F16>(mn, mx, z, sc, bits, x);
+#pragma unroll
+          for (int j = 0; j < 3; ++j) thr[j * NPAR + item] = (uint16_t)x[j];
+        }
+        const size_t grp = (size_t)bh * cap_g + (tq0 / G + gl);  // per group: D scales, then D zero-points
+        const int pos = k_meta_position(d, D);
+        meta[grp * 2 * D + pos] = sh;
+        meta[grp * 2 * D + D + pos] = zh;
       }
     }
-    if (t0 < p.win_count) {
+  } else {
+    // values: one group per (token, run of G channels); consecutive threads take consecutive tokens
+    __half* meta = reinterpret_cast<__half*>(pl.L.v_meta);
 #pragma unroll
-      for (int st = 0; st < Ti::STEPS; ++st) refill<2>(p, pl.L.win_k, pl.K_in, bh, t0 + st * TS + sub, d0);
-    }
-    scatter_step<8>(mn, LR, sub & 1, min2);
-    scatter_step<8>(mx, LR, sub & 1, max2);
-    scatter_step<4>(mn, 2 * LR, sub & 2, min2);
-    scatter_step<4>(mx, 2 * LR, sub & 2, max2);
-    int q0 = 4 * (sub & 1) + (sub & 2);
-    if constexpr (TS == 8) {
-      scatter_step<2>(mn, 4 * LR, sub & 4, min2);
-      scatter_step<2>(mx, 4 * LR, sub & 4, max2);
-      q0 += sub >> 2;
-    }
-    constexpr int PAIRS = 8 / TS;  // pairs of channels that are this lane's now
-    __half* meta = reinterpret_cast<__half*>(pl.L.k_meta) + ((size_t)bh * (p.dm.nq_cap / G) + tq0 / G) * (2 * D);
-    uint32_t thr[2][3] = {{0u, 0u, 0u}, {0u, 0u, 0u}};
-#pragma unroll 1
-    for (int g = 0; g < 2 * PAIRS; ++g) {  // (rolled, for the instruction cache)
-      const int h = g & 1;
-      const bool second = PAIRS == 2 && g >= 2;
-      const uint32_t mnw = second ? mn[1] : mn[0], mxw = second ? mx[1] : mx[0];
-      const float lo = h ? I16::hi(mnw) : I16::lo(mnw), hi = h ? I16::hi(mxw) : I16::lo(mxw);
-      float z, sc;
-      __half zh, sh;
-      group_params(lo, hi, pl.L.bk, pl.eta_k, z, sc, zh, sh);
-      const int pos = k_meta_position(d0 + 2 * q0 + g, D);
-      meta[pos] = sh;
-      meta[D + pos] = zh;
-      if (pl.own_k) {
-        uint32_t tt[3];
-        group_thresholds<F16>(lo, hi, z, sc, pl.L.bk, tt);
+    for (int k = 0; k < (T * NG + PACK_THREADS - 1) / PACK_THREADS; ++k) {
+      const int item = tid + k * PACK_THREADS;
+      if (item < T * NG) {
+        const int tl = item % T, gi = item / T;
+        const uint4* row = reinterpret_cast<const uint4*>(tile + tl * ROWB + gi * G * 2);
+        V2 mn2, mx2;
+        {
+          uint4 v = row[0];
+          const V2* e = reinterpret_cast<const V2*>(&v);
+          mn2 = __hmin2(__hmin2(e[0], e[1]), __hmin2(e[2], e[3]));
+          mx2 = __hmax2(__hmax2(e[0], e[1]), __hmax2(e[2], e[3]));
+        }
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          const uint32_t v = tt[j] << (16 * h);
-          if (second) thr[1][j] |= v; else thr[0][j] |= v;
+        for (int j = 1; j < G / 8; ++j) {
+          uint4 v = row[j];
+          const V2* e = reinterpret_cast<const V2*>(&v);
+          mn2 = __hmin2(mn2, __hmin2(__hmin2(e[0], e[1]), __hmin2(e[2], e[3])));
+          mx2 = __hmax2(mx2, __hmax2(__hmax2(e[0], e[1]), __hmax2(e[2], e[3])));
+        }
+        const uint32_t mnw = *reinterpret_cast<const uint32_t*>(&mn2), mxw = *reinterpret_cast<const uint32_t*>(&mx2);
+        const float mn = fminf(I16::lo(mnw), I16::hi(mnw));
+        const float mx = fmaxf(I16::lo(mxw), I16::hi(mxw));
+        float z, sc;
+        __half zh, sh;
+        group_params(mn, mx, bits, eta, z, sc, zh, sh);
+        if (own) {
+          uint32_t x[3];
+          group_thresholds<F16>(mn, mx, z, sc, bits, x);
+#pragma unroll
+          for (int j = 0; j < 3; ++j) thr[j * NPAR + gi * T + tl] = (uint16_t)x[j];
+        }
+        const int tabs = tq0 + tl;
+        __half* mine = meta + (size_t)bh * dm.nq_cap * 2 * NG;
+        mine[v_scale_index(tabs, gi, NG)] = sh;
+        mine[v_zero_index(tabs, gi, NG)] = zh;
+      }
+    }
+  }
+  if (!own) return;  // PseudoQuantize: parameters only
+  __syncthreads();
+
+  // codes
+  uint32_t* codes = kind ? pl.L.v_codes : pl.L.k_codes;
+  const bool merge = (own & 2) != 0, stats = (own & 4) != 0, store = (own & 3) != 0;
+  uint32_t hist[4] = {0u, 0u, 0u, 0u};
+  const size_t stream_words = (size_t)dm.nq_cap * D * bits / 32;
+  auto build = [&](auto bits_c) {
+    constexpr int BITS = decltype(bits_c)::value;
+    constexpr int N = 32 / BITS;        // codes per word
+    if (kind == 0) {
+      constexpr int NW = D * BITS / 32;  // words per token row
+      const size_t w0 = k_code_position(tq0, 0, BITS, D).word;  // the tile's words are one contiguous run
+#pragma unroll
+      for (int k = 0; k < (T * NW + PACK_THREADS - 1) / PACK_THREADS; ++k) {
+        const int item = tid + k * PACK_THREADS;
+        if (item < T * NW) {
+          const int tl = item % T, i = item / T, gl = tl / G;
+          const uint8_t* row = tile + tl * ROWB;
+          uint32_t word = 0u;
+#pragma unroll
+          for (int s4 = 0; s4 < N / 4; ++s4) {
+            const int d = i * N + 4 * s4;  // four consecutive channels: four groups
+            const uint2 xx = *reinterpret_cast<const uint2*>(row + d * 2);
+            const uint2 t1 = *reinterpret_cast<const uint2*>(thr + gl * D + d);
+            uint2 t2 = t1, t3 = t1;
+            if constexpr (BITS == 2) {
+              t2 = *reinterpret_cast<const uint2*>(thr + NPAR + gl * D + d);
+              t3 = *reinterpret_cast<const uint2*>(thr + 2 * NPAR + gl * D + d);
+            }
+            const uint32_t lo = code_pair<BITS, V2>(xx.x, t1.x, t2.x, t3.x), hi = code_pair<BITS, V2>(xx.y, t1.y, t2.y, t3.y);
+            word |= __byte_perm(lo, hi, 0x6420) << (BITS * s4);
+          }
+          wbuf[k_code_position(tq0 + tl, i * N, BITS, D).word - w0] = word;
+        }
+      }
+      __syncthreads();
+      uint4* dst = reinterpret_cast<uint4*>(codes + (size_t)bh * stream_words + w0);
+      for (int v = tid; v < T * NW / 4; v += PACK_THREADS) {
+        uint4 w = reinterpret_cast<const uint4*>(wbuf)[v];
+        if (merge || stats) {  // the dominant layer's codes of these positions are in place
+          const uint4 o = dst[v];
+          if (stats) {
+            delta_count<BITS>(o.x, w.x, hist); delta_count<BITS>(o.y, w.y, hist);
+            delta_count<BITS>(o.z, w.z, hist); delta_count<BITS>(o.w, w.w, hist);
+          }
+          const uint32_t lut = p.merge_lut[BITS - 1];
+          w = make_uint4(merge_words<BITS>(o.x, w.x, lut), merge_words<BITS>(o.y, w.y, lut),
+                         merge_words<BITS>(o.z, w.z, lut), merge_words<BITS>(o.w, w.w, lut));
+        }
+        if (store) dst[v] = w;
+      }
+    } else {
+      constexpr int WPC = T / N;  // words per channel over the tile's tokens
+#pragma unroll
+      for (int k = 0; k < (D * WPC + PACK_THREADS - 1) / PACK_THREADS; ++k) {
+        const int item = tid + k * PACK_THREADS;
+        if (item < D * WPC) {
+          const int d = item % D, wi = item / D, gi = d / G;
+          uint32_t word = 0u;
+#pragma unroll
+          for (int s4 = 0; s4 < N / 4; ++s4) {
+            const int tl = wi * N + 4 * s4;  // four consecutive tokens: four groups
+            const uint8_t* src = tile + tl * ROWB + d * 2;
+            const uint32_t x0 = *reinterpret_cast<const uint16_t*>(src), x1 = *reinterpret_cast<const uint16_t*>(src + ROWB);
+            const uint32_t x2 = *reinterpret_cast<const uint16_t*>(src + 2 * ROWB), x3 = *reinterpret_cast<const uint16_t*>(src + 3 * ROWB);
+            const uint2 t1 = *reinterpret_cast<const uint2*>(thr + gi * T + tl);
+            uint2 t2 = t1, t3 = t1;
+            if constexpr (BITS == 2) {
+              t2 = *reinterpret_cast<const uint2*>(thr + NPAR + gi * T + tl);
+              t3 = *reinterpret_cast<const uint2*>(thr + 2 * NPAR + gi * T + tl);
+            }
+            const uint32_t lo = code_pair<BITS, V2>(x0 | (x1 << 16), t1.x, t2.x, t3.x);
+            const uint32_t hi = code_pair<BITS, V2>(x2 | (x3 << 16), t1.y, t2.y, t3.y);
+            word |= __byte_perm(lo, hi, 0x6420) << (BITS * s4);
+          }
+          uint32_t* dst = codes + (size_t)bh * stream_words + v_code_position(tq0 + wi * N, d, BITS, D).word;
+          if (merge || stats) {
+            const uint32_t o = *dst;
+            if (stats) delta_count<BITS>(o, word, hist);
+            word = merge_words<BITS>(o, word, p.merge_lut[BITS - 1]);
+          }
+          if (store) *dst = word;
         }
       }
     }
-    if (!pl.own_k) return;  // PseudoQuantize: parameters only
-    if (pl.L.bk == 2) key_codes<2>(p, pl, x, thr, tq0, d0, bh, i, sub, hist);
-    else key_codes<1>(p, pl, x, thr, tq0, d0, bh, i, sub, hist);
-  }
-
-  template <int BITS>
-  static __device__ __forceinline__ void value_codes(const PackParams& p, const PackLayer& pl, const uint32_t (&x)[16][Ti::CPL / 2],
-                                                     const uint32_t (&ta)[Ti::TPL], const uint32_t (&tb)[Ti::TPL], int tq0, int d0,
-                                                     int bh, int lane, uint32_t (&hist)[4]) {
-    constexpr int NP = Ti::CPL / 2, LG = Ti::LG;
-    uint32_t acc[4][NP];  // [token % 4][channel pair]: the codes' bits of that byte, a channel in each half
-#pragma unroll
-    for (int b = 0; b < 4; ++b)
-#pragma unroll
-      for (int c = 0; c < NP; ++c) acc[b][c] = 0u;
-#pragma unroll
-    for (int t = 0; t < 16; ++t) {
-      // token t was left with the lane of the group that has these bits, as its value t % TPL
-      int owner = 0;
-#pragma unroll
-      for (int k = 0, n = 8; n >= Ti::TPL; n >>= 1, ++k) owner |= ((t & n) ? 1 : 0) << k;
-      const int src = (lane & ~(LG - 1)) | owner;
-      const uint32_t a = __shfl_sync(0xffffffffu, ta[t % Ti::TPL], src);
-      const uint32_t t1 = __byte_perm(a, a, 0x1010);
-      uint32_t t2 = 0u, t3 = 0u;
-      if constexpr (BITS == 2) {
-        t2 = __byte_perm(a, a, 0x3232);
-        t3 = __shfl_sync(0xffffffffu, tb[t % Ti::TPL], src);
-      }
-#pragma unroll
-      for (int c = 0; c < NP; ++c) acc[t % 4][c] += code_pair<BITS, V2>(x[t][c], t1, t2, t3) << (BITS * (t / 4));
-    }
-    uint32_t w[Ti::CPL];
-#pragma unroll
-    for (int c = 0; c < NP; ++c) {
-      const uint32_t a = __byte_perm(acc[0][c], acc[1][c], 0x6240), b = __byte_perm(acc[2][c], acc[3][c], 0x6240);
-      w[2 * c] = __byte_perm(a, b, 0x5410);
-      w[2 * c + 1] = __byte_perm(a, b, 0x7632);
-    }
-    uint32_t* codes = pl.L.v_codes + (size_t)bh * ((size_t)p.dm.nq_cap * D * BITS / 32);
-    const uint32_t lut = p.merge_lut[BITS - 1];
-    const int half = lane >> 4;
-    if constexpr (BITS == 2) {
-      put_words<2>(w, Ti::CPL, pl.own_v, lut, hist,
-                   [&](int c) { return codes + v_code_position(tq0 + 16 * half, d0 + c, 2, D).word; });
-    } else {  // a word is both halves' tokens: each half completes half of the channels
-#pragma unroll
-      for (int c = 0; c < Ti::CPL; ++c) w[c] <<= 4 * half;
-      scatter_step<Ti::CPL>(w, 16, half, [](uint32_t a, uint32_t b) { return a | b; });
-      put_words<1>(w, NP, pl.own_v, lut, hist,
-                   [&](int c) { return codes + v_code_position(tq0, d0 + half * NP + c, 1, D).word; });
-    }
-  }
-
-  static __device__ __forceinline__ void values(const PackParams& p, const PackLayer& pl, int tile, int bh, int lane, uint32_t (&hist)[4]) {
-    constexpr int NP = Ti::CPL / 2, NG = D / G, LG = Ti::LG, TPL = Ti::TPL;
-    const int half = lane >> 4, d0 = (lane & 15) * Ti::CPL, t0 = tile * 32, tq0 = p.nq_old + t0;
-    uint32_t x[16][NP];
-#pragma unroll
-    for (int t = 0; t < 16; ++t) {
-      const uint16_t* src = row(p, pl.L.win_v, pl.V_in, bh, tq0 + 16 * half + t) + d0;
-      if constexpr (NP == 4) {
-        const uint4 a = *reinterpret_cast<const uint4*>(src);
-        x[t][0] = a.x; x[t][1] = a.y; x[t][2] = a.z; x[t][3] = a.w;
-      } else {
-        const uint2 a = *reinterpret_cast<const uint2*>(src);
-        x[t][0] = a.x; x[t][1] = a.y;
-      }
-    }
-    // per token (minimum, -maximum) of this lane's channels, then of the group's: one packed minimum for both
-    uint32_t st[16];
-#pragma unroll
-    for (int t = 0; t < 16; ++t) {
-      uint32_t mn = x[t][0], mx = x[t][0];
-#pragma unroll
-      for (int c = 1; c < NP; ++c) {
-        mn = min2(mn, x[t][c]);
-        mx = max2(mx, x[t][c]);
-      }
-      mx ^= 0x80008000u;
-      st[t] = min2(__byte_perm(mn, mx, 0x5410), __byte_perm(mn, mx, 0x7632));
-    }
-    if (t0 < p.win_count) {
-#pragma unroll
-      for (int t = 0; t < 16; ++t) refill<NP == 4 ? 1 : 0>(p, pl.L.win_v, pl.V_in, bh, t0 + 16 * half + t, d0);
-    }
-    int tk = 0;  // first of the tokens that are left with this lane
-    scatter_step<16>(st, 1, lane & 1, min2); tk += 8 * (lane & 1);
-    scatter_step<8>(st, 2, (lane >> 1) & 1, min2); tk += 4 * ((lane >> 1) & 1);
-    if constexpr (LG >= 8) { scatter_step<4>(st, 4, (lane >> 2) & 1, min2); tk += 2 * ((lane >> 2) & 1); }
-    if constexpr (LG >= 16) { scatter_step<2>(st, 8, (lane >> 3) & 1, min2); tk += (lane >> 3) & 1; }
-    __half* meta = reinterpret_cast<__half*>(pl.L.v_meta) + (size_t)bh * p.dm.nq_cap * 2 * NG;
-    uint32_t ta[TPL], tb[TPL];  // X_1 and X_2; X_3 twice
-#pragma unroll
-    for (int k = 0; k < TPL; ++k) ta[k] = tb[k] = 0u;
-#pragma unroll 1
-    for (int g = 0; g < TPL; ++g) {
-      uint32_t w = st[0];
-#pragma unroll
-      for (int k = 1; k < TPL; ++k) w = g == k ? st[k] : w;
-      const float mn = I16::lo(w), mx = -I16::hi(w);
-      float z, sc;
-      __half zh, sh;
-      group_params(mn, mx, pl.L.bv, pl.eta_v, z, sc, zh, sh);
-      const int tabs = tq0 + 16 * half + tk + g, gi = d0 / G;
-      meta[v_scale_index(tabs, gi, NG)] = sh;
-      meta[v_zero_index(tabs, gi, NG)] = zh;
-      if (pl.own_v) {
-        uint32_t tt[3];
-        group_thresholds<F16>(mn, mx, z, sc, pl.L.bv, tt);
-        const uint32_t a = tt[0] | (tt[1] << 16), b = tt[2] * 0x10001u;
-#pragma unroll
-        for (int k = 0; k < TPL; ++k)
-          if (g == k) { ta[k] = a; tb[k] = b; }
-      }
-    }
-    if (!pl.own_v) return;
-    if (pl.L.bv == 2) value_codes<2>(p, pl, x, ta, tb, tq0, d0, bh, lane, hist);
-    else value_codes<1>(p, pl, x, ta, tb, tq0, d0, bh, lane, hist);
-  }
-};
-
-// blockIdx.x even: keys, odd: values, a tile per warp; blockIdx.y the (sequence, kv head) stream, blockIdx.z the layer
-// of the launch.  With p.win_count > 0 the warps of the first block also copy the new window rows over those they read.
-template <int D, int G, bool F16>
-__global__ void __launch_bounds__(PACK_THREADS, 4) pack_kernel(const __grid_constant__ PackParams p) {
-  using Ti = Tiles<D, G>;
-  const int lane = threadIdx.x & 31, tile = (blockIdx.x >> 1) * (PACK_THREADS / 32) + (threadIdx.x >> 5);
-  const bool values = blockIdx.x & 1;
-  const int tokens = p.n_blocks * p.dm.R;
-  grid_dependency_wait();  // the inputs come from the preceding kernel, and earlier kernels may still read the cache
-  grid_dependents_go();    // the next kernel may get its CTAs placed; it waits for this one before it reads the cache
-  if (tile >= (values ? tokens / 32 : tokens / G * (D / Ti::C))) return;
-  const PackLayer& pl = p.layer[blockIdx.z];
-  uint32_t hist[4] = {0u, 0u, 0u, 0u};
-  if (values) Packer<D, G, F16>::values(p, pl, tile, blockIdx.y, lane, hist);
-  else Packer<D, G, F16>::keys(p, pl, tile, blockIdx.y, lane, hist);
-  if ((values ? pl.own_v : pl.own_k) & 4) {
-    unsigned long long* out = values ? pl.delta_v : pl.delta_k;
+  };
+  if (bits == 2) build(std::integral_constant<int, 2>{}); else build(std::integral_constant<int, 1>{});
+  if (stats) {
+    unsigned long long* out = kind ? pl.delta_v : pl.delta_k;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const uint32_t tot = __reduce_add_sync(0xffffffffu, hist[k]);
-      if (lane == 0 && tot) atomicAdd(out + k, (unsigned long long)tot);
+      if ((tid & 31) == 0 && tot) atomicAdd(out + k, (unsigned long long)tot);
     }
   }
 }
 
 template <int D, int G, bool F16>
 cudaError_t launch_pack_t(const PackParams& p, cudaStream_t st) {
-  using Ti = Tiles<D, G>;
-  const int tokens = p.n_blocks * p.dm.R;
-  const int tiles_k = tokens / G * (D / Ti::C), tiles_v = tokens / 32, tiles = tiles_k > tiles_v ? tiles_k : tiles_v;
-  constexpr int W = PACK_THREADS / 32;
-  return launch_dependent(pack_kernel<D, G, F16>, dim3(2 * ((tiles + W - 1) / W), p.dm.B * p.dm.Hkv, p.n_layers),
+  // a tile is one key group long: 32 or 64 tokens, whole words of either kind
+  return launch_dependent(pack_kernel<D, G, G, F16>, dim3(2 * p.n_blocks * (p.dm.R / G), p.dm.B * p.dm.Hkv, p.n_layers),
                           dim3(PACK_THREADS), 0, st, p);
 }
 
