@@ -131,8 +131,9 @@ __device__ __forceinline__ float quotient(const Quot& g, float x) {
 // rounding, exactly.  x at or above z + a* satisfies RN(x - z) >= a*; x below it only if it is closer to it than half an
 // ulp of a*.  So X_k is the first lattice point at or above z + a* (1 - 2^-23) if that point passes the test, and else
 // the next one if that one lies above z + a* (the midpoint of minimum and maximum, k = 2, is a lattice point itself
-// more often than not).  Where several lattice points lie between (a threshold next to zero under a large |z|) c
-// itself decides, by bisection.  Groups whose scale takes the division (safe_rcp) are bisected from the
+// more often than not).  Several lattice points lie between only where z + a* all but cancels (one group in fifty:
+// minimum and maximum of equal magnitude); z + a* is then exact and so is w, half an ulp of a* below it: X_k is the
+// first lattice point at or above w (above it, where a* is odd: the tie goes down).  Groups whose scale takes the division (safe_rcp) are bisected from the
 // group's ends (c(mn) = 0, c(mx) = 2^B - 1).
 template <bool F16>
 __device__ __noinline__ uint32_t bisect16(float z, float sc, float y, int k, int lo, int hi) {
@@ -156,6 +157,13 @@ __device__ __forceinline__ uint32_t threshold16(const Quot& g, float mn, float m
   const bool passes = __fsub_rn(In16<F16>::one((uint16_t)up_lo), g.z) >= as;
   const bool next = up == ((up_lo & 0x8000u) ? up_lo - 1u : up_lo + 1u);
   if (g.fast && up != INF16 && (passes || next || up == up_lo)) return passes ? up_lo : up;
+  const float d = __fadd_rn(g.z, as);
+  if (g.fast && fabsf(d) < __fmul_rn(as, 0x1p-10f)) {
+    const float w = __fsub_rn(d, __fmul_rn(0.5f, __fsub_rn(as, __uint_as_float(__float_as_uint(as) - 1u))));
+    const uint32_t x = In16<F16>::bits_up(w);
+    const bool above = (__float_as_uint(as) & 1u) && In16<F16>::one((uint16_t)x) == w;
+    return above ? pat16(ord16(x) + 1) : x;
+  }
   const int lo = g.fast ? ord16(up_lo) - 1 : ord16(In16<F16>::bits(mn));
   const int hi = g.fast && up != INF16 ? ord16(up) : ord16(In16<F16>::bits(mx));  // (a bound beyond the largest finite value)
   return bisect16<F16>(g.z, g.s, g.y, K, lo, hi);
@@ -179,24 +187,19 @@ __device__ __forceinline__ void group_thresholds(float mn, float mx, float z, fl
   }
 }
 
-// Codes of two packed 16-bit elements against their groups' packed thresholds: code of the low element at bit 0,
-// of the high element at bit 16.
+// Codes of two packed 16-bit elements against their groups' packed thresholds, accumulated: acc += S << shift.  A mask
+// is 0xffff per element that passed, so S, the sum of the three masks, is -(low count) + 2^16 (low count - high count):
+// linear in the counts, and finish() turns the accumulated sum into (low counts) + 2^16 (high counts), every count at
+// its shift, with one multiplication.
 template <int BITS, typename V2>
-__device__ __forceinline__ uint32_t code_pair(uint32_t x, uint32_t t1, uint32_t t2, uint32_t t3) {
+__device__ __forceinline__ void add_codes(uint32_t& acc, int shift, uint32_t x, uint32_t t1, uint32_t t2, uint32_t t3) {
   const V2 xv = *reinterpret_cast<const V2*>(&x);
-  const uint32_t m1 = __hge2_mask(xv, *reinterpret_cast<const V2*>(&t1));
-  if constexpr (BITS == 1) {
-    return m1 & 0x00010001u;
-  } else {
-    const uint32_t m2 = __hge2_mask(xv, *reinterpret_cast<const V2*>(&t2));
-    const uint32_t m3 = __hge2_mask(xv, *reinterpret_cast<const V2*>(&t3));
-    // A mask is 0xffff per element that passed.  n = -(m1 + m2 + m3) holds the low element's count in its low
-    // half and (high count - low count) in its high half (the low half borrows); n * 0x10001 adds the low count
-    // back to the high half.
-    const uint32_t n = 0u - m1 - m2 - m3;
-    return n * 0x10001u;
-  }
+  uint32_t sum = __hge2_mask(xv, *reinterpret_cast<const V2*>(&t1));
+  if constexpr (BITS == 2)
+    sum += __hge2_mask(xv, *reinterpret_cast<const V2*>(&t2)) + __hge2_mask(xv, *reinterpret_cast<const V2*>(&t3));
+  acc += sum << shift;
 }
+__device__ __forceinline__ uint32_t finish(uint32_t acc) { return acc * (0u - 0x10001u); }
 
 // Adds to hist[d] the number of fields of the two words whose codes differ by d.
 template <int BITS>
@@ -223,12 +226,15 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __grid_constan
   using V2 = typename I16::V2;
   constexpr int ROWB = D * 2 + PACK_ROW_PAD;
   constexpr int NG = D / G;
-  constexpr int NPAR = (T * NG > (T / G) * D) ? T * NG : (T / G) * D;  // groups of the tile, either kind
+  constexpr int KG = (T / G) * D;                                      // key groups of the tile
   constexpr int KP = PACK_THREADS / ((T / G) * (D / 2));               // token parts of a key group in the statistics
   static_assert(KP >= 1 && G % KP == 0, "key statistics: 128 threads over (group, channel pair, token part)");
   __shared__ __align__(16) uint8_t tile[T * ROWB];
-  // thresholds X_1..X_3 of a group: [k][group]; keys: group = [token group][channel], values: [channel group][token]
-  __shared__ __align__(16) uint16_t thr[3 * NPAR];
+  // thresholds X_1..X_3 of a group: keys [k][token group][channel]; values [token][channel group] of four words, each
+  // threshold in both halves of one
+  constexpr int NTHR = 3 * (T / G) * D * 2 > T * NG * 16 ? 3 * (T / G) * D * 2 : T * NG * 16;
+  __shared__ __align__(16) uint8_t thr_mem[NTHR];
+  uint16_t* const thr = reinterpret_cast<uint16_t*>(thr_mem);
   // packed words (at most T * D * 2 / 32); before that, the key statistics' partial (min, max) pairs, two words per thread
   constexpr int NWBUF = (T * D * 2 / 32) > 2 * PACK_THREADS ? (T * D * 2 / 32) : 2 * PACK_THREADS;
   __shared__ __align__(16) uint32_t wbuf[NWBUF];
@@ -319,7 +325,7 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __grid_constan
           uint32_t x[3];
           group_thresholds<F16>(mn, mx, z, sc, bits, x);
 #pragma unroll
-          for (int j = 0; j < 3; ++j) thr[j * NPAR + item] = (uint16_t)x[j];
+          for (int j = 0; j < 3; ++j) thr[j * KG + item] = (uint16_t)x[j];
         }
         const size_t grp = (size_t)bh * cap_g + (tq0 / G + gl);  // per group: D scales, then D zero-points
         const int pos = k_meta_position(d, D);
@@ -360,7 +366,8 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __grid_constan
           uint32_t x[3];
           group_thresholds<F16>(mn, mx, z, sc, bits, x);
 #pragma unroll
-          for (int j = 0; j < 3; ++j) thr[j * NPAR + gi * T + tl] = (uint16_t)x[j];
+          for (int j = 0; j < 3; ++j) x[j] *= 0x10001u;
+          reinterpret_cast<uint4*>(thr_mem)[tl * NG + gi] = make_uint4(x[0], x[1], x[2], 0u);
         }
         const int tabs = tq0 + tl;
         __half* mine = meta + (size_t)bh * dm.nq_cap * 2 * NG;
@@ -383,28 +390,30 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __grid_constan
     if (kind == 0) {
       constexpr int NW = D * BITS / 32;  // words per token row
       const size_t w0 = k_code_position(tq0, 0, BITS, D).word;  // the tile's words are one contiguous run
+      // a thread takes word i of every TS-th token: consecutive threads consecutive words
+      constexpr int TS = PACK_THREADS / NW;
+      const int i = tid % NW, d0 = i * N;
 #pragma unroll
-      for (int k = 0; k < (T * NW + PACK_THREADS - 1) / PACK_THREADS; ++k) {
-        const int item = tid + k * PACK_THREADS;
-        if (item < T * NW) {
-          const int tl = item % T, i = item / T, gl = tl / G;
-          const uint8_t* row = tile + tl * ROWB;
-          uint32_t word = 0u;
+      for (int k = 0; k < (T + TS - 1) / TS; ++k) {
+        const int tl = tid / NW + k * TS, gl = tl / G;
+        if (TS > T && tl >= T) break;
+        const uint4* row = reinterpret_cast<const uint4*>(tile + tl * ROWB + d0 * 2);
+        const uint4* th = reinterpret_cast<const uint4*>(thr + gl * D + d0);  // thresholds k: KG * 2 bytes apart
+        uint32_t a0 = 0u, a1 = 0u;  // channels 4 e, 4 e + 1; 4 e + 2, 4 e + 3
 #pragma unroll
-          for (int s4 = 0; s4 < N / 4; ++s4) {
-            const int d = i * N + 4 * s4;  // four consecutive channels: four groups
-            const uint2 xx = *reinterpret_cast<const uint2*>(row + d * 2);
-            const uint2 t1 = *reinterpret_cast<const uint2*>(thr + gl * D + d);
-            uint2 t2 = t1, t3 = t1;
-            if constexpr (BITS == 2) {
-              t2 = *reinterpret_cast<const uint2*>(thr + NPAR + gl * D + d);
-              t3 = *reinterpret_cast<const uint2*>(thr + 2 * NPAR + gl * D + d);
-            }
-            const uint32_t lo = code_pair<BITS, V2>(xx.x, t1.x, t2.x, t3.x), hi = code_pair<BITS, V2>(xx.y, t1.y, t2.y, t3.y);
-            word |= __byte_perm(lo, hi, 0x6420) << (BITS * s4);
+        for (int v = 0; v < N / 8; ++v) {
+          const uint4 x = row[v], t1 = th[v];
+          uint4 t2 = t1, t3 = t1;
+          if constexpr (BITS == 2) {
+            t2 = th[KG / 8 + v];
+            t3 = th[2 * (KG / 8) + v];
           }
-          wbuf[k_code_position(tq0 + tl, i * N, BITS, D).word - w0] = word;
+          add_codes<BITS, V2>(a0, BITS * (2 * v), x.x, t1.x, t2.x, t3.x);
+          add_codes<BITS, V2>(a1, BITS * (2 * v), x.y, t1.y, t2.y, t3.y);
+          add_codes<BITS, V2>(a0, BITS * (2 * v + 1), x.z, t1.z, t2.z, t3.z);
+          add_codes<BITS, V2>(a1, BITS * (2 * v + 1), x.w, t1.w, t2.w, t3.w);
         }
+        wbuf[k_code_position(tq0 + tl, d0, BITS, D).word - w0] = __byte_perm(finish(a0), finish(a1), 0x6420);
       }
       __syncthreads();
       uint4* dst = reinterpret_cast<uint4*>(codes + (size_t)bh * stream_words + w0);
@@ -424,35 +433,35 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __grid_constan
       }
     } else {
       constexpr int WPC = T / N;  // words per channel over the tile's tokens
+      // a thread takes a word of two neighbouring channels
 #pragma unroll
-      for (int k = 0; k < (D * WPC + PACK_THREADS - 1) / PACK_THREADS; ++k) {
+      for (int k = 0; k < (D / 2 * WPC + PACK_THREADS - 1) / PACK_THREADS; ++k) {
         const int item = tid + k * PACK_THREADS;
-        if (item < D * WPC) {
-          const int d = item % D, wi = item / D, gi = d / G;
-          uint32_t word = 0u;
+        if (item < D / 2 * WPC) {
+          const int d = item % (D / 2) * 2, wi = item / (D / 2), gi = d / G;
+          const uint8_t* col = tile + wi * N * ROWB + d * 2;
+          const uint4* th = reinterpret_cast<const uint4*>(thr_mem) + wi * N * NG + gi;
+          uint32_t acc[4] = {0u, 0u, 0u, 0u};  // tokens t % 4: the codes' bits of that byte
 #pragma unroll
-          for (int s4 = 0; s4 < N / 4; ++s4) {
-            const int tl = wi * N + 4 * s4;  // four consecutive tokens: four groups
-            const uint8_t* src = tile + tl * ROWB + d * 2;
-            const uint32_t x0 = *reinterpret_cast<const uint16_t*>(src), x1 = *reinterpret_cast<const uint16_t*>(src + ROWB);
-            const uint32_t x2 = *reinterpret_cast<const uint16_t*>(src + 2 * ROWB), x3 = *reinterpret_cast<const uint16_t*>(src + 3 * ROWB);
-            const uint2 t1 = *reinterpret_cast<const uint2*>(thr + gi * T + tl);
-            uint2 t2 = t1, t3 = t1;
-            if constexpr (BITS == 2) {
-              t2 = *reinterpret_cast<const uint2*>(thr + NPAR + gi * T + tl);
-              t3 = *reinterpret_cast<const uint2*>(thr + 2 * NPAR + gi * T + tl);
+          for (int t = 0; t < N; ++t) {
+            const uint32_t x = *reinterpret_cast<const uint32_t*>(col + t * ROWB);
+            const uint4 tt = th[t * NG];
+            add_codes<BITS, V2>(acc[t % 4], BITS * (t / 4), x, tt.x, tt.y, tt.z);
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[j] = finish(acc[j]);
+          const uint32_t a = __byte_perm(acc[0], acc[1], 0x6240), b = __byte_perm(acc[2], acc[3], 0x6240);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            uint32_t word = __byte_perm(a, b, h ? 0x7632 : 0x5410);
+            uint32_t* dst = codes + (size_t)bh * stream_words + v_code_position(tq0 + wi * N, d + h, BITS, D).word;
+            if (merge || stats) {
+              const uint32_t o = *dst;
+              if (stats) delta_count<BITS>(o, word, hist);
+              word = merge_words<BITS>(o, word, p.merge_lut[BITS - 1]);
             }
-            const uint32_t lo = code_pair<BITS, V2>(x0 | (x1 << 16), t1.x, t2.x, t3.x);
-            const uint32_t hi = code_pair<BITS, V2>(x2 | (x3 << 16), t1.y, t2.y, t3.y);
-            word |= __byte_perm(lo, hi, 0x6420) << (BITS * s4);
+            if (store) *dst = word;
           }
-          uint32_t* dst = codes + (size_t)bh * stream_words + v_code_position(tq0 + wi * N, d, BITS, D).word;
-          if (merge || stats) {
-            const uint32_t o = *dst;
-            if (stats) delta_count<BITS>(o, word, hist);
-            word = merge_words<BITS>(o, word, p.merge_lut[BITS - 1]);
-          }
-          if (store) *dst = word;
         }
       }
     }
