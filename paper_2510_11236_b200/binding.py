@@ -241,6 +241,8 @@ class Cache:
         import torch
         self.cfg = cfg
         self.device = torch.device(device)
+        self._index = torch.cuda.current_device() if self.device.index is None else self.device.index
+        self._raw_stream = torch._C._cuda_getCurrentRawStream  # the current stream without a Stream object around it
         nbytes = xq_workspace_bytes(cfg)
         if nbytes == 0:
             raise XQError(XQ_ERR_CONFIG, "xq_workspace_bytes")
@@ -253,8 +255,7 @@ class Cache:
             raise XQError(rc, "xq_create")
 
     def _stream(self) -> int:
-        import torch
-        return torch.cuda.current_stream(self.device).cuda_stream
+        return self._raw_stream(self._index)
 
     def close(self):
         if getattr(self, "handle", None):

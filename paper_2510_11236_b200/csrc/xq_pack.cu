@@ -220,8 +220,8 @@ __device__ __forceinline__ void delta_count(uint32_t w0, uint32_t w1, uint32_t (
 // G: group size; T: a multiple of G and of 32; F16: the 16-bit type is IEEE half precision.
 // blockIdx.y is the (sequence, kv head) stream, blockIdx.z the layer of the launch.  With p.win_count > 0 the CTAs of the first block also copy
 // the new window rows that replace the rows they staged.
-template <int D, int G, int T, bool F16>
-__global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __grid_constant__ PackParams p) {
+template <int D, int G, int T, bool F16, int LAYERS>
+__global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __grid_constant__ PackParamsOf<LAYERS> p) {
   using I16 = In16<F16>;
   using V2 = typename I16::V2;
   constexpr int ROWB = D * 2 + PACK_ROW_PAD;
@@ -480,8 +480,12 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __grid_constan
 template <int D, int G, bool F16>
 cudaError_t launch_pack_t(const PackParams& p, cudaStream_t st) {
   // a tile is one key group long: 32 or 64 tokens, whole words of either kind
-  return launch_dependent(pack_kernel<D, G, G, F16>, dim3(2 * p.n_blocks * (p.dm.R / G), p.dm.B * p.dm.Hkv, p.n_layers),
-                          dim3(PACK_THREADS), 0, st, p);
+  const dim3 grid(2 * p.n_blocks * (p.dm.R / G), p.dm.B * p.dm.Hkv, p.n_layers), block(PACK_THREADS);
+  if (p.n_layers > 1) return launch_dependent(pack_kernel<D, G, G, F16, PACK_MAX_LAYERS>, grid, block, 0, st, p);
+  PackParamsOf<1> one;
+  static_cast<PackCommon&>(one) = p;
+  one.layer[0] = p.layer[0];
+  return launch_dependent(pack_kernel<D, G, G, F16, 1>, grid, block, 0, st, one);
 }
 
 cudaError_t launch_pack(const PackParams& p, cudaStream_t st) {
