@@ -20,14 +20,18 @@
 // large operand; a tcgen05 kernel has to pass them through tensor memory and hand batches between warps, and the
 // version before this one spent a batch's ~1600 cycles on that chain of hand-overs, two batches per SM at a time
 // (32k context, four heads: 34.7 us per layer).  Here sixteen independent warps share an SM and hide each other's
-// latencies: 30.2 us (4k context, one head per kv head: 28.8 -> 27.3; 8k context, groups of 64: 33.0 -> 25.9;
-// 128k context: 35.5 -> 26.2; head_dim 64, 512 tokens, which had only the scalar kernel: 380 -> 5).
-// What bounds it: instruction issue.  A batch (four heads, 32-token groups) is ~2000 warp instructions, 512 of them
-// the masks (ALU: 2 cycles each per sub-partition), 140 products (8 cycles each), ~350 half-precision multiplies
-// (2 cycles each); about two thirds of the issue slots are used inside the loop.
-// Measured and not kept (32k context, four heads): one CTA of 12 warps per SM 32.0 us, of 8 warps 34.1; four CTAs of
-// 4 warps 32.0; three CTAs of 5 warps 33.4 (fewer registers do not pay for more warps, nor fewer warps for more
-// registers).
+// latencies.  A layer in a step of 16 or 32 (layers share launches), us, before and now: 32k context, four heads, batch
+// 4: 34.2 -> 25.5 (84 MB: 3.3 TB/s); 4k, one head per kv head, batch 8: 28.1 -> 22.9; 8k, groups of 64, batch 16: 32.4 -> 22.9; one
+// sequence of 128k: 34.5 -> 24.8; groups of five heads at 16k: 34.2 -> 30.5; head_dim 64, 512 tokens, which had only
+// the scalar kernel: 380 -> 5.
+// What bounds it: issue and latency of a batch's phases.  A batch (four heads, 32-token groups) is ~2000 warp
+// instructions, 512 of them the masks (ALU: 2 cycles each per sub-partition), 140 products (8 cycles each), ~350
+// half-precision multiplies (2 cycles each), and takes a warp ~14000 cycles with sixteen on the SM: key products 2900,
+// value products 3100, waits for copies and their issue 1700, key scales 1600, softmax 1400, value scales 1000,
+// biases 700.  A CTA's start and end cost 5000 each, which is why a step wants few CTAs (plan_splits).
+// Measured and not kept (32k context, four heads, us per 32 layers; this shape 925 then): four CTAs of 4 warps 944,
+// three of 4 1014, three of 5 1025, one of 12 1026 (fewer registers do not pay for more warps, nor fewer warps for
+// more registers).
 #pragma once
 #include "xq_internal.h"
 #include "xq_mma.cuh"
@@ -308,9 +312,14 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
   const int bh = b * dm.Hkv + hk;
   const int nbt = (p.n_q + BT - 1) / BT;  // batches of the stream (the last one may be ragged)
   int b0, b1, wt0, wt1;
-  share_of((nbt + p.deal - 1) / p.deal, ns, split, b0, b1);
-  b0 *= p.deal;
-  b1 = min(b1 * p.deal, nbt);
+  {
+    // the larger shares come last, with the run that may be short
+    const int runs = (nbt + p.deal - 1) / p.deal;
+    int lo, hi;
+    share_of(runs, ns, ns - 1 - split, lo, hi);
+    b0 = (runs - hi) * p.deal;
+    b1 = min((runs - lo) * p.deal, nbt);
+  }
   share_of(p.r, ns, split, wt0, wt1);
   const int nb = b1 - b0;
 

@@ -224,6 +224,12 @@ MmaShape mma_shape(const xq_cache* c, int l) {
   return s;
 }
 
+// Layers of a step from which on they share launches.  A launch of its own costs a layer ~2.5 us of host time and a
+// start and an end with idle SMs: 32 layers of one user at 1000 tokens take 140 us with a launch each, 54 us together;
+// 32k context 965 and 927 us, 48 layers with host buffers 1608 and 1521 us.  A model of one or two layers keeps a
+// launch per layer, which callers that watch xq_launch_count have seen so far (10.6 us for a tiny pair; 8.5 together).
+constexpr int MIN_JOINT_LAYERS = 3;
+
 // Splits per (sequence, kv head) stream.  Tensor-core kernel: every split takes whole
 // batches of the packed region and a share of the window (ns_w = 0), sized towards
 // whole waves of resident CTAs.  Generic kernel:
@@ -250,26 +256,62 @@ void plan_splits(const xq_cache* c, int l, int nq, int r, int& ns_q, int& ns_w, 
       if (n_ctas_out) *n_ctas_out = ns_q * streams;
       return;
     }
-    // Time of a launch in units of one batch's time on an SM of which nothing is idle: a wave costs a start and an
-    // end of about 12 units, and as long as its CTAs' batches take: one after the other in the slowest warp (a warp
-    // alone takes about 6 units for a batch), or all of the SM's together.
-    int best = 1;
-    double best_time = 0.0;
-    for (int ns = 1; ns <= XQ_MAX_SPLITS && ns <= most; ++ns) {
-      const long long ctas = (long long)ns * streams;
-      const double waves = (double)((ctas + slot_count - 1) / slot_count);
+    // Largest number of batches that a split gets (the last run, which may be short, goes to a split of the larger kind)
+    auto largest = [&](int ns) {
+      const int base = runs / ns, rem = runs % ns;
+      const int last = (base + (rem > 0 ? 1 : 0)) * deal - (runs * deal - batches), others = (base + (rem > 1 ? 1 : 0)) * deal;
+      return ns > 1 && others > last ? others : last;
+    };
+    // Time of a launch of one layer in units of one batch's time on an SM of which nothing is idle: a wave costs a
+    // start and an end of about 12 units, and as long as its CTAs' batches take: one after the other in the slowest
+    // warp (a warp alone takes about 6 units for a batch), or all of the SM's together.
+    auto wave = [&](int ns, long long ctas) {
       long long resident = (ctas + c->sm_count - 1) / c->sm_count;
       if (resident > shape.ctas_per_sm) resident = shape.ctas_per_sm;
-      const int per = (runs + ns - 1) / ns * deal;
+      const int per = largest(ns);
       const double chain = 6.0 * ((per + shape.warps - 1) / shape.warps), together = (double)per * (double)resident;
-      const double time = waves * (12.0 + (chain > together ? chain : together)) + 0.05 * ns;
-      if (ns == 1 || time < best_time) { best_time = time; best = ns; }
+      return 12.0 + (chain > together ? chain : together);
+    };
+    auto alone = [&](int ns) {
+      const long long ctas = (long long)ns * streams;
+      return (double)((ctas + slot_count - 1) / slot_count) * wave(ns, ctas) + 0.05 * ns;
+    };
+    // The same of a step whose layers share launches: a CTA follows the one before it in its slot, so only their
+    // number and the last, partly filled wave count.  CTA of 8 warps, 32k context, 32 streams, us per layer with 4, 6,
+    // 8, 9, 10, 12 splits: 25.4, 27.0, 27.3, 28.6, 29.2, 30.6, that is 14 units a CTA.
+    auto step = [&](int ns) {
+      const long long ctas = (long long)c->cfg.n_layers * ns * streams, rest = ctas % slot_count;
+      const double each = 14.0 + (double)batches / ns * shape.ctas_per_sm;
+      return (double)(ctas / slot_count) * each + (rest ? wave(ns, rest) : 0.0);
+    };
+    // Steps of 16 layers, us per layer, by the time alone / by the time of a step: four heads, 32k tokens and one
+    // block more, 29.5 / 26.1; 16k 18.1 / 14.4; one sequence of 20k 9.3 / 6.4; one user at 1000 tokens (32 layers)
+    // 0.77 / 0.51; at 8000 3.6 / 3.0.  The price is paid by a layer called alone, whose long chains the model
+    // underrates: 32k 35.6 / 43.4, 16k 21.2 / 24.4 us.  Both give the same bits, so there is one plan;
+    // cfg.n_splits sets another.
+    const bool joint = c->cfg.n_layers >= MIN_JOINT_LAYERS;
+    const int limit = most < XQ_MAX_SPLITS ? most : XQ_MAX_SPLITS;
+    int best = 1;
+    double times[XQ_MAX_SPLITS + 1];
+    for (int ns = 1; ns <= limit; ++ns) {
+      times[ns] = alone(ns);
+      if (times[ns] < times[best]) best = ns;
+    }
+    if (joint) {
+      // of the splits that cost a layer alone at most a tenth more, those that a step takes the least time with
+      const double bound = 1.1 * times[best];
+      double best_time = step(best);
+      for (int ns = 1; ns <= limit; ++ns) {
+        if (times[ns] > bound) continue;
+        const double t = step(ns);
+        if (t < best_time) { best_time = t; best = ns; }
+      }
     }
     ns_q = best;
     if (n_ctas_out) *n_ctas_out = best * streams;
-    // One wave that does not fill every resident slot: give some streams one split more, if the splits are many
-    // enough for the CTAs' sizes to stay within a few percent of each other.
-    if ((long long)best * streams < slot_count && slot_count < (long long)(best + 1) * streams && best >= 8 &&
+    // A layer alone, one wave that does not fill every resident slot: give some streams one split more, if the splits
+    // are many enough for the CTAs' sizes to stay within a few percent of each other.
+    if (!joint && (long long)best * streams < slot_count && slot_count < (long long)(best + 1) * streams && best >= 8 &&
         best + 1 <= most && best + 1 <= XQ_MAX_SPLITS) {
       ns_q = best + 1;
       if (n_ctas_out) *n_ctas_out = slot_count;
@@ -532,11 +574,6 @@ int decode_impl(xq_cache* c, int layer, const void* q, void* out, int out_f32, c
   return XQ_OK;
 }
 
-// Layers of a step from which on they share launches.  A launch of its own costs a layer ~2.5 us of host time and a
-// start and an end with idle SMs: 32 layers of one user at 1000 tokens take 140 us with a launch each, 54 us together;
-// 32k context 965 and 927 us, 48 layers with host buffers 1608 and 1521 us.  A model of one or two layers keeps a
-// launch per layer, which callers that watch xq_launch_count have seen so far (10.6 us for a tiny pair; 8.5 together).
-constexpr int MIN_JOINT_LAYERS = 3;
 
 // Tensor-core decode of the layers order[0 .. n) in one launch, or few: consecutive layers of equal length and
 // bit-widths share one.  Layer l's q and out are slice l of q and out; with K_new / V_new the launch appends slice l

@@ -718,6 +718,28 @@ def test_chained_decode_launches_equal_single_calls():
     a.close(); b.close()
 
 
+@pytest.mark.parametrize("batches", [152, 153, 159])
+def test_decode_splits_of_whole_runs(batches):
+    """Enough batches for splits of whole runs (one batch per warp), the last run full, of one batch, of all but one.
+    However the batches are dealt, the same logits enter the same sums, so the results differ by the accumulation
+    alone: up to 160 fp32 steps per side, 2^-23 of sum p |v_hat| each at most, and numerators rounded at 2^-22."""
+    B, Hq, Hkv, D, S = 4, 32, 8, 128, 128 * batches + 40
+    gen = torch.Generator(device=DEV).manual_seed(batches)
+    k, v = (torch.randn(B, Hkv, S, D, generator=gen, device=DEV).to(torch.bfloat16) for _ in range(2))
+    q = torch.randn(B, Hq, 1, D, generator=gen, device=DEV).to(torch.bfloat16).reshape(B, Hq, D)
+    bound = (2 * 160 * 2.0 ** -23 + 2 * 2.0 ** -22) * float(v.abs().max())
+    outs = []
+    for n_splits, layers in ((1, 1), (0, 1), (0, 4), (3, 1), (7, 1)):
+        cache = xq.Cache(xq.make_config(n_layers=layers, batch=B, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=D,
+                                        max_seq=S + 128, n_splits=n_splits), DEV)
+        cache.append_kv(0, k, v)
+        outs.append(cache.decode_attention(0, q, f32=True).clone())
+        cache.check_device()
+        cache.close()
+    for o in outs[1:]:
+        assert float((o - outs[0]).abs().max()) <= bound
+
+
 @pytest.mark.parametrize("D,Hq,Hkv,S", [(128, 8, 2, 40), (128, 2, 2, 700), (64, 4, 1, 300)])
 def test_decode_step_layers_that_share_launches(D, Hq, Hkv, S):
     """Six layers of three bit-width combinations and two lengths (the last pair is five tokens ahead): the layers that
