@@ -36,7 +36,7 @@ BULK_MIN, BULK_MAX = 16, 64  # between 16 and 64 window blocks per call
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of the decode kernel (ncu, same launch shape as the
 # timed one; see profiles/), with the SHA-256 of the kernel's sources at the time the counters were taken: the
 # figure is reported only while the sources still hash to that.
-NCU_TRAFFIC = {"c2": {"bytes": 84.05e6 + 2.60e6,
+NCU_TRAFFIC = {"c2": {"bytes": 84.69e6 + 2.50e6,
                       "sources_sha256": "aafe1f3193d74c1d55e9d1a4309874d6a8a793292f0d4dcb65080bbb7dc7a849"}}
 KERNEL_SOURCES = ("xq_decode_mma.cuh", "xq_mma.cuh", "xq_layout.cuh", "xq_internal.h")
 
@@ -372,11 +372,11 @@ def main():
     bytes_pass2 = step_bytes(seq_before2 + 1, K)
     peak, peak_kind = _peaks()
     isolated = bytes_pass2 / (dec["total_ms"] * 1e-3) / 1e9 if dec["launches"] else 0.0
-    # The decode launches of pass 1 run back to back (each starts its prologue while its predecessor drains), so
-    # their average duration over that timed region is the region's time over their number; the few other kernels
-    # of the region (the steps that quantize a window block) are charged to them.
-    decode_launches_pass1 = K * L
-    avg_launch_us = ms / decode_launches_pass1 * 1e3
+    # The layers of a step share decode launches, which run back to back, so a layer call's duration is the timed
+    # region's time over the number of layer calls; the few other kernels of the region (the steps that quantize a
+    # window block) are charged to them.
+    layer_calls_pass1 = K * L
+    avg_launch_us = ms / layer_calls_pass1 * 1e3
     achieved = bytes_pass1 / (ms * 1e-3) / 1e9
 
     # ---- pass 3: end to end through the C ABI with host buffers
@@ -417,7 +417,7 @@ def main():
     chunk = {"n_q_tokens": CHUNK_T, "layers": chunk_layers, "context": S_now,
              "us_per_query_token_and_layer": ms_chunk * 1e3 / (CHUNK_T * chunk_layers),
              "attended_tokens_per_s": world * B * CHUNK_T * chunk_layers * (S_now - (CHUNK_T - 1) / 2.0) / (ms_chunk * 1e-3),
-             "how": "one decode launch per query token with its visibility limit"}
+             "how": "one launch per chunk: all its query rows share one pass over the cache"}
     rc, nsq, nsw = xq.xq_split_plan(cache.handle, 0)  # the decode launches' split plan (before the appends below)
 
     # ---- pass 4: the quantize-and-pack path: every layer receives whole window blocks (R tokens per call), so each
@@ -465,7 +465,7 @@ def main():
         line = {
             "metric": METRIC, "value": value, "unit": "GB/s", "n_gpus": world, "steps": K, "warmup": Wm,
             "ms_per_step": ms_max / K, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": "u8 x u8 -> s32 tensor-core products (24-bit fixed-point operands), f32 softmax, bf16 io",
+            "dtype": "f16 tensor-core products (codes exact, other operand as hi + lo pairs), f32 accumulation and softmax, bf16 io",
             "data": "synthetic",
             "config": _config_block(args, w),
             "run": {"equiv_bits": xq.xq_equiv_bits(cfg), "layer_order": args.layer_order,
@@ -483,12 +483,12 @@ def main():
                          "peak_source": peak_kind, "unit": "GB/s", "frac": achieved / peak,
                          "frac_of_8TBps": achieved / 8000.0,
                          "traffic": _ncu_traffic(args.config) if not (args.layers or args.seq or args.splits) else None,
-                         "algorithmic_bytes_per_launch": bytes_pass1 / decode_launches_pass1,
-                         "avg_launch_us": avg_launch_us, "launches": decode_launches_pass1,
-                         "timing": "CUDA events around the timed region of back-to-back launches, divided by the decode launches in it",
+                         "algorithmic_bytes_per_launch": bytes_pass1 / layer_calls_pass1,
+                         "avg_launch_us": avg_launch_us, "launches": layer_calls_pass1,
+                         "timing": "CUDA events around the timed region of back-to-back launches, per layer call (a launch serves up to 32 layers)",
                          "isolated": {"avg_launch_us": dec["avg_us"], "achieved": isolated, "frac": isolated / peak,
                                       "launches": dec["launches"],
-                                      "timing": "CUDA events around every launch (no overlap of a launch's prologue with its predecessor's tail)"}},
+                                      "timing": "CUDA events around every launch (the layers of a step that share it)"}},
             "chunk": chunk,
             "kernels": kinds,
             "flush_step": {"what": "the step on which every layer's window block fills: one quantize-and-pack launch for "
