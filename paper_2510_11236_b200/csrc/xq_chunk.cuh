@@ -11,16 +11,15 @@
 // accumulated in fp32 in tensor memory.  Two groups of four warps (thread = row = tensor-memory lane) take the softmax
 // of the even and of the odd tiles; the softmax reference of a row goes from one to the other through shared memory
 // and is raised only when a logit exceeds it by more than 8 (log2 units), which rescales O (rare).  One warp issues the
-// products: keys of tile i + 2, then values of tile i.  Tokens of the 16-bit window are expanded into the same pairs (exactly).  Split partials are
-// merged by the last CTA of a row tile, as in the decode kernel.
+// products: keys of tile i + 2, then values of tile i.  Tokens of the 16-bit window are expanded into the same pairs
+// (exactly).  Split partials are merged by the last CTA of a row tile, as in the decode kernel.
 //
 // What bounds it: the expanding warps, ~2800-3300 cycles per tile (the products: ~1650), and with them the instruction
-// cache: hot code above ~30 KB runs slower, so the loops are rolled.  Four more expanding warps, at 80 registers a
-// thread, were slower (969 / 532 / 125 us in the order below); two softmax groups because one row per thread takes
-// longer than a tile's products; four S buffers
-// so that the keys of two tiles are ahead (two: 1108 / 532 / 137 -> 1056 / 506 / 136 then).  Against one decode launch per query token, us: 16 tokens behind 32k, batch 4, four
-// layers, 2278 -> 922; 250 tokens behind 8k, two layers, 6063 -> 499; a prompt of 1024, 32 kv heads, two layers,
-// 10516 -> 123.
+// cache: hot code above ~30 KB runs slower, so the loops are rolled.  Against one decode launch per query token, us:
+// 16 tokens behind 32k, batch 4, four layers, 2278 -> 922; 250 tokens behind 8k, two layers, 6063 -> 499; a prompt of
+// 1024, 32 kv heads, two layers, 10516 -> 123.  In the same order: four more expanding warps, at 80 registers a thread,
+// were slower, 969 / 532 / 125; four S buffers, so that the keys of two tiles are ahead, took 1108 / 532 / 137 to
+// 1056 / 506 / 136, softmax in two passes of 32 columns those to 922 / 499 / 123.
 //
 // Every wait on an mbarrier is bounded: a thread that gives up sets a flag in shared memory that makes every other
 // wait of the CTA give up too; the CTA then waits for its products in flight, frees its tensor memory, reports through
