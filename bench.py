@@ -33,11 +33,11 @@ METRIC = "decode-attention GB/s at 32k ctx"
 APPEND_BLOCKS = 6  # window blocks quantized per layer in the append pass, one block per call
 BULK_BYTES = 256e6  # then two calls per layer of about this much 16-bit input each (a prefill-sized append):
 BULK_MIN, BULK_MAX = 16, 64  # between 16 and 64 window blocks per call
-# dram__bytes_read.sum + dram__bytes_write.sum of one launch of the decode kernel (ncu, same launch shape as the
-# timed one; see profiles/), with the SHA-256 of the kernel's sources at the time the counters were taken: the
+# dram__bytes_read.sum + dram__bytes_write.sum of one layer call of the decode kernel (ncu, a launch of four layers;
+# see profiles/), with the SHA-256 of the kernel's sources at the time the counters were taken: the
 # figure is reported only while the sources still hash to that.
-NCU_TRAFFIC = {"c2": {"bytes": 84.69e6 + 2.50e6,
-                      "sources_sha256": "aafe1f3193d74c1d55e9d1a4309874d6a8a793292f0d4dcb65080bbb7dc7a849"}}
+NCU_TRAFFIC = {"c2": {"bytes": 335.5e6 / 4 + 4.3e6 / 4,
+                      "sources_sha256": "ae02fb3b34429808aeaa77f676da84500e03c8005f0fe6ad7ae914e8046b8f9e"}}
 KERNEL_SOURCES = ("xq_decode_mma.cuh", "xq_mma.cuh", "xq_layout.cuh", "xq_internal.h")
 
 
