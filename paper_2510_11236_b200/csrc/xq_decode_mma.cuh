@@ -178,10 +178,14 @@ __device__ __forceinline__ void window_tile(uint32_t wbuf, int n_valid, const ui
   const float f = ex2(m - mn);
   const float p0 = ex2(x0 - mn), p1 = ex2(x1 - mn);
   m = mn;
-  // numerators as a 16-bit pair hi + lo (at least 16 bits of precision), transposed into B-operand order
+  // Numerators as unevaluated sums of three 16-bit numbers (bfloat16: 24 bits, all of an fp32 numerator; a pair would
+  // leave errors of 2^-17, four times what everything else here adds up to), the first two in the two columns of the
+  // head, the third beside a zero; transposed into B-operand order.
   const uint32_t h0 = pack_io2<F16>(p0, 0.f), h1 = pack_io2<F16>(p1, 0.f);
-  const uint32_t l0 = pack_io2<F16>(p0 - io2_lo<F16>(h0), 0.f), l1 = pack_io2<F16>(p1 - io2_lo<F16>(h1), 0.f);
-  const uint32_t bh0 = movmatrix_trans(h0), bh1 = movmatrix_trans(h1), bl0 = movmatrix_trans(l0), bl1 = movmatrix_trans(l1);
+  const float e0 = p0 - io2_lo<F16>(h0), e1 = p1 - io2_lo<F16>(h1);
+  const uint32_t m0 = pack_io2<F16>(p0, e0), m1 = pack_io2<F16>(p1, e1);
+  const uint32_t l0 = pack_io2<F16>(e0 - io2_hi<F16>(m0), 0.f), l1 = pack_io2<F16>(e1 - io2_hi<F16>(m1), 0.f);
+  const uint32_t bh0 = movmatrix_trans(m0), bh1 = movmatrix_trans(m1), bl0 = movmatrix_trans(l0), bl1 = movmatrix_trans(l1);
   float ps = p0 + p1;
 #pragma unroll
   for (int k = 4; k < 32; k <<= 1) ps += __shfl_xor_sync(0xffffffffu, ps, k);
@@ -192,11 +196,11 @@ __device__ __forceinline__ void window_tile(uint32_t wbuf, int n_valid, const ui
   for (int mt = 0; mt < KS; ++mt) {
     uint32_t a0, a1, a2, a3;
     ldmatrix_x4_trans(va + mt * 32, a0, a1, a2, a3);
-    float acc[4] = {o[mt][0] * f, 0.f, o[mt][1] * f, 0.f};
-    mma16816<F16>(acc, a0, a1, a2, a3, bh0, bh1);
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
     mma16816<F16>(acc, a0, a1, a2, a3, bl0, bl1);
-    o[mt][0] = acc[0];
-    o[mt][1] = acc[2];
+    mma16816<F16>(acc, a0, a1, a2, a3, bh0, bh1);
+    o[mt][0] = fmaf(o[mt][0], f, acc[0] + acc[1]);
+    o[mt][1] = fmaf(o[mt][1], f, acc[2] + acc[3]);
   }
 }
 

@@ -868,3 +868,26 @@ def _full_size_pair(name, w, pair):
             worst = max(worst, err)
     print(f"{name}: splits {nsq}+{nsw}, worst fp32 attention error over sampled streams {worst:.2e}")
     cache.close()
+
+
+def _exact_attention(q, K, V):
+    """fp64 attention of q [B, Hq, D] over K, V [B, Hkv, S, D] as they are."""
+    B, Hq, D = q.shape
+    G = Hq // K.shape[1]
+    K, V = K.double().repeat_interleave(G, 1), V.double().repeat_interleave(G, 1)
+    p = torch.softmax((q.double()[:, :, None] * K).sum(-1) / D ** 0.5, -1)
+    return (p[..., None] * V).sum(2)
+
+
+@pytest.mark.parametrize("D,G,S", [(64, 1, 31), (64, 4, 100), (128, 1, 17), (128, 4, 128), (128, 5, 100)])
+def test_window_attention_to_single_precision(D, G, S):
+    # Nothing is quantized: every factor of the fp32 result is exact but the logits (|x| < 16, a few roundings of 2^-24),
+    # the exponentials (2^-22) and the sums, which random signs add to about 2^-22 of the result; bound: twice that.
+    w = dict(n_layers=2, batch=4, n_q_heads=2 * G, n_kv_heads=2, head_dim=D, seq=S, residual_len=128, group_size=32,
+             kq=2, vq=2, km=0, vm=0, n_outliers=3, outlier_scale=4.0, seed=21, n_splits=0)
+    cache = xq.Cache(W.make_xq_config(w), DEV)
+    K, V = _fill(cache, w, [0], S)[0]
+    q = W.queries(w, 0, 0, DEV)
+    ref = _exact_attention(q, K, V)
+    err = (cache.decode_attention(0, q, f32=True).double() - ref).norm() / ref.norm()
+    assert err.item() <= 2.0 ** -21
