@@ -3,8 +3,12 @@
 //
 // Every warp works alone on batches of 128 tokens: nothing in the loop waits for another warp.  Codes are expanded
 // straight into A fragments of mma.sync.m16n8k16 (fp16): four codes of a row sit at one bit offset of the four bytes
-// of a packed word, so `word & 0x00030003 << 2e` is a pair of fp16 subnormals, code * 4^e * 2^-24, for one logic
-// instruction per two codes.  Scale and zero-point are folded out of the inner products,
+// of a packed word, so `word << 2 & 0x000c000c << 2e` is a pair of fp16 subnormals, code * 4^e * 2^-22, for one logic
+// instruction per two codes (and a shift per word: the tensor core aligns a product by the exponent fields of its
+// operands, so every leading zero of a subnormal costs the sum a bit; codes at the very foot of the fraction, without
+// the shift, put the fp32 results four to seven times farther off: 4.2e-4 of the result's norm at 32k, 2-bit, now
+// 0.6e-4; multiplying them up into normal numbers, 0.3e-4, costs 17 % of the time, the shift 1.5 %).  Scale and
+// zero-point are folded out of the inner products,
 //
 //   q . k_hat_t = sum_d (q_d s_d) c_td + sum_d q_d z_d        (keys, per channel)
 //   sum_t p_t v_hat_td = sum_t (p_t s_tg) c_td + sum_t p_t z_tg  (values, per token)
@@ -42,6 +46,7 @@ namespace {
 constexpr int BT = 128;            // tokens per batch
 constexpr float TAU = 3.f;         // log2 units a logit may exceed the softmax reference before it is raised
 constexpr int P_EXP = 11;          // numerators are carried times 2^P_EXP (at most 2^(P_EXP + TAU) as fp16)
+constexpr int CODE_EXP = 22;       // a code operand is code * 4^e * 2^-CODE_EXP (1-bit: 2^e)
 constexpr int Q_BIAS_EXP = 8;      // exponent of the largest |q| in the zero-point products
 
 // Shared-memory plan.  D: head dim, GS: quantization group, BK / BV: bits.  The eight operand columns are four column
@@ -86,7 +91,7 @@ struct Plan {
   static_assert(TOTAL <= LIMIT, "shared memory");
 };
 
-// log2 of the weight that the code of k-slot (step ks, any tig, any pair) carries in its fp16 pattern, beside 2^-24
+// log2 of the weight that the code of k-slot (step ks, any tig, any pair) carries in its fp16 pattern, beside 2^-CODE_EXP
 template <int D, int BK>
 __device__ __forceinline__ constexpr int k_weight(int ks) { return BK == 2 ? 2 * (ks % 4) : (D == 128 ? ks : ks % 4); }
 // channel of k-slot c (pairs (0, 2) and (1, 3)) of step ks for lane column tig
@@ -440,7 +445,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
         qk[n][ks][0] = *reinterpret_cast<const uint32_t*>(&h0);
         qk[n][ks][1] = *reinterpret_cast<const uint32_t*>(&h1);
       }
-      ck[n] = cq[n] * pow2i(24 - e);
+      ck[n] = cq[n] * pow2i(CODE_EXP - e);
     }
   };
 
@@ -543,18 +548,21 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
       }
     }
     // ---- keys: q . c ----
-    auto load_rows = [&](int u, int kw, uint32_t (&w)[2][2], uint32_t (&w8)[2][2]) {  // packed words of rows gid, gid + 8
+    // packed words of rows gid, gid + 8: even bytes, odd bytes
+    auto load_rows = [&](int u, int kw, uint32_t (&w)[2][2], uint32_t (&w8)[2][2]) {
 #pragma unroll
       for (int t = 0; t < 2; ++t)
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
           const int tk = 16 * t + 2 * r;
-          if constexpr (BK == 1 && D == 64) w[t][r] = lds32(kc_lane + u * 256 + tk * 8) >> (4 * (tig & 1));
-          else w[t][r] = lds32(kc_lane + u * (32 * D * BK / 8) + kw * 512 + tk * 16);
-          w8[t][r] = high_bytes(w[t][r]);
+          uint32_t raw;
+          if constexpr (BK == 1 && D == 64) raw = lds32(kc_lane + u * 256 + tk * 8) >> (4 * (tig & 1));
+          else raw = lds32(kc_lane + u * (32 * D * BK / 8) + kw * 512 + tk * 16);
+          w[t][r] = even_bytes_up(raw);
+          w8[t][r] = odd_bytes_up(raw);
         }
     };
-    auto key_mask = [](int k) { return BK == 2 ? 0x00030003u << (2 * (k & 3)) : 0x00010001u << k; };
+    auto key_mask = [](int k) { return BK == 2 ? 0x000c000cu << (2 * (k & 3)) : 0x00040004u << k; };
     constexpr int KPW = KS / KWORDS;  // k-steps a word serves
     if constexpr (GC == 1) {
       constexpr int UG = GS / 32;  // units of a group
@@ -800,18 +808,20 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
     // ---- values: one chunk of packed words at a time (lane column tig owns word tig of every channel row) ----
 #pragma unroll
     for (int c = 0; c < VCH; ++c) {
-      uint32_t w[KS][2], w8[KS][2];  // rows (channels) 16 mt + gid, + 8
+      uint32_t w[KS][2], w8[KS][2];  // even and odd bytes of rows (channels) 16 mt + gid, + 8
       const uint32_t va = st + Pl::OFF_VC + c * D * 16 + gid * 16 + tig * 4;
 #pragma unroll
       for (int mt = 0; mt < KS; ++mt) {
-        w[mt][0] = lds32(va + mt * 256);
-        w[mt][1] = lds32(va + mt * 256 + 128);
-        w8[mt][0] = high_bytes(w[mt][0]);
-        w8[mt][1] = high_bytes(w[mt][1]);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const uint32_t raw = lds32(va + mt * 256 + r * 128);
+          w[mt][r] = even_bytes_up(raw);
+          w8[mt][r] = odd_bytes_up(raw);
+        }
       }
 #pragma unroll
       for (int e = 0; e < VE; ++e) {
-        const uint32_t msk = BV == 2 ? 0x00030003u << (2 * e) : 0x00010001u << e;
+        const uint32_t msk = BV == 2 ? 0x000c000cu << (2 * e) : 0x00040004u << e;
         constexpr int VB = CP / GC;  // operands of a step: parts GC * vb + slot
         uint32_t sp[2][VB];
         const uint32_t sa = vs_lane + pair_row(32 * c) * Pl::VSROW + 2 * e * Pl::VSROW, sb = sa + Pl::VSROW;
@@ -863,7 +873,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
   float o[NT][KS][2], l[NT];
 #pragma unroll
   for (int n = 0; n < NT; ++n) {
-    const float ua = pow2i(24 - P_EXP - Ev), uz = pow2i(-P_EXP);
+    const float ua = pow2i(CODE_EXP - P_EXP - Ev), uz = pow2i(-P_EXP);
     const float z = (zacc[n][0] + zacc[n][1]) * uz;  // row gid < NG: channel group gid; row NG: the sum
     l[n] = __shfl_sync(0xffffffffu, z, NG * 4 + tig);
 #pragma unroll

@@ -195,7 +195,17 @@ __device__ __forceinline__ uint32_t product_part(uint32_t a, uint32_t s, int low
       "@p fma.rn.f16x2 t, %1, %2, n;\nmov.b32 %0, t;\n}\n" : "=r"(d) : "r"(a), "r"(s), "r"(low));
   return d;
 }
-// w >> 8 as a byte permutation (a shift would be merged into the masks that follow it, once per mask)
-__device__ __forceinline__ uint32_t high_bytes(uint32_t w) { return __byte_perm(w, 0u, 0x4321); }
+// A packed word with the codes of bytes 0 and 2, or 1 and 3, two bits above the foot of each half.  (Opaque to the
+// compiler, which would merge the shift into the masks that follow it, once per mask.)
+__device__ __forceinline__ uint32_t even_bytes_up(uint32_t w) {
+  uint32_t d;
+  asm("shl.b32 %0, %1, 2;\n" : "=r"(d) : "r"(w));
+  return d;
+}
+__device__ __forceinline__ uint32_t odd_bytes_up(uint32_t w) {
+  uint32_t d;
+  asm("shr.b32 %0, %1, 6;\n" : "=r"(d) : "r"(w));
+  return d;
+}
 
 }  // namespace xq

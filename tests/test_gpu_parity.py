@@ -891,3 +891,29 @@ def test_window_attention_to_single_precision(D, G, S):
     ref = _exact_attention(q, K, V)
     err = (cache.decode_attention(0, q, f32=True).double() - ref).norm() / ref.norm()
     assert err.item() <= 2.0 ** -21
+
+
+def _relative_error(cache, cfg, kv, layer, q):
+    """2-norm of the fp32 result's error over that of the result, all streams."""
+    out = cache.decode_attention(layer, q, f32=True).double().cpu().numpy()
+    G = cfg.n_q_heads // cfg.n_kv_heads
+    num = den = 0.0
+    for b in range(cfg.batch):
+        for hk in range(cfg.n_kv_heads):
+            oc = util.oracle_for_stream(cfg, [layer], b, hk, kv)
+            ref = oc.decode(layer, util.bits_of(q[b:b + 1, hk * G:(hk + 1) * G]))[0]
+            num += ((out[b, hk * G:(hk + 1) * G] - ref) ** 2).sum()
+            den += (ref ** 2).sum()
+    return (num / den) ** 0.5
+
+
+@pytest.mark.parametrize("G,g,S", [(4, 64, 4000), (1, 32, 4000), (8, 32, 4000)])
+def test_two_bit_values_keep_sixteen_bits_of_the_sums(G, g, S):
+    # A code operand has at most eight leading zeros in its fp16 fraction: the sums of products keep 24 - 8 bits, and
+    # scale and zero-point parts that cancel leave about 1 / 8 of their size here: bound 2^-16 * 8 = 1.2e-4
+    w = dict(n_layers=2, batch=1, n_q_heads=2 * G, n_kv_heads=2, head_dim=128, seq=S, residual_len=128, group_size=g,
+             kq=2, vq=2, km=0, vm=0, n_outliers=3, outlier_scale=10.0, seed=22, n_splits=0)
+    cfg = W.make_xq_config(w)
+    cache = xq.Cache(cfg, DEV)
+    kv = _fill(cache, w, [0], S)
+    assert _relative_error(cache, cfg, kv, 0, W.queries(w, 0, 0, DEV)) <= 1.2e-4
