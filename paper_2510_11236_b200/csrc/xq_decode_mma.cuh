@@ -46,7 +46,6 @@ namespace {
 constexpr int BT = 128;            // tokens per batch
 constexpr float TAU = 3.f;         // log2 units a logit may exceed the softmax reference before it is raised
 constexpr int P_EXP = 11;          // numerators are carried times 2^P_EXP (at most 2^(P_EXP + TAU) as fp16)
-constexpr int CODE_EXP = 22;       // a code operand is code * 4^e * 2^-CODE_EXP (1-bit: 2^e)
 constexpr int Q_BIAS_EXP = 8;      // exponent of the largest |q| in the zero-point products
 
 // Shared-memory plan.  D: head dim, GS: quantization group, BK / BV: bits.  The eight operand columns are four column
@@ -67,7 +66,10 @@ struct Plan {
   // value scales, then zero-points, as they are reordered over VM: [pair of tokens][NG] half2, one more row after
   // the pairs of a lane column (bank conflicts)
   static constexpr int VSROW = 4 * NG, VS = 64 * VSROW + 4 * VSROW;
-  static constexpr int STAGE = KC + KM + VC + 2 * VS;
+  // centered codes: the second halves of the zero-points, of the values (as VS), of the keys (as the second half of KM)
+  static constexpr bool CENTERED = D == 64;
+  static constexpr int OFF_KL = OFF_VM + 3 * VS, KL = NGT * 2 * D;
+  static constexpr int STAGE = CENTERED ? OFF_KL + KL : OFF_VM + 2 * VS;
   // numerators: [head][pair of tokens (t, t + 2)] of (hi pair, lo pair), 16 bytes more after every 16 pairs and 32
   // more after every head against bank conflicts
   static constexpr int PH = 64 * 8 + 4 * 16 + 32;
@@ -80,7 +82,7 @@ struct Plan {
   static_assert(HP * NT * MS * 4 <= WARP, "a warp's state rows fit its own memory");
   // after the warps' parts: B fragments of the zero-point products; fp16 ones, read in place of zero-points for the
   // sum of the numerators; q as it came
-  static constexpr int QB = NT * KS * 32 * 4, ONES = 64 * VSROW, QS = HP * NT * D * 2;
+  static constexpr int QB = NT * KS * 32 * 4, ONES = CENTERED ? 0 : 64 * VSROW, QS = HP * NT * D * 2;
   static constexpr int room(int w) { return w * WARP + QB + ONES + QS; }
   // Two CTAs per SM, each of as many warps as registers (128, or 168 for eight heads) and shared memory allow.
   static constexpr int CTAS = 2;
@@ -91,7 +93,41 @@ struct Plan {
   static_assert(TOTAL <= LIMIT, "shared memory");
 };
 
-// log2 of the weight that the code of k-slot (step ks, any tig, any pair) carries in its fp16 pattern, beside 2^-CODE_EXP
+// Code operands.  head_dim 128: the masked code bits as they are, fp16 subnormals code * weight * 2^-22.  head_dim 64:
+// (code - center) * weight * 2^-9, normal numbers, center = (2^BITS - 1) / 2, and zero-points plus center scales, as
+// pairs of fp16, in place of the zero-points: both sums are then as small as the result, and no digit of it is lost where
+// they cancel.  That makes the kernel as exact as the scalar one, which served head_dim 64 before it (fp32 result against
+// fp64, of its norm: scalar 3.6-5.5e-7, this one 4.7-5.6e-7, with operands as for head_dim 128 1.0-2.5e-5) and costs a
+// layer of a step 0.4 us (2.8 to 3.3 us at 2048 tokens, 32 streams, four heads; scalar 500).
+template <int D>
+struct Code {
+  static constexpr bool CENTERED = D == 64;
+  static constexpr int EXP = CENTERED ? 9 : 22;
+  template <int BITS>
+  static __device__ __forceinline__ float center() { return 0.5f * (float)((1 << BITS) - 1); }
+  // the operand pair of the code bits at 2 + BITS * i of both halves of w; their weight is 2^(BITS * i)
+  template <int BITS>
+  static __device__ __forceinline__ uint32_t pair(uint32_t w, int i) {
+    const uint32_t m = w & ((BITS == 2 ? 0x000c000cu : 0x00040004u) << (BITS * i));
+    if constexpr (CENTERED) {
+      // times 2^13, less center * weight * 2^-9: 1.5 or 0.5 at exponent field 15 - 9 + BITS * i
+      const uint32_t c = BITS == 2 ? 0x8200u + ((uint32_t)(6 + 2 * i) << 10) : 0x8000u + ((uint32_t)(5 + i) << 10);
+      return hfma2(m, 0x70007000u, c * 0x10001u);
+    } else {
+      return m;
+    }
+  }
+};
+// z + center s of a pair of groups as an unevaluated sum of two fp16
+template <int D, int BITS>
+__device__ __forceinline__ void centered_zero(uint32_t s, uint32_t z, uint32_t& hi, uint32_t& lo) {
+  const float a = fmaf(Code<D>::template center<BITS>(), io2_lo<true>(s), io2_lo<true>(z));
+  const float b = fmaf(Code<D>::template center<BITS>(), io2_hi<true>(s), io2_hi<true>(z));
+  hi = pack_io2<true>(a, b);
+  lo = pack_io2<true>(a - io2_lo<true>(hi), b - io2_hi<true>(hi));
+}
+
+// log2 of the weight that the code of k-slot (step ks, any tig, any pair) carries in its operand
 template <int D, int BK>
 __device__ __forceinline__ constexpr int k_weight(int ks) { return BK == 2 ? 2 * (ks % 4) : (D == 128 ? ks : ks % 4); }
 // channel of k-slot c (pairs (0, 2) and (1, 3)) of step ks for lane column tig
@@ -275,6 +311,7 @@ template <int D, int BK, int BV, int GS, int HP, int NT>
 __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<D, BK, BV, GS, HP, NT>::CTAS)
     decode_mma_kernel(const __grid_constant__ DecodeParams p) {
   using Pl = Plan<D, BK, BV, GS, HP, NT>;
+  using Cd = Code<D>;
   constexpr int KS = Pl::KS, NG = Pl::NG, NGT = Pl::NGT, W = Pl::WARPS, WROW = Pl::WROW, GC = Pl::GC, CP = Pl::CP;
   constexpr int KWORDS = (BK == 2 && D == 128) ? 2 : 1;  // packed words of a token row that a thread expands
   constexpr int VCH = BV;                               // 16-byte chunks of a channel row (128 / BV tokens each)
@@ -445,18 +482,20 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
         qk[n][ks][0] = *reinterpret_cast<const uint32_t*>(&h0);
         qk[n][ks][1] = *reinterpret_cast<const uint32_t*>(&h1);
       }
-      ck[n] = cq[n] * pow2i(CODE_EXP - e);
+      ck[n] = cq[n] * pow2i(Cd::EXP - e);
     }
   };
 
   // softmax state: reference m (log2 units, an integer; -infinity before the first batch, where mr is 0 instead).
-  // Row gid of zacc: the zero-point products of channel group gid (gid < NG), the sum of the numerators (gid >= NG).
-  float m[NT], mr[NT], acc[NT][KS][4], zacc[NT][4];
+  // Row gid of zacc: the zero-point products of channel group gid (gid < NG), the sum of the numerators (gid >= NG;
+  // with centered codes lsum, of this thread's tokens).
+  float m[NT], mr[NT], acc[NT][KS][4], zacc[NT][4], lsum[NT];
   int Ev = -100;  // value scales are taken times 2^Ev
 #pragma unroll
   for (int n = 0; n < NT; ++n) {
     m[n] = -CUDART_INF_F;
     mr[n] = 0.f;
+    lsum[n] = 0.f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       zacc[n][i] = 0.f;
@@ -467,11 +506,12 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
   // weights of this lane's tokens in the value words (row gid of row tile mt is pair q = gid + 8 mt of 32 tokens)
   const int wt_a = BV == 1 ? gid >> 1 : 2 * ((gid >> 1) & 3), wt_b = BV == 1 ? wt_a + 4 : wt_a;
   const float off[2] = {(float)(P_EXP - wt_a), (float)(P_EXP - wt_b)};
+  const float weight_a = pow2i(wt_a), weight_b = pow2i(wt_b);
   const int tok0 = 4 * (gid >> 1) + (gid & 1);                       // token of row gid, tile 0; the other rows: + 2, + 16
   const uint32_t kc_lane = st + tok0 * (BK == 1 && D == 64 ? 8 : 16) + (BK == 1 && D == 64 ? (tig >> 1) : tig) * 4;
   const uint32_t vs_lane = st + Pl::OFF_VM + pair_row(BV == 1 ? 16 * tig : 8 * tig) * Pl::VSROW;  // first pair of the lane's word
   // zero-points of channel group gid, or ones (row NG and up: the sum of the numerators)
-  const uint32_t vz_lane = gid < NG ? vs_lane + Pl::VS + 4 * gid : ones;
+  const uint32_t vz_lane = gid < NG || Cd::CENTERED ? vs_lane + Pl::VS + 4 * (gid % NG) : ones;
   const uint32_t p_st = pbuf + my_head * Pl::PH + my_slot * 144 + gid * 8;  // + pair offset
   const uint32_t p_ld = pbuf + col_head * Pl::PH + tig * (BV == 1 ? 144 : 64) + (BV == 2 ? (tig >> 1) * 16 : 0);
 
@@ -505,6 +545,16 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
       for (int g = 0; g < NGT; ++g)
 #pragma unroll
         for (int j = 0; j < V / 2; ++j) mx = __vmaxu2(mx, s[g][j]);
+      if constexpr (Cd::CENTERED) {
+#pragma unroll
+        for (int g = 0; g < NGT; ++g) {
+          const uint32_t a = st + Pl::OFF_KM + g * 4 * D + 2 * D + lane * 4;
+          uint32_t hi, lo;
+          centered_zero<D, BK>(s[g][0], lds32(a), hi, lo);
+          sts32(a, hi);
+          sts32(st + Pl::OFF_KL + g * 2 * D + lane * 4, lo);
+        }
+      }
       __syncwarp();
 #pragma unroll
       for (int j = 0; j < V; ++j) {
@@ -524,6 +574,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
     // ---- zero-points: sum_d q_d z_d per token group and head (rows: groups, first and second half of the channels) ----
     {
       const uint32_t za = st + Pl::OFF_KM + (gid & (NGT - 1)) * 4 * D + 2 * D + (gid >> 2) * D + tig * 16;
+      const uint32_t zl = st + Pl::OFF_KL + (gid & (NGT - 1)) * 2 * D + (gid >> 2) * D + tig * 16;
       float zc[NT][4];
 #pragma unroll
       for (int n = 0; n < NT; ++n)
@@ -535,6 +586,11 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
           const uint2 q0 = lds64(qb + ((n * KS / 2 + 2 * kp) * 32 + lane) * 8), q1 = lds64(qb + ((n * KS / 2 + 2 * kp + 1) * 32 + lane) * 8);
+          if constexpr (Cd::CENTERED) {
+            const uint4 l = lds128(zl + kp * 64);
+            mma_f16(zc[n], l.x, l.x, l.y, l.y, q0.x, q0.y);
+            mma_f16(zc[n], l.z, l.z, l.w, l.w, q1.x, q1.y);
+          }
           mma_f16(zc[n], a.x, a.x, a.y, a.y, q0.x, q0.y);  // (rows 8 and up: the same again)
           mma_f16(zc[n], a.z, a.z, a.w, a.w, q1.x, q1.y);
         }
@@ -562,7 +618,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
           w8[t][r] = odd_bytes_up(raw);
         }
     };
-    auto key_mask = [](int k) { return BK == 2 ? 0x000c000cu << (2 * (k & 3)) : 0x00040004u << k; };
+    auto key_pair = [](uint32_t w, int k) { return Cd::template pair<BK>(w, BK == 2 ? k & 3 : k); };
     constexpr int KPW = KS / KWORDS;  // k-steps a word serves
     if constexpr (GC == 1) {
       constexpr int UG = GS / 32;  // units of a group
@@ -604,8 +660,8 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
               for (int u = 0; u < UG; ++u)
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
-                  const uint32_t a0 = w[u][t][0] & key_mask(k), a1 = w[u][t][1] & key_mask(k);
-                  const uint32_t a2 = w8[u][t][0] & key_mask(k), a3 = w8[u][t][1] & key_mask(k);
+                  const uint32_t a0 = key_pair(w[u][t][0], k), a1 = key_pair(w[u][t][1], k);
+                  const uint32_t a2 = key_pair(w8[u][t][0], k), a3 = key_pair(w8[u][t][1], k);
                   if (ks == 0) mma_f16_first(c[n][2 * u + t], a0, a1, a2, a3, p0, p1);
                   else mma_f16(c[n][2 * u + t], a0, a1, a2, a3, p0, p1);
                 }
@@ -649,8 +705,8 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
             for (int k = 0; k < KPW; ++k)
 #pragma unroll
               for (int t = 0; t < 2; ++t) {
-                const uint32_t a0 = w[t][0] & key_mask(k), a1 = w[t][1] & key_mask(k);
-                const uint32_t a2 = w8[t][0] & key_mask(k), a3 = w8[t][1] & key_mask(k);
+                const uint32_t a0 = key_pair(w[t][0], k), a1 = key_pair(w[t][1], k);
+                const uint32_t a2 = key_pair(w8[t][0], k), a3 = key_pair(w8[t][1], k);
                 if (kw + k == 0) mma_f16_first(c[t], a0, a1, a2, a3, pp[0][0], pp[0][1]);
                 else mma_f16(c[t], a0, a1, a2, a3, pp[kw * KPW + k][0], pp[kw * KPW + k][1]);
               }
@@ -709,6 +765,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
         for (int ux = 0; ux < HP; ++ux)
 #pragma unroll
           for (int k = 0; k < 4; ++k) x[n][ux][k] -= up;
+        lsum[n] *= f;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           zacc[n][k] *= f;
@@ -725,6 +782,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
           const float pa = ex2(x[n][ux][2 * t]), pb = ex2(x[n][ux][2 * t + 1]);
+          if constexpr (Cd::CENTERED) lsum[n] = fmaf(pa + pb, t ? weight_b : weight_a, lsum[n]);
           const uint32_t h = pack_io2<true>(pa, pb);
           const uint32_t lo = pack_io2<true>(pa - io2_lo<true>(h), pb - io2_hi<true>(h));
           sts64(p_st + n * HP * Pl::PH + ux * GC * 144 + t * 64, h, lo);
@@ -792,6 +850,14 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const uint32_t dst = vm + pair_row(32 * h) * Pl::VSROW + pair_row(lane) * Pl::VSROW;
+        if constexpr (Cd::CENTERED) {
+#pragma unroll
+          for (int g = 0; g < NG; ++g) {
+            uint32_t lo;
+            centered_zero<D, BV>(sp[h][g], zp[h][g], zp[h][g], lo);
+            sts32(dst + 2 * Pl::VS + 4 * g, lo);
+          }
+        }
         if constexpr (NG == 4) {
           sts128(dst, hmul2(sp[h][0], e2), hmul2(sp[h][1], e2), hmul2(sp[h][2], e2), hmul2(sp[h][3], e2));
           sts128(dst + Pl::VS, zp[h][0], zp[h][1], zp[h][2], zp[h][3]);
@@ -821,7 +887,6 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
       }
 #pragma unroll
       for (int e = 0; e < VE; ++e) {
-        const uint32_t msk = BV == 2 ? 0x000c000cu << (2 * e) : 0x00040004u << e;
         constexpr int VB = CP / GC;  // operands of a step: parts GC * vb + slot
         uint32_t sp[2][VB];
         const uint32_t sa = vs_lane + pair_row(32 * c) * Pl::VSROW + 2 * e * Pl::VSROW, sb = sa + Pl::VSROW;
@@ -844,7 +909,12 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
           const uint4 hp = lds128(p_ld + n * HP * Pl::PH + c * 288 + e * 16);  // (hi, lo) of pairs 2 e and 2 e + 1
-          mma_f16(zacc[n], z0, z0, z1, z1, hmul2(low ? hp.y : hp.x, we), hmul2(low ? hp.w : hp.z, we));
+          const uint32_t pz0 = hmul2(low ? hp.y : hp.x, we), pz1 = hmul2(low ? hp.w : hp.z, we);
+          if constexpr (Cd::CENTERED) {
+            const uint32_t y0 = lds32(zo + Pl::VS), y1 = lds32(zo + Pl::VS + Pl::VSROW);
+            mma_f16(zacc[n], y0, y0, y1, y1, pz0, pz1);
+          }
+          mma_f16(zacc[n], z0, z0, z1, z1, pz0, pz1);
           // fma(l, s, fma(h, s, hn * s)): hi where hn = l = 0, lo where hn = -h
           const uint32_t hn0 = (hp.x ^ 0x80008000u) & low_mask, hn1 = (hp.z ^ 0x80008000u) & low_mask;
           const uint32_t l0 = hp.y & low_mask, l1 = hp.w & low_mask;
@@ -855,7 +925,8 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
             constexpr int MT = GC * KS / CP;
 #pragma unroll
             for (int mt = vb * MT; mt < (vb + 1) * MT; ++mt)
-              mma_f16(acc[n][mt], w[mt][0] & msk, w[mt][1] & msk, w8[mt][0] & msk, w8[mt][1] & msk, p0, p1);
+              mma_f16(acc[n][mt], Cd::template pair<BV>(w[mt][0], e), Cd::template pair<BV>(w[mt][1], e),
+                      Cd::template pair<BV>(w8[mt][0], e), Cd::template pair<BV>(w8[mt][1], e), p0, p1);
           }
         }
       }
@@ -873,9 +944,15 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
   float o[NT][KS][2], l[NT];
 #pragma unroll
   for (int n = 0; n < NT; ++n) {
-    const float ua = pow2i(CODE_EXP - P_EXP - Ev), uz = pow2i(-P_EXP);
+    const float ua = pow2i(Cd::EXP - P_EXP - Ev), uz = pow2i(-P_EXP);
     const float z = (zacc[n][0] + zacc[n][1]) * uz;  // row gid < NG: channel group gid; row NG: the sum
-    l[n] = __shfl_sync(0xffffffffu, z, NG * 4 + tig);
+    if constexpr (Cd::CENTERED) {
+#pragma unroll
+      for (int k = HP; k < 32; k <<= 1) lsum[n] += __shfl_xor_sync(0xffffffffu, lsum[n], k);
+      l[n] = lsum[n] * uz;
+    } else {
+      l[n] = __shfl_sync(0xffffffffu, z, NG * 4 + tig);
+    }
 #pragma unroll
     for (int mt = 0; mt < KS; ++mt) {
       const float zg = __shfl_sync(0xffffffffu, z, (mt * 16 / GS) * 4 + tig);

@@ -917,3 +917,16 @@ def test_two_bit_values_keep_sixteen_bits_of_the_sums(G, g, S):
     cache = xq.Cache(cfg, DEV)
     kv = _fill(cache, w, [0], S)
     assert _relative_error(cache, cfg, kv, 0, W.queries(w, 0, 0, DEV)) <= 1.2e-4
+
+
+@pytest.mark.parametrize("G,kq,vq,g,S", [(1, 2, 2, 32, 512), (3, 0, 0, 32, 1000), (4, 2, 0, 64, 2000), (8, 0, 2, 32, 1000),
+                                         (2, 2, 2, 64, 777)])
+def test_head_dim_64_to_single_precision(G, kq, vq, g, S):
+    # Every operand is exact or a pair of 22 bits, sums and result are of one size: a few roundings of 2^-24 on logits
+    # below 2^4, 2^-22 on the numerators, random signs; bound: 2^-20 of the result's norm
+    w = dict(n_layers=2, batch=2, n_q_heads=2 * G, n_kv_heads=2, head_dim=64, seq=S, residual_len=64, group_size=g,
+             kq=kq, vq=vq, km=0, vm=0, n_outliers=3, outlier_scale=8.0, seed=23, n_splits=0)
+    cfg = W.make_xq_config(w)
+    cache = xq.Cache(cfg, DEV)
+    kv = _fill(cache, w, [0], S)
+    assert _relative_error(cache, cfg, kv, 0, W.queries(w, 0, 0, DEV)) <= 2.0 ** -20
