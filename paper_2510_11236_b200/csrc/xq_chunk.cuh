@@ -113,8 +113,15 @@ struct ChunkPlan {
   static constexpr int RAW_VC = (D / 4) * 8 * BV, V_QUAD = 16 * NG + 16, RAW_V = RAW_VC + CT / 4 * V_QUAD;
   static constexpr int OFF_RAW = OFF_V + VBUFS * 2 * MAT;
   static constexpr int TOTAL = OFF_RAW + 4 * C_STAGES * (RAW_K + RAW_V);
-  // tensor memory columns: q, S (then numerators) of four tiles, O
-  static constexpr uint32_t COL_Q = 0, COL_S = 64, COL_O = 320;
+  // tensor memory columns: q, S (then numerators) of four tiles, O; head_dim 64: the sum of earlier O
+  static constexpr uint32_t COL_Q = 0, COL_S = 64, COL_O = 320, COL_T = 384;
+  // Tiles after which O is added to the sum (in fp32) and starts over, 0: never.  Every product's addition to O drops
+  // what lies below its last digit, always in one direction: after 8000 tokens, 1500 products, the fp32 result was 8.8e-6
+  // of its norm off.  With head_dim 64, where the scalar kernel is the measure (4.1, 5.3, 7.8e-7 at 512, 2000, 8000
+  // tokens), sums of 8 tiles leave 15.6e-7 at 8000, of 4 10.8e-7, of 2 8.5e-7, and those with the small products first
+  // 4.4, 5.8, 7.6e-7.  300 query tokens at 2048: 49 us without, 50, 52, 56 us.  (head_dim 128 has no columns left; its
+  // measure, one decode call per token, is 1.0-1.7e-4.)
+  static constexpr int FLUSH = D == 64 ? 2 : 0;
   static_assert(TOTAL <= 226 * 1024, "shared memory");
 };
 
@@ -286,6 +293,13 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         r[i] = pack_io2<true>(io_to_f(w[32 * c + i] & 0xffffu, p.f16) * f, io_to_f(w[32 * c + i] >> 16, p.f16) * f);
       tmem_st32(row_t + Pl::COL_Q + 32 * c, r);
     }
+    if constexpr (Pl::FLUSH != 0) {
+      uint32_t zero[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) zero[i] = 0u;
+#pragma unroll
+      for (int c = 0; c < D; c += 32) tmem_st32(row_t + Pl::COL_T + c, zero);
+    }
     tc_wait_st();
     cq_sm[tid] = p.scale * 1.4426950408889634f * pow2i(-e);
     m_sm[tid] = -CUDART_INF_F;
@@ -309,12 +323,12 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         tc_fence_after();
         if (ok && elect_one()) {
           const uint32_t base = smu + (i & 1) * 2 * Pl::MAT, dS = tb + Pl::COL_S + (i & 3) * 64;
+          // the small products first, here and below: a sum drops what lies below its own last digit
           const uint64_t kh = smem_desc(base, Pl::CORE, Pl::K_SBO), kl = smem_desc(base + Pl::MAT, Pl::CORE, Pl::K_SBO);
 #pragma unroll
-          for (int ks = 0; ks < D / 16; ++ks) {
-            umma_f16(dS, tb + Pl::COL_Q + 8 * ks, kh + KSTEP * ks, IDK, ks > 0);
-            umma_f16(dS, tb + Pl::COL_Q + 8 * ks, kl + KSTEP * ks, IDK, true);
-          }
+          for (int ks = 0; ks < D / 16; ++ks) umma_f16(dS, tb + Pl::COL_Q + 8 * ks, kl + KSTEP * ks, IDK, ks > 0);
+#pragma unroll
+          for (int ks = 0; ks < D / 16; ++ks) umma_f16(dS, tb + Pl::COL_Q + 8 * ks, kh + KSTEP * ks, IDK, true);
           umma_commit(bar_s + 8 * (i & 3));
           umma_commit(bar_kfree + 8 * (i & 1));
         }
@@ -332,10 +346,11 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
 #pragma unroll
           for (int ks = 0; ks < CT / 16; ++ks) {
             const uint32_t ph = pt + 32 * (ks >> 1) + 8 * (ks & 1), pl = ph + 16;
-            umma_f16(dO, ph, vh + KSTEP * ks, IDV, j > 0 || ks > 0);
-            umma_f16(dO, ph, vl + KSTEP * ks, IDV, true);
+            umma_f16(dO, ph, vl + KSTEP * ks, IDV, j > 0 || ks > 0);
             umma_f16(dO, pl, vh + KSTEP * ks, IDV, true);
           }
+#pragma unroll
+          for (int ks = 0; ks < CT / 16; ++ks) umma_f16(dO, pt + 32 * (ks >> 1) + 8 * (ks & 1), vh + KSTEP * ks, IDV, true);
           umma_commit(bar_o + 8 * (j & 3));
           umma_commit(bar_vfree + 8 * (j % 3));
         }
@@ -403,6 +418,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         if (i > 0) {
           const int4 e1 = *reinterpret_cast<const int4*>(v_exp[i & 3]), e0 = *reinterpret_cast<const int4*>(v_exp[(i - 1) & 3]);
           change |= e1.x != e0.x || e1.y != e0.y || e1.z != e0.z || e1.w != e0.w;
+          if constexpr (Pl::FLUSH != 0) change |= i % Pl::FLUSH == 0;
         }
         if (__any_sync(0xffffffffu, change)) {
           m_sm[r] = m;
@@ -417,9 +433,21 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
               const float fz = f * pow2i(v_exp[i & 3][qz] - v_exp[(i - 1) & 3][qz]);
               uint32_t s[32];
               tmem_ld32(row_t + Pl::COL_O + c, s);
-              tc_wait_ld();
+              if constexpr (Pl::FLUSH != 0) {
+                uint32_t sum[32];
+                tmem_ld32(row_t + Pl::COL_T + c, sum);
+                tc_wait_ld();
 #pragma unroll
-              for (int k = 0; k < 32; ++k) s[k] = __float_as_uint(__uint_as_float(s[k]) * (k < 16 ? fa : fz));
+                for (int k = 0; k < 32; ++k) {
+                  sum[k] = __float_as_uint((__uint_as_float(sum[k]) + __uint_as_float(s[k])) * (k < 16 ? fa : fz));
+                  s[k] = 0u;
+                }
+                tmem_st32(row_t + Pl::COL_T + c, sum);
+              } else {
+                tc_wait_ld();
+#pragma unroll
+                for (int k = 0; k < 32; ++k) s[k] = __float_as_uint(__uint_as_float(s[k]) * (k < 16 ? fa : fz));
+              }
               tmem_st32(row_t + Pl::COL_O + c, s);
             }
             tc_wait_st();
@@ -681,6 +709,13 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         if (N > 0) {
           tmem_ld32(row_t + Pl::COL_O + cb, o);
           tc_wait_ld();
+          if constexpr (Pl::FLUSH != 0) {
+            uint32_t sum[32];
+            tmem_ld32(row_t + Pl::COL_T + cb, sum);
+            tc_wait_ld();
+#pragma unroll
+            for (int k = 0; k < 32; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) + __uint_as_float(sum[k]));
+          }
         }
         float f[2];  // of the two channel quarters that 32 channels can span
         f[0] = (N > 0 ? pow2i(-v_exp[(N - 1) & 3][cb / DQ]) : 0.f) * inv;

@@ -930,3 +930,23 @@ def test_head_dim_64_to_single_precision(G, kq, vq, g, S):
     cache = xq.Cache(cfg, DEV)
     kv = _fill(cache, w, [0], S)
     assert _relative_error(cache, cfg, kv, 0, W.queries(w, 0, 0, DEV)) <= 2.0 ** -20
+
+
+@pytest.mark.parametrize("D,G,S,T", [(64, 1, 8000, 24), (64, 4, 2000, 70), (128, 4, 100, 100)])
+def test_chunks_to_single_precision(D, G, S, T):
+    # head_dim 64, and any head_dim over the window alone: as test_head_dim_64_to_single_precision
+    w = dict(n_layers=2, batch=1, n_q_heads=2 * G, n_kv_heads=2, head_dim=D, seq=S, residual_len=128, group_size=32,
+             kq=2, vq=0, km=0, vm=0, n_outliers=3, outlier_scale=10.0, seed=24, n_splits=0)
+    cfg = W.make_xq_config(w)
+    cache = xq.Cache(cfg, DEV)
+    kv = _fill(cache, w, [0], S)
+    gen = torch.Generator(device="cpu").manual_seed(T)
+    q = torch.randn(T, 1, 2 * G, D, generator=gen).to(torch.bfloat16).to(DEV)
+    out = cache.attention_chunk(0, q, f32=True).double().cpu().numpy()
+    num = den = 0.0
+    for hk in range(2):
+        oc = util.oracle_for_stream(cfg, [0], 0, hk, kv)
+        ref = oc.attention_chunk(0, util.bits_of(q[:, :, hk * G:(hk + 1) * G]))[:, 0]
+        num += ((out[:, 0, hk * G:(hk + 1) * G] - ref) ** 2).sum()
+        den += (ref ** 2).sum()
+    assert (num / den) ** 0.5 <= 2.0 ** -20
