@@ -80,6 +80,7 @@ struct Plan {
   static constexpr int WARP = ((BODY > WIN ? BODY : WIN) + 127) / 128 * 128;
   static constexpr int MS = D + 4;               // state row: acc[D], m, l
   static_assert(HP * NT * MS * 4 <= WARP, "a warp's state rows fit its own memory");
+  static_assert(MS % 4 == 0, "state rows are read as vectors");
   // after the warps' parts: B fragments of the zero-point products; fp16 ones, read in place of zero-points for the
   // sum of the numerators; q as it came
   static constexpr int QB = NT * KS * 32 * 4, ONES = CENTERED ? 0 : 64 * VSROW, QS = HP * NT * D * 2;
@@ -91,6 +92,7 @@ struct Plan {
   static constexpr int WARPS = room(MOST) <= LIMIT ? MOST : (room(MOST - 1) <= LIMIT ? MOST - 1 : MOST - 2);
   static constexpr int TOTAL = room(WARPS);
   static_assert(TOTAL <= LIMIT, "shared memory");
+  static_assert(WARPS * WARP >= HP * NT * (256 + 1) * 4, "the merge's weights");
 };
 
 // Code operands.  head_dim 128: the masked code bits as they are, fp16 subnormals code * weight * 2^-22.  head_dim 64:
@@ -245,19 +247,29 @@ __device__ __forceinline__ void window_tile(uint32_t wbuf, int n_valid, const ui
   }
 }
 
+// four channels c .. c + 3 of query head hq's result
 template <int D>
-__device__ __forceinline__ void store_out(const DecodeParams& p, const DecodeLayer& L, size_t hq, int c, float v) {
-  if (p.out_f32) reinterpret_cast<float*>(L.out)[hq * D + c] = v;
-  else if (p.f16) reinterpret_cast<__half*>(L.out)[hq * D + c] = __float2half_rn(v);
-  else reinterpret_cast<__nv_bfloat16*>(L.out)[hq * D + c] = __float2bfloat16_rn(v);
+__device__ __forceinline__ void store_out(const DecodeParams& p, const DecodeLayer& L, size_t hq, int c, float4 v) {
+  if (p.out_f32) {
+    *reinterpret_cast<float4*>(reinterpret_cast<float*>(L.out) + hq * D + c) = v;
+  } else {
+    uint2 w;
+    if (p.f16) w = make_uint2(pack_io2<true>(v.x, v.y), pack_io2<true>(v.z, v.w));
+    else w = make_uint2(pack_io2<false>(v.x, v.y), pack_io2<false>(v.z, v.w));
+    *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(L.out) + hq * D + c) = w;
+  }
 }
 
 // Split-K merge by the last CTA of a stream: the CTA takes a ticket after its partials are visible device-wide; the
 // CTA that draws the last ticket reads all partials from L2 and writes
 // out = sum_s acc_s 2^(m_s-M) / sum_s l_s 2^(m_s-M).  No CTA ever waits for another.
+// What it takes is two trips to L2, one for all (m, l) and one for the partials: a warp that went through its share of
+// the heads one after the other, both trips for each, made it 2.3 us with four heads and 5.1 us with eight.
+// weights: G * (ns + 1) floats of shared memory.
 template <int D>
 __device__ __forceinline__ void ticket_merge(const DecodeParams& p, const DecodeLayer& L, int ns, int hk, int b,
-                                             const float* part_acc, const float* part_ml, unsigned* ticket, int* s_flag) {
+                                             const float* part_acc, const float* part_ml, unsigned* ticket, int* s_flag,
+                                             float* weights) {
   const Dims& dm = p.dm;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
   // The barrier orders every thread's partial stores before thread 0's ticket; the ticket is a release (cumulative
@@ -271,38 +283,57 @@ __device__ __forceinline__ void ticket_merge(const DecodeParams& p, const Decode
   }
   __syncthreads();
   if (!*s_flag) return;
-  // a warp takes 64 channels of a head
-  for (int item = warp; item < dm.G * (D / 64); item += n_warps) {
-    const int a = item / (D / 64), c0 = (item % (D / 64)) * 64 + lane * 2;
-    const size_t hq = (size_t)b * dm.Hq + hk * dm.G + a;
-    const float* ml = part_ml + hq * p.ns_q * 2;
-    const float* pa = part_acc + hq * p.ns_q * D + c0;
-    float M = -CUDART_INF_F;
-    for (int s = lane; s < ns; s += 32) M = fmaxf(M, ld_cg(ml + 2 * s));
+  const size_t hq0 = (size_t)b * dm.Hq + hk * dm.G;
+  // weights[h][s] = 2^(m_s - M), weights[h][ns] = 1 / sum_s l_s 2^(m_s - M)
+#pragma unroll 2
+  for (int h = warp; h < dm.G; h += n_warps) {
+    const float* ml = part_ml + (hq0 + h) * p.ns_q * 2;
+    float* w = weights + h * (ns + 1);
+    float M = -CUDART_INF_F, Ls = 0.f;
+    if (ns <= 32) {
+      const float2 x = lane < ns ? ld_cg2(ml + 2 * lane) : make_float2(-CUDART_INF_F, 0.f);
+      M = x.x;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-    float ax = 0.f, ay = 0.f, Ls = 0.f;
-    for (int s0 = 0; s0 < ns; s0 += 16) {
-      float2 v[16];
+      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+      const float f = lane < ns ? ex2(x.x - M) : 0.f;
+      Ls = x.y * f;
+      if (lane < ns) w[lane] = f;
+    } else {
+      for (int s = lane; s < ns; s += 32) M = fmaxf(M, ld_cg(ml + 2 * s));
 #pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = s0 + i < ns ? ld_cg2(pa + (size_t)(s0 + i) * D) : make_float2(0.f, 0.f);
-      float f = 0.f;  // lane i < 16: weight of partial s0 + i
-      if (lane < 16 && s0 + lane < ns) {
-        f = ex2(ld_cg(ml + 2 * (s0 + lane)) - M);
-        Ls = fmaf(ld_cg(ml + 2 * (s0 + lane) + 1), f, Ls);
-      }
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const float fi = __shfl_sync(0xffffffffu, f, i);
-        ax = fmaf(v[i].x, fi, ax);
-        ay = fmaf(v[i].y, fi, ay);
+      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+      for (int s = lane; s < ns; s += 32) {
+        const float2 x = ld_cg2(ml + 2 * s);
+        const float f = ex2(x.x - M);
+        Ls = fmaf(x.y, f, Ls);
+        w[s] = f;
       }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) Ls += __shfl_xor_sync(0xffffffffu, Ls, o);
-    const float inv = 1.0f / Ls;
-    store_out<D>(p, L, hq, c0, ax * inv);
-    store_out<D>(p, L, hq, c0 + 1, ay * inv);
+    if (lane == 0) w[ns] = 1.0f / Ls;
+  }
+  __syncthreads();
+  for (int item = threadIdx.x; item < dm.G * (D / 4); item += blockDim.x) {
+    const int h = item / (D / 4), c = item % (D / 4) * 4;
+    const float* pa = part_acc + (hq0 + h) * p.ns_q * D + c;
+    const float* w = weights + h * (ns + 1);
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < ns; s0 += 16) {
+      float4 v[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[i] = s0 + i < ns ? ld_cg4(pa + (size_t)(s0 + i) * D) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const float f = s0 + i < ns ? w[s0 + i] : 0.f;
+        a.x = fmaf(v[i].x, f, a.x);
+        a.y = fmaf(v[i].y, f, a.y);
+        a.z = fmaf(v[i].z, f, a.z);
+        a.w = fmaf(v[i].w, f, a.w);
+      }
+    }
+    const float inv = w[ns];
+    store_out<D>(p, L, hq0 + h, c, make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv));
   }
   if (threadIdx.x == 0) *ticket = 0u;  // ready for the next launch on this stream
 }
@@ -1021,30 +1052,36 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
   const size_t slot = (size_t)blockIdx.y * ((size_t)dm.B * dm.Hq) * p.ns_q;  // this layer's partials in the scratch
   float* const part_acc = p.part_acc + slot * D;
   float* const part_ml = p.part_ml + slot * 2;
-  for (int item = tid; item < G * D; item += W * 32) {
-    const int h = item / D, d = item % D;
+  for (int item = tid; item < G * (D / 4); item += W * 32) {
+    const int h = item / (D / 4), d = item % (D / 4) * 4;
+    auto row = [&](int w) { return reinterpret_cast<const float*>(smem + w * Pl::WARP) + h * Pl::MS; };
     float M = -CUDART_INF_F;
 #pragma unroll
-    for (int w = 0; w < W; ++w) M = fmaxf(M, reinterpret_cast<const float*>(smem + w * Pl::WARP)[h * Pl::MS + D]);
-    float A = 0.f, Ls = 0.f;
+    for (int w = 0; w < W; ++w) M = fmaxf(M, row(w)[D]);
+    float4 A = make_float4(0.f, 0.f, 0.f, 0.f);
+    float Ls = 0.f;
 #pragma unroll
     for (int w = 0; w < W; ++w) {
-      const float* row = reinterpret_cast<const float*>(smem + w * Pl::WARP) + h * Pl::MS;
-      const float mw = row[D];
+      const float4 v = *reinterpret_cast<const float4*>(row(w) + d);
+      const float mw = row(w)[D];
       const float f = mw == -CUDART_INF_F ? 0.f : ex2(mw - M);  // a warp without tokens
-      A = fmaf(row[d], f, A);
-      Ls = fmaf(row[D + 1], f, Ls);
+      A.x = fmaf(v.x, f, A.x);
+      A.y = fmaf(v.y, f, A.y);
+      A.z = fmaf(v.z, f, A.z);
+      A.w = fmaf(v.w, f, A.w);
+      Ls = fmaf(row(w)[D + 1], f, Ls);
     }
     const size_t hq = (size_t)b * dm.Hq + hk * G + h;
     if (ns == 1) {
-      store_out<D>(p, L, hq, d, A / Ls);
+      store_out<D>(p, L, hq, d, make_float4(A.x / Ls, A.y / Ls, A.z / Ls, A.w / Ls));
     } else {
-      part_acc[(hq * p.ns_q + split) * D + d] = A;
+      *reinterpret_cast<float4*>(part_acc + (hq * p.ns_q + split) * D + d) = A;
       if (d == 0) *reinterpret_cast<float2*>(part_ml + (hq * p.ns_q + split) * 2) = make_float2(M, Ls);
     }
   }
   if (ns > 1)
-    ticket_merge<D>(p, L, ns, hk, b, part_acc, part_ml, p.tickets + (size_t)blockIdx.y * (dm.B * dm.Hkv) + bh, &s_flag);
+    ticket_merge<D>(p, L, ns, hk, b, part_acc, part_ml, p.tickets + (size_t)blockIdx.y * (dm.B * dm.Hkv) + bh, &s_flag,
+                    reinterpret_cast<float*>(smem));
 }
 
 template <int D, int BK, int BV, int GS, int HP, int NT>
