@@ -84,7 +84,11 @@ struct Plan {
   // after the warps' parts: B fragments of the zero-point products; fp16 ones, read in place of zero-points for the
   // sum of the numerators; q as it came
   static constexpr int QB = NT * KS * 32 * 4, ONES = CENTERED ? 0 : 64 * VSROW, QS = HP * NT * D * 2;
-  static constexpr int room(int w) { return w * WARP + QB + ONES + QS; }
+  // four or eight heads: q as operand fragments, for all warps (else each keeps them in registers; 16 or 32 a thread,
+  // which spilled 80-580 bytes: a step's layer at 32k, four heads 25.8 -> 25.1 us, groups of five at 16k 31.2 -> 28.7)
+  static constexpr bool Q_SHARED = HP == 4 && D == 128;
+  static constexpr int QF = Q_SHARED ? NT * KS * 32 * 8 : 0;
+  static constexpr int room(int w) { return w * WARP + QB + ONES + QS + QF; }
   // Two CTAs per SM, each of as many warps as registers (128, or 168 for eight heads) and shared memory allow.
   static constexpr int CTAS = 2;
   static constexpr int MOST = NT == 1 ? 8 : 6;
@@ -405,6 +409,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
   const uint32_t pbuf = st + Pl::STAGE;
   const uint32_t qb = sm_base + W * Pl::WARP, ones = qb + Pl::QB;
   uint16_t* const q_sm = reinterpret_cast<uint16_t*>(smem + W * Pl::WARP + Pl::QB + Pl::ONES);  // zeros for absent heads
+  const uint32_t qf = ones + Pl::ONES + Pl::QS + lane * 8;  // this lane's fragments of q
   const uint32_t bar_k = (uint32_t)__cvta_generic_to_shared(&bar_mem[0]) + 16 * warp, bar_v = bar_k + 8;
 
   // Copies of batch j of this CTA's range into this warp's stage (one lane; the stage is free)
@@ -486,6 +491,15 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
     const __half2 h0 = __floats2half2_rn(v[0], v[1]), h1 = __floats2half2_rn(v[2], v[3]);
     sts64(qb + (i * 32 + lane) * 8, *reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
   }
+  if constexpr (Pl::Q_SHARED) {  // largest |q| in [2^14, 2^15); the key scales carry the rest of the exponent
+    for (int i = warp; i < NT * KS; i += W) {
+      const int ks = i % KS, h = HP * (i / KS) + col_head;
+      const float e2 = pow2i(__shfl_sync(0xffffffffu, eq_lane, h) + 14 - k_weight<D, BK>(ks));
+      const uint2 v = *reinterpret_cast<const uint2*>(q_sm + h * D + k_channel<D, BK>(ks, tig, 0));
+      sts64(qf + i * 256, pack_io2<true>(io_to_f(v.x & 0xffffu, p.f16) * e2, io_to_f(v.y & 0xffffu, p.f16) * e2),
+            pack_io2<true>(io_to_f(v.x >> 16, p.f16) * e2, io_to_f(v.y >> 16, p.f16) * e2));
+    }
+  }
   __syncthreads();
   float cq[NT];
 #pragma unroll
@@ -494,13 +508,17 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
 
   const uint32_t low_mask = low ? 0xffffffffu : 0u;
   // q of this lane's operand column as fp16 pairs, times 2^Ek and divided by the weights of the codes
-  uint32_t qk[NT][KS][2];
-  int Ek = -100;  // not set
+  uint32_t qk[Pl::Q_SHARED ? 1 : NT][Pl::Q_SHARED ? 1 : KS][2];
+  int Ek = -100;  // not set; with Q_SHARED the scales are taken times 2^Ek instead
   float ck[NT];
   auto set_ek = [&](int e) {
     Ek = e;
 #pragma unroll
     for (int n = 0; n < NT; ++n) {
+      if constexpr (Pl::Q_SHARED) {
+        ck[n] = cq[n] * pow2i(Cd::EXP - 14 - e);
+        continue;
+      }
       const int h = HP * n + col_head;
       const int eh = e + __shfl_sync(0xffffffffu, eq_lane, h);
       const uint16_t* qh = q_sm + h * D;
@@ -586,6 +604,21 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
           sts32(st + Pl::OFF_KL + g * 2 * D + lane * 4, lo);
         }
       }
+      // |q s| below 2^15 and its largest at least 2^8 (where 2^14 |q| allows): exponents of q move only outside that
+      const float smax = f16_to_f(redux_max_u32(max(mx & 0xffffu, mx >> 16)));
+      const int es = smax > 0.f ? exponent_of(smax) : -24;
+      if constexpr (Pl::Q_SHARED) {
+        // |q s| below 2^15; a scale keeps its 11 bits down to 2^-10 of the largest
+        if (es > -1 - Ek || (es < -4 - Ek && Ek < 15) || Ek == -100) set_ek(min(15, -1 - es));
+        const float ek = pow2i(Ek);
+        const __half2 ek2 = __floats2half2_rn(ek, ek);
+#pragma unroll
+        for (int g = 0; g < NGT; ++g)
+#pragma unroll
+          for (int j = 0; j < V / 2; ++j) s[g][j] = hmul2(s[g][j], *reinterpret_cast<const uint32_t*>(&ek2));
+      } else {
+        if (es > 13 - Ek || (es < 7 - Ek && Ek < 14) || Ek == -100) set_ek(min(14, 13 - es));
+      }
       __syncwarp();
 #pragma unroll
       for (int j = 0; j < V; ++j) {
@@ -593,10 +626,6 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
 #pragma unroll
         for (int g = 0; g < NGT; ++g) sts16(dst + g * 4 * D, j & 1 ? s[g][j / 2] >> 16 : s[g][j / 2]);
       }
-      // |q s| below 2^15 and its largest at least 2^8 (where 2^14 |q| allows): exponents of q move only outside that
-      const float smax = f16_to_f(redux_max_u32(max(mx & 0xffffu, mx >> 16)));
-      const int es = smax > 0.f ? exponent_of(smax) : -24;
-      if (es > 13 - Ek || (es < 7 - Ek && Ek < 14) || Ek == -100) set_ek(min(14, 13 - es));
       __syncwarp();
     }
     // Units of 32 tokens: this thread's logits are those of units GC * ux + my_slot, ux = 0 .. HP - 1, of its head:
@@ -655,7 +684,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
       constexpr int UG = GS / 32;  // units of a group
       // fma(q, s, qn * s) is hi where qn = 0 and lo where qn = -q
       uint32_t qn[KS][2];
-      if constexpr (NT == 1) {
+      if constexpr (!Pl::Q_SHARED && NT == 1) {
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks) {
           qn[ks][0] = (qk[0][ks][0] ^ 0x80008000u) & low_mask;
@@ -680,7 +709,11 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
 #pragma unroll
             for (int n = 0; n < NT; ++n) {
               uint32_t p0, p1;
-              if constexpr (NT == 1) {
+              if constexpr (Pl::Q_SHARED) {
+                const uint2 q = lds64(qf + (n * KS + ks) * 256);
+                p0 = product_part(q.x, s0, low);
+                p1 = product_part(q.y, s1, low);
+              } else if constexpr (NT == 1) {
                 p0 = hfma2(qk[n][ks][0], s0, hmul2(qn[ks][0], s0));
                 p1 = hfma2(qk[n][ks][1], s1, hmul2(qn[ks][1], s1));
               } else {

@@ -950,3 +950,24 @@ def test_chunks_to_single_precision(D, G, S, T):
         num += ((out[:, 0, hk * G:(hk + 1) * G] - ref) ** 2).sum()
         den += (ref ** 2).sum()
     assert (num / den) ** 0.5 <= 2.0 ** -20
+
+
+@pytest.mark.parametrize("G,kq,f16", [(1, 0, True), (4, 0, True), (4, 2, False), (8, 0, True), (5, 2, False)])
+@pytest.mark.parametrize("kind", ["small", "spread"])
+def test_key_scales_far_from_one(G, kq, f16, kind):
+    # Key scales near 2^-14 (fp16's smallest normal number) with queries that bring the logits back to one, and key
+    # channels 2^9 apart with queries the other way round, so that all count alike.  A scale keeps its 11 bits down to
+    # 2^-10 of the batch's largest, products q s lose 2^-25 of 2^8 at most: what counts is the sums' 16 bits, as in
+    # test_two_bit_values_keep_sixteen_bits_of_the_sums.
+    S, D = 1000, 128
+    w = dict(n_layers=2, batch=1, n_q_heads=2 * G, n_kv_heads=2, head_dim=D, seq=S, residual_len=128, group_size=32,
+             kq=kq, vq=0, km=0, vm=0, n_outliers=3, outlier_scale=4.0, seed=25, n_splits=0)
+    cfg = W.make_xq_config(w, io_dtype=int(f16))
+    dt = torch.float16 if f16 else torch.bfloat16
+    f = torch.full((D,), 2.0 ** -13) if kind == "small" else torch.exp2(-9.0 * (torch.arange(D) % 2))
+    K, V, _, _ = W.pair_tokens(w, 0, 0, S, DEV)
+    K, V = (K.float() * f.to(DEV)).to(dt), V.to(dt)
+    q = (W.queries(w, 0, 0, DEV).float() / f.to(DEV)).to(dt)
+    cache = xq.Cache(cfg, DEV)
+    cache.append_kv(0, K, V)
+    assert _relative_error(cache, cfg, {0: (K, V)}, 0, q) <= 1.2e-4
