@@ -369,27 +369,11 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
   // successor never starts before the work this kernel waited for has completed.
   if (p.late_wait) grid_dependents_go();
 
-  // CTA -> (stream, split): p.n_ctas CTAs dealt to the streams in order; the first n_ctas % streams streams get one
-  // split more than the others
-  int split, ns, hk, b;
-  {
-    const unsigned n_streams = (unsigned)(dm.B * dm.Hkv), c = blockIdx.x;
-    const unsigned base = (unsigned)p.n_ctas / n_streams, rem = (unsigned)p.n_ctas - base * n_streams;
-    const unsigned big = rem * (base + 1u);
-    unsigned stream;
-    if (c < big) {
-      stream = c / (base + 1u);
-      split = (int)(c - stream * (base + 1u));
-      ns = (int)base + 1;
-    } else {
-      const unsigned c2 = c - big;
-      stream = rem + c2 / base;
-      split = (int)(c2 - (c2 / base) * base);
-      ns = (int)base;
-    }
-    hk = (int)(stream % (unsigned)dm.Hkv);
-    b = (int)(stream / (unsigned)dm.Hkv);
-  }
+  // CTA -> (stream, split), the splits of a stream side by side
+  const int ns = p.ns_q;
+  const unsigned stream = blockIdx.x / (unsigned)ns;
+  const int split = (int)(blockIdx.x - stream * (unsigned)ns);
+  const int hk = (int)(stream % (unsigned)dm.Hkv), b = (int)(stream / (unsigned)dm.Hkv);
   const int bh = b * dm.Hkv + hk;
   const int nbt = (p.n_q + BT - 1) / BT;  // batches of the stream (the last one may be ragged)
   int b0, b1, wt0, wt1;
@@ -1120,7 +1104,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
 template <int D, int BK, int BV, int GS, int HP, int NT>
 cudaError_t launch_one(const DecodeParams& p, cudaStream_t st) {
   using Pl = Plan<D, BK, BV, GS, HP, NT>;
-  return launch_dependent(decode_mma_kernel<D, BK, BV, GS, HP, NT>, dim3(p.n_ctas, p.n_layers), dim3(Pl::WARPS * 32),
+  return launch_dependent(decode_mma_kernel<D, BK, BV, GS, HP, NT>, dim3((unsigned)(p.ns_q * p.dm.B * p.dm.Hkv), p.n_layers), dim3(Pl::WARPS * 32),
                           (size_t)Pl::TOTAL, st, p);
 }
 

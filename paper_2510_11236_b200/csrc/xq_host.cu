@@ -124,6 +124,8 @@ constexpr int TIMING_POOL = 1 << 15;
 
 struct EventPair { cudaEvent_t a, b; int kind; };
 
+struct MmaPlan { int batches, ns, deal; };
+
 }  // namespace
 
 // Scratch of xq_decode_attention_static: part of the library image, one copy per
@@ -162,6 +164,7 @@ struct xq_cache {
   bool delta_clean;    // the code-difference counters have been zeroed on a stream
   std::vector<uint8_t> repacked;  // per layer: codes or parameters it reads were written since its last decode
   MmaShape mma_shape[2][2];  // the tensor-core kernel by (key bits - 1, value bits - 1); warps 0 = not asked yet
+  MmaPlan mma_plan[2][2];    // and the splits of the latest number of batches asked for; batches 0 = none yet
   // timing
   bool timing;
   std::vector<EventPair> pool;
@@ -230,92 +233,113 @@ MmaShape mma_shape(const xq_cache* c, int l) {
 // launch per layer, which callers that watch xq_launch_count have seen so far (10.6 us for a tiny pair; 8.5 together).
 constexpr int MIN_JOINT_LAYERS = 3;
 
+// Times of the tensor-core kernel, us, as plan_splits adds them up: fitted to 30 shapes (head_dim 64 and 128, one to
+// eight heads, 4 to 512 streams of 1000 to 131072 tokens), each with up to 29 numbers of splits.
+struct DecodeTimes {
+  double launch;         // start and end of a launch that runs alone
+  double round, warp;    // a warp's batch, while w warps of its SM work: round + warp * w
+  double floor;          // host time of a call: no plan makes a layer alone faster
+  double cta, batch;     // with other CTAs waiting for the slot: a CTA's start and end, and a batch's share of the SM
+};
+DecodeTimes decode_times(const Dims& dm) {
+  if (dm.D == 64) return {6.5, 1.0, 0.19, 9.0, 4.0, 0.25};
+  if (dm.G == 1) return {8.0, 0.6, 0.3, 11.0, 6.5, 0.4};
+  if (dm.G == 2) return {9.0, 1.24, 0.295, 11.0, 6.0, 0.42};
+  if (dm.G <= 4) return {8.0, 1.46, 0.325, 11.0, 6.0, 0.415};
+  return {12.8, 2.6, 0.57, 0.0, 5.5, 0.93};
+}
+
+// Number of splits of a stream's batches, and the runs in which they are dealt, for the tensor-core kernel; splits > 0:
+// that many are wanted.  xq_decode_step promises the bits of single calls, and those depend on the plan, so both kinds
+// of call use the same one: xq_decode_attention, a launch for each layer (what a model that feeds one layer's result to
+// the next can call), which wants the CTAs of one full wave, and xq_decode_step, whose layers share launches and which
+// wants few CTAs.  The single call counts: of the plans that cost a layer alone at most ALONE_BOUND times the best, the
+// one that a step takes the least time with.  us per layer, alone / in a step, with the plan a step would choose for
+// itself and with this one: 32k, four heads 40.7 / 25.1, 33.2 / 26.5; 16k 24.8 / 14.3, 21.6 / 15.5; one sequence of 128k
+// 42.0 / 25.3, 35.0 / 27.3; groups of five at 16k 52.9 / 29.0, 38.6 / 28.6; MHA at 4k, batch 8, 30.5 / 23.2 with either.
+constexpr double ALONE_BOUND = 1.07;  // what the model is worth: measured times are within 1.07 of it
+constexpr double MERGE = 0.03;  // us of a launch's end for each partial of a stream
+void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int splits, int& ns_out, int& deal_out) {
+  const Dims& dm = c->plan.dm;
+  const long long streams = (long long)dm.B * dm.Hkv, slots = (long long)c->sm_count * shape.ctas_per_sm;
+  const DecodeTimes t = decode_times(dm);
+  const bool joint = c->cfg.n_layers >= MIN_JOINT_LAYERS;
+  struct Candidate { int ns, deal; double alone, step; };
+  Candidate all[2 * XQ_MAX_SPLITS];
+  int n = 0;
+  double alone_min = 0.0;
+  // batches are dealt to the splits one by one, or in runs of one per warp: no warp of a CTA then waits for another's
+  // last batch
+  for (int deal : {1, shape.warps}) {
+    const int runs = (batches + deal - 1) / deal;
+    const int limit = runs < XQ_MAX_SPLITS ? runs : XQ_MAX_SPLITS;
+    for (int ns = splits > 0 ? splits : 1; ns <= (splits > 0 ? splits : limit); ++ns) {
+      if (ns > limit) continue;
+      // batches of the largest split (the last run, which may be short, goes to a split of the larger kind)
+      const int base = runs / ns, rem = runs % ns;
+      const int last = (base + (rem > 0 ? 1 : 0)) * deal - (runs * deal - batches), others = (base + (rem > 1 ? 1 : 0)) * deal;
+      const int per = ns > 1 && others > last ? others : last;
+      // the last wave: a start and an end, and the rounds of a CTA, whose last one may leave warps without a batch
+      auto wave = [&](long long ctas) {
+        long long resident = (ctas + c->sm_count - 1) / c->sm_count;
+        if (resident > shape.ctas_per_sm) resident = shape.ctas_per_sm;
+        const int rounds = per / shape.warps;
+        double left = (double)batches / ns - rounds * shape.warps;  // on average: the SM's CTAs share its rate
+        if (left < 0.0 || per % shape.warps == 0) left = 0.0;
+        return t.launch + MERGE * ns + rounds * (t.round + t.warp * resident * shape.warps) + (left > 0.0 ? t.round + t.warp * resident * left : 0.0);
+      };
+      // earlier waves: a CTA follows the one before it in its slot; the warps that have no batch in its last round idle
+      const int idle = deal == 1 ? (shape.warps - per % shape.warps) % shape.warps : 0;
+      const double each = t.cta + ((double)batches / ns * shape.ctas_per_sm + idle) * t.batch;
+      auto launch = [&](long long ctas) {
+        const long long last_wave = (ctas - 1) % slots + 1;
+        return (double)((ctas - last_wave) / slots) * each + wave(last_wave);
+      };
+      Candidate k{ns, deal, launch(streams * ns), joint ? launch(streams * ns * c->cfg.n_layers) / c->cfg.n_layers : 1.0};
+      if (k.alone < t.floor) k.alone = t.floor;
+      if (n == 0 || k.alone < alone_min) alone_min = k.alone;
+      all[n++] = k;
+    }
+  }
+  const Candidate* best = nullptr;
+  for (int i = 0; i < n; ++i) {
+    const Candidate& k = all[i];
+    if (k.alone > ALONE_BOUND * alone_min) continue;
+    if (!best || (joint ? k.step < best->step : k.alone < best->alone)) best = &k;
+  }
+  ns_out = best->ns;
+  deal_out = best->deal;
+}
+
 // Splits per (sequence, kv head) stream.  Tensor-core kernel: every split takes whole
-// batches of the packed region and a share of the window (ns_w = 0), sized towards
-// whole waves of resident CTAs.  Generic kernel:
+// batches of the packed region and a share of the window (ns_w = 0; plan_batches).  Generic kernel:
 // separate splits for the packed region and for the window, in proportion to their bytes.
 // nq packed tokens and r window tokens are visible to the call.
-void plan_splits(const xq_cache* c, int l, int nq, int r, int& ns_q, int& ns_w, int* n_ctas_out = nullptr, int* deal_out = nullptr) {
+void plan_splits(const xq_cache* c, int l, int nq, int r, int& ns_q, int& ns_w, int* deal_out = nullptr) {
   const Dims& dm = c->plan.dm;
   int units = (nq + 31) / 32, tiles = (r + 15) / 16;
   const int streams = dm.B * dm.Hkv;
   if (uses_mma(c)) {
-    // the tensor-core kernel: a CTA takes whole 128-token batches, dealt to its warps, and a share of the window
     const MmaShape shape = mma_shape(c, l);
     const int batches = (nq + XQ_BATCH - 1) / XQ_BATCH;
-    // Batches are dealt to the CTAs in runs of one per warp where there are plenty (no warp of a CTA then waits for
-    // another's last batch; the CTAs that got fewer runs make room for the next layer), else one by one.
-    const int slot_count = c->sm_count * shape.ctas_per_sm;
-    const int deal = (long long)batches * streams >= 2LL * slot_count * shape.warps ? shape.warps : 1;
-    const int runs = (batches + deal - 1) / deal;
-    const int most = batches > 0 ? runs : tiles;  // no CTA without tokens
     ns_w = 0;
-    if (deal_out) *deal_out = deal;
-    if (c->cfg.n_splits > 0) {
-      ns_q = c->cfg.n_splits < most ? c->cfg.n_splits : most;
-      if (n_ctas_out) *n_ctas_out = ns_q * streams;
-      return;
-    }
-    // Largest number of batches that a split gets (the last run, which may be short, goes to a split of the larger kind)
-    auto largest = [&](int ns) {
-      const int base = runs / ns, rem = runs % ns;
-      const int last = (base + (rem > 0 ? 1 : 0)) * deal - (runs * deal - batches), others = (base + (rem > 1 ? 1 : 0)) * deal;
-      return ns > 1 && others > last ? others : last;
-    };
-    // Time of a launch of one layer in units of one batch's time on an SM of which nothing is idle: a wave costs a
-    // start and an end of about 12 units, and as long as its CTAs' batches take: one after the other in the slowest
-    // warp (a warp alone takes about 6 units for a batch), or all of the SM's together.
-    auto wave = [&](int ns, long long ctas) {
-      long long resident = (ctas + c->sm_count - 1) / c->sm_count;
-      if (resident > shape.ctas_per_sm) resident = shape.ctas_per_sm;
-      const int per = largest(ns);
-      const double chain = 6.0 * ((per + shape.warps - 1) / shape.warps), together = (double)per * (double)resident;
-      return 12.0 + (chain > together ? chain : together);
-    };
-    auto alone = [&](int ns) {
-      const long long ctas = (long long)ns * streams;
-      return (double)((ctas + slot_count - 1) / slot_count) * wave(ns, ctas) + 0.05 * ns;
-    };
-    // The same of a step whose layers share launches: a CTA follows the one before it in its slot, so only their
-    // number and the last, partly filled wave count.  CTA of 8 warps, 32k context, 32 streams, us per layer with 4, 6,
-    // 8, 9, 10, 12 splits: 25.4, 27.0, 27.3, 28.6, 29.2, 30.6, that is 14 units a CTA.
-    auto step = [&](int ns) {
-      const long long ctas = (long long)c->cfg.n_layers * ns * streams, rest = ctas % slot_count;
-      const double each = 14.0 + (double)batches / ns * shape.ctas_per_sm;
-      return (double)(ctas / slot_count) * each + (rest ? wave(ns, rest) : 0.0);
-    };
-    // Steps of 16 layers, us per layer, by the time alone / by the time of a step: four heads, 32k tokens and one
-    // block more, 29.5 / 26.1; 16k 18.1 / 14.4; one sequence of 20k 9.3 / 6.4; one user at 1000 tokens (32 layers)
-    // 0.77 / 0.51; at 8000 3.6 / 3.0.  The price is paid by a layer called alone, whose long chains the model
-    // underrates: 32k 35.6 / 43.4, 16k 21.2 / 24.4 us.  Both give the same bits, so there is one plan;
-    // cfg.n_splits sets another.
-    const bool joint = c->cfg.n_layers >= MIN_JOINT_LAYERS;
-    const int limit = most < XQ_MAX_SPLITS ? most : XQ_MAX_SPLITS;
-    int best = 1;
-    double times[XQ_MAX_SPLITS + 1];
-    for (int ns = 1; ns <= limit; ++ns) {
-      times[ns] = alone(ns);
-      if (times[ns] < times[best]) best = ns;
-    }
-    if (joint) {
-      // of the splits that cost a layer alone at most a tenth more, those that a step takes the least time with
-      const double bound = 1.1 * times[best];
-      double best_time = step(best);
-      for (int ns = 1; ns <= limit; ++ns) {
-        if (times[ns] > bound) continue;
-        const double t = step(ns);
-        if (t < best_time) { best_time = t; best = ns; }
+    int deal = 1;
+    if (batches == 0) {
+      // the window alone, a tile a warp; no CTA without tokens
+      ns_q = c->cfg.n_splits > 0 ? c->cfg.n_splits : (tiles + shape.warps - 1) / shape.warps;
+      if (ns_q > tiles) ns_q = tiles;
+      if (ns_q > XQ_MAX_SPLITS) ns_q = XQ_MAX_SPLITS;
+    } else {
+      // the plan of a number of batches is kept: making it costs the host about 10 us at 32k
+      MmaPlan& memo = const_cast<xq_cache*>(c)->mma_plan[layer_bits(l, c->cfg.kq) - 1][layer_bits(l, c->cfg.vq) - 1];
+      if (memo.batches != batches) {
+        memo.batches = batches;
+        plan_batches(c, shape, batches, c->cfg.n_splits < batches ? c->cfg.n_splits : batches, memo.ns, memo.deal);
       }
+      ns_q = memo.ns;
+      deal = memo.deal;
     }
-    ns_q = best;
-    if (n_ctas_out) *n_ctas_out = best * streams;
-    // A layer alone, one wave that does not fill every resident slot: give some streams one split more, if the splits
-    // are many enough for the CTAs' sizes to stay within a few percent of each other.
-    if (!joint && (long long)best * streams < slot_count && slot_count < (long long)(best + 1) * streams && best >= 8 &&
-        best + 1 <= most && best + 1 <= XQ_MAX_SPLITS) {
-      ns_q = best + 1;
-      if (n_ctas_out) *n_ctas_out = slot_count;
-    }
+    if (deal_out) *deal_out = deal;
     return;
   }
   double qb, wb;
@@ -407,9 +431,8 @@ int prepare_decode(const xq_cache* c, int layer, const void* q, void* out, int o
   p.layer[0] = {layer_ptrs(c, layer), (const uint16_t*)q, out, (const uint16_t*)K_new, (const uint16_t*)V_new};
   p.n_q = nq;
   p.r = r;
-  p.n_ctas = 0;
   p.deal = 1;
-  plan_splits(c, layer, nq, r, p.ns_q, p.ns_w, &p.n_ctas, &p.deal);
+  plan_splits(c, layer, nq, r, p.ns_q, p.ns_w, &p.deal);
   p.scale = c->scale;
   p.out_f32 = out_f32;
   p.early_fetch = 0;
@@ -663,6 +686,7 @@ int xq_create(const xq_config* cfg, void* dev_workspace, size_t bytes, xq_cache*
   c->device = -1;
   c->static_base = nullptr;
   memset(c->mma_shape, 0, sizeof(c->mma_shape));
+  memset(c->mma_plan, 0, sizeof(c->mma_plan));
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) == cudaSuccess &&
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) {

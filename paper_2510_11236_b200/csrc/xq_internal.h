@@ -93,7 +93,6 @@ struct DecodeParams {
   int n_q;            // quantized tokens
   int r;              // window tokens
   int ns_q, ns_w;     // splits over the quantized region (most of any stream) / over the window
-  int n_ctas;         // tensor-core kernel: CTAs of a layer over all streams (n_ctas / streams splits each, or one more)
   int deal;           // tensor-core kernel: batches of 128 tokens are dealt to the splits in runs of this many
   float scale;
   float* part_acc;    // [n_layers,B,Hq,ns,D]

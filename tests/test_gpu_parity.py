@@ -971,3 +971,16 @@ def test_key_scales_far_from_one(G, kq, f16, kind):
     cache = xq.Cache(cfg, DEV)
     cache.append_kv(0, K, V)
     assert _relative_error(cache, cfg, {0: (K, V)}, 0, q) <= 1.2e-4
+
+
+@pytest.mark.parametrize("B,Hkv,G,S", [(4, 8, 4, 32768), (1, 8, 4, 131072), (4, 8, 5, 16384), (16, 2, 1, 20000)])
+def test_splits_of_many_layers_fill_one_wave(B, Hkv, G, S):
+    # A layer alone (xq_decode_attention) is fastest with the CTAs of one wave, two an SM, however many layers the model
+    # has; a step, which would take fewer, uses the same splits
+    cfg = xq.make_config(n_layers=4, batch=B, n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=128, max_seq=S, vq=0)
+    cache = xq.Cache(cfg, DEV)
+    k = torch.zeros(B, Hkv, S, 128, dtype=torch.bfloat16, device=DEV)
+    cache.append_kv(0, k, k)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rc, ns, ns_w = xq.xq_split_plan(cache.handle, 0)
+    assert rc == 0 and ns_w == 0 and 1.5 * sms < ns * B * Hkv <= 2 * sms
