@@ -984,3 +984,15 @@ def test_splits_of_many_layers_fill_one_wave(B, Hkv, G, S):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     rc, ns, ns_w = xq.xq_split_plan(cache.handle, 0)
     assert rc == 0 and ns_w == 0 and 1.5 * sms < ns * B * Hkv <= 2 * sms
+
+
+def test_number_of_splits_as_configured():
+    # 156 batches of 32 streams: enough to deal them in runs of one per warp, which must not limit the splits asked for
+    S = 20000
+    for n_splits in (1, 20, 100, 156, 256):
+        cfg = xq.make_config(n_layers=1, batch=1, n_q_heads=32, n_kv_heads=32, head_dim=128, max_seq=S, n_splits=n_splits, km=1, vm=1)
+        cache = xq.Cache(cfg, DEV)
+        k = torch.zeros(1, 32, S, 128, dtype=torch.bfloat16, device=DEV)
+        cache.append_kv(0, k, k)
+        assert xq.xq_split_plan(cache.handle, 0) == (0, min(n_splits, 156), 0)
+        cache.close()
