@@ -124,7 +124,8 @@ constexpr int TIMING_POOL = 1 << 15;
 
 struct EventPair { cudaEvent_t a, b; int kind; };
 
-struct MmaPlan { int batches, ns, deal; };
+// modelled times, us: of a launch alone, and of one more in a row of launches that overlap
+struct MmaPlan { int batches, ns, deal; double alone, next; };
 
 }  // namespace
 
@@ -243,7 +244,7 @@ struct DecodeTimes {
 };
 DecodeTimes decode_times(const Dims& dm) {
   if (dm.D == 64) return {6.5, 1.0, 0.19, 9.0, 4.0, 0.25};
-  if (dm.G == 1) return {8.0, 0.6, 0.3, 11.0, 6.5, 0.4};
+  if (dm.G == 1) return {8.0, 0.6, 0.3, 11.0, 5.5, 0.34};
   if (dm.G == 2) return {9.0, 1.24, 0.295, 11.0, 6.0, 0.42};
   if (dm.G <= 4) return {8.0, 1.46, 0.325, 11.0, 6.0, 0.415};
   return {12.8, 2.6, 0.57, 0.0, 5.5, 0.93};
@@ -259,12 +260,12 @@ DecodeTimes decode_times(const Dims& dm) {
 // 42.0 / 25.3, 35.0 / 27.3; groups of five at 16k 52.9 / 29.0, 38.6 / 28.6; MHA at 4k, batch 8, 30.5 / 23.2 with either.
 constexpr double ALONE_BOUND = 1.07;  // what the model is worth: measured times are within 1.07 of it
 constexpr double MERGE = 0.03;  // us of a launch's end for each partial of a stream
-void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int splits, int& ns_out, int& deal_out) {
+void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int splits, MmaPlan& out) {
   const Dims& dm = c->plan.dm;
   const long long streams = (long long)dm.B * dm.Hkv, slots = (long long)c->sm_count * shape.ctas_per_sm;
   const DecodeTimes t = decode_times(dm);
   const bool joint = c->cfg.n_layers >= MIN_JOINT_LAYERS;
-  struct Candidate { int ns, deal; double alone, step; };
+  struct Candidate { int ns, deal; double alone, step, next; };
   Candidate all[2 * XQ_MAX_SPLITS];
   int n = 0;
   double alone_min = 0.0;
@@ -295,7 +296,8 @@ void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int spl
         const long long last_wave = (ctas - 1) % slots + 1;
         return (double)((ctas - last_wave) / slots) * each + wave(last_wave);
       };
-      Candidate k{ns, deal, launch(streams * ns), joint ? launch(streams * ns * c->cfg.n_layers) / c->cfg.n_layers : 1.0};
+      Candidate k{ns, deal, launch(streams * ns), joint ? launch(streams * ns * c->cfg.n_layers) / c->cfg.n_layers : 1.0,
+                  (dm.G > 4 ? 5.5 : 2.5) + (double)(streams * ns) / slots * each};
       if (k.alone < t.floor) k.alone = t.floor;
       if (n == 0 || k.alone < alone_min) alone_min = k.alone;
       all[n++] = k;
@@ -307,8 +309,14 @@ void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int spl
     if (k.alone > ALONE_BOUND * alone_min) continue;
     if (!best || (joint ? k.step < best->step : k.alone < best->alone)) best = &k;
   }
-  ns_out = best->ns;
-  deal_out = best->deal;
+  out = {batches, best->ns, best->deal, best->alone, best->next};
+}
+
+// The plan of a number of batches is kept: making it costs the host about 10 us at 32k.
+const MmaPlan& batches_plan(const xq_cache* c, int l, int batches) {
+  MmaPlan& plan = const_cast<xq_cache*>(c)->mma_plan[layer_bits(l, c->cfg.kq) - 1][layer_bits(l, c->cfg.vq) - 1];
+  if (plan.batches != batches) plan_batches(c, mma_shape(c, l), batches, c->cfg.n_splits < batches ? c->cfg.n_splits : batches, plan);
+  return plan;
 }
 
 // Splits per (sequence, kv head) stream.  Tensor-core kernel: every split takes whole
@@ -330,14 +338,9 @@ void plan_splits(const xq_cache* c, int l, int nq, int r, int& ns_q, int& ns_w, 
       if (ns_q > tiles) ns_q = tiles;
       if (ns_q > XQ_MAX_SPLITS) ns_q = XQ_MAX_SPLITS;
     } else {
-      // the plan of a number of batches is kept: making it costs the host about 10 us at 32k
-      MmaPlan& memo = const_cast<xq_cache*>(c)->mma_plan[layer_bits(l, c->cfg.kq) - 1][layer_bits(l, c->cfg.vq) - 1];
-      if (memo.batches != batches) {
-        memo.batches = batches;
-        plan_batches(c, shape, batches, c->cfg.n_splits < batches ? c->cfg.n_splits : batches, memo.ns, memo.deal);
-      }
-      ns_q = memo.ns;
-      deal = memo.deal;
+      const MmaPlan& plan = batches_plan(c, l, batches);
+      ns_q = plan.ns;
+      deal = plan.deal;
     }
     if (deal_out) *deal_out = deal;
     return;
@@ -401,20 +404,20 @@ struct Scratch {
   int* status;
 };
 
-// Checks a decode call and fills the kernel parameters (everything but the scratch).  Touches no state.
-// K_new / V_new: one new token per stream that the tensor-core kernel appends itself; S_eff is the layer's
-// length with that token counted.  vis >= 0: only the first vis tokens are visible to the query (a query token of
-// a chunk that is followed by later tokens in the cache).
-int prepare_decode(const xq_cache* c, int layer, const void* q, void* out, int out_f32, const void* K_new,
-                   const void* V_new, int S_eff, DecodeParams& p, bool& use_mma, int vis = -1) {
+// Checks a decode call; nq packed and r window tokens are visible to it.  Touches no state.
+// K_new / V_new: one new token per stream that the tensor-core kernel appends itself; S is the layer's length with that
+// token counted.  vis >= 0: only the first vis tokens are visible to the query (a query token of a chunk that is
+// followed by later tokens in the cache).
+int check_decode(const xq_cache* c, int layer, const void* q, const void* out, const void* K_new, const void* V_new, int S,
+                 int vis, int& nq, int& r, bool& use_mma) {
   if (!c || !q || !out) return XQ_ERR_ARG;
   if (layer < 0 || layer >= c->cfg.n_layers) return XQ_ERR_ARG;
   if (((uintptr_t)q & 15) || ((uintptr_t)out & 15)) return XQ_ERR_ARG;
   if (((uintptr_t)K_new & 15) || ((uintptr_t)V_new & 15)) return XQ_ERR_ARG;
   const Dims& dm = c->plan.dm;
-  const int S = S_eff;
   if (S < 1) return XQ_ERR_ARG;
-  int r = residual_count(S, dm.R), nq = S - r;
+  r = residual_count(S, dm.R);
+  nq = S - r;
   if (vis >= 0) {
     if (vis < 1 || vis > S) return XQ_ERR_ARG;
     if (vis < nq) { nq = vis; r = 0; } else { r = vis - nq; }
@@ -426,6 +429,16 @@ int prepare_decode(const xq_cache* c, int layer, const void* q, void* out, int o
   use_mma = uses_mma(c);
   if (c->cfg.kernel >= XQ_KERNEL_MMA && !use_mma) return XQ_ERR_CONFIG;
   if (K_new && !use_mma) return XQ_ERR_ARG;
+  return XQ_OK;
+}
+
+// Checks a decode call and fills the kernel parameters (everything but the scratch).  Touches no state.
+int prepare_decode(const xq_cache* c, int layer, const void* q, void* out, int out_f32, const void* K_new,
+                   const void* V_new, int S, DecodeParams& p, bool& use_mma, int vis = -1) {
+  int nq = 0, r = 0;
+  const int rc = check_decode(c, layer, q, out, K_new, V_new, S, vis, nq, r, use_mma);
+  if (rc != XQ_OK) return rc;
+  const Dims& dm = c->plan.dm;
   p.dm = dm;
   p.n_layers = 1;
   p.layer[0] = {layer_ptrs(c, layer), (const uint16_t*)q, out, (const uint16_t*)K_new, (const uint16_t*)V_new};
@@ -791,6 +804,25 @@ int plan_chunk(const xq_cache* c, int S, int T, int row_tiles) {
   return best;
 }
 
+// Whether T query tokens take less time as one decode launch each, chained, than as one launch of the chunk kernel,
+// which expands every tile of 64 tokens whatever T is.  Modelled times in us, fitted to T = 2 .. 16 on 19 shapes:
+// decode, as plan_batches has them; chunk, 14 for a wave (head_dim 64: 9), 1.47 (1.1) for a tile, 4 and 0.02 for each
+// partial of a row where splits merge.
+// Tokens from which on the chunk kernel is chosen / was measured to be the faster: four heads, 32k, batch 4 7 / 8; one
+// sequence of 1000 6 / 8, of 8000 6 / 7, of 128k 13 / 14; MHA at 4k, batch 8 9 / 11; groups of five at 16k 3 / 4, of
+// eight at 8k 3 / 4.  Two tokens at 32k, batch 4: 64 us a layer, in the chunk kernel 217.
+bool tokens_one_by_one(const xq_cache* c, int layer, int T) {
+  if (T > 16) return false;  // (and the host's 2 us a launch)
+  const Dims& dm = c->plan.dm;
+  const int S = c->seq[layer], batches = (S - residual_count(S, dm.R) + XQ_BATCH - 1) / XQ_BATCH;
+  const MmaPlan window{0, 0, 1, decode_times(dm).launch, 2.5}, &plan = batches > 0 ? batches_plan(c, layer, batches) : window;
+  const int row_tiles = (T * dm.G + CHUNK_ROWS - 1) / CHUNK_ROWS, ns = plan_chunk(c, S, T, row_tiles);
+  const double waves = ceil((double)dm.B * dm.Hkv * row_tiles * ns / c->sm_count), tiles = S / 64.0 + 1.0;
+  const double merge = ns > 1 ? 4.0 + 0.02 * (T * dm.G < CHUNK_ROWS ? T * dm.G : CHUNK_ROWS) * ns : 0.0;
+  const double chunk = waves * ((dm.D == 64 ? 9.0 : 14.0) + (dm.D == 64 ? 1.1 : 1.47) * tiles / ns) + merge;
+  return plan.alone + (T - 1) * plan.next < chunk;
+}
+
 int launch_chunk(xq_cache* c, int layer, const void* q, void* out, int T, int out_f32, cudaStream_t st) {
   int rc = ensure_clean_scratch(c, st);
   if (rc != XQ_OK) return rc;
@@ -829,8 +861,8 @@ int launch_chunk(xq_cache* c, int layer, const void* q, void* out, int T, int ou
   return XQ_OK;
 }
 
-// Query token j of n sees the cache up to its own position.  The tensor-core kernels: one launch for the chunk;
-// otherwise (the scalar kernel, a single token) one decode launch per token, all on the same stream.
+// Query token j of n sees the cache up to its own position.  One launch of the chunk kernel, or (few tokens, the scalar
+// kernel) one decode launch per token, all on the same stream.
 int chunk_impl(xq_cache* c, int layer, const void* q, void* out, int n, int out_f32, void* stream) {
   if (!c || !q || !out) return XQ_ERR_ARG;
   if (layer < 0 || layer >= c->cfg.n_layers) return XQ_ERR_ARG;
@@ -841,12 +873,12 @@ int chunk_impl(xq_cache* c, int layer, const void* q, void* out, int n, int out_
   bool use_mma;
   // everything that can be refused is the same for every token: check the first and the last before any launch
   {
-    DecodeParams p;
-    int rc = prepare_decode(c, layer, q, out, out_f32, nullptr, nullptr, S, p, use_mma, S - n + 1);
-    if (rc == XQ_OK) rc = prepare_decode(c, layer, q, out, out_f32, nullptr, nullptr, S, p, use_mma, S);
+    int nq, r;
+    int rc = check_decode(c, layer, q, out, nullptr, nullptr, S, S - n + 1, nq, r, use_mma);
+    if (rc == XQ_OK) rc = check_decode(c, layer, q, out, nullptr, nullptr, S, S, nq, r, use_mma);
     if (rc != XQ_OK) return rc;
   }
-  if (use_mma && n > 1) return launch_chunk(c, layer, q, out, n, out_f32, (cudaStream_t)stream);
+  if (use_mma && n > 1 && !tokens_one_by_one(c, layer, n)) return launch_chunk(c, layer, q, out, n, out_f32, (cudaStream_t)stream);
   const size_t row = (size_t)dm.B * dm.Hq * dm.D;  // elements of one token's queries: [batch, heads, head_dim]
   bool chain = false;  // launches after the first read what the first one waited for and write their own rows
   for (int j = 0; j < n; ++j) {

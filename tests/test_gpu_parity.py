@@ -986,6 +986,27 @@ def test_splits_of_many_layers_fill_one_wave(B, Hkv, G, S):
     assert rc == 0 and ns_w == 0 and 1.5 * sms < ns * B * Hkv <= 2 * sms
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,D,S,few,many", [(1, 32, 8, 128, 8000, 3, 30), (2, 8, 8, 128, 3000, 5, 40),
+                                                   (1, 8, 1, 128, 20000, 2, 16), (1, 6, 2, 64, 2000, 2, 30), (1, 4, 4, 128, 90, 3, 20)])
+def test_few_query_tokens_take_a_decode_launch_each(B, Hq, Hkv, D, S, few, many):
+    # A tile of the chunk kernel costs the same for one query token and for many: a few go one by one, and each of their
+    # rows is then a decode call that sees the tokens before it; the last is xq_decode_attention itself
+    cfg = xq.make_config(n_layers=1, batch=B, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=D, max_seq=S, km=1, vm=1)
+    cache = xq.Cache(cfg, DEV)
+    gen = torch.Generator(device=DEV).manual_seed(S)
+    k, v = (torch.randn(B, Hkv, S, D, generator=gen, device=DEV).to(torch.bfloat16) for _ in range(2))
+    cache.append_kv(0, k, v)
+    q = torch.randn(many, B, Hq, D, generator=gen, device=DEV).to(torch.bfloat16)
+    n0 = xq.xq_launch_count(cache.handle)
+    whole = cache.attention_chunk(0, q, f32=True)
+    n1 = xq.xq_launch_count(cache.handle)
+    part = cache.attention_chunk(0, q[many - few:], f32=True)
+    assert (n1 - n0, xq.xq_launch_count(cache.handle) - n1) == (1, few)
+    assert torch.equal(part[few - 1], cache.decode_attention(0, q[many - 1], f32=True))
+    assert (part - whole[many - few:]).abs().max().item() <= util.ATTN_TOL
+    cache.check_device()
+
+
 def test_number_of_splits_as_configured():
     # 156 batches of 32 streams: enough to deal them in runs of one per warp, which must not limit the splits asked for
     S = 20000
