@@ -256,6 +256,9 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
     dead_sm = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
+  // Tensor memory is asked for after the wait: a CTA of the preceding kernel that shares the SM may still have to get
+  // its own, and with all columns taken here it would wait for this CTA, which waits for it.
+  grid_dependency_wait();
   if (warp == 8 + C_EXPAND) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                      (uint32_t)__cvta_generic_to_shared(&tmem_base_sm)), "r"(512u) : "memory");
@@ -266,7 +269,6 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
   tc_fence_after();
   const uint32_t tbase = tmem_base_sm;
   const uint32_t row_t = tbase + ((uint32_t)((warp & 3) * 32) << 16);
-  grid_dependency_wait();
 
   if (warp < 4) {
     // ---- q: this thread's row as fp16 scaled by a power of two into [1, 2), to tensor memory ----

@@ -1017,3 +1017,23 @@ def test_number_of_splits_as_configured():
         cache.append_kv(0, k, k)
         assert xq.xq_split_plan(cache.handle, 0) == (0, min(n_splits, 156), 0)
         cache.close()
+
+
+def test_chunk_right_after_a_matrix_product_on_the_same_stream():
+    # The chunk kernel takes all of an SM's tensor memory; it may be placed while the kernel before it in the stream
+    # still runs, and must leave that kernel the tensor memory it has yet to ask for (head_dim 64: both fit an SM)
+    D, S, T = 64, 600, 200
+    cfg = xq.make_config(n_layers=1, batch=1, n_q_heads=16, n_kv_heads=4, head_dim=D, max_seq=S, km=1, vm=1)
+    cache = xq.Cache(cfg, DEV)
+    gen = torch.Generator(device=DEV).manual_seed(3)
+    k, v = (torch.randn(1, 4, S, D, generator=gen, device=DEV).to(torch.bfloat16) for _ in range(2))
+    cache.append_kv(0, k, v)
+    a = torch.randn(2048, 1024, generator=gen, device=DEV).to(torch.bfloat16)
+    wq = (torch.randn(1024, 16 * D, generator=gen, device=DEV) / 32).to(torch.bfloat16)
+    want = cache.attention_chunk(0, (a @ wq)[:T].reshape(T, 1, 16, D).contiguous(), f32=True)
+    torch.cuda.synchronize()
+    for _ in range(20):
+        q = torch.mm(a, wq)[:T].view(T, 1, 16, D)
+        got = cache.attention_chunk(0, q, f32=True)
+    cache.check_device()
+    assert torch.equal(got, want)
