@@ -175,14 +175,21 @@ __device__ __forceinline__ void expand_block(const uint32_t (&w)[8], int sh, con
            __byte_perm(t[j].lo[0], t[j].lo[1], s1), __byte_perm(t[j].lo[0], t[j].lo[1], u1));
   }
 }
-// eight fp32 values as hi and lo rows of 16 bytes
+// eight fp32 values as hi and lo rows of 16 bytes (the difference of an infinity and its hi is not a number; the lo of
+// a number below 2^15 is below 64)
 __device__ __forceinline__ void store_row(const float (&v)[8], uint32_t dst, uint32_t lo_off) {
   uint32_t hi[4], lo[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) split2(v[2 * k], v[2 * k + 1], hi[k], lo[k]);
+  for (int k = 0; k < 4; ++k) {
+    hi[k] = pack_io2<true>(v[2 * k], v[2 * k + 1]);
+    lo[k] = pack_io2<true>(fminf(v[2 * k] - io2_lo<true>(hi[k]), 64.f), fminf(v[2 * k + 1] - io2_hi<true>(hi[k]), 64.f));
+  }
   sts128(dst, hi[0], hi[1], hi[2], hi[3]);
   sts128(dst + lo_off, lo[0], lo[1], lo[2], lo[3]);
 }
+constexpr uint32_t INF32 = 0x7f800000u;  // |x| as bits: at or above, x is not a number or infinite
+__device__ __forceinline__ uint32_t abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+__device__ __forceinline__ uint32_t finite_bits(float x) { return abs_bits(x) < INF32 ? abs_bits(x) : 0u; }
 // 2^e that puts mx below 2^15 and, unless it is there already, above 2^14
 __device__ __forceinline__ int key_exponent(float mx) {
   return mx >= 1.f && mx < 32768.f ? 0 : (mx > 0.f ? 14 - exponent_of(mx) : 0);
@@ -198,6 +205,10 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
   __shared__ __align__(16) int v_exp[4][4];               // [tile % 4][channel quarter]: the expanded values are times 2^v_exp
   __shared__ float cq_sm[CM], m_sm[CM];     // logits from products of the scaled q; softmax reference (-infinity: none)
   __shared__ float l_sm[2][CM], ml_sm[2][CM];
+  // Values that are not finite: a row that does not see their token must not get them, and its zero numerator does not
+  // keep them out of a product.  They are expanded as zeros; rows that do see them get a NaN in those channels at the end.
+  __shared__ uint32_t row_bad[CM][4];       // [row][channel quarter]: channels in which a row sees any
+  __shared__ int any_bad;
   __shared__ uint32_t tmem_base_sm;
   __shared__ int s_flag;
   __shared__ volatile int dead_sm;
@@ -303,6 +314,9 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
       for (int c = 0; c < D; c += 32) tmem_st32(row_t + Pl::COL_T + c, zero);
     }
     tc_wait_st();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) row_bad[tid][k] = 0u;
+    if (tid == 0) any_bad = 0;
     cq_sm[tid] = p.scale * 1.4426950408889634f * pow2i(-e);
     m_sm[tid] = -CUDART_INF_F;
   }
@@ -534,14 +548,22 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
     int ev = 0;
     bool ev_set = false;
     // exponent of the values in use: the largest |v| times 2^ev in [2^4, 2^14); it moves only outside that
-    auto value_exponent = [&](float mx) {
-      mx = __uint_as_float(redux_max_u32(__float_as_uint(mx)));
+    auto value_exponent = [&](uint32_t mb) {
+      const float mx = __uint_as_float(mb);
       const int em = mx > 0.f ? exponent_of(mx) : -100;
       if (em > -100 && (!ev_set || em + ev > 13 || em + ev < 4)) {
         ev = 9 - em;
         ev_set = true;
       }
       return pow2i(ev);
+    };
+    // the rows that see token tok (counted from the layer's first) see values that are not finite, in channels `mask` of
+    // this lane's half of the quarter
+    auto mark = [&](int tok, uint32_t mask) {
+#pragma unroll 1
+      for (int r = 0; mask != 0u && r < CM; ++r)
+        if (tok < vis0 + (row0 + r) / G) atomicOr(&row_bad[r][ew & 3], mask << (v_h * (DQ / 2)));
+      if (mask != 0u) any_bad = 1;
     };
     fetch(0);
     fetch(1);
@@ -593,15 +615,14 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
           const int w0 = (t - pk_tiles) * CT;
           const uint2* rows = reinterpret_cast<const uint2*>(p.L.win_k + (size_t)bh * dm.R * D) + k_q;
           const int r0 = w0 + 32 * (ew >> 1);
-          float mx = 0.f;
+          uint32_t mb = 0u;
 #pragma unroll 1
-          for (int x = k_b; x < 32; x += 128 / D) {  // the unit is that of 32 tokens
+          for (int x = k_b; x < 32; x += 128 / D) {  // the unit is that of 32 tokens, and of their finite elements
             const uint2 v = r0 + x < p.r ? rows[(size_t)(r0 + x) * (D / 4)] : make_uint2(0u, 0u);
-            mx = fmaxf(mx, fmaxf(fmaxf(fabsf(io_to_f(v.x & 0xffffu, p.f16)), fabsf(io_to_f(v.x >> 16, p.f16))),
-                                 fmaxf(fabsf(io_to_f(v.y & 0xffffu, p.f16)), fabsf(io_to_f(v.y >> 16, p.f16)))));
+            mb = max(mb, max(max(finite_bits(io_to_f(v.x & 0xffffu, p.f16)), finite_bits(io_to_f(v.x >> 16, p.f16))),
+                             max(finite_bits(io_to_f(v.y & 0xffffu, p.f16)), finite_bits(io_to_f(v.y >> 16, p.f16)))));
           }
-          mx = __uint_as_float(redux_max_u32(__float_as_uint(mx)));
-          const int e = key_exponent(mx);
+          const int e = key_exponent(__uint_as_float(redux_max_u32(mb)));
           if (lane == 0) k_unit[i & 7][ew >> 1] = pow2i(-e);
           const float f = pow2i(e);
 #pragma unroll 1
@@ -623,15 +644,31 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         const uint32_t dst = sm + Pl::OFF_V + (i % 3) * 2 * Pl::MAT + (c0 + v_h * (DQ / 2)) / 8 * Pl::V_SBO + v_dst;
         if (t < n_pk) {
           const bool exists = t * CT + 4 * v_q < p.n_q;
-          float s[4], z[4], mx = 0.f;
+          float s[4], z[4];
+          uint32_t mb = 0u;
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             const uint32_t a = src + Pl::RAW_VC + v_q * Pl::V_QUAD + j * 4 * NG + 2 * (c0 / GS);
             s[j] = exists ? f16_to_f(lds16(a)) : 0.f;
             z[j] = exists ? f16_to_f(lds16(a + 2 * NG)) : 0.f;
-            mx = fmaxf(mx, fmaf((float)((1 << BV) - 1), s[j], fabsf(z[j])));
+            mb = max(mb, abs_bits(fmaf((float)((1 << BV) - 1), s[j], fabsf(z[j]))));
           }
-          const float f = value_exponent(mx);
+          mb = redux_max_u32(mb);
+          if (mb >= INF32) {
+            uint32_t tokens = 0u;
+            mb = 0u;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const uint32_t b = abs_bits(fmaf((float)((1 << BV) - 1), s[j], fabsf(z[j])));
+              tokens |= (uint32_t)(b >= INF32) << j;
+              mb = max(mb, b < INF32 ? b : 0u);
+              if (b >= INF32) s[j] = z[j] = 0.f;
+            }
+#pragma unroll 1
+            for (int j = 0; j < 4; ++j) mark(t * CT + 4 * v_q + j, (tokens >> j) & 1u ? (1u << (DQ / 2)) - 1u : 0u);
+            mb = redux_max_u32(mb);
+          }
+          const float f = value_exponent(mb);
           if (lane == 0) v_exp[i & 3][ew & 3] = ev;
           Table tab[4];
 #pragma unroll
@@ -652,16 +689,21 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
           auto piece = [&](int tok, int c) {  // 8 channels of a window row
             return w0 + tok < p.r ? rows[(size_t)(w0 + tok) * (D / 8) + c / 8] : make_uint4(0u, 0u, 0u, 0u);
           };
-          float mx = 0.f;
+          uint32_t mb = 0u;
 #pragma unroll 1
           for (int x = 0; x < 4 * KB; ++x) {
             const uint4 u = piece(4 * v_q + (x & 3), c0 + v_h * (DQ / 2) + 8 * (x >> 2));
             const uint32_t y[4] = {u.x, u.y, u.z, u.w};
+            uint32_t mask = 0u;
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-              mx = fmaxf(mx, fmaxf(fabsf(io_to_f(y[k] & 0xffffu, p.f16)), fabsf(io_to_f(y[k] >> 16, p.f16))));
+            for (int c = 0; c < 8; ++c) {
+              const uint32_t a = abs_bits(io_to_f(c & 1 ? y[c / 2] >> 16 : y[c / 2] & 0xffffu, p.f16));
+              mb = max(mb, a < INF32 ? a : 0u);
+              mask |= (uint32_t)(a >= INF32) << c;
+            }
+            if (mask != 0u) mark(p.n_q + w0 + 4 * v_q + (x & 3), mask << (8 * (x >> 2)));
           }
-          const float f = value_exponent(mx);
+          const float f = value_exponent(redux_max_u32(mb));
           if (lane == 0) v_exp[i & 3][ew & 3] = ev;
 #pragma unroll 1
           for (int x = 0; x < 4 * KB; ++x) {
@@ -671,8 +713,9 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
             float v[8];
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-              v[2 * c] = io_to_f(y[c] & 0xffffu, p.f16) * f;
-              v[2 * c + 1] = io_to_f(y[c] >> 16, p.f16) * f;
+              const float a = io_to_f(y[c] & 0xffffu, p.f16), b = io_to_f(y[c] >> 16, p.f16);
+              v[2 * c] = abs_bits(a) < INF32 ? a * f : 0.f;
+              v[2 * c + 1] = abs_bits(b) < INF32 ? b * f : 0.f;
             }
             store_row(v, dst + k * Pl::V_SBO + 16 * j, Pl::MAT);
           }
@@ -725,6 +768,12 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         float v[32];
 #pragma unroll
         for (int k = 0; k < 32; ++k) v[k] = N > 0 ? __uint_as_float(o[k]) * f[k / 16] : 0.f;
+        if (any_bad != 0) {
+          const uint32_t ba = row_bad[r][cb / DQ], bz = row_bad[r][(cb + 31) / DQ];
+#pragma unroll
+          for (int k = 0; k < 32; ++k)
+            if (((k < 16 ? ba : bz) >> ((cb + k) % DQ)) & 1u) v[k] = CUDART_NAN_F;
+        }
         if (r < n_rows) {
           if (p.ns > 1) {
             float4* dst = reinterpret_cast<float4*>(p.part_acc + ((part0 + r) * p.ns + split) * D + cb);

@@ -1037,3 +1037,45 @@ def test_chunk_right_after_a_matrix_product_on_the_same_stream():
         got = cache.attention_chunk(0, q, f32=True)
     cache.check_device()
     assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("D,Hq,Hkv,R,S,T,at,f16", [
+    (128, 8, 2, 128, 300, 40, 290, False),   # in the window
+    (64, 6, 2, 64, 300, 40, 295, True),
+    (128, 4, 4, 256, 250, 250, 100, False),  # a whole prompt in the window, several tiles
+    (128, 8, 2, 32, 400, 150, 300, True),    # in a packed block
+    (64, 4, 1, 32, 900, 700, 500, False),
+])
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+def test_chunk_rows_do_not_see_later_tokens_that_are_not_finite(D, Hq, Hkv, R, S, T, at, f16, value):
+    # Query tokens before token `at` must get what they get with an ordinary token there, bit for bit (in a packed block:
+    # those before its key group of 32 tokens); those from it on a NaN where it sees one (quantized, a NaN is dropped)
+    cfg = xq.make_config(n_layers=1, batch=1, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=D, max_seq=S, residual_len=R,
+                         io_dtype=int(f16), km=1, vm=1)
+    dt = torch.float16 if f16 else torch.bfloat16
+    gen = torch.Generator(device=DEV).manual_seed(S)
+    k, v = (torch.randn(1, Hkv, S, D, generator=gen, device=DEV).to(dt) for _ in range(2))
+    k[:, :, at] = 0
+    v[:, :, at] = 0
+    q = torch.randn(T, 1, Hq, D, generator=gen, device=DEV).to(dt)
+    outs = []
+    for kind in ("finite", "key", "value"):
+        kk, vv = k.clone(), v.clone()
+        if kind == "key":
+            kk[:, :, at, 3] = value
+        if kind == "value":
+            vv[:, :, at, 5] = value
+        cache = xq.Cache(cfg, DEV)
+        cache.workspace.zero_()
+        cache.append_kv(0, kk, vv)
+        n0 = xq.xq_launch_count(cache.handle)
+        outs.append(cache.attention_chunk(0, q, f32=True))
+        assert xq.xq_launch_count(cache.handle) == n0 + 1
+        cache.check_device()
+        packed = at < cache.quantized_len(0)
+        cache.close()
+    before = (at // 32 * 32 if packed else at) - (S - T)  # query token j sees the tokens up to S - T + j
+    assert 0 < before < T and torch.isfinite(outs[0]).all()
+    for o in outs[1:]:
+        assert torch.equal(o[:before], outs[0][:before])
+    assert torch.isnan(outs[2][at - (S - T):, ..., 5]).all() or (packed and value != value)
