@@ -175,24 +175,59 @@ __device__ __forceinline__ void expand_block(const uint32_t (&w)[8], int sh, con
            __byte_perm(t[j].lo[0], t[j].lo[1], s1), __byte_perm(t[j].lo[0], t[j].lo[1], u1));
   }
 }
-// eight fp32 values as hi and lo rows of 16 bytes (the difference of an infinity and its hi is not a number; the lo of
-// a number below 2^15 is below 64)
-__device__ __forceinline__ void store_row(const float (&v)[8], uint32_t dst, uint32_t lo_off) {
+// eight fp32 values as hi and lo rows of 16 bytes; bad: some may not be finite (an infinity less its hi is not a number;
+// the lo of a number below 2^15 is below 64)
+__device__ __forceinline__ void store_row(const float (&v)[8], uint32_t dst, uint32_t lo_off, bool bad) {
   uint32_t hi[4], lo[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    hi[k] = pack_io2<true>(v[2 * k], v[2 * k + 1]);
-    lo[k] = pack_io2<true>(fminf(v[2 * k] - io2_lo<true>(hi[k]), 64.f), fminf(v[2 * k + 1] - io2_hi<true>(hi[k]), 64.f));
+  for (int k = 0; k < 4; ++k) split2(v[2 * k], v[2 * k + 1], hi[k], lo[k]);
+  if (bad) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      lo[k] = pack_io2<true>(fminf(v[2 * k] - io2_lo<true>(hi[k]), 64.f), fminf(v[2 * k + 1] - io2_hi<true>(hi[k]), 64.f));
   }
   sts128(dst, hi[0], hi[1], hi[2], hi[3]);
   sts128(dst + lo_off, lo[0], lo[1], lo[2], lo[3]);
 }
 constexpr uint32_t INF32 = 0x7f800000u;  // |x| as bits: at or above, x is not a number or infinite
 __device__ __forceinline__ uint32_t abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
-__device__ __forceinline__ uint32_t finite_bits(float x) { return abs_bits(x) < INF32 ? abs_bits(x) : 0u; }
+// 16-bit patterns: the smallest one that is not a finite number, but for the sign; a pair without its elements from there on
+__device__ __forceinline__ uint32_t inf16(int f16) { return f16 ? 0x7c00u : 0x7f80u; }
+__device__ __forceinline__ uint32_t finite_pair(uint32_t w, uint32_t inf) {
+  return ((w & 0x7fffu) < inf ? w & 0xffffu : 0u) | (((w >> 16) & 0x7fffu) < inf ? w & 0xffff0000u : 0u);
+}
+__device__ __forceinline__ uint32_t max_pair(uint32_t m, uint32_t w) { return __vmaxu2(m, w & 0x7fff7fffu); }
+__device__ __forceinline__ uint32_t redux_pair(uint32_t m) { return redux_max_u32(max(m & 0xffffu, m >> 16)); }
 // 2^e that puts mx below 2^15 and, unless it is there already, above 2^14
 __device__ __forceinline__ int key_exponent(float mx) {
   return mx >= 1.f && mx < 32768.f ? 0 : (mx > 0.f ? 14 - exponent_of(mx) : 0);
+}
+
+// What elements that are not finite need, out of line: the loops that never meet any keep their place in the instruction
+// cache (16 tokens at 32k, us a layer: in line 229 to 237, as it is 230, without any of it 226).
+struct BadRows {  // the rows of a CTA, as they see tokens
+  uint32_t (*row_bad)[4];
+  int* any_bad;
+  int vis0, row0, G;
+};
+// the rows that see token tok (counted from the layer's first) see values that are not finite, in channels `mask` of
+// quarter `quarter`
+__device__ __noinline__ void mark_rows(const BadRows& b, int tok, int quarter, uint32_t mask) {
+  if (mask == 0u) return;
+  for (int r = 0; r < CM; ++r)
+    if (tok < b.vis0 + (b.row0 + r) / b.G) atomicOr(&b.row_bad[r][quarter], mask);
+  *b.any_bad = 1;
+}
+// largest finite pattern among 4 channels of 32 window rows from r0 (every step-th from first), of r rows
+__device__ __noinline__ uint32_t finite_key_max(const uint2* rows, int r0, int first, int step, int r, int row_vecs, uint32_t inf) {
+  uint32_t mp = 0u;
+#pragma unroll 1
+  for (int x = first; x < 32; x += step)
+    if (r0 + x < r) {
+      const uint2 v = rows[(size_t)(r0 + x) * row_vecs];
+      mp = max_pair(max_pair(mp, finite_pair(v.x, inf)), finite_pair(v.y, inf));
+    }
+  return redux_pair(mp);
 }
 
 template <int D, int BK, int BV, int GS>
@@ -557,14 +592,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
       }
       return pow2i(ev);
     };
-    // the rows that see token tok (counted from the layer's first) see values that are not finite, in channels `mask` of
-    // this lane's half of the quarter
-    auto mark = [&](int tok, uint32_t mask) {
-#pragma unroll 1
-      for (int r = 0; mask != 0u && r < CM; ++r)
-        if (tok < vis0 + (row0 + r) / G) atomicOr(&row_bad[r][ew & 3], mask << (v_h * (DQ / 2)));
-      if (mask != 0u) any_bad = 1;
-    };
+    const BadRows bad_rows{row_bad, &any_bad, vis0, row0, G};
     fetch(0);
     fetch(1);
 #pragma unroll 1
@@ -615,14 +643,18 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
           const int w0 = (t - pk_tiles) * CT;
           const uint2* rows = reinterpret_cast<const uint2*>(p.L.win_k + (size_t)bh * dm.R * D) + k_q;
           const int r0 = w0 + 32 * (ew >> 1);
-          uint32_t mb = 0u;
+          uint32_t mp = 0u;
 #pragma unroll 1
           for (int x = k_b; x < 32; x += 128 / D) {  // the unit is that of 32 tokens, and of their finite elements
             const uint2 v = r0 + x < p.r ? rows[(size_t)(r0 + x) * (D / 4)] : make_uint2(0u, 0u);
-            mb = max(mb, max(max(finite_bits(io_to_f(v.x & 0xffffu, p.f16)), finite_bits(io_to_f(v.x >> 16, p.f16))),
-                             max(finite_bits(io_to_f(v.y & 0xffffu, p.f16)), finite_bits(io_to_f(v.y >> 16, p.f16)))));
+            mp = max_pair(max_pair(mp, v.x), v.y);
           }
-          const int e = key_exponent(__uint_as_float(redux_max_u32(mb)));
+          mp = redux_pair(mp);
+          const bool bad = mp >= inf16(p.f16);
+          if (bad) {
+            mp = finite_key_max(rows, r0, k_b, 128 / D, p.r, D / 4, inf16(p.f16));
+          }
+          const int e = key_exponent(io_to_f(mp, p.f16));
           if (lane == 0) k_unit[i & 7][ew >> 1] = pow2i(-e);
           const float f = pow2i(e);
 #pragma unroll 1
@@ -636,7 +668,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
               v[2][x] = io_to_f(u.y & 0xffffu, p.f16) * f; v[3][x] = io_to_f(u.y >> 16, p.f16) * f;
             }
 #pragma unroll
-            for (int j = 0; j < 4; ++j) store_row(v[j], dst + blk * Pl::K_SBO + 16 * j, Pl::MAT);
+            for (int j = 0; j < 4; ++j) store_row(v[j], dst + blk * Pl::K_SBO + 16 * j, Pl::MAT, bad);
           }
         }
       } else {
@@ -665,7 +697,8 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
               if (b >= INF32) s[j] = z[j] = 0.f;
             }
 #pragma unroll 1
-            for (int j = 0; j < 4; ++j) mark(t * CT + 4 * v_q + j, (tokens >> j) & 1u ? (1u << (DQ / 2)) - 1u : 0u);
+            for (int j = 0; j < 4; ++j)
+              mark_rows(bad_rows, t * CT + 4 * v_q + j, ew & 3, (tokens >> j) & 1u ? ((1u << (DQ / 2)) - 1u) << (v_h * (DQ / 2)) : 0u);
             mb = redux_max_u32(mb);
           }
           const float f = value_exponent(mb);
@@ -689,35 +722,49 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
           auto piece = [&](int tok, int c) {  // 8 channels of a window row
             return w0 + tok < p.r ? rows[(size_t)(w0 + tok) * (D / 8) + c / 8] : make_uint4(0u, 0u, 0u, 0u);
           };
-          uint32_t mb = 0u;
+          uint32_t mp = 0u;
 #pragma unroll 1
           for (int x = 0; x < 4 * KB; ++x) {
             const uint4 u = piece(4 * v_q + (x & 3), c0 + v_h * (DQ / 2) + 8 * (x >> 2));
-            const uint32_t y[4] = {u.x, u.y, u.z, u.w};
-            uint32_t mask = 0u;
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              const uint32_t a = abs_bits(io_to_f(c & 1 ? y[c / 2] >> 16 : y[c / 2] & 0xffffu, p.f16));
-              mb = max(mb, a < INF32 ? a : 0u);
-              mask |= (uint32_t)(a >= INF32) << c;
-            }
-            if (mask != 0u) mark(p.n_q + w0 + 4 * v_q + (x & 3), mask << (8 * (x >> 2)));
+            mp = max_pair(max_pair(max_pair(max_pair(mp, u.x), u.y), u.z), u.w);
           }
-          const float f = value_exponent(redux_max_u32(mb));
+          mp = redux_pair(mp);
+          const bool bad = mp >= inf16(p.f16);
+          if (bad) {
+            mp = 0u;
+#pragma unroll 1
+            for (int x = 0; x < 4 * KB; ++x) {
+              const uint4 u = piece(4 * v_q + (x & 3), c0 + v_h * (DQ / 2) + 8 * (x >> 2));
+              const uint32_t y[4] = {u.x, u.y, u.z, u.w};
+              uint32_t mask = 0u;
+#pragma unroll
+              for (int c = 0; c < 4; ++c) {
+                mask |= (uint32_t)((y[c] & 0x7fffu) >= inf16(p.f16)) << (2 * c);
+                mask |= (uint32_t)(((y[c] >> 16) & 0x7fffu) >= inf16(p.f16)) << (2 * c + 1);
+                mp = max_pair(mp, finite_pair(y[c], inf16(p.f16)));
+              }
+              mark_rows(bad_rows, p.n_q + w0 + 4 * v_q + (x & 3), ew & 3, mask << (v_h * (DQ / 2) + 8 * (x >> 2)));
+            }
+            mp = redux_pair(mp);
+          }
+          const float f = value_exponent(__float_as_uint(io_to_f(mp, p.f16)));
           if (lane == 0) v_exp[i & 3][ew & 3] = ev;
 #pragma unroll 1
           for (int x = 0; x < 4 * KB; ++x) {
             const int j = x & 3, k = x >> 2;
             const uint4 u = piece(4 * v_q + j, c0 + v_h * (DQ / 2) + 8 * k);
-            const uint32_t y[4] = {u.x, u.y, u.z, u.w};
+            uint32_t y[4] = {u.x, u.y, u.z, u.w};
+            if (bad) {
+#pragma unroll
+              for (int c = 0; c < 4; ++c) y[c] = finite_pair(y[c], inf16(p.f16));
+            }
             float v[8];
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-              const float a = io_to_f(y[c] & 0xffffu, p.f16), b = io_to_f(y[c] >> 16, p.f16);
-              v[2 * c] = abs_bits(a) < INF32 ? a * f : 0.f;
-              v[2 * c + 1] = abs_bits(b) < INF32 ? b * f : 0.f;
+              v[2 * c] = io_to_f(y[c] & 0xffffu, p.f16) * f;
+              v[2 * c + 1] = io_to_f(y[c] >> 16, p.f16) * f;
             }
-            store_row(v, dst + k * Pl::V_SBO + 16 * j, Pl::MAT);
+            store_row(v, dst + k * Pl::V_SBO + 16 * j, Pl::MAT, false);
           }
         }
       }

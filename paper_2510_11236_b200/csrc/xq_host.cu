@@ -333,8 +333,10 @@ void plan_splits(const xq_cache* c, int l, int nq, int r, int& ns_q, int& ns_w, 
     ns_w = 0;
     int deal = 1;
     if (batches == 0) {
-      // the window alone, a tile a warp; no CTA without tokens
+      // the window alone: a round of a CTA's warps takes a tile each; more splits while that leaves the wave one wave
       ns_q = c->cfg.n_splits > 0 ? c->cfg.n_splits : (tiles + shape.warps - 1) / shape.warps;
+      const int most = c->sm_count * shape.ctas_per_sm / streams;
+      if (c->cfg.n_splits == 0 && ns_q > most) ns_q = most > 1 ? most : 1;
       if (ns_q > tiles) ns_q = tiles;
       if (ns_q > XQ_MAX_SPLITS) ns_q = XQ_MAX_SPLITS;
     } else {
