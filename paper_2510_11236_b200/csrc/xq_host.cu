@@ -234,8 +234,8 @@ MmaShape mma_shape(const xq_cache* c, int l) {
 // launch per layer, which callers that watch xq_launch_count have seen so far (10.6 us for a tiny pair; 8.5 together).
 constexpr int MIN_JOINT_LAYERS = 3;
 
-// Times of the tensor-core kernel, us, as plan_splits adds them up: fitted to 30 shapes (head_dim 64 and 128, one to
-// eight heads, 4 to 512 streams of 1000 to 131072 tokens), each with up to 29 numbers of splits.
+// Times of the tensor-core kernel, us, as plan_batches adds them up: fitted to 75 shapes (one to eight heads, 6 to 256
+// streams of 1500 to 131072 tokens; head_dim 64 by two), each with up to 29 numbers of splits; rms error 6 %.
 struct DecodeTimes {
   double launch;         // start and end of a launch that runs alone
   double round, warp;    // a warp's batch, while w warps of its SM work: round + warp * w
@@ -244,10 +244,10 @@ struct DecodeTimes {
 };
 DecodeTimes decode_times(const Dims& dm) {
   if (dm.D == 64) return {6.5, 1.0, 0.19, 9.0, 4.0, 0.25};
-  if (dm.G == 1) return {8.0, 0.6, 0.3, 11.0, 5.5, 0.34};
-  if (dm.G == 2) return {9.0, 1.24, 0.295, 11.0, 6.0, 0.42};
-  if (dm.G <= 4) return {8.0, 1.46, 0.325, 11.0, 6.0, 0.415};
-  return {12.8, 2.6, 0.57, 0.0, 5.5, 0.93};
+  if (dm.G == 1) return {7.3, 0.48, 0.34, 10.0, 3.8, 0.37};
+  if (dm.G == 2) return {7.0, 0.71, 0.36, 10.0, 4.1, 0.40};
+  if (dm.G <= 4) return {7.2, 0.91, 0.37, 10.0, 4.0, 0.44};
+  return {8.3, 2.4, 0.63, 10.0, 5.0, 0.86};
 }
 
 // Number of splits of a stream's batches, and the runs in which they are dealt, for the tensor-core kernel; splits > 0:
@@ -255,10 +255,11 @@ DecodeTimes decode_times(const Dims& dm) {
 // of call use the same one: xq_decode_attention, a launch for each layer (what a model that feeds one layer's result to
 // the next can call), which wants the CTAs of one full wave, and xq_decode_step, whose layers share launches and which
 // wants few CTAs.  The single call counts: of the plans that cost a layer alone at most ALONE_BOUND times the best, the
-// one that a step takes the least time with.  us per layer, alone / in a step, with the plan a step would choose for
-// itself and with this one: 32k, four heads 40.7 / 25.1, 33.2 / 26.5; 16k 24.8 / 14.3, 21.6 / 15.5; one sequence of 128k
-// 42.0 / 25.3, 35.0 / 27.3; groups of five at 16k 52.9 / 29.0, 38.6 / 28.6; MHA at 4k, batch 8, 30.5 / 23.2 with either.
-constexpr double ALONE_BOUND = 1.07;  // what the model is worth: measured times are within 1.07 of it
+// one with the smallest sum of the time alone, relative to the best, and STEP_WEIGHT times that in a step.  us per layer,
+// alone / in a step, with the plan a step would choose for itself and with this one: 32k, four heads 40.7 / 25.1,
+// 33.1 / 27.8; 16k 24.8 / 14.3, 20.4 / 16.7; one sequence of 128k 42.0 / 25.3, 33.7 / 27.5; groups of five at 16k
+// 52.9 / 29.0, 36.5 / 30.9; MHA at 4k, batch 8, 30.5 / 23.1 with either.
+constexpr double ALONE_BOUND = 1.10, STEP_WEIGHT = 0.5;
 constexpr double MERGE = 0.03;  // us of a launch's end for each partial of a stream
 void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int splits, MmaPlan& out) {
   const Dims& dm = c->plan.dm;
@@ -268,7 +269,7 @@ void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int spl
   struct Candidate { int ns, deal; double alone, step, next; };
   Candidate all[2 * XQ_MAX_SPLITS];
   int n = 0;
-  double alone_min = 0.0;
+  double alone_min = 0.0, step_min = 0.0;
   // batches are dealt to the splits one by one, or in runs of one per warp: no warp of a CTA then waits for another's
   // last batch
   for (int deal : {1, shape.warps}) {
@@ -300,14 +301,18 @@ void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int spl
                   (dm.G > 4 ? 5.5 : 2.5) + (double)(streams * ns) / slots * each};
       if (k.alone < t.floor) k.alone = t.floor;
       if (n == 0 || k.alone < alone_min) alone_min = k.alone;
+      if (n == 0 || k.step < step_min) step_min = k.step;
       all[n++] = k;
     }
   }
   const Candidate* best = nullptr;
+  double best_score = 0.0;
   for (int i = 0; i < n; ++i) {
     const Candidate& k = all[i];
-    if (k.alone > ALONE_BOUND * alone_min) continue;
-    if (!best || (joint ? k.step < best->step : k.alone < best->alone)) best = &k;
+    const double score = k.alone / alone_min + (joint ? STEP_WEIGHT * k.step / step_min : 0.0);
+    if (k.alone > ALONE_BOUND * alone_min || (best && score >= best_score)) continue;
+    best = &k;
+    best_score = score;
   }
   out = {batches, best->ns, best->deal, best->alone, best->next};
 }
