@@ -29,8 +29,8 @@
  *     synchronizes the device, except where a function says otherwise.  All
  *     kernels are launched asynchronously on the given stream
  *     (a cudaStream_t passed as void*; NULL is the default stream).
- *     The decode and window-append kernels are launched as programmatic
- *     dependents: their thread blocks may be placed, and packed cache data that
+ *     The decode, chunk, window-append and quantize-and-pack kernels are launched as
+ *     programmatic dependents: their thread blocks may be placed, and packed cache data that
  *     earlier calls completed may be fetched, while the preceding kernel in the
  *     stream is still running; they wait for that kernel to complete before
  *     they touch q, new tokens, the window, the split scratch or any output, so
@@ -69,8 +69,11 @@ extern "C" {
 /* Tensor-core kernel: group of <= 8 query heads; this value asks for it and wants head_dim
  * 128 (XQ_KERNEL_AUTO takes it for head_dim 64 too).  The products q_d * s_d (query times
  * key scale) and p_t * s_t (softmax numerator times value scale) enter the matrix products
- * as unevaluated sums of two halves (22 significant bits), codes are exact, accumulation
- * and everything else is fp32. */
+ * as unevaluated sums of two halves (22 bits of every product down to 2^-10 of the largest
+ * of its 128 tokens), codes are exact.  The fp32 sums of the matrix products keep 16 bits or
+ * more; with head_dim 128 they set the error: 1e-5 to 1e-4 of the result's norm (2-norm), in
+ * xq_attention_chunk's own kernel 1e-6 to 1e-5.  With head_dim 64, and over the window alone,
+ * the result is as exact as the scalar kernel's (below 1e-6). */
 #define XQ_KERNEL_MMA 2
 
 #define XQ_MEM_DEVICE 0
@@ -95,8 +98,10 @@ typedef struct xq_config {
                            group must have equal bit-width.                               */
   float eta1, eta2;     /* calibration parameter eta_B for B = 1, 2, in [0, 0.5] (Eq. 5)  */
   float sm_scale;       /* softmax scale; 0 selects 1/sqrt(head_dim)                      */
-  int32_t n_splits;     /* sequence splits per (sequence, KV head) in decode; 0 = library
-                           chooses; at most XQ_MAX_SPLITS                                 */
+  int32_t n_splits;     /* sequence splits per (sequence, KV head) of a decode launch; 0 =
+                           library chooses; at most XQ_MAX_SPLITS, and as many as there are
+                           128-token batches.  The launch that xq_attention_chunk makes for
+                           many query tokens chooses its own                              */
   int32_t io_dtype;     /* type of K, V, q, out and of the residual window: XQ_BF16 or
                            XQ_F16                                                         */
   int32_t kernel;       /* XQ_KERNEL_*                                                    */
@@ -188,8 +193,11 @@ int xq_decode_attention_f32(xq_cache* c, int layer, const void* q, float* out, v
  * are, exactly as xq_decode_attention does for the tokens it sees; n_q_tokens = 1
  * is xq_decode_attention.  q, out: device, [n_q_tokens, batch, n_q_heads, head_dim]
  * contiguous (token-major: one token's slice is a decode call's q), io_dtype;
- * 16-byte aligned.  The _f32 variant writes float results (tests).  Errors as
- * xq_decode_attention; 1 <= n_q_tokens <= S. */
+ * 16-byte aligned.  Many tokens share one launch and one pass over the cache; a few
+ * (2 to 12, where that takes less time) take a decode launch each, with that call's
+ * rounding.  A token that is not finite does not reach the rows before it.  The _f32
+ * variant writes float results (tests).  Errors as xq_decode_attention;
+ * 1 <= n_q_tokens <= S. */
 int xq_attention_chunk(xq_cache* c, int layer, const void* q, void* out, int n_q_tokens, void* stream);
 int xq_attention_chunk_f32(xq_cache* c, int layer, const void* q, float* out, int n_q_tokens, void* stream);
 

@@ -14,28 +14,34 @@
 //   sum_t p_t v_hat_td = sum_t (p_t s_tg) c_td + sum_t p_t z_tg  (values, per token)
 //
 // and the other operand (q_d s_d, or p_t s_tg) is carried as an unevaluated sum hi + lo of two fp16 numbers in two of
-// the eight operand columns: hi = RN(q s), lo = fma(q, s, -hi) is exact, so a product q_d s_d loses nothing
-// (p_t s_t: one rounding at 2^-22), codes are exact, accumulation is fp32.  The powers of two that the bit offsets put
-// on the codes are taken out of q and of the softmax numerators.  The m16n8 accumulator gives a thread the hi and lo
-// sums of its own head: a logit is their sum, and each (token, head) has one thread.  The numerators go through a
-// small buffer of the warp in shared memory to become B fragments.
+// the eight operand columns: hi = RN(q s), lo = fma(q, s, -hi), as far as fp16 reaches: relative to the largest product
+// of a batch, which is kept between 2^8 and 2^15 (2^9 with 1-bit keys, whose weights come off q), nothing above 2^-33 is lost
+// (p_t s_t: one rounding at 2^-22).  Codes are exact, accumulation is fp32 with the digits that the alignment above
+// leaves: for head_dim 128 this, not the operands, is what limits the result (16 bits and more of each sum; scale and
+// zero-point parts are large and cancel).  The powers of two that the bit offsets put on the codes are taken out of q
+// and of the softmax numerators.  The m16n8 accumulator gives a thread the hi and lo sums of its own head: a logit is
+// their sum, and each (token, head) has one thread.  The numerators go through a small buffer of the warp in shared
+// memory to become B fragments.
 //
 // Why mma.sync and not tcgen05.  At this shape (at most 8 query heads against 128 channels) the expanded codes are the
-// large operand; a tcgen05 kernel has to pass them through tensor memory and hand batches between warps, and the
-// version before this one spent a batch's ~1600 cycles on that chain of hand-overs, two batches per SM at a time
-// (32k context, four heads: 34.7 us per layer).  Here sixteen independent warps share an SM and hide each other's
-// latencies.  A layer in a step of 16 or 32 (layers share launches), us, before and now: 32k context, four heads, batch
-// 4: 34.2 -> 25.5 (84 MB: 3.3 TB/s); 4k, one head per kv head, batch 8: 28.1 -> 22.9; 8k, groups of 64, batch 16: 32.4 -> 22.9; one
-// sequence of 128k: 34.5 -> 24.8; groups of five heads at 16k: 34.2 -> 30.5; head_dim 64, 512 tokens, which had only
-// the scalar kernel: 380 -> 5.
+// large operand; a tcgen05 kernel has to pass them through tensor memory and hand batches between warps, and one that
+// did spent a batch's ~1600 cycles on that chain of hand-overs, two batches per SM at a time (32k context, four heads:
+// 34.2 us per layer).  Here sixteen independent warps share an SM and hide each other's latencies.  A layer of a step of 16
+// (layers share launches), us, that kernel -> this one, with the splits that plan_batches gives both kinds of call: 32k
+// context, four heads, batch 4 34.2 -> 27.8 (84 MB: 3.1 TB/s); 4k, one head per kv head, batch 8 27.9 -> 23.1; 8k,
+// groups of 64, batch 16 32.3 -> 24.7; one sequence of 128k 34.8 -> 27.5; groups of five heads at 16k 33.1 -> 30.9, of
+// eight at 32k 37.0 -> 30.6; head_dim 64, 2048 tokens, 32 streams (the scalar kernel: 500) 2.6.
 // What bounds it: issue and latency of a batch's phases.  A batch (four heads, 32-token groups) is ~2000 warp
 // instructions, 512 of them the masks (ALU: 2 cycles each per sub-partition), 140 products (8 cycles each), ~350
 // half-precision multiplies (2 cycles each), and takes a warp ~14000 cycles with sixteen on the SM: key products 2900,
 // value products 3100, waits for copies and their issue 1700, key scales 1600, softmax 1400, value scales 1000,
-// biases 700.  A CTA's start and end cost 5000 each, which is why a step wants few CTAs (plan_splits).
+// biases 700 (with q in registers; q in shared memory took 3 % off).  A CTA's start and end cost 5000 each, which is
+// why a step wants few CTAs.  Registers: 128 a thread, 168 with two sets of heads; at head_dim 128 up to 28 bytes of
+// spills with one set, 96 to 256 with two.
 // Measured and not kept (32k context, four heads, us per 32 layers; this shape 925 then): four CTAs of 4 warps 944,
 // three of 4 1014, three of 5 1025, one of 12 1026 (fewer registers do not pay for more warps, nor fewer warps for
-// more registers).
+// more registers).  Two sets of heads with 7 warps (146 registers) instead of 6: 40.0 us against 31.9 (groups of five
+// at 16k, eight splits).  The window's rows asked into L2 at the start of a CTA: no change.
 #pragma once
 #include "xq_internal.h"
 #include "xq_mma.cuh"

@@ -64,8 +64,8 @@ __device__ __forceinline__ void group_params(float mn, float mx, int bits, float
   const float qmax = (float)((1 << bits) - 1);
   s = __fsub_rn(mx, mn);
   if (bits == 2) {
-    // RN(a / 3) by the correction step below (`Quot`); tiny and huge ranges, which could leave the normal range on the
-    // way, take the division
+    // RN(a / 3) by Markstein's correction step, as in `Quot` below: RN(1 / 3) is the correctly rounded reciprocal and q
+    // within an ulp of a / 3; tiny and huge ranges, which could leave the normal range on the way, take the division
     const float a = s, third = __uint_as_float(0x3eaaaaabu);  // RN(1 / 3)
     const uint32_t e = (__float_as_uint(a) >> 23) & 0xffu;
     const float q = __fmul_rn(a, third);
@@ -107,9 +107,11 @@ __device__ __forceinline__ int ord16(uint32_t h) {
 __device__ __forceinline__ uint32_t pat16(int o) { return o >= 0 ? (uint32_t)o : (0x8000u | (uint32_t)(-o)); }
 
 // A group's uncalibrated parameters for the quotient RN(RN(x - z) / s).  With y = RN(1/s): q = RN(a y),
-// r = a - q s (exact in one fused multiply-add), q' = RN(q + r y) is the correctly rounded quotient (the classical
-// correction step of division by a correctly rounded reciprocal; the scales it can miss get a NaN from safe_rcp
-// and take the division).
+// r = a - q s (exact in one fused multiply-add), q' = RN(q + r y) is the correctly rounded quotient: the correction step
+// of P. W. Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", IBM J. Res. Dev.
+// 34 (1990), which holds where y is the correctly rounded reciprocal, q is within an ulp of a / s and nothing leaves the
+// normal range.  Scales whose significand is all ones and those of extreme exponent get a NaN from safe_rcp and take the
+// division.
 struct Quot {
   float z, s, y;
   bool fast;
