@@ -28,9 +28,9 @@
 // did spent a batch's ~1600 cycles on that chain of hand-overs, two batches per SM at a time (32k context, four heads:
 // 34.2 us per layer).  Here sixteen independent warps share an SM and hide each other's latencies.  A layer of a step of 16
 // (layers share launches), us, that kernel -> this one, with the splits that plan_batches gives both kinds of call: 32k
-// context, four heads, batch 4 34.2 -> 27.8 (84 MB: 3.1 TB/s); 4k, one head per kv head, batch 8 27.9 -> 23.1; 8k,
-// groups of 64, batch 16 32.3 -> 24.7; one sequence of 128k 34.8 -> 27.5; groups of five heads at 16k 33.1 -> 30.9, of
-// eight at 32k 37.0 -> 30.6; head_dim 64, 2048 tokens, 32 streams (the scalar kernel: 500) 2.6.
+// context, four heads, batch 4 34.2 -> 26.5 (84 MB: 3.2 TB/s); 4k, one head per kv head, batch 8 27.9 -> 23.1; 8k,
+// groups of 64, batch 16 32.3 -> 24.7; one sequence of 128k 34.8 -> 27.5; groups of five heads at 16k 33.1 -> 28.6, of
+// eight at 32k 37.0 -> 28.4; head_dim 64, 2048 tokens, 32 streams (the scalar kernel: 500) 2.6.
 // What bounds it: issue and latency of a batch's phases.  A batch (four heads, 32-token groups) is ~2000 warp
 // instructions, 512 of them the masks (ALU: 2 cycles each per sub-partition), 140 products (8 cycles each), ~350
 // half-precision multiplies (2 cycles each), and takes a warp ~14000 cycles with sixteen on the SM: key products 2900,

@@ -255,8 +255,10 @@ DecodeTimes decode_times(const Dims& dm) {
 // of call use the same one: xq_decode_attention, a launch for each layer (what a model that feeds one layer's result to
 // the next can call), which wants the CTAs of one full wave, and xq_decode_step, whose layers share launches and which
 // wants few CTAs.  The single call counts: of the plans that cost a layer alone at most ALONE_BOUND times the best, the
-// one with the smallest sum of the time alone, relative to the best, and STEP_WEIGHT times that in a step (half as much
-// for more than four heads, whose launches alone have nothing to spare against the kernel before this one).
+// one with the smallest sum of the time alone, relative to the best, and STEP_WEIGHT times that in a step.  us per layer,
+// alone / in a step, with the plan a step would choose for itself and with this one: 32k, four heads 40.7 / 25.1,
+// 34.8 / 26.5; 16k 24.8 / 14.3, 21.6 / 15.5; one sequence of 128k 42.0 / 25.3, 33.7 / 27.5; groups of five at 16k
+// 52.9 / 29.0, 38.6 / 28.6; MHA at 4k, batch 8, 30.5 / 23.1 with either.
 constexpr double ALONE_BOUND = 1.10, STEP_WEIGHT = 1.2;
 constexpr double MERGE = 0.03;  // us of a launch's end for each partial of a stream
 void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int splits, MmaPlan& out) {
@@ -305,7 +307,7 @@ void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int spl
   }
   const Candidate* best = nullptr;
   double best_score = 0.0;
-  const double step_weight = !joint ? 0.0 : (dm.G > 4 ? 0.5 * STEP_WEIGHT : STEP_WEIGHT);
+  const double step_weight = joint ? STEP_WEIGHT : 0.0;
   for (int i = 0; i < n; ++i) {
     const Candidate& k = all[i];
     const double score = k.alone / alone_min + step_weight * k.step / step_min;
