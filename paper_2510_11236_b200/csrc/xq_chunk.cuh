@@ -41,31 +41,7 @@ constexpr int C_PEXP = 6;          // numerators are carried times 2^C_PEXP (at 
 constexpr int C_EXPAND = 8;        // expanding warps (8 .. 15): keys 0 .. 3, values 4 .. 7
 constexpr int C_THREADS = (8 + C_EXPAND + 1) * 32;
 
-// ---- tensor memory and tcgen05 ----
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
-__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
-      "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};\n" ::"r"(taddr),
-      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]),
-      "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
-      "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
-      : "memory");
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
-      "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr) : "memory");
-}
+// ---- tcgen05 ----
 // shared-memory matrix descriptor, N-major, no swizzle: core matrices of 8 K-rows x 16 bytes of N;
 // lbo / sbo: byte distance between core matrices along K / along N
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
@@ -306,9 +282,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
   // its own, and with all columns taken here it would wait for this CTA, which waits for it.
   grid_dependency_wait();
   if (warp == 8 + C_EXPAND) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                     (uint32_t)__cvta_generic_to_shared(&tmem_base_sm)), "r"(512u) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    tmem_alloc((uint32_t)__cvta_generic_to_shared(&tmem_base_sm), 512u);
   }
   tc_fence_before();
   __syncthreads();
@@ -339,14 +313,14 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
 #pragma unroll
       for (int i = 0; i < 32; ++i)
         r[i] = pack_io2<true>(io_to_f(w[32 * c + i] & 0xffffu, p.f16) * f, io_to_f(w[32 * c + i] >> 16, p.f16) * f);
-      tmem_st32(row_t + Pl::COL_Q + 32 * c, r);
+      tmem_st<32>(row_t + Pl::COL_Q + 32 * c, r);
     }
     if constexpr (Pl::FLUSH != 0) {
       uint32_t zero[32];
 #pragma unroll
       for (int i = 0; i < 32; ++i) zero[i] = 0u;
 #pragma unroll
-      for (int c = 0; c < D; c += 32) tmem_st32(row_t + Pl::COL_T + c, zero);
+      for (int c = 0; c < D; c += 32) tmem_st<32>(row_t + Pl::COL_T + c, zero);
     }
     tc_wait_st();
 #pragma unroll
@@ -443,7 +417,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         const bool masked = __any_sync(0xffffffffu, n_valid < CT);
         // 32 columns of S at a time, here and below: the loops stay small (the instruction cache bounds this kernel)
         auto load = [&](int c, uint32_t (&s)[32]) {
-          tmem_ld32(s_t + 32 * c, s);
+          tmem_ld<32>(s_t + 32 * c, s);
           tc_wait_ld();
           if (masked) {
 #pragma unroll
@@ -483,23 +457,23 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
               const float fa = f * pow2i(v_exp[i & 3][qa] - v_exp[(i - 1) & 3][qa]);
               const float fz = f * pow2i(v_exp[i & 3][qz] - v_exp[(i - 1) & 3][qz]);
               uint32_t s[32];
-              tmem_ld32(row_t + Pl::COL_O + c, s);
+              tmem_ld<32>(row_t + Pl::COL_O + c, s);
               if constexpr (Pl::FLUSH != 0) {
                 uint32_t sum[32];
-                tmem_ld32(row_t + Pl::COL_T + c, sum);
+                tmem_ld<32>(row_t + Pl::COL_T + c, sum);
                 tc_wait_ld();
 #pragma unroll
                 for (int k = 0; k < 32; ++k) {
                   sum[k] = __float_as_uint((__uint_as_float(sum[k]) + __uint_as_float(s[k])) * (k < 16 ? fa : fz));
                   s[k] = 0u;
                 }
-                tmem_st32(row_t + Pl::COL_T + c, sum);
+                tmem_st<32>(row_t + Pl::COL_T + c, sum);
               } else {
                 tc_wait_ld();
 #pragma unroll
                 for (int k = 0; k < 32; ++k) s[k] = __float_as_uint(__uint_as_float(s[k]) * (k < 16 ? fa : fz));
               }
-              tmem_st32(row_t + Pl::COL_O + c, s);
+              tmem_st<32>(row_t + Pl::COL_O + c, s);
             }
             tc_wait_st();
           }
@@ -524,7 +498,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
             split2(a, d, o[k], o[16 + k]);
           }
           l += la + lb;
-          tmem_st32(s_t + 32 * c, o);
+          tmem_st<32>(s_t + 32 * c, o);
         }
         tc_wait_st();
       }
@@ -799,11 +773,11 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
         const int cb = w * (D / 2) + 32 * h;
         uint32_t o[32];
         if (N > 0) {
-          tmem_ld32(row_t + Pl::COL_O + cb, o);
+          tmem_ld<32>(row_t + Pl::COL_O + cb, o);
           tc_wait_ld();
           if constexpr (Pl::FLUSH != 0) {
             uint32_t sum[32];
-            tmem_ld32(row_t + Pl::COL_T + cb, sum);
+            tmem_ld<32>(row_t + Pl::COL_T + cb, sum);
             tc_wait_ld();
 #pragma unroll
             for (int k = 0; k < 32; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) + __uint_as_float(sum[k]));
@@ -849,7 +823,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) chunk_kernel(const __grid_consta
   __syncthreads();
   tc_fence_after();
   if (warp == 8 + C_EXPAND)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tbase), "r"(512u) : "memory");
+    tmem_dealloc(tbase, 512u);
   if (dead_sm != 0) {
     if (tid == 0) atomicExch(p.status, 1);
     return;

@@ -50,59 +50,77 @@ namespace xq {
 namespace {
 
 constexpr int BT = 128;            // tokens per batch
+constexpr int TT = 64;             // tokens of a round: half a batch
 constexpr float TAU = 3.f;         // log2 units a logit may exceed the softmax reference before it is raised
 constexpr int P_EXP = 11;          // numerators are carried times 2^P_EXP (at most 2^(P_EXP + TAU) as fp16)
 constexpr int Q_BIAS_EXP = 8;      // exponent of the largest |q| in the zero-point products
+constexpr uint32_t ONES = 0x3C003C00u;
 
-// Shared-memory plan.  D: head dim, GS: quantization group, BK / BV: bits.  The eight operand columns are four column
-// pairs (hi, lo) of HP heads (1, 2 or 4) times GC = 4 / HP slots: with fewer heads, one operand serves GC token units
-// of the keys (or GC channel parts of the values) at once, each row tile reading the columns of its own slot.
-// NT: sets of four heads (HP = 4).
-template <int D, int BK, int BV, int GS, int HP, int NT>
+// Shared-memory plan.  D: head dim, GS: quantization group, BK / BV: bits, HP: query heads per kv head and layer (1, 2,
+// 4, 8; a G in between is padded), NL: layers that share their codes (1 or 2).  A CTA's "heads" are the VH = HP * NL
+// heads of its layers.  Up to four of them: the eight operand columns are four column pairs (hi, lo) of VH heads times
+// GC = 4 / VH slots: with fewer heads, one operand serves GC token units of the keys (or GC channel parts of the values)
+// at once, each row tile reading the columns of its own slot.  Eight (WIDE): a column is a head, hi and lo are operands
+// of two products.
+template <int D, int BK, int BV, int GS, int HP, int NL>
 struct Plan {
-  static_assert(NT == 1 || HP == 4, "several sets only of four heads");
-  static constexpr int NGT = BT / GS;            // token groups of the keys in a batch
+  static constexpr int VH = HP * NL;
+  static_assert(VH == 1 || VH == 2 || VH == 4 || VH == 8, "heads of a CTA");
+  static constexpr bool WIDE = VH == 8;
+  static constexpr int NSET = WIDE ? 2 : 1;      // sets of up to four heads
+  static constexpr int SH = WIDE ? 4 : VH;       // heads of a set
+  static constexpr int NCOL = WIDE ? 2 : 1;      // heads of a thread's accumulator columns
+  static constexpr int NGT = TT / GS;            // token groups of the keys in a round
   static constexpr int NG = D / GS;              // channel groups of a value row
   static constexpr int KS = D / 16;              // k-steps of the key products, row tiles of the value products
-  static constexpr int GC = 4 / HP;              // slots
+  static constexpr int GC = WIDE ? 1 : 4 / VH;   // slots
+  static constexpr int NE = WIDE ? 4 : 4 / GC;   // row tiles of 16 tokens whose logits a thread has, of the four of a round
   static constexpr int CP = NG > GC ? NG : GC;   // channel parts of the value products: one scale per token each
-  static constexpr int KC = BT * D * BK / 8, KM = NGT * 4 * D;  // key codes; scales and zero-points
-  static constexpr int VC = BT * D * BV / 8, VM = BT * 4 * NG;  // the same of the values
-  static constexpr int OFF_KM = KC, OFF_VC = KC + KM, OFF_VM = KC + KM + VC;
-  // value scales, then zero-points, as they are reordered over VM: [pair of tokens][NG] half2, one more row after
-  // the pairs of a lane column (bank conflicts)
-  static constexpr int VSROW = 4 * NG, VS = 64 * VSROW + 4 * VSROW;
-  // centered codes: the second halves of the zero-points, of the values (as VS), of the keys (as the second half of KM)
+  static constexpr int KCODES = TT * D * BK / 8;  // codes of a round; values in 1 bit: of its whole batch
+  static constexpr int VCODES = 16 * D;
+  static constexpr int KM = NGT * 4 * D, VM = TT * 4 * NG;  // scales and zero-points of a round and layer: keys, values
   static constexpr bool CENTERED = D == 64;
-  static constexpr int OFF_KL = OFF_VM + 3 * VS, KL = NGT * 2 * D;
-  static constexpr int STAGE = CENTERED ? OFF_KL + KL : OFF_VM + 2 * VS;
-  // numerators: [head][pair of tokens (t, t + 2)] of (hi pair, lo pair), 16 bytes more after every 16 pairs and 32
-  // more after every head against bank conflicts
-  static constexpr int PH = 64 * 8 + 4 * 16 + 32;
-  static constexpr int PBUF = HP * NT * PH;
+  static_assert(!CENTERED || NL == 1, "layers share codes only with head_dim 128");
+  // value scales, then zero-points, as they are reordered over the copy: [channel group][pair of tokens] half2, a
+  // group's zero-points 8 bytes longer (bank conflicts); centered codes: second halves of the zero-points, of the
+  // values (as the first), of the keys (as the zero-points of the copy)
+  static constexpr int VZROW = TT / 2 * 4 + 8, VZ = NG * (TT / 2) * 4;
+  static constexpr int VL = VZ + NG * VZROW;
+  static constexpr int VROOM = ((CENTERED ? VL + NG * VZROW : VL) + 15) / 16 * 16;
+  static_assert(VROOM >= VM, "the copy fits");
+  // numerators: [head][tile of 16 tokens][pair of tokens (t, t + 2)] of (hi pair, lo pair), 16 bytes more after every
+  // tile and 32 more after every head against bank conflicts (WIDE: 16-byte cells in an order without any).  Two layers:
+  // over the key scales and zero-points, whose next copies then come after the value products.
+  static constexpr int PT = 8 * 8 + 16, PH = 4 * PT + 32;
+  static constexpr int PBUF = WIDE ? 8 * 256 : VH * PH;
+  static constexpr bool P_OVER = NL == 2;
+  static constexpr int OFF_V = 16 * D, OFF_KM = 2 * 16 * D;
+  static constexpr int OFF_VM = OFF_KM + (P_OVER && NL * KM < PBUF ? PBUF : NL * KM);
+  static constexpr int OFF_KL = OFF_VM + NL * VROOM, KL = CENTERED ? NGT * 2 * D : 0;
+  static constexpr int OFF_P = P_OVER ? OFF_KM : (OFF_KL + KL + 127) / 128 * 128;
+  static_assert(OFF_P % 128 == 0, "cells are found by exclusive or");
   static constexpr int WROW = 2 * D + 16;        // a staged window row
   static constexpr int WIN = 32 * WROW;          // 16 key rows, then 16 value rows (over the stage of the warp)
-  static constexpr int BODY = STAGE + PBUF;
+  static constexpr int BODY = P_OVER ? OFF_KL + KL : OFF_P + PBUF;
   static constexpr int WARP = ((BODY > WIN ? BODY : WIN) + 127) / 128 * 128;
   static constexpr int MS = D + 4;               // state row: acc[D], m, l
-  static_assert(HP * NT * MS * 4 <= WARP, "a warp's state rows fit its own memory");
+  static_assert(2 * VH * MS * 4 <= WARP, "a warp's state rows, of the packed tokens and of the window, fit its own memory");
   static_assert(MS % 4 == 0, "state rows are read as vectors");
-  // after the warps' parts: B fragments of the zero-point products; fp16 ones, read in place of zero-points for the
-  // sum of the numerators; q as it came
-  static constexpr int QB = NT * KS * 32 * 4, ONES = CENTERED ? 0 : 64 * VSROW, QS = HP * NT * D * 2;
-  // four or eight heads: q as operand fragments, for all warps (else each keeps them in registers; 16 or 32 a thread,
-  // which spilled 80-580 bytes: a step's layer at 32k, four heads 25.8 -> 25.1 us, groups of five at 16k 31.2 -> 28.7)
-  static constexpr bool Q_SHARED = HP == 4 && D == 128;
-  static constexpr int QF = Q_SHARED ? NT * KS * 32 * 8 : 0;
-  static constexpr int room(int w) { return w * WARP + QB + ONES + QS + QF; }
-  // Two CTAs per SM, each of as many warps as registers (128, or 168 for eight heads) and shared memory allow.
-  static constexpr int CTAS = 2;
-  static constexpr int MOST = NT == 1 ? 8 : 6;
-  static constexpr int LIMIT = 228 * 1024 / CTAS - 1024 - 512;
-  static constexpr int WARPS = room(MOST) <= LIMIT ? MOST : (room(MOST - 1) <= LIMIT ? MOST - 1 : MOST - 2);
+  // after the warps' parts: B fragments of the zero-point products; q as it came; with head_dim 128 q as operand
+  // fragments, for all warps (else each keeps them in registers)
+  static constexpr int QB = NSET * KS * 32 * 4, QS = VH * D * 2;
+  static constexpr bool Q_SHARED = D == 128;
+  static constexpr int QF = Q_SHARED ? KS * 32 * 8 : 0;
+  static constexpr int room(int w) { return w * WARP + QB + QS + QF; }
+  // Three CTAs per SM, each of eight warps of 80 registers.
+  static constexpr int CTAS = 3, WARPS = 8;
+  // Tensor memory: the value sums of a warp between its rounds, 4 columns a row tile (WIDE: 4 more, of the lo products)
+  static constexpr int TCOLS = KS * 4 * NCOL, TUSED = (WARPS + 3) / 4 * TCOLS;
+  static constexpr int TMEM = TUSED <= 32 ? 32 : TUSED <= 64 ? 64 : TUSED <= 128 ? 128 : 256;
+  static_assert(TUSED <= TMEM && CTAS * TMEM <= 512, "tensor memory");
   static constexpr int TOTAL = room(WARPS);
-  static_assert(TOTAL <= LIMIT, "shared memory");
-  static_assert(WARPS * WARP >= HP * NT * (256 + 1) * 4, "the merge's weights");
+  static_assert(TOTAL <= 228 * 1024 / CTAS - 1024 - 512, "shared memory");
+  static_assert(WARPS * WARP >= VH * (256 + 1) * 4, "the merge's weights");
 };
 
 // Code operands.  head_dim 128: the masked code bits as they are, fp16 subnormals code * weight * 2^-22.  head_dim 64:
@@ -114,21 +132,22 @@ struct Plan {
 template <int D>
 struct Code {
   static constexpr bool CENTERED = D == 64;
-  static constexpr int EXP = CENTERED ? 9 : 22;
   template <int BITS>
   static __device__ __forceinline__ float center() { return 0.5f * (float)((1 << BITS) - 1); }
-  // the operand pair of the code bits at 2 + BITS * i of both halves of w; their weight is 2^(BITS * i)
-  template <int BITS>
+  // the operand pair of the code bits at BASE + BITS * i of both halves of w; their weight is 2^(BITS * i)
+  template <int BITS, int BASE>
   static __device__ __forceinline__ uint32_t pair(uint32_t w, int i) {
-    const uint32_t m = w & ((BITS == 2 ? 0x000c000cu : 0x00040004u) << (BITS * i));
+    const uint32_t m = w & (((BITS == 2 ? 0x00030003u : 0x00010001u) << BASE) << (BITS * i));
     if constexpr (CENTERED) {
-      // times 2^13, less center * weight * 2^-9: 1.5 or 0.5 at exponent field 15 - 9 + BITS * i
+      // times 2^(15 - BASE), less center * weight * 2^-9: 1.5 or 0.5 at exponent field 15 - 9 + BITS * i
       const uint32_t c = BITS == 2 ? 0x8200u + ((uint32_t)(6 + 2 * i) << 10) : 0x8000u + ((uint32_t)(5 + i) << 10);
-      return hfma2(m, 0x70007000u, c * 0x10001u);
+      return hfma2(m, ((uint32_t)(30 - BASE) << 10) * 0x10001u, c * 0x10001u);
     } else {
       return m;
     }
   }
+  // exponent of the operand of a code with weight 1
+  static __host__ __device__ constexpr int exp(int base) { return CENTERED ? 9 : 24 - base; }
 };
 // z + center s of a pair of groups as an unevaluated sum of two fp16
 template <int D, int BITS>
@@ -158,9 +177,9 @@ __device__ __forceinline__ int k_slot(int d) {
   else { tig = (d >> 4) & 3; ks = 4 * (d >> 6) + ((d >> 2) & 3); }
   return ((ks >> 1) * 4 + tig) * 8 + (ks & 1) * 4 + (c & 1) * 2 + (c >> 1);
 }
-// Row of the reordered value scales that holds token pair p (tokens t = 4 (p / 2) + p % 2 and t + 2) of a batch: a
-// spare row after every 16 pairs, so that the rows which the lane columns read together fall into different banks.
-__device__ __forceinline__ constexpr int pair_row(int p) { return p + (p >> 4); }
+// k_slot of channel d + 32 j less that of channel d < 32
+template <int D, int BK>
+__device__ __forceinline__ constexpr int k_slot_step(int j) { return BK == 1 && D == 128 ? 8 * j : 16 * (j & 1) + 64 * (j >> 1); }
 
 // One warp stages window tokens [tb, tb + 16) (rows at or beyond t1 are zero-filled); no commit.  With a fused
 // append the newest row (index r - 1) is not in the window yet: it comes from the step's input.
@@ -275,9 +294,9 @@ __device__ __forceinline__ void store_out(const DecodeParams& p, const DecodeLay
 // out = sum_s acc_s 2^(m_s-M) / sum_s l_s 2^(m_s-M).  No CTA ever waits for another.
 // What it takes is two trips to L2, one for all (m, l) and one for the partials: a warp that went through its share of
 // the heads one after the other, both trips for each, made it 2.3 us with four heads and 5.1 us with eight.
-// weights: G * (ns + 1) floats of shared memory.
-template <int D>
-__device__ __forceinline__ void ticket_merge(const DecodeParams& p, const DecodeLayer& L, int ns, int hk, int b,
+// L, part_acc, part_ml: of the first of the CTA's NL layers; weights: NL * G * (ns + 1) floats of shared memory.
+template <int D, int NL>
+__device__ __forceinline__ void ticket_merge(const DecodeParams& p, const DecodeLayer* L, int ns, int hk, int b,
                                              const float* part_acc, const float* part_ml, unsigned* ticket, int* s_flag,
                                              float* weights) {
   const Dims& dm = p.dm;
@@ -293,12 +312,13 @@ __device__ __forceinline__ void ticket_merge(const DecodeParams& p, const Decode
   }
   __syncthreads();
   if (!*s_flag) return;
-  const size_t hq0 = (size_t)b * dm.Hq + hk * dm.G;
-  // weights[h][s] = 2^(m_s - M), weights[h][ns] = 1 / sum_s l_s 2^(m_s - M)
+  const size_t hq0 = (size_t)b * dm.Hq + hk * dm.G, layer_rows = (size_t)dm.B * dm.Hq;
+  auto row_of = [&](int v) { return NL == 1 || v < dm.G ? hq0 + v : layer_rows + hq0 + (v - dm.G); };  // head v of the CTA
+  // weights[v][s] = 2^(m_s - M), weights[v][ns] = 1 / sum_s l_s 2^(m_s - M)
 #pragma unroll 2
-  for (int h = warp; h < dm.G; h += n_warps) {
-    const float* ml = part_ml + (hq0 + h) * p.ns_q * 2;
-    float* w = weights + h * (ns + 1);
+  for (int v = warp; v < NL * dm.G; v += n_warps) {
+    const float* ml = part_ml + row_of(v) * p.ns_q * 2;
+    float* w = weights + v * (ns + 1);
     float M = -CUDART_INF_F, Ls = 0.f;
     if (ns <= 32) {
       const float2 x = lane < ns ? ld_cg2(ml + 2 * lane) : make_float2(-CUDART_INF_F, 0.f);
@@ -324,153 +344,170 @@ __device__ __forceinline__ void ticket_merge(const DecodeParams& p, const Decode
     if (lane == 0) w[ns] = 1.0f / Ls;
   }
   __syncthreads();
-  for (int item = threadIdx.x; item < dm.G * (D / 4); item += blockDim.x) {
-    const int h = item / (D / 4), c = item % (D / 4) * 4;
-    const float* pa = part_acc + (hq0 + h) * p.ns_q * D + c;
-    const float* w = weights + h * (ns + 1);
+  for (int item = threadIdx.x; item < NL * dm.G * (D / 4); item += blockDim.x) {
+    const int v = item / (D / 4), c = item % (D / 4) * 4;
+    const float* pa = part_acc + row_of(v) * p.ns_q * D + c;
+    const float* w = weights + v * (ns + 1);
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int s0 = 0; s0 < ns; s0 += 16) {
-      float4 v[16];
+      float4 x[16];
 #pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = s0 + i < ns ? ld_cg4(pa + (size_t)(s0 + i) * D) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int i = 0; i < 16; ++i) x[i] = s0 + i < ns ? ld_cg4(pa + (size_t)(s0 + i) * D) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
         const float f = s0 + i < ns ? w[s0 + i] : 0.f;
-        a.x = fmaf(v[i].x, f, a.x);
-        a.y = fmaf(v[i].y, f, a.y);
-        a.z = fmaf(v[i].z, f, a.z);
-        a.w = fmaf(v[i].w, f, a.w);
+        a.x = fmaf(x[i].x, f, a.x);
+        a.y = fmaf(x[i].y, f, a.y);
+        a.z = fmaf(x[i].z, f, a.z);
+        a.w = fmaf(x[i].w, f, a.w);
       }
     }
     const float inv = w[ns];
-    store_out<D>(p, L, hq0 + h, c, make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv));
+    const int l = NL == 1 || v < dm.G ? 0 : 1;
+    store_out<D>(p, L[l], hq0 + (v - l * dm.G), c, make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv));
   }
   if (threadIdx.x == 0) *ticket = 0u;  // ready for the next launch on this stream
 }
 
-template <int D, int BK, int BV, int GS, int HP, int NT>
-__global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<D, BK, BV, GS, HP, NT>::CTAS)
+template <int D, int BK, int BV, int GS, int HP, int NL>
+__global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<D, BK, BV, GS, HP, NL>::CTAS)
     decode_mma_kernel(const __grid_constant__ DecodeParams p) {
-  using Pl = Plan<D, BK, BV, GS, HP, NT>;
+  using Pl = Plan<D, BK, BV, GS, HP, NL>;
   using Cd = Code<D>;
+  constexpr bool WIDE = Pl::WIDE;
   constexpr int KS = Pl::KS, NG = Pl::NG, NGT = Pl::NGT, W = Pl::WARPS, WROW = Pl::WROW, GC = Pl::GC, CP = Pl::CP;
+  constexpr int VH = Pl::VH, SH = Pl::SH, NSET = Pl::NSET, NCOL = Pl::NCOL, NE = Pl::NE;
   constexpr int KWORDS = (BK == 2 && D == 128) ? 2 : 1;  // packed words of a token row that a thread expands
-  constexpr int VCH = BV;                               // 16-byte chunks of a channel row (128 / BV tokens each)
-  constexpr int VE = 8 / BV;                            // k-steps of a value chunk
+  constexpr int KBASE = 2, VBASE = BV == 2 ? 2 : 4;      // where the codes of an operand begin in its halves
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) unsigned long long bar_mem[2 * W];
-  __shared__ const uint8_t* src_sm[4];  // the CTA's packed data: key codes, key parameters, value codes, value parameters
+  // the CTA's packed data: key codes, value codes, and of each layer key parameters, value parameters
+  __shared__ const uint8_t* src_sm[2 + 2 * NL];
+  __shared__ __align__(16) int place_sm[8];  // what follows from the CTA's index
+  __shared__ int eq_sm[VH];
   __shared__ int s_flag;
+  __shared__ uint32_t tmem_base_sm;
   __shared__ volatile int dead_sm;
 
   const Dims& dm = p.dm;
-  const DecodeLayer& L = p.layer[blockIdx.y];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gid = lane >> 2, tig = lane & 3, low = gid & 1;
-  // operand column gid: head col_head, slot col_slot; accumulator columns 2 tig and 2 tig + 1: head my_head, slot my_slot
-  const int col_head = (gid >> 1) % HP, col_slot = (gid >> 1) / HP, my_head = tig % HP, my_slot = tig / HP;
+  const DecodeLayer* const LL = &p.layer[NL * blockIdx.y];
+  // (the shuffle tells the compiler that the warp's index, and all that follows from it, is the same in all lanes)
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int gid = lane >> 2, tig = lane & 3, low = gid & 1;
+  // head v of the CTA: head v % HP of layer v / HP.  Operand column gid: head col_head (WIDE: gid), slot col_slot;
+  // accumulator columns 2 tig and 2 tig + 1: head my_head, slot my_slot (WIDE: heads 2 tig, 2 tig + 1, of layer my_layer)
+  const int col_head = WIDE ? gid : (gid >> 1) % VH, col_slot = WIDE ? 0 : (gid >> 1) / VH;
+  const int my_head = WIDE ? 2 * tig : tig % VH, my_slot = WIDE ? 0 : tig / VH;
+  const int col_layer = NL == 1 ? 0 : col_head / HP, my_layer = NL == 1 ? 0 : my_head / HP;
   const int G = dm.G;
-
-  // The next kernel in the stream may be scheduled at once when all work before this kernel's own predecessor is
-  // known to be complete (a chained launch); otherwise only after this kernel's own wait (below), so that a chained
-  // successor never starts before the work this kernel waited for has completed.
-  if (p.late_wait) grid_dependents_go();
-
-  // CTA -> (stream, split), the splits of a stream side by side
-  const int ns = p.ns_q;
-  const unsigned stream = blockIdx.x / (unsigned)ns;
-  const int split = (int)(blockIdx.x - stream * (unsigned)ns);
-  const int hk = (int)(stream % (unsigned)dm.Hkv), b = (int)(stream / (unsigned)dm.Hkv);
-  const int bh = b * dm.Hkv + hk;
-  const int nbt = (p.n_q + BT - 1) / BT;  // batches of the stream (the last one may be ragged)
-  int b0, b1, wt0, wt1;
-  {
-    // the larger shares come last, with the run that may be short
-    const int runs = (nbt + p.deal - 1) / p.deal;
-    int lo, hi;
-    share_of(runs, ns, ns - 1 - split, lo, hi);
-    b0 = (runs - hi) * p.deal;
-    b1 = min((runs - lo) * p.deal, nbt);
-  }
-  share_of(p.r, ns, split, wt0, wt1);
-  const int nb = b1 - b0;
 
   const uint32_t sm_base = (uint32_t)__cvta_generic_to_shared(smem);
   const uint32_t st = sm_base + warp * Pl::WARP;                     // this warp's stage
-  const uint32_t pbuf = st + Pl::STAGE;
-  const uint32_t qb = sm_base + W * Pl::WARP, ones = qb + Pl::QB;
-  uint16_t* const q_sm = reinterpret_cast<uint16_t*>(smem + W * Pl::WARP + Pl::QB + Pl::ONES);  // zeros for absent heads
-  const uint32_t qf = ones + Pl::ONES + Pl::QS + lane * 8;  // this lane's fragments of q
+  const uint32_t pbuf = st + Pl::OFF_P;
+  const uint32_t qb = sm_base + W * Pl::WARP;
+  uint16_t* const q_sm = reinterpret_cast<uint16_t*>(smem + W * Pl::WARP + Pl::QB);  // zeros for absent heads
+  const uint32_t qf = qb + Pl::QB + Pl::QS + lane * 8;  // this lane's fragments of q
   const uint32_t bar_k = (uint32_t)__cvta_generic_to_shared(&bar_mem[0]) + 16 * warp, bar_v = bar_k + 8;
 
-  // Copies of batch j of this CTA's range into this warp's stage (one lane; the stage is free)
-  auto load_keys = [&](int j) {
-    const uint8_t *gk = src_sm[0] + (size_t)(unsigned)j * Pl::KC, *gm = src_sm[1] + (size_t)(unsigned)j * Pl::KM;
-    mbar_expect_tx(bar_k, Pl::KC + Pl::KM);
-    bulk_load(st, gk, Pl::KC, bar_k);
-    bulk_load(st + Pl::OFF_KM, gm, Pl::KM, bar_k);
-  };
-  auto load_values = [&](int j) {
-    const uint8_t *gv = src_sm[2] + (size_t)(unsigned)j * Pl::VC, *gm = src_sm[3] + (size_t)(unsigned)j * Pl::VM;
-    mbar_expect_tx(bar_v, Pl::VC + Pl::VM);
-    bulk_load(st + Pl::OFF_VC, gv, Pl::VC, bar_v);
-    bulk_load(st + Pl::OFF_VM, gm, Pl::VM, bar_v);
-  };
-
   if (tid == 0) {
+    // CTA -> (stream, split), the splits of a stream side by side
+    const unsigned stream = blockIdx.x / (unsigned)p.ns_q;
+    const int split = (int)(blockIdx.x - stream * (unsigned)p.ns_q);
+    const int bh = (int)stream, b = (int)(stream / (unsigned)dm.Hkv);
+    const int nbt = (p.n_q + BT - 1) / BT;  // batches of the stream (the last one may be ragged)
+    // the larger shares come last, with the run that may be short
+    const int runs = p.deal == 1 ? nbt : (nbt + p.deal - 1) / p.deal;
+    int lo, hi, wt0, wt1;
+    share_of(runs, p.ns_q, p.ns_q - 1 - split, lo, hi);
+    const int b0 = (runs - hi) * p.deal, b1 = min((runs - lo) * p.deal, nbt);
+    share_of(p.r, p.ns_q, split, wt0, wt1);
+    // half batches (the last half of the stream's last batch may be empty)
+    const int halves = b1 > b0 ? 2 * (b1 - b0) - (b1 == nbt && nbt * BT - p.n_q >= TT ? 1 : 0) : 0;
+    place_sm[0] = b0; place_sm[1] = halves; place_sm[2] = wt0; place_sm[3] = wt1;
+    place_sm[4] = b; place_sm[5] = bh - b * dm.Hkv; place_sm[6] = split;
     dead_sm = 0;
-    src_sm[0] = reinterpret_cast<const uint8_t*>(L.L.k_codes) + (size_t)bh * ((size_t)dm.nq_cap * (D * BK / 8)) + (size_t)b0 * Pl::KC;
-    src_sm[1] = reinterpret_cast<const uint8_t*>(L.L.k_meta) + (size_t)bh * ((size_t)(dm.nq_cap / GS) * (4 * D)) + (size_t)b0 * Pl::KM;
-    src_sm[2] = reinterpret_cast<const uint8_t*>(L.L.v_codes) + (size_t)bh * ((size_t)dm.nq_cap * (D * BV / 8)) + (size_t)b0 * Pl::VC;
-    src_sm[3] = reinterpret_cast<const uint8_t*>(L.L.v_meta) + (size_t)bh * ((size_t)dm.nq_cap * 4 * NG) + (size_t)b0 * Pl::VM;
+    src_sm[0] = reinterpret_cast<const uint8_t*>(LL[0].L.k_codes) + (size_t)bh * ((size_t)dm.nq_cap * (D * BK / 8)) + (size_t)b0 * (BT * D * BK / 8);
+    src_sm[1] = reinterpret_cast<const uint8_t*>(LL[0].L.v_codes) + (size_t)bh * ((size_t)dm.nq_cap * (D * BV / 8)) + (size_t)b0 * (BT * D * BV / 8);
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+      src_sm[2 + 2 * l] = reinterpret_cast<const uint8_t*>(LL[l].L.k_meta) + (size_t)bh * ((size_t)(dm.nq_cap / GS) * (4 * D)) + (size_t)b0 * (BT / GS * 4 * D);
+      src_sm[3 + 2 * l] = reinterpret_cast<const uint8_t*>(LL[l].L.v_meta) + (size_t)bh * ((size_t)dm.nq_cap * 4 * NG) + (size_t)b0 * (BT * 4 * NG);
+    }
   }
   if (lane == 0) {
-    mbar_init(bar_k, 1);
+    mbar_init(bar_k, 2);  // codes; scales and zero-points
     mbar_init(bar_v, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   __syncthreads();
+  const int4 place = *reinterpret_cast<const int4*>(place_sm), place2 = *reinterpret_cast<const int4*>(place_sm + 4);
+  const int ns = p.ns_q;
+  // uniform in a warp, as its index is
+  const int b0 = __shfl_sync(0xffffffffu, place.x, 0), halves = __shfl_sync(0xffffffffu, place.y, 0);
+  // the rounds of a warp are the half batches warp, warp + W, ... of the CTA's range
+  const int rounds = warp < halves ? (halves - 1 - warp) / W + 1 : 0;
+  static_assert(W % 2 == 0, "a warp's rounds are all first, or all second halves");
+
+  // Copies of round r into this warp's stage (one lane; the stage is free)
+  auto half_of = [&](int r) { return (unsigned)(warp + W * r); };
+  auto load_key_codes = [&](int r) {
+    mbar_expect_tx(bar_k, Pl::KCODES);
+    bulk_load(st, src_sm[0] + (size_t)half_of(r) * Pl::KCODES, Pl::KCODES, bar_k);
+  };
+  auto load_key_params = [&](int r) {
+    mbar_expect_tx(bar_k, NL * Pl::KM);
+#pragma unroll
+    for (int l = 0; l < NL; ++l) bulk_load(st + Pl::OFF_KM + l * Pl::KM, src_sm[2 + 2 * l] + (size_t)half_of(r) * Pl::KM, Pl::KM, bar_k);
+  };
+  auto load_values = [&](int r) {
+    mbar_expect_tx(bar_v, NL * Pl::VM + Pl::VCODES);
+    bulk_load(st + Pl::OFF_V, src_sm[1] + (size_t)(BV == 2 ? half_of(r) : half_of(r) >> 1) * Pl::VCODES, Pl::VCODES, bar_v);
+#pragma unroll
+    for (int l = 0; l < NL; ++l) bulk_load(st + Pl::OFF_VM + l * Pl::VROOM, src_sm[3 + 2 * l] + (size_t)half_of(r) * Pl::VM, Pl::VM, bar_v);
+  };
+
   if (lane == 0) {
     // Packed data that earlier calls completed may be fetched while the preceding kernel still runs; when a pack
     // kernel may have written it since this layer's last decode, the first copies wait for that kernel.
     if (!p.early_fetch) grid_dependency_wait();
-    if (warp < nb) {
-      load_keys(warp);
-      load_values(warp);
+    if (rounds > 0) {
+      load_key_codes(0);
+      load_key_params(0);
+      load_values(0);
     }
   }
   __syncwarp();
-  if (!p.late_wait) {
-    grid_dependency_wait();  // q may come from the preceding kernel
-    grid_dependents_go();    // whatever this kernel waited for is complete for its successor too
+  if (!p.late_wait) grid_dependency_wait();  // q may come from the preceding kernel
+  // Tensor memory is asked for after the wait (a chained launch: its predecessor, a launch of this kernel, waited, and
+  // the tensor memory of an SM serves all of their CTAs that fit it): a CTA of the preceding kernel that shares the SM may
+  // still have to get its own, and this CTA, which waits for it, would be in its way.  For the same reason the next kernel
+  // in the stream may be scheduled only from here on: whatever this kernel waited for is complete for it too.
+  if (warp == W - 1) {
+    tmem_alloc((uint32_t)__cvta_generic_to_shared(&tmem_base_sm), Pl::TMEM);
+    grid_dependents_go();
   }
 
-  // ---- q ----
-  for (int i = tid; i < HP * NT * D / 8; i += W * 32) {
-    const bool real = i / (D / 8) < G;
-    const uint4* src = reinterpret_cast<const uint4*>(L.q + ((size_t)b * dm.Hq + hk * G) * D);
-    reinterpret_cast<uint4*>(q_sm)[i] = real ? src[i] : make_uint4(0u, 0u, 0u, 0u);
+  // ---- q, and the exponents that put a head's largest |q| into [1, 2) ----
+  static_assert(VH * D / 8 <= W * 32, "a vector a thread");
+  if (tid < VH * D / 8) {
+    const int v = tid / (D / 8), layer = v / HP, h = v % HP;
+    uint4 x = make_uint4(0u, 0u, 0u, 0u);
+    if (h < G) x = reinterpret_cast<const uint4*>(LL[layer].q + ((size_t)place2.x * dm.Hq + place2.y * G + h) * D)[tid % (D / 8)];
+    reinterpret_cast<uint4*>(q_sm)[tid] = x;
+    const uint32_t sign = 0x7fff7fffu;  // both formats order like their bits without the sign
+    uint32_t mx = __vmaxu2(__vmaxu2(x.x & sign, x.y & sign), __vmaxu2(x.z & sign, x.w & sign));
+#pragma unroll
+    for (int k = 1; k < D / 8; k <<= 1) mx = __vmaxu2(mx, __shfl_xor_sync(VH * D / 8 >= 32 ? 0xffffffffu : (1u << (VH * D / 8 & 31)) - 1u, mx, k));
+    const float qmax = io_to_f(max(mx & 0xffffu, mx >> 16), p.f16);
+    if (tid % (D / 8) == 0) eq_sm[v] = qmax > 0.f ? max(-100, min(100, -exponent_of(qmax))) : 0;
   }
-  for (int i = tid; i < Pl::ONES / 4; i += W * 32) sts32(ones + 4 * i, 0x3C003C00u);
   __syncthreads();
-  // exponents that put a head's largest |q| into [1, 2): each warp finds those of all heads; lane h keeps head h's
-  int eq_lane = 0;
-#pragma unroll
-  for (int h = 0; h < HP * NT; ++h) {
-    float am = 0.f;
-#pragma unroll
-    for (int j = 0; j < D / 64; ++j) {
-      const uint32_t v = reinterpret_cast<const uint32_t*>(q_sm + h * D)[lane + 32 * j];
-      am = fmaxf(am, fmaxf(fabsf(io_to_f(v & 0xffffu, p.f16)), fabsf(io_to_f(v >> 16, p.f16))));
-    }
-    const float qmax = __uint_as_float(redux_max_u32(__float_as_uint(am)));
-    if (lane == h) eq_lane = qmax > 0.f ? max(-100, min(100, -exponent_of(qmax))) : 0;
-  }
   // B fragments of the zero-point products, for zero-points as they are stored (position pos holds channel
-  // (pos % (D / 32)) * 32 + pos / (D / 32)): rows = token groups; even columns take the first half of the positions,
-  // odd columns the second (whose zero-points sit in rows 4 and up).
-  for (int i = warp; i < NT * KS / 2; i += W) {
-    const int kp = i % (KS / 2), h = HP * (i / (KS / 2)) + col_head;
-    const float e2 = pow2i(__shfl_sync(0xffffffffu, eq_lane, h) + Q_BIAS_EXP);
+  // (pos % (D / 32)) * 32 + pos / (D / 32)), for a set of heads: rows = token groups; even columns take the first half
+  // of the positions, odd columns the second (whose zero-points sit in rows 4 and up).
+  for (int i = warp; i < NSET * KS / 2; i += W) {
+    const int kp = i % (KS / 2), h = SH * (i / (KS / 2)) + (gid >> 1) % SH;
+    const float e2 = pow2i(eq_sm[h] + Q_BIAS_EXP);
     float v[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
@@ -478,592 +515,748 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
       const int d = (pos % (D / 32)) * 32 + pos / (D / 32);
       v[c] = io_to_f(q_sm[h * D + d], p.f16) * e2;
     }
-    const __half2 h0 = __floats2half2_rn(v[0], v[1]), h1 = __floats2half2_rn(v[2], v[3]);
-    sts64(qb + (i * 32 + lane) * 8, *reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+    sts64(qb + ((i >> 1) * 32 + lane) * 16 + (i & 1) * 8, pack_io2<true>(v[0], v[1]), pack_io2<true>(v[2], v[3]));
   }
   if constexpr (Pl::Q_SHARED) {  // largest |q| in [2^14, 2^15); the key scales carry the rest of the exponent
-    for (int i = warp; i < NT * KS; i += W) {
-      const int ks = i % KS, h = HP * (i / KS) + col_head;
-      const float e2 = pow2i(__shfl_sync(0xffffffffu, eq_lane, h) + 14 - k_weight<D, BK>(ks));
-      const uint2 v = *reinterpret_cast<const uint2*>(q_sm + h * D + k_channel<D, BK>(ks, tig, 0));
-      sts64(qf + i * 256, pack_io2<true>(io_to_f(v.x & 0xffffu, p.f16) * e2, io_to_f(v.y & 0xffffu, p.f16) * e2),
+    for (int ks = warp; ks < KS; ks += W) {
+      const float e2 = pow2i(eq_sm[col_head] + 14 - k_weight<D, BK>(ks));
+      const uint2 v = *reinterpret_cast<const uint2*>(q_sm + col_head * D + k_channel<D, BK>(ks, tig, 0));
+      sts64(qf + ks * 256, pack_io2<true>(io_to_f(v.x & 0xffffu, p.f16) * e2, io_to_f(v.y & 0xffffu, p.f16) * e2),
             pack_io2<true>(io_to_f(v.x >> 16, p.f16) * e2, io_to_f(v.y >> 16, p.f16) * e2));
     }
   }
+  tc_fence_before();
   __syncthreads();
-  float cq[NT];
+  tc_fence_after();
+  float cq[NCOL];  // of the heads of this thread's columns; of the head whose zero-point products it adds up
 #pragma unroll
-  for (int n = 0; n < NT; ++n)
-    cq[n] = p.scale * 1.4426950408889634f * pow2i(-__shfl_sync(0xffffffffu, eq_lane, HP * n + my_head));
+  for (int j = 0; j < NCOL; ++j) cq[j] = p.scale * 1.4426950408889634f * pow2i(-eq_sm[my_head + j]);
+  const float cz = WIDE ? p.scale * 1.4426950408889634f * pow2i(-eq_sm[4 * (lane >> 4) + tig]) : cq[0];
 
   const uint32_t low_mask = low ? 0xffffffffu : 0u;
-  // q of this lane's operand column as fp16 pairs, times 2^Ek and divided by the weights of the codes
-  uint32_t qk[Pl::Q_SHARED ? 1 : NT][Pl::Q_SHARED ? 1 : KS][2];
-  int Ek = -100;  // not set; with Q_SHARED the scales are taken times 2^Ek instead
-  float ck[NT];
+  // q of this lane's operand column as fp16 pairs, times 2^Ek and divided by the weights of the codes (head_dim 64)
+  uint32_t qk[Pl::Q_SHARED ? 1 : KS][2];
+  int Ek = -100;  // not set
+  // With Q_SHARED the scales are taken times 2^Ek of their layer instead: ek2, a pair of fp16 (0: not set).
+  uint32_t ek2[NL];
+  float ck[NCOL];
+#pragma unroll
+  for (int j = 0; j < NCOL; ++j) ck[j] = 0.f;
+  auto set_unit = [&](int l, int e) {
+    const float unit = pow2i(Cd::exp(KBASE) - e);
+#pragma unroll
+    for (int j = 0; j < NCOL; ++j) ck[j] = NL == 1 || my_layer == l ? cq[j] * unit : ck[j];
+  };
   auto set_ek = [&](int e) {
     Ek = e;
+    set_unit(0, e);
+    const int eh = e + eq_sm[col_head];
 #pragma unroll
-    for (int n = 0; n < NT; ++n) {
-      if constexpr (Pl::Q_SHARED) {
-        ck[n] = cq[n] * pow2i(Cd::EXP - 14 - e);
-        continue;
-      }
-      const int h = HP * n + col_head;
-      const int eh = e + __shfl_sync(0xffffffffu, eq_lane, h);
-      const uint16_t* qh = q_sm + h * D;
-#pragma unroll
-      for (int ks = 0; ks < KS; ++ks) {
-        const float e2 = pow2i(eh - k_weight<D, BK>(ks));
-        const uint2 v = *reinterpret_cast<const uint2*>(qh + k_channel<D, BK>(ks, tig, 0));
-        const __half2 h0 = __floats2half2_rn(io_to_f(v.x & 0xffffu, p.f16) * e2, io_to_f(v.y & 0xffffu, p.f16) * e2);
-        const __half2 h1 = __floats2half2_rn(io_to_f(v.x >> 16, p.f16) * e2, io_to_f(v.y >> 16, p.f16) * e2);
-        qk[n][ks][0] = *reinterpret_cast<const uint32_t*>(&h0);
-        qk[n][ks][1] = *reinterpret_cast<const uint32_t*>(&h1);
-      }
-      ck[n] = cq[n] * pow2i(Cd::EXP - e);
+    for (int ks = 0; ks < (Pl::Q_SHARED ? 0 : KS); ++ks) {
+      const float e2 = pow2i(eh - k_weight<D, BK>(ks));
+      const uint2 v = *reinterpret_cast<const uint2*>(q_sm + col_head * D + k_channel<D, BK>(ks, tig, 0));
+      qk[ks][0] = pack_io2<true>(io_to_f(v.x & 0xffffu, p.f16) * e2, io_to_f(v.y & 0xffffu, p.f16) * e2);
+      qk[ks][1] = pack_io2<true>(io_to_f(v.x >> 16, p.f16) * e2, io_to_f(v.y >> 16, p.f16) * e2);
     }
   };
+  auto q_pair = [&](int ks) {
+    if constexpr (Pl::Q_SHARED) return lds64(qf + ks * 256);
+    else return make_uint2(qk[ks][0], qk[ks][1]);
+  };
 
-  // softmax state: reference m (log2 units, an integer; -infinity before the first batch, where mr is 0 instead).
-  // Row gid of zacc: the zero-point products of channel group gid (gid < NG), the sum of the numerators (gid >= NG;
-  // with centered codes lsum, of this thread's tokens).
-  float m[NT], mr[NT], acc[NT][KS][4], zacc[NT][4], lsum[NT];
-  int Ev = -100;  // value scales are taken times 2^Ev
+  // Softmax state of the heads of this thread's columns: reference mr (log2 units, an integer; 0 until the first round
+  // sets it).  Value sums, in tensor memory between the rounds: of row tile mt the products' four (WIDE: of hi, then of
+  // lo).  zacc[part]: rows gid: the zero-point products of layer gid / 4, channel group gid % 4 (one layer: gid % NG), rows
+  // 8 and up: the sum of the numerators (with centered codes lsum, of this thread's tokens); columns hi and lo (WIDE:
+  // columns heads, hi and lo apart).
+  const uint32_t t_acc = tmem_base_sm + ((uint32_t)(warp & 3) << 21) + (warp >> 2) * Pl::TCOLS;
+  constexpr int MT = GC * KS / CP;                          // row tiles of a channel part of the value products
+  constexpr int MTS = MT < 2 ? MT : 2, TV = MTS * 4 * NCOL;  // that are taken at a time; their columns
+  float mr[NCOL], zacc[NCOL][4], lsum[NCOL];
+  uint32_t ev2[NL];  // value scales are taken times 2^Ev: a pair of fp16 (0: not set)
 #pragma unroll
-  for (int n = 0; n < NT; ++n) {
-    m[n] = -CUDART_INF_F;
-    mr[n] = 0.f;
-    lsum[n] = 0.f;
+  for (int l = 0; l < NL; ++l) ek2[l] = ev2[l] = 0u;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      zacc[n][i] = 0.f;
+  for (int j = 0; j < NCOL; ++j) {
+    mr[j] = 0.f;
+    lsum[j] = 0.f;
 #pragma unroll
-      for (int mt = 0; mt < KS; ++mt) acc[n][mt][i] = 0.f;
-    }
+    for (int i = 0; i < 4; ++i) zacc[j][i] = 0.f;
   }
-  // weights of this lane's tokens in the value words (row gid of row tile mt is pair q = gid + 8 mt of 32 tokens)
-  const int wt_a = BV == 1 ? gid >> 1 : 2 * ((gid >> 1) & 3), wt_b = BV == 1 ? wt_a + 4 : wt_a;
-  const float off[2] = {(float)(P_EXP - wt_a), (float)(P_EXP - wt_b)};
-  const float weight_a = pow2i(wt_a), weight_b = pow2i(wt_b);
-  const int tok0 = 4 * (gid >> 1) + (gid & 1);                       // token of row gid, tile 0; the other rows: + 2, + 16
-  const uint32_t kc_lane = st + tok0 * (BK == 1 && D == 64 ? 8 : 16) + (BK == 1 && D == 64 ? (tig >> 1) : tig) * 4;
-  const uint32_t vs_lane = st + Pl::OFF_VM + pair_row(BV == 1 ? 16 * tig : 8 * tig) * Pl::VSROW;  // first pair of the lane's word
-  // zero-points of channel group gid, or ones (row NG and up: the sum of the numerators)
-  const uint32_t vz_lane = gid < NG || Cd::CENTERED ? vs_lane + Pl::VS + 4 * (gid % NG) : ones;
-  const uint32_t p_st = pbuf + my_head * Pl::PH + my_slot * 144 + gid * 8;  // + pair offset
-  const uint32_t p_ld = pbuf + col_head * Pl::PH + tig * (BV == 1 ? 144 : 64) + (BV == 2 ? (tig >> 1) * 16 : 0);
-
-  int last_k = 0, last_v = 0;  // number of the copy that each barrier was armed for last
+  // all value sums of columns j times f[j] (rare)
+  auto scale_sums = [&](const float (&f)[NCOL]) {
+    tc_wait_st();
 #pragma unroll 1
-  for (int i = warp, it = 0; i < nb; i += W, ++it) {
-    const int valid = min(BT, p.n_q - (b0 + i) * BT);  // < BT only in the stream's last batch
-    if (!__all_sync(0xffffffffu, mbar_wait(bar_k, it & 1, &dead_sm))) break;
-
-    // ---- keys: scales into the order of the operand slots (in place), the largest of them ----
-    {
-      constexpr int V = D / 32;
-      uint32_t s[NGT][V / 2], mx = 0u;
+    for (int c = 0; c < Pl::TCOLS; c += 8) {
+      uint32_t a[8];
+      tmem_ld<8>(t_acc + c, a);
+      tc_wait_ld();
 #pragma unroll
-      for (int g = 0; g < NGT; ++g) {
-        const uint32_t a = st + Pl::OFF_KM + g * 4 * D + lane * 2 * V;
-        if constexpr (V == 4) {
-          const uint2 x = lds64(a);
-          s[g][0] = x.x; s[g][1] = x.y;
-        } else {
-          s[g][0] = lds32(a);
-        }
+      for (int i = 0; i < 8; ++i) a[i] = __float_as_uint(__uint_as_float(a[i]) * f[WIDE ? i & 1 : 0]);
+      tmem_st<8>(t_acc + c, a);
+    }
+    tc_wait_st();
+  };
+  {
+    uint32_t zero[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) zero[i] = 0u;
+#pragma unroll
+    for (int c = 0; c < Pl::TCOLS; c += 8) tmem_st<8>(t_acc + c, zero);
+  }
+  const unsigned layer0 = NL == 2 ? __ballot_sync(0xffffffffu, my_layer == 0) : 0xffffffffu;
+  const unsigned my_lanes = my_layer == 0 ? layer0 : ~layer0;  // lanes with heads of this thread's layer
+  // weight of the codes of this lane's tokens in the value words (the token of row gid is in quad (gid >> 1) of its tile)
+  const int wt = BV == 1 ? gid >> 1 : 2 * (gid >> 1);
+  const float off = (float)(P_EXP - wt), weight = pow2i(wt);
+  const int tok0 = 4 * (gid >> 1) + (gid & 1);                       // token of row gid, tile 0; the other rows: + 2, + 16
+  const uint32_t kz_lane = st + Pl::OFF_KM + (gid & (NGT - 1)) * 4 * D + 2 * D + (gid >> 2) * D + tig * 16;  // zero-points of its row
+  const uint32_t qb_lane = qb + lane * 16;
+  const uint32_t kc_lane = st + tok0 * (BK == 1 && D == 64 ? 8 : 16) + (BK == 1 && D == 64 ? (tig >> 1) : tig) * 4;
+  const uint32_t km_read = st + Pl::OFF_KM + lane * (D / 16), km_write = st + Pl::OFF_KM + 2 * k_slot<D, BK>(lane);
+  const uint32_t km_lane = st + Pl::OFF_KM + (NL == 2 ? col_layer * Pl::KM : 0) + tig * 16;
+  // Lane column tig owns the tokens 16 tig ... of a round in the value products: in 2 bits word tig of a channel's chunk,
+  // in 1 bit a half of word tig / 2 (of the two that this half of the batch has), shifted so that its codes begin at bit
+  // VBASE.
+  const uint32_t vc_lane = st + Pl::OFF_V + gid * 16 + (BV == 2 ? tig : 2 * (warp & 1) + (tig >> 1)) * 4;
+  const int shift_up = BV == 2 ? 2 : (tig & 1 ? 0 : 4), shift_down = BV == 2 ? 6 : (tig & 1 ? 8 : 4);
+  const uint32_t vm_read = st + Pl::OFF_VM + (4 * (lane >> 1) + (lane & 1)) * (4 * NG), vm_write = st + Pl::OFF_VM + 4 * lane;
+  const uint32_t vs_lane = st + Pl::OFF_VM + (NL == 2 ? col_layer * Pl::VROOM : 0) + tig * 32;  // the scales of its pairs
+  const uint32_t vz_lane = st + Pl::OFF_VM + (NL == 2 ? (gid >> 2) * Pl::VROOM : 0) + Pl::VZ + (NL == 2 ? (gid & 3) % NG : gid % NG) * Pl::VZROW + tig * 32;
+  // Numerators.  WIDE: 16-byte cells (two pairs of tokens) of head v, tile s, quad k in the tile: 128 bytes for each
+  // (v >> 1, k), in it the cell of (s, v & 1), exclusive-or'ed with (v >> 1, k & 1), so that the cells which a warp reads
+  // or writes together fall into different banks.
+  const uint32_t p_st = WIDE ? pbuf + ((tig * 4 + (gid >> 1)) << 7) + ((tig << 1 | ((gid >> 1) & 1)) << 4) + (gid & 1) * 8
+                             : pbuf + my_head * Pl::PH + gid * 8;
+  const uint32_t p_ld = WIDE ? pbuf + ((gid >> 1) << 9) + ((((tig << 1) | (gid & 1)) ^ ((gid >> 1) << 1)) << 4)
+                             : pbuf + col_head * Pl::PH + tig * Pl::PT;
+  // row tile of 16 tokens (of the round's four) of this thread's logits x[n]
+  auto tile_of = [&](int n) { return GC == 1 ? n : (GC == 2 ? 2 * my_slot + n : 2 * (my_slot & 1) + (my_slot >> 1)); };
+
+  int last_k = 0, last_v = 0;  // rounds whose key codes, values were copied last
+#pragma unroll 1
+  for (int r = 0; r < rounds; ++r) {
+    const int valid = min(TT, p.n_q - b0 * BT - (warp + W * r) * TT);  // < TT only in the stream's last round
+    if (!__all_sync(0xffffffffu, mbar_wait(bar_k, r & 1, &dead_sm))) break;
+
+    if (valid < TT) {  // what no token has reached may be anything: no scale, no zero-point
+      for (int i = lane; i < NL * NGT * D; i += 32) {
+        const int l = i / (NGT * D), g = i / D % NGT;
+        if (g * GS >= valid) sts32(st + Pl::OFF_KM + l * Pl::KM + g * 4 * D + 4 * (i % D), 0u);
       }
-      if (valid < BT) {
+      __syncwarp();
+    }
+    // ---- keys: scales into the order of the operand slots (in place), times 2^Ek ----
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+      constexpr int V = D / 32;
+      uint32_t s[NGT][V / 2];
+      auto read = [&]() {
+#pragma unroll
+        for (int g = 0; g < NGT; ++g) {
+          if constexpr (V == 4) {
+            const uint2 x = lds64(km_read + l * Pl::KM + g * 4 * D);
+            s[g][0] = x.x; s[g][1] = x.y;
+          } else {
+            s[g][0] = lds32(km_read + l * Pl::KM + g * 4 * D);
+          }
+        }
+      };
+      auto scale = [&]() {
 #pragma unroll
         for (int g = 0; g < NGT; ++g)
 #pragma unroll
-          for (int j = 0; j < V / 2; ++j) s[g][j] = g * GS < valid ? s[g][j] : 0u;
+          for (int j = 0; j < V / 2; ++j) s[g][j] = hmul2(s[g][j], ek2[l]);
+      };
+      auto largest = [&]() {  // the bits of an fp16
+        uint32_t mx = 0u;
+#pragma unroll
+        for (int g = 0; g < NGT; ++g)
+#pragma unroll
+          for (int j = 0; j < V / 2; ++j) mx = __vmaxu2(mx, s[g][j]);
+        return redux_max_u32(max(mx & 0xffffu, mx >> 16));
+      };
+      read();
+      if constexpr (Pl::Q_SHARED) {
+        // The largest scale of the round times 2^Ek in [2^-4, 1): |q s| below 2^15, and a scale keeps its 11 bits down to
+        // 2^-10 of the largest.  Ek moves only outside that, and no further than 15.
+        scale();
+        if (largest() - 0x2c00u >= 0x1000u) {
+          read();
+          const float smax = f16_to_f(largest());
+          const int es = smax > 0.f ? exponent_of(smax) : -24, e = min(15, -1 - es);
+          const float f = pow2i(e);
+          ek2[l] = pack_io2<true>(f, f);
+          set_unit(l, 14 + e);
+          scale();
+        }
+      } else {
+        // |q s| below 2^15 and its largest at least 2^8 (where 2^14 |q| allows): exponents of q move only outside that
+        const float smax = f16_to_f(largest());
+        const int es = smax > 0.f ? exponent_of(smax) : -24;
+        if (es > 13 - Ek || (es < 7 - Ek && Ek < 14) || Ek == -100) set_ek(min(14, 13 - es));
       }
-#pragma unroll
-      for (int g = 0; g < NGT; ++g)
-#pragma unroll
-        for (int j = 0; j < V / 2; ++j) mx = __vmaxu2(mx, s[g][j]);
       if constexpr (Cd::CENTERED) {
 #pragma unroll
         for (int g = 0; g < NGT; ++g) {
-          const uint32_t a = st + Pl::OFF_KM + g * 4 * D + 2 * D + lane * 4;
+          const uint32_t a = km_read + g * 4 * D + 2 * D;
           uint32_t hi, lo;
           centered_zero<D, BK>(s[g][0], lds32(a), hi, lo);
           sts32(a, hi);
           sts32(st + Pl::OFF_KL + g * 2 * D + lane * 4, lo);
         }
       }
-      // |q s| below 2^15 and its largest at least 2^8 (where 2^14 |q| allows): exponents of q move only outside that
-      const float smax = f16_to_f(redux_max_u32(max(mx & 0xffffu, mx >> 16)));
-      const int es = smax > 0.f ? exponent_of(smax) : -24;
-      if constexpr (Pl::Q_SHARED) {
-        // |q s| below 2^15; a scale keeps its 11 bits down to 2^-10 of the largest
-        if (es > -1 - Ek || (es < -4 - Ek && Ek < 15) || Ek == -100) set_ek(min(15, -1 - es));
-        const float ek = pow2i(Ek);
-        const __half2 ek2 = __floats2half2_rn(ek, ek);
-#pragma unroll
-        for (int g = 0; g < NGT; ++g)
-#pragma unroll
-          for (int j = 0; j < V / 2; ++j) s[g][j] = hmul2(s[g][j], *reinterpret_cast<const uint32_t*>(&ek2));
-      } else {
-        if (es > 13 - Ek || (es < 7 - Ek && Ek < 14) || Ek == -100) set_ek(min(14, 13 - es));
-      }
       __syncwarp();
 #pragma unroll
-      for (int j = 0; j < V; ++j) {
-        const uint32_t dst = st + Pl::OFF_KM + 2 * k_slot<D, BK>(lane + 32 * j);
+      for (int g = 0; g < NGT; ++g)
 #pragma unroll
-        for (int g = 0; g < NGT; ++g) sts16(dst + g * 4 * D, j & 1 ? s[g][j / 2] >> 16 : s[g][j / 2]);
-      }
-      __syncwarp();
+        for (int j = 0; j < V; ++j)
+          sts16(km_write + l * Pl::KM + g * 4 * D + 2 * k_slot_step<D, BK>(j), j & 1 ? s[g][j / 2] >> 16 : s[g][j / 2]);
     }
-    // Units of 32 tokens: this thread's logits are those of units GC * ux + my_slot, ux = 0 .. HP - 1, of its head:
-    // [row gid, gid + 8 of the unit's first tile, of its second]; less the reference and with the exponents `off`.
-    float x[NT][HP][4];
-    // ---- zero-points: sum_d q_d z_d per token group and head (rows: groups, first and second half of the channels) ----
+    __syncwarp();
+    // Logits x[n][r][j] of row gid + 8 r (tokens 2 r further) of tile tile_of(n), head my_head + j; less the reference and
+    // with the exponent `off`.
+    float x[NE][2][NCOL];
+    float zb;  // zero-points: sum_d q_d z_d, lane 16 * set + 4 * group + head of the set
     {
-      const uint32_t za = st + Pl::OFF_KM + (gid & (NGT - 1)) * 4 * D + 2 * D + (gid >> 2) * D + tig * 16;
-      const uint32_t zl = st + Pl::OFF_KL + (gid & (NGT - 1)) * 2 * D + (gid >> 2) * D + tig * 16;
-      float zc[NT][4];
+      // Rows: groups, first and second half of the channels.  A vector of zero-points is an operand as it is: rows gid get
+      // its first and third words, rows gid + 8 its second and fourth; the products with their q, of rows gid in zc, of
+      // rows gid + 8 in zd (the rest of both is of no use).
+      float zc[2][4], zd[2][4];
 #pragma unroll
-      for (int n = 0; n < NT; ++n)
+      for (int n = 0; n < 2; ++n)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) zc[n][k] = 0.f;
+        for (int k = 0; k < 4; ++k) zc[n][k] = zd[n][k] = 0.f;
 #pragma unroll
-      for (int kp = 0; kp < KS / 4; ++kp) {
-        const uint4 a = lds128(za + kp * 64);
+      for (int n = 0; n < (WIDE ? NSET : NL); ++n) {
+        const int l = NL == 2 ? n : 0, set = WIDE ? n : 0;
+        const uint32_t za = kz_lane + l * Pl::KM, zl = st + Pl::OFF_KL + (gid & (NGT - 1)) * 2 * D + (gid >> 2) * D + tig * 16;
 #pragma unroll
-        for (int n = 0; n < NT; ++n) {
-          const uint2 q0 = lds64(qb + ((n * KS / 2 + 2 * kp) * 32 + lane) * 8), q1 = lds64(qb + ((n * KS / 2 + 2 * kp + 1) * 32 + lane) * 8);
+        for (int kp = 0; kp < KS / 4; ++kp) {
+          const uint4 a = lds128(za + kp * 64);
+          const uint4 q = lds128(qb_lane + (set * KS / 4 + kp) * 512);
           if constexpr (Cd::CENTERED) {
-            const uint4 l = lds128(zl + kp * 64);
-            mma_f16(zc[n], l.x, l.x, l.y, l.y, q0.x, q0.y);
-            mma_f16(zc[n], l.z, l.z, l.w, l.w, q1.x, q1.y);
+            const uint4 c = lds128(zl + kp * 64);
+            mma_f16(zc[n], c.x, c.y, c.z, c.w, q.x, q.z);
+            mma_f16(zd[n], c.x, c.y, c.z, c.w, q.y, q.w);
           }
-          mma_f16(zc[n], a.x, a.x, a.y, a.y, q0.x, q0.y);  // (rows 8 and up: the same again)
-          mma_f16(zc[n], a.z, a.z, a.w, a.w, q1.x, q1.y);
+          mma_f16(zc[n], a.x, a.y, a.z, a.w, q.x, q.z);
+          mma_f16(zd[n], a.x, a.y, a.z, a.w, q.y, q.w);
         }
       }
-#pragma unroll
-      for (int n = 0; n < NT; ++n) {
-        const float zb = (zc[n][0] + __shfl_xor_sync(0xffffffffu, zc[n][1], 16)) * (cq[n] * (1.f / (float)(1 << Q_BIAS_EXP)));
-#pragma unroll
-        for (int ux = 0; ux < HP; ++ux)
-          x[n][ux][0] = __shfl_sync(0xffffffffu, zb, ((GC * ux + my_slot) * 32 / GS) * 4 + tig) - mr[n];
+      auto row = [&](int n, int col) { return zc[n][col] + zd[n][2 + col]; };
+      if constexpr (WIDE) {  // lanes 0 .. 15 add up the first set, the others the second
+        const float v = __shfl_xor_sync(0xffffffffu, lane < 16 ? row(1, 0) : row(0, 1), 16);
+        zb = (lane < 16 ? row(0, 0) : row(1, 1)) + v;
+      } else {
+        const float z0 = NL == 2 && my_layer == 1 ? row(1, 0) : row(0, 0), z1 = NL == 2 && my_layer == 1 ? row(1, 1) : row(0, 1);
+        zb = z0 + __shfl_xor_sync(0xffffffffu, z1, 16);
       }
+      zb *= cz * (1.f / (float)(1 << Q_BIAS_EXP));
     }
     // ---- keys: q . c ----
-    // packed words of rows gid, gid + 8: even bytes, odd bytes
+    // packed words of rows gid, gid + 8 of both tiles of unit u (32 tokens): even bytes, odd bytes
     auto load_rows = [&](int u, int kw, uint32_t (&w)[2][2], uint32_t (&w8)[2][2]) {
 #pragma unroll
       for (int t = 0; t < 2; ++t)
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          const int tk = 16 * t + 2 * r;
+        for (int h = 0; h < 2; ++h) {
+          const int tk = 16 * t + 2 * h;
           uint32_t raw;
           if constexpr (BK == 1 && D == 64) raw = lds32(kc_lane + u * 256 + tk * 8) >> (4 * (tig & 1));
           else raw = lds32(kc_lane + u * (32 * D * BK / 8) + kw * 512 + tk * 16);
-          w[t][r] = even_bytes_up(raw);
-          w8[t][r] = odd_bytes_up(raw);
+          w[t][h] = byte_pair_up(raw, 2);
+          w8[t][h] = byte_pair_down(raw, 6);
         }
     };
-    auto key_pair = [](uint32_t w, int k) { return Cd::template pair<BK>(w, BK == 2 ? k & 3 : k); };
+    auto key_pair = [](uint32_t w, int k) { return Cd::template pair<BK, KBASE>(w, BK == 2 ? k & 3 : k); };
     constexpr int KPW = KS / KWORDS;  // k-steps a word serves
-    if constexpr (GC == 1) {
-      constexpr int UG = GS / 32;  // units of a group
-      // fma(q, s, qn * s) is hi where qn = 0 and lo where qn = -q
-      uint32_t qn[KS][2];
-      if constexpr (!Pl::Q_SHARED && NT == 1) {
+    if constexpr (WIDE) {
 #pragma unroll
-        for (int ks = 0; ks < KS; ++ks) {
-          qn[ks][0] = (qk[0][ks][0] ^ 0x80008000u) & low_mask;
-          qn[ks][1] = (qk[0][ks][1] ^ 0x80008000u) & low_mask;
-        }
-      }
-#pragma unroll
-      for (int g = 0; g < NGT; ++g) {
-        float c[NT][2 * UG][4];
+      for (int u = 0; u < 2; ++u) {
+        float chi[2][4], clo[2][4];
 #pragma unroll
         for (int kw = 0; kw < KWORDS; ++kw) {
-          uint32_t w[UG][2][2], w8[UG][2][2];
-#pragma unroll
-          for (int u = 0; u < UG; ++u) load_rows(g * UG + u, kw, w[u], w8[u]);
-          const uint32_t sa = st + Pl::OFF_KM + g * 4 * D + tig * 16 + kw * (KPW / 2) * 64;
+          uint32_t w[2][2], w8[2][2];
+          load_rows(u, kw, w, w8);
+          const uint32_t sa = km_lane + u * 32 / GS * 4 * D + kw * (KPW / 2) * 64;
           uint4 sv;
 #pragma unroll
           for (int k = 0; k < KPW; ++k) {
             if ((k & 1) == 0) sv = lds128(sa + (k / 2) * 64);
             const uint32_t s0 = k & 1 ? sv.z : sv.x, s1 = k & 1 ? sv.w : sv.y;
             const int ks = kw * KPW + k;
+            const uint2 q = q_pair(ks);
+            const uint32_t h0 = hmul2(q.x, s0), h1 = hmul2(q.y, s1), l0 = product_rest(q.x, s0, h0), l1 = product_rest(q.y, s1, h1);
 #pragma unroll
-            for (int n = 0; n < NT; ++n) {
-              uint32_t p0, p1;
-              if constexpr (Pl::Q_SHARED) {
-                const uint2 q = lds64(qf + (n * KS + ks) * 256);
-                p0 = product_part(q.x, s0, low);
-                p1 = product_part(q.y, s1, low);
-              } else if constexpr (NT == 1) {
-                p0 = hfma2(qk[n][ks][0], s0, hmul2(qn[ks][0], s0));
-                p1 = hfma2(qk[n][ks][1], s1, hmul2(qn[ks][1], s1));
+            for (int t = 0; t < 2; ++t) {
+              const uint32_t a0 = key_pair(w[t][0], k), a1 = key_pair(w[t][1], k);
+              const uint32_t a2 = key_pair(w8[t][0], k), a3 = key_pair(w8[t][1], k);
+              if (ks == 0) {
+                mma_f16_first(chi[t], a0, a1, a2, a3, h0, h1);
+                mma_f16_first(clo[t], a0, a1, a2, a3, l0, l1);
               } else {
-                p0 = product_part(qk[n][ks][0], s0, low);
-                p1 = product_part(qk[n][ks][1], s1, low);
+                mma_f16(chi[t], a0, a1, a2, a3, h0, h1);
+                mma_f16(clo[t], a0, a1, a2, a3, l0, l1);
               }
-#pragma unroll
-              for (int u = 0; u < UG; ++u)
-#pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                  const uint32_t a0 = key_pair(w[u][t][0], k), a1 = key_pair(w[u][t][1], k);
-                  const uint32_t a2 = key_pair(w8[u][t][0], k), a3 = key_pair(w8[u][t][1], k);
-                  if (ks == 0) mma_f16_first(c[n][2 * u + t], a0, a1, a2, a3, p0, p1);
-                  else mma_f16(c[n][2 * u + t], a0, a1, a2, a3, p0, p1);
-                }
             }
           }
         }
 #pragma unroll
-        for (int n = 0; n < NT; ++n)
+        for (int j = 0; j < NCOL; ++j) {
+          const int g = u * 32 / GS;
+          const float bias = (__shfl_sync(0xffffffffu, zb, 16 * (tig >> 1) + 4 * g + 2 * (tig & 1) + j) - mr[j]) + off;
 #pragma unroll
-          for (int u = 0; u < UG; ++u) {
-            float* xu = x[n][g * UG + u];
-            const float bias[2] = {xu[0] + off[0], xu[0] + off[1]};
+          for (int t = 0; t < 2; ++t)
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-              xu[k] = fmaf(c[n][2 * u + k / 2][2 * (k & 1)] + c[n][2 * u + k / 2][2 * (k & 1) + 1], ck[n], bias[k >> 1]);
-          }
-      }
-    } else {
-      // one operand for GC units, each in its own column slot; a unit's logits are in the threads of its slot
-#pragma unroll
-      for (int ux = 0; ux < HP; ++ux) {
-        uint32_t pp[KS][2];
-        const uint32_t sa = st + Pl::OFF_KM + ((GC * ux + col_slot) * 32 / GS) * 4 * D + tig * 16;
-#pragma unroll
-        for (int kp = 0; kp < KS / 2; ++kp) {
-          const uint4 sv = lds128(sa + kp * 64);
-          pp[2 * kp][0] = product_part(qk[0][2 * kp][0], sv.x, low);
-          pp[2 * kp][1] = product_part(qk[0][2 * kp][1], sv.y, low);
-          pp[2 * kp + 1][0] = product_part(qk[0][2 * kp + 1][0], sv.z, low);
-          pp[2 * kp + 1][1] = product_part(qk[0][2 * kp + 1][1], sv.w, low);
+            for (int h = 0; h < 2; ++h) x[2 * u + t][h][j] = fmaf(chi[t][2 * h + j] + clo[t][2 * h + j], ck[j], bias);
         }
-        const float bias[2] = {x[0][ux][0] + off[0], x[0][ux][0] + off[1]};
+      }
+    } else if constexpr (GC == 1) {
+      constexpr int UG = GS / 32;  // units of a group
 #pragma unroll
-        for (int j = 0; j < GC; ++j) {
-          float c[2][4];
+      for (int g = 0; g < NGT; ++g) {
+        float c[2 * UG][4];
 #pragma unroll
-          for (int kw = 0; kw < KWORDS; ++kw) {
-            uint32_t w[2][2], w8[2][2];
-            load_rows(GC * ux + j, kw, w, w8);
+        for (int kw = 0; kw < KWORDS; ++kw) {
+          uint32_t w[UG][2][2], w8[UG][2][2];
 #pragma unroll
-            for (int k = 0; k < KPW; ++k)
+          for (int u = 0; u < UG; ++u) load_rows(g * UG + u, kw, w[u], w8[u]);
+          const uint32_t sa = km_lane + g * 4 * D + kw * (KPW / 2) * 64;
+          uint4 sv;
+#pragma unroll
+          for (int k = 0; k < KPW; ++k) {
+            if ((k & 1) == 0) sv = lds128(sa + (k / 2) * 64);
+            const uint32_t s0 = k & 1 ? sv.z : sv.x, s1 = k & 1 ? sv.w : sv.y;
+            const int ks = kw * KPW + k;
+            const uint2 q = q_pair(ks);
+            const uint32_t p0 = product_part(q.x, s0, low), p1 = product_part(q.y, s1, low);
+#pragma unroll
+            for (int u = 0; u < UG; ++u)
 #pragma unroll
               for (int t = 0; t < 2; ++t) {
-                const uint32_t a0 = key_pair(w[t][0], k), a1 = key_pair(w[t][1], k);
-                const uint32_t a2 = key_pair(w8[t][0], k), a3 = key_pair(w8[t][1], k);
-                if (kw + k == 0) mma_f16_first(c[t], a0, a1, a2, a3, pp[0][0], pp[0][1]);
-                else mma_f16(c[t], a0, a1, a2, a3, pp[kw * KPW + k][0], pp[kw * KPW + k][1]);
+                const uint32_t a0 = key_pair(w[u][t][0], k), a1 = key_pair(w[u][t][1], k);
+                const uint32_t a2 = key_pair(w8[u][t][0], k), a3 = key_pair(w8[u][t][1], k);
+                if (ks == 0) mma_f16_first(c[2 * u + t], a0, a1, a2, a3, p0, p1);
+                else mma_f16(c[2 * u + t], a0, a1, a2, a3, p0, p1);
               }
           }
+        }
+        const float bias = (__shfl_sync(0xffffffffu, zb, 4 * g + tig) - mr[0]) + off;
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float v = fmaf(c[k / 2][2 * (k & 1)] + c[k / 2][2 * (k & 1) + 1], ck[0], bias[k >> 1]);
-            x[0][ux][k] = j == 0 || my_slot == j ? v : x[0][ux][k];
+        for (int n = 0; n < 2 * UG; ++n)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) x[2 * g * UG + n][h][0] = fmaf(c[n][2 * h] + c[n][2 * h + 1], ck[0], bias);
+      }
+    } else {
+      // one operand for both units, each in its own column slot (four slots: twice); a unit's logits are in the threads
+      // of its slot (four slots: those of a tile)
+      uint32_t pp[KS][2];
+      const uint32_t sa = km_lane + ((col_slot & 1) * 32 / GS) * 4 * D;
+#pragma unroll
+      for (int kp = 0; kp < KS / 2; ++kp) {
+        const uint4 sv = lds128(sa + kp * 64);
+        const uint2 q0 = q_pair(2 * kp), q1 = q_pair(2 * kp + 1);
+        pp[2 * kp][0] = product_part(q0.x, sv.x, low);
+        pp[2 * kp][1] = product_part(q0.y, sv.y, low);
+        pp[2 * kp + 1][0] = product_part(q1.x, sv.z, low);
+        pp[2 * kp + 1][1] = product_part(q1.y, sv.w, low);
+      }
+      const float bias = (__shfl_sync(0xffffffffu, zb, 4 * ((my_slot & 1) * 32 / GS) + tig) - mr[0]) + off;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        float c[2][4];
+#pragma unroll
+        for (int kw = 0; kw < KWORDS; ++kw) {
+          uint32_t w[2][2], w8[2][2];
+          load_rows(u, kw, w, w8);
+#pragma unroll
+          for (int k = 0; k < KPW; ++k)
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+              const uint32_t a0 = key_pair(w[t][0], k), a1 = key_pair(w[t][1], k);
+              const uint32_t a2 = key_pair(w8[t][0], k), a3 = key_pair(w8[t][1], k);
+              if (kw + k == 0) mma_f16_first(c[t], a0, a1, a2, a3, pp[0][0], pp[0][1]);
+              else mma_f16(c[t], a0, a1, a2, a3, pp[kw * KPW + k][0], pp[kw * KPW + k][1]);
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if constexpr (GC == 2) {
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+              const float v = fmaf(c[t][2 * h] + c[t][2 * h + 1], ck[0], bias);
+              x[t][h][0] = u == 0 || my_slot == 1 ? v : x[t][h][0];
+            }
+          } else {
+            const float v = fmaf(my_slot < 2 ? c[0][2 * h] + c[0][2 * h + 1] : c[1][2 * h] + c[1][2 * h + 1], ck[0], bias);
+            x[0][h][0] = u == 0 || (my_slot & 1) == 1 ? v : x[0][h][0];
           }
         }
       }
     }
-    // the key half of the stage is free: fetch the keys of this warp's next batch
+    // the key half of the stage is free: fetch the keys of this warp's next round
     proxy_fence();
     __syncwarp();
-    if (i + W < nb) {
-      if (lane == 0) load_keys(i + W);
-      last_k = it + 1;
+    if (r + 1 < rounds) {
+      if (lane == 0) {
+        load_key_codes(r + 1);
+        if (!Pl::P_OVER) load_key_params(r + 1);
+      }
+      last_k = r + 1;
     }
 
-    if (valid < BT) {
+    if (valid < TT) {
+      __syncwarp();  // (a branch, and not a selection that every round would execute)
 #pragma unroll
-      for (int ux = 0; ux < HP; ++ux)
+      for (int n = 0; n < NE; ++n)
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (32 * (GC * ux + my_slot) + tok0 + 16 * (k >> 1) + 2 * (k & 1) >= valid) {
+        for (int h = 0; h < 2; ++h)
+          if (16 * tile_of(n) + tok0 + 2 * h >= valid) {
 #pragma unroll
-            for (int n = 0; n < NT; ++n) x[n][ux][k] = -CUDART_INF_F;
+            for (int j = 0; j < NCOL; ++j) x[n][h][j] = -CUDART_INF_F;
           }
     }
-    // ---- softmax: raise the reference when a logit exceeds it by more than TAU (rare) ----
-    float xm[NT];
+    // ---- softmax: raise the references of a layer when a logit exceeds one by more than TAU (rare) ----
+    float xm[NCOL];
     bool need = false;
 #pragma unroll
-    for (int n = 0; n < NT; ++n) {
-      float v[2];
+    for (int j = 0; j < NCOL; ++j) {
+      xm[j] = fmaxf(x[0][0][j], x[0][1][j]);
 #pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        v[t] = fmaxf(x[n][0][2 * t], x[n][0][2 * t + 1]);
-#pragma unroll
-        for (int ux = 1; ux < HP; ++ux) v[t] = fmaxf(fmaxf(v[t], x[n][ux][2 * t]), x[n][ux][2 * t + 1]);
-      }
-      xm[n] = fmaxf(v[0] - off[0], v[1] - off[1]);  // above the reference
-      need |= xm[n] > (m[n] == mr[n] ? TAU : -CUDART_INF_F);
+      for (int n = 1; n < NE; ++n) xm[j] = fmaxf(fmaxf(xm[j], x[n][0][j]), x[n][1][j]);
+      xm[j] -= off;  // above the reference
+      need |= xm[j] > TAU;
     }
-    if (__any_sync(0xffffffffu, need)) {
+    const unsigned needed = __ballot_sync(0xffffffffu, need || r == 0);
+    if (needed != 0u) {
+      float f[NCOL];
 #pragma unroll
-      for (int n = 0; n < NT; ++n) {
-        float v = xm[n];
+      for (int j = 0; j < NCOL; ++j) {
+        float v = xm[j];
 #pragma unroll
-        for (int k = HP; k < 32; k <<= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, k));
-        const float up = m[n] != mr[n] || v > TAU - 1.f ? ceilf(v) : 0.f;
-        const float f = m[n] != mr[n] ? 0.f : ex2(-up);  // (nothing has been accumulated yet)
-        m[n] = mr[n] = mr[n] + up;
+        for (int k = WIDE ? 4 : VH; k < 32; k <<= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, k));
+        const float up = (needed & my_lanes) != 0u && (r == 0 || v > TAU - 1.f) ? ceilf(v) : 0.f;
+        f[j] = ex2(-up);
+        mr[j] += up;
 #pragma unroll
-        for (int ux = 0; ux < HP; ++ux)
-#pragma unroll
-          for (int k = 0; k < 4; ++k) x[n][ux][k] -= up;
-        lsum[n] *= f;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          zacc[n][k] *= f;
-#pragma unroll
-          for (int mt = 0; mt < KS; ++mt) acc[n][mt][k] *= f;
+        for (int n = 0; n < NE; ++n) {
+          x[n][0][j] -= up;
+          x[n][1][j] -= up;
         }
+      }
+      if (r > 0) {  // (else nothing has been accumulated yet)
+#pragma unroll
+        for (int j = 0; j < NCOL; ++j) {
+          lsum[j] *= f[j];
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if constexpr (WIDE) zacc[k & 1][2 * (k >> 1) + j] *= f[j];
+            else zacc[0][k] *= f[j];
+        }
+        scale_sums(f);
       }
     }
     // numerators times 2^P_EXP and divided by the weight of the token's value code, as hi + lo pairs (t, t + 2)
 #pragma unroll
-    for (int n = 0; n < NT; ++n) {
+    for (int j = 0; j < NCOL; ++j)
 #pragma unroll
-      for (int ux = 0; ux < HP; ++ux)
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-          const float pa = ex2(x[n][ux][2 * t]), pb = ex2(x[n][ux][2 * t + 1]);
-          if constexpr (Cd::CENTERED) lsum[n] = fmaf(pa + pb, t ? weight_b : weight_a, lsum[n]);
-          const uint32_t h = pack_io2<true>(pa, pb);
-          const uint32_t lo = pack_io2<true>(pa - io2_lo<true>(h), pb - io2_hi<true>(h));
-          sts64(p_st + n * HP * Pl::PH + ux * GC * 144 + t * 64, h, lo);
-        }
-    }
+      for (int n = 0; n < NE; ++n) {
+        const float pa = ex2(x[n][0][j]), pb = ex2(x[n][1][j]);
+        if constexpr (Cd::CENTERED) lsum[j] = fmaf(pa + pb, weight, lsum[j]);
+        const uint32_t h = pack_io2<true>(pa, pb);
+        const uint32_t lo = pack_io2<true>(pa - io2_lo<true>(h), pb - io2_hi<true>(h));
+        if constexpr (WIDE) sts64(p_st ^ ((n << 1 | j) << 4), h, lo);
+        else sts64(p_st + tile_of(n) * Pl::PT, h, lo);
+      }
 
     // ---- values: scales and zero-points as pairs of tokens (t, t + 2), in place ----
-    if (!__all_sync(0xffffffffu, mbar_wait(bar_v, it & 1, &dead_sm))) break;
-    {
-      uint32_t sp[2][NG], zp[2][NG], mx = 0u;
-      const uint32_t vm = st + Pl::OFF_VM;
+    if (!__all_sync(0xffffffffu, mbar_wait(bar_v, r & 1, &dead_sm))) break;
+    if (valid < TT) {
+      for (int i = lane; i < NL * TT * NG; i += 32)
+        if (i / NG % TT >= valid) sts32(st + Pl::OFF_VM + i / (TT * NG) * Pl::VROOM + i % (TT * NG) * 4, 0u);
+      __syncwarp();
+    }
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int pr = lane + 32 * h, ta = 4 * (pr >> 1) + (pr & 1);
-        uint32_t ra[NG], rb[NG];  // raw rows of the two tokens: NG scales, NG zero-points
-        if constexpr (NG == 4) {
-          const uint4 a = lds128(vm + ta * 16), c = lds128(vm + ta * 16 + 32);
-          ra[0] = a.x; ra[1] = a.y; ra[2] = a.z; ra[3] = a.w;
-          rb[0] = c.x; rb[1] = c.y; rb[2] = c.z; rb[3] = c.w;
-        } else if constexpr (NG == 2) {
-          const uint2 a = lds64(vm + ta * 8), c = lds64(vm + ta * 8 + 16);
-          ra[0] = a.x; ra[1] = a.y; rb[0] = c.x; rb[1] = c.y;
-        } else {
-          ra[0] = lds32(vm + ta * 4); rb[0] = lds32(vm + ta * 4 + 8);
-        }
-        if (valid < BT) {
-#pragma unroll
-          for (int g = 0; g < NG; ++g) {
-            if (ta >= valid) ra[g] = 0u;
-            if (ta + 2 >= valid) rb[g] = 0u;
-          }
-        }
+    for (int l = 0; l < NL; ++l) {
+      uint32_t sp[NG], zp[NG];
+      {  // raw rows of the two tokens: NG scales, NG zero-points
+        const uint32_t a = vm_read + l * Pl::VROOM;
         if constexpr (NG == 1) {
-          sp[h][0] = __byte_perm(ra[0], rb[0], 0x5410);
-          zp[h][0] = __byte_perm(ra[0], rb[0], 0x7632);
+          const uint32_t ra = lds32(a), rb = lds32(a + 8);
+          sp[0] = __byte_perm(ra, rb, 0x5410);
+          zp[0] = __byte_perm(ra, rb, 0x7632);
         } else {
+          uint32_t ra[NG], rb[NG];
+          if constexpr (NG == 4) {
+            const uint4 x4 = lds128(a), y4 = lds128(a + 32);
+            ra[0] = x4.x; ra[1] = x4.y; ra[2] = x4.z; ra[3] = x4.w;
+            rb[0] = y4.x; rb[1] = y4.y; rb[2] = y4.z; rb[3] = y4.w;
+          } else {
+            const uint2 x2 = lds64(a), y2 = lds64(a + 16);
+            ra[0] = x2.x; ra[1] = x2.y; rb[0] = y2.x; rb[1] = y2.y;
+          }
 #pragma unroll
           for (int g = 0; g < NG; ++g) {
             const uint32_t sel = g & 1 ? 0x7632 : 0x5410;
-            sp[h][g] = __byte_perm(ra[g / 2], rb[g / 2], sel);
-            zp[h][g] = __byte_perm(ra[NG / 2 + g / 2], rb[NG / 2 + g / 2], sel);
+            sp[g] = __byte_perm(ra[g / 2], rb[g / 2], sel);
+            zp[g] = __byte_perm(ra[NG / 2 + g / 2], rb[NG / 2 + g / 2], sel);
           }
         }
-#pragma unroll
-        for (int g = 0; g < NG; ++g) mx = __vmaxu2(mx, sp[h][g]);
       }
-      // the largest scale times 2^Ev in [2^-6, 1): the exponent moves only outside that
-      const float smax = f16_to_f(redux_max_u32(max(mx & 0xffffu, mx >> 16)));
-      const int es = smax > 0.f ? exponent_of(smax) : -24;
-      if (es >= -Ev || (es < -6 - Ev && Ev < 15) || Ev == -100) {
-        const int e = min(15, -1 - es);
-        const float f = Ev == -100 ? 0.f : pow2i(e - Ev);
-        Ev = e;
+      uint32_t se[NG];
+      auto scale = [&]() {
 #pragma unroll
-        for (int n = 0; n < NT; ++n)
+        for (int g = 0; g < NG; ++g) se[g] = hmul2(sp[g], ev2[l]);
+      };
+      auto largest = [&](const uint32_t (&v)[NG]) {  // the bits of an fp16
+        uint32_t mx = 0u;
 #pragma unroll
-          for (int mt = 0; mt < KS; ++mt)
+        for (int g = 0; g < NG; ++g) mx = __vmaxu2(mx, v[g]);
+        return redux_max_u32(max(mx & 0xffffu, mx >> 16));
+      };
+      scale();
+      // the largest scale times 2^Ev in [2^-6, 1): the exponent moves only outside that, and no further than 15
+      if (largest(se) - 0x2400u >= 0x1800u) {
+        const float smax = f16_to_f(largest(sp));
+        const int es = smax > 0.f ? exponent_of(smax) : -24, e = min(15, -1 - es), before = exponent_of(f16_to_f(ev2[l] & 0xffffu));
+        float f[NCOL];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) acc[n][mt][k] *= f;
+        for (int j = 0; j < NCOL; ++j) f[j] = NL == 2 && my_layer != l ? 1.f : pow2i(e - before);
+        if (r > 0) scale_sums(f);
+        const float ev = pow2i(e);
+        ev2[l] = pack_io2<true>(ev, ev);
+        scale();
       }
-      const float ev = pow2i(Ev);
-      const __half2 ev2 = __floats2half2_rn(ev, ev);
-      const uint32_t e2 = *reinterpret_cast<const uint32_t*>(&ev2);
       __syncwarp();
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const uint32_t dst = vm + pair_row(32 * h) * Pl::VSROW + pair_row(lane) * Pl::VSROW;
+      for (int g = 0; g < NG; ++g) {
         if constexpr (Cd::CENTERED) {
-#pragma unroll
-          for (int g = 0; g < NG; ++g) {
-            uint32_t lo;
-            centered_zero<D, BV>(sp[h][g], zp[h][g], zp[h][g], lo);
-            sts32(dst + 2 * Pl::VS + 4 * g, lo);
-          }
+          uint32_t lo;
+          centered_zero<D, BV>(sp[g], zp[g], zp[g], lo);
+          sts32(vm_write + Pl::VL + g * Pl::VZROW, lo);
         }
-        if constexpr (NG == 4) {
-          sts128(dst, hmul2(sp[h][0], e2), hmul2(sp[h][1], e2), hmul2(sp[h][2], e2), hmul2(sp[h][3], e2));
-          sts128(dst + Pl::VS, zp[h][0], zp[h][1], zp[h][2], zp[h][3]);
-        } else if constexpr (NG == 2) {
-          sts64(dst, hmul2(sp[h][0], e2), hmul2(sp[h][1], e2));
-          sts64(dst + Pl::VS, zp[h][0], zp[h][1]);
-        } else {
-          sts32(dst, hmul2(sp[h][0], e2));
-          sts32(dst + Pl::VS, zp[h][0]);
-        }
+        sts32(vm_write + l * Pl::VROOM + g * (TT / 2 * 4), se[g]);
+        sts32(vm_write + l * Pl::VROOM + Pl::VZ + g * Pl::VZROW, zp[g]);
       }
-      __syncwarp();
     }
-    // ---- values: one chunk of packed words at a time (lane column tig owns word tig of every channel row) ----
+    __syncwarp();
+    // ---- values: the numerators of this lane's column, zero-point products ----
+    // of the two pairs (t, t + 2), (t + 1, t + 3) of a quad of tokens e: hi, and what the lo operand needs
+    uint32_t ph[4][2], pn[4][2], pl[4][2];
 #pragma unroll
-    for (int c = 0; c < VCH; ++c) {
-      uint32_t w[KS][2], w8[KS][2];  // even and odd bytes of rows (channels) 16 mt + gid, + 8
-      const uint32_t va = st + Pl::OFF_VC + c * D * 16 + gid * 16 + tig * 4;
-#pragma unroll
-      for (int mt = 0; mt < KS; ++mt) {
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          const uint32_t raw = lds32(va + mt * 256 + r * 128);
-          w[mt][r] = even_bytes_up(raw);
-          w8[mt][r] = odd_bytes_up(raw);
+    for (int e = 0; e < 4; ++e) {
+      constexpr uint32_t STEP = BV == 2 ? 0x0800u : 0x0400u;
+      const uint32_t we = (0x3C00u + e * STEP) * 0x10001u;  // the weight of this step's codes as a pair of fp16
+      uint4 hp;
+      if constexpr (WIDE) hp = lds128((p_ld ^ ((e & 1) << 4)) + (e << 7));
+      else hp = lds128(p_ld + e * 16);
+      const uint32_t zo = vz_lane + e * 8;
+      const uint2 z = lds64(zo);
+      ph[e][0] = hp.x; ph[e][1] = hp.z;
+      if constexpr (WIDE) {
+        pl[e][0] = hp.y; pl[e][1] = hp.w;
+        const uint32_t h0 = hmul2(hp.x, we), h1 = hmul2(hp.z, we), l0 = hmul2(hp.y, we), l1 = hmul2(hp.w, we);
+        if constexpr (Cd::CENTERED) {
+          const uint2 y = lds64(zo + Pl::VL - Pl::VZ);
+          mma_f16(zacc[0], y.x, 0u, y.y, 0u, h0, h1);
+          mma_f16(zacc[1], y.x, 0u, y.y, 0u, l0, l1);
         }
+        mma_f16(zacc[0], z.x, ONES, z.y, ONES, h0, h1);
+        mma_f16(zacc[1], z.x, ONES, z.y, ONES, l0, l1);
+      } else {
+        // fma(l, s, fma(h, s, hn * s)): hi where hn = l = 0, lo where hn = -h
+        pn[e][0] = (hp.x ^ 0x80008000u) & low_mask; pn[e][1] = (hp.z ^ 0x80008000u) & low_mask;
+        pl[e][0] = hp.y & low_mask; pl[e][1] = hp.w & low_mask;
+        const uint32_t pz0 = hmul2(low ? hp.y : hp.x, we), pz1 = hmul2(low ? hp.w : hp.z, we);
+        if constexpr (Cd::CENTERED) {
+          const uint2 y = lds64(zo + Pl::VL - Pl::VZ);
+          mma_f16(zacc[0], y.x, 0u, y.y, 0u, pz0, pz1);
+        }
+        mma_f16(zacc[0], z.x, ONES, z.y, ONES, pz0, pz1);
       }
+    }
+    // ---- values: p . c, one channel part after the other ----
+    auto value_pair = [](uint32_t w, int e) { return Cd::template pair<BV, VBASE>(w, e); };
+    tc_wait_st();
 #pragma unroll
-      for (int e = 0; e < VE; ++e) {
-        constexpr int VB = CP / GC;  // operands of a step: parts GC * vb + slot
-        uint32_t sp[2][VB];
-        const uint32_t sa = vs_lane + pair_row(32 * c) * Pl::VSROW + 2 * e * Pl::VSROW, sb = sa + Pl::VSROW;
-        if constexpr (GC == 1 && NG == 4) {
-          const uint4 a = lds128(sa), d = lds128(sb);
-          sp[0][0] = a.x; sp[0][1] = a.y; sp[0][2] = a.z; sp[0][3] = a.w;
-          sp[1][0] = d.x; sp[1][1] = d.y; sp[1][2] = d.z; sp[1][3] = d.w;
-        } else {
+    for (int vb = 0; vb < CP / GC; ++vb) {
+      uint32_t sums[TV];
+      tmem_ld<TV>(t_acc + vb * (MT * 4 * NCOL), sums);
+      const uint32_t sa = vs_lane + (GC * vb + col_slot) * NG / CP * (TT / 2 * 4);
+      const uint4 s01 = lds128(sa), s23 = lds128(sa + 16);
+      const uint32_t sc[4][2] = {{s01.x, s01.y}, {s01.z, s01.w}, {s23.x, s23.y}, {s23.z, s23.w}};
+      uint32_t ps[4][2], pr[4][2];  // p s: hi (not WIDE: hi or lo, by column), lo
 #pragma unroll
-          for (int vb = 0; vb < VB; ++vb) {
-            const uint32_t o = ((GC * vb + col_slot) * NG / CP) * 4;
-            sp[0][vb] = lds32(sa + o);
-            sp[1][vb] = lds32(sb + o);
+      for (int e = 0; e < 4; ++e)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const uint32_t s = sc[e][k];
+          if constexpr (WIDE) {
+            ps[e][k] = hmul2(ph[e][k], s);
+            pr[e][k] = hfma2(pl[e][k], s, product_rest(ph[e][k], s, ps[e][k]));
+          } else {
+            ps[e][k] = hfma2(pl[e][k], s, hfma2(ph[e][k], s, hmul2(pn[e][k], s)));
           }
         }
-        const uint32_t zo = vz_lane + pair_row(32 * c) * Pl::VSROW + 2 * e * Pl::VSROW;
-        const uint32_t z0 = lds32(zo), z1 = lds32(zo + Pl::VSROW);
-        constexpr uint32_t ONE = 0x3C00u, STEP = BV == 2 ? 0x0800u : 0x0400u;
-        const uint32_t we = (ONE + e * STEP) * 0x10001u;  // the weight of this step's codes as a pair of fp16
 #pragma unroll
-        for (int n = 0; n < NT; ++n) {
-          const uint4 hp = lds128(p_ld + n * HP * Pl::PH + c * 288 + e * 16);  // (hi, lo) of pairs 2 e and 2 e + 1
-          const uint32_t pz0 = hmul2(low ? hp.y : hp.x, we), pz1 = hmul2(low ? hp.w : hp.z, we);
-          if constexpr (Cd::CENTERED) {
-            const uint32_t y0 = lds32(zo + Pl::VS), y1 = lds32(zo + Pl::VS + Pl::VSROW);
-            mma_f16(zacc[n], y0, y0, y1, y1, pz0, pz1);
+      for (int m0 = vb * MT; m0 < (vb + 1) * MT; m0 += MTS) {
+        if (m0 > vb * MT) tmem_ld<TV>(t_acc + m0 * (4 * NCOL), sums);
+        uint32_t w[MTS][2], w8[MTS][2];  // even and odd bytes of rows (channels) 16 mt + gid, + 8
+#pragma unroll
+        for (int i = 0; i < MTS; ++i)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const uint32_t raw = lds32(vc_lane + (m0 + i) * 256 + h * 128);
+            w[i][h] = byte_pair_up(raw, shift_up);
+            w8[i][h] = byte_pair_down(raw, shift_down);
           }
-          mma_f16(zacc[n], z0, z0, z1, z1, pz0, pz1);
-          // fma(l, s, fma(h, s, hn * s)): hi where hn = l = 0, lo where hn = -h
-          const uint32_t hn0 = (hp.x ^ 0x80008000u) & low_mask, hn1 = (hp.z ^ 0x80008000u) & low_mask;
-          const uint32_t l0 = hp.y & low_mask, l1 = hp.w & low_mask;
+        tc_wait_ld();
+        float acc[MTS * NCOL][4];
 #pragma unroll
-          for (int vb = 0; vb < VB; ++vb) {
-            const uint32_t p0 = hfma2(l0, sp[0][vb], hfma2(hp.x, sp[0][vb], hmul2(hn0, sp[0][vb])));
-            const uint32_t p1 = hfma2(l1, sp[1][vb], hfma2(hp.z, sp[1][vb], hmul2(hn1, sp[1][vb])));
-            constexpr int MT = GC * KS / CP;
+        for (int i = 0; i < TV; ++i) acc[i / 4][i % 4] = __uint_as_float(sums[i]);
 #pragma unroll
-            for (int mt = vb * MT; mt < (vb + 1) * MT; ++mt)
-              mma_f16(acc[n][mt], Cd::template pair<BV>(w[mt][0], e), Cd::template pair<BV>(w[mt][1], e),
-                      Cd::template pair<BV>(w8[mt][0], e), Cd::template pair<BV>(w8[mt][1], e), p0, p1);
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+          for (int i = 0; i < MTS; ++i) {
+            const uint32_t a0 = value_pair(w[i][0], e), a1 = value_pair(w[i][1], e), a2 = value_pair(w8[i][0], e), a3 = value_pair(w8[i][1], e);
+            mma_f16(acc[NCOL * i], a0, a1, a2, a3, ps[e][0], ps[e][1]);
+            if constexpr (WIDE) mma_f16(acc[NCOL * i + 1], a0, a1, a2, a3, pr[e][0], pr[e][1]);
           }
-        }
+#pragma unroll
+        for (int i = 0; i < TV; ++i) sums[i] = __float_as_uint(acc[i / 4][i % 4]);
+        tmem_st<TV>(t_acc + m0 * (4 * NCOL), sums);
       }
     }
     // the value half of the stage and the numerators are free
     proxy_fence();
     __syncwarp();
-    if (i + W < nb) {
-      if (lane == 0) load_values(i + W);
-      last_v = it + 1;
+    if (r + 1 < rounds) {
+      if (lane == 0) {
+        if (Pl::P_OVER) load_key_params(r + 1);
+        load_values(r + 1);
+      }
+      last_v = r + 1;
     }
   }
 
-  // ---- this warp's result so far in true units: channels 16 mt + gid, + 8 of head HP n + my_head ----
-  float o[NT][KS][2], l[NT];
-#pragma unroll
-  for (int n = 0; n < NT; ++n) {
-    const float ua = pow2i(Cd::EXP - P_EXP - Ev), uz = pow2i(-P_EXP);
-    const float z = (zacc[n][0] + zacc[n][1]) * uz;  // row gid < NG: channel group gid; row NG: the sum
-    if constexpr (Cd::CENTERED) {
-#pragma unroll
-      for (int k = HP; k < 32; k <<= 1) lsum[n] += __shfl_xor_sync(0xffffffffu, lsum[n], k);
-      l[n] = lsum[n] * uz;
-    } else {
-      l[n] = __shfl_sync(0xffffffffu, z, NG * 4 + tig);
-    }
-#pragma unroll
-    for (int mt = 0; mt < KS; ++mt) {
-      const float zg = __shfl_sync(0xffffffffu, z, (mt * 16 / GS) * 4 + tig);
-      float s0 = acc[n][mt][0] + acc[n][mt][1], s1 = acc[n][mt][2] + acc[n][mt][3];
-      if constexpr (GC > 1) {  // the threads of the tile's slot hold it
-        const int src = (lane & ~3) + (mt / (KS / CP)) % GC * HP + my_head;
-        s0 = __shfl_sync(0xffffffffu, s0, src);
-        s1 = __shfl_sync(0xffffffffu, s1, src);
-      }
-      o[n][mt][0] = fmaf(s0, ua, zg);
-      o[n][mt][1] = fmaf(s1, ua, zg);
-    }
-  }
-  // ---- the CTA's share of the 16-bit window, tile by tile, first to the warps with the fewest batches ----
+  // ---- state rows, over the stage: acc, m, l of each head from the packed tokens, then from the window ----
+  const int wt0 = place.z, wt1 = place.w, hk = place2.y, b = place2.x, split = place2.z, bh = b * dm.Hkv + hk;
+  // The CTA's share of the 16-bit window goes tile by tile to its warps, first to those with the fewest rounds.
+  const int wtiles = (wt1 - wt0 + 15) / 16;
+  auto window_turn = [&](int w) { const int t = w - halves % W; return t < 0 ? t + W : t; };
   if (dead_sm == 0) {  // (else a wait gave up somewhere: copies may be in flight, the stage is not reused)
-    int t = warp - nb % W;
-    if (t < 0) t += W;
-    for (int tb = wt0 + 16 * t; tb < wt1; tb += 16 * W) {
-      window_stage<D, WROW>(p, L, tb, wt1, bh, st, lane);
-      cp_async_commit();
-      cp_async_wait_all();
-      __syncwarp();
-      if (L.K_new != nullptr && tb + 16 > p.r - 1 && wt1 == p.r) window_store_new<D, WROW>(p, L, tb, bh, st, lane);
+    float* const ws = reinterpret_cast<float*>(smem + warp * Pl::WARP);
+    if (window_turn(warp) < wtiles) {
       const float scale2 = p.scale * 1.4426950408889634f;
+      float o[NSET][KS][2], l[NSET], ms[NSET];  // channels 16 mt + gid, + 8 of head SH * s + tig % SH
 #pragma unroll
-      for (int n = 0; n < NT; ++n) {
-        const int h = HP * n + col_head;
-        const bool real = low == 0 && col_slot == 0 && h < G;
-        const uint16_t* qrow = q_sm + h * D;
-        if (p.f16) window_tile<D, WROW, true>(st, wt1 - tb, qrow, real, scale2, o[n], m[n], l[n], lane);
-        else window_tile<D, WROW, false>(st, wt1 - tb, qrow, real, scale2, o[n], m[n], l[n], lane);
+      for (int s = 0; s < NSET; ++s) {
+        ms[s] = -CUDART_INF_F;
+        l[s] = 0.f;
+#pragma unroll
+        for (int mt = 0; mt < KS; ++mt) o[s][mt][0] = o[s][mt][1] = 0.f;
       }
-      __syncwarp();
+#pragma unroll 1
+      for (int layer = 0; layer < NL; ++layer) {
+        const DecodeLayer& L = LL[layer];
+#pragma unroll 1
+        for (int tb = wt0 + 16 * window_turn(warp); tb < wt1; tb += 16 * W) {
+          window_stage<D, WROW>(p, L, tb, wt1, bh, st, lane);
+          cp_async_commit();
+          cp_async_wait_all();
+          __syncwarp();
+          if (L.K_new != nullptr && tb + 16 > p.r - 1 && wt1 == p.r) window_store_new<D, WROW>(p, L, tb, bh, st, lane);
+#pragma unroll
+          for (int s = 0; s < NSET; ++s) {
+            if (WIDE && NL == 2 && s != layer) continue;
+            const int v = SH * s + (gid >> 1) % SH;  // head of operand column gid
+            const bool real = low == 0 && (gid >> 1) / SH == 0 && v % HP < G && v / HP == layer;
+            const uint16_t* qrow = q_sm + v * D;
+            // layers that share a set: only the threads of this layer's heads take the result
+            const bool mine = WIDE || NL == 1 || my_layer == layer;
+            float o2[KS][2], m2 = ms[s], l2 = l[s];
+#pragma unroll
+            for (int mt = 0; mt < KS; ++mt) o2[mt][0] = o[s][mt][0], o2[mt][1] = o[s][mt][1];
+            if (p.f16) window_tile<D, WROW, true>(st, wt1 - tb, qrow, real, scale2, o2, m2, l2, lane);
+            else window_tile<D, WROW, false>(st, wt1 - tb, qrow, real, scale2, o2, m2, l2, lane);
+            if (mine) {
+              ms[s] = m2;
+              l[s] = l2;
+#pragma unroll
+              for (int mt = 0; mt < KS; ++mt) o[s][mt][0] = o2[mt][0], o[s][mt][1] = o2[mt][1];
+            }
+          }
+          __syncwarp();
+        }
+      }
+#pragma unroll
+      for (int s = 0; s < NSET; ++s) {
+        float* const row = ws + (VH + SH * s + tig % SH) * Pl::MS;
+        if (tig / SH == 0) {
+#pragma unroll
+          for (int mt = 0; mt < KS; ++mt) {
+            row[16 * mt + gid] = o[s][mt][0];
+            row[16 * mt + gid + 8] = o[s][mt][1];
+          }
+          if (gid == 0) {
+            row[D] = ms[s];
+            row[D + 1] = l[s];
+          }
+        }
+      }
     }
     __syncwarp();
-    float* ws = reinterpret_cast<float*>(smem + warp * Pl::WARP);  // state rows, over the stage
+    // the packed tokens, in true units
+    const float uz = pow2i(-P_EXP);
+    const float ua = pow2i(Cd::exp(VBASE) - P_EXP - exponent_of(f16_to_f((NL == 2 && my_layer == 1 ? ev2[NL - 1] : ev2[0]) & 0xffffu)));
+    float z[NCOL];  // row gid < 4 NL: channel group of a layer
+    tc_wait_st();
 #pragma unroll
-    for (int n = 0; n < NT; ++n) {
-      const int h = HP * n + my_head;
-      if (h < G && my_slot == 0) {
+    for (int j = 0; j < NCOL; ++j) {
+      z[j] = (WIDE ? zacc[0][j] + zacc[1 % NCOL][j] : zacc[0][0] + zacc[0][1]) * uz;
+      float sum = (WIDE ? zacc[0][2 + j] + zacc[1 % NCOL][2 + j] : zacc[0][2] + zacc[0][3]) * uz;
+      if constexpr (Cd::CENTERED) {
 #pragma unroll
-        for (int mt = 0; mt < KS; ++mt) {
-          ws[h * Pl::MS + 16 * mt + gid] = o[n][mt][0];
-          ws[h * Pl::MS + 16 * mt + gid + 8] = o[n][mt][1];
-        }
-        if (gid == 0) {
-          ws[h * Pl::MS + D] = m[n];
-          ws[h * Pl::MS + D + 1] = l[n];
-        }
+        for (int k = WIDE ? 4 : VH; k < 32; k <<= 1) lsum[j] += __shfl_xor_sync(0xffffffffu, lsum[j], k);
+        sum = lsum[j] * uz;
+      }
+      if (gid == 0 && my_slot == 0) {
+        ws[(my_head + j) * Pl::MS + D] = rounds > 0 ? mr[j] : -CUDART_INF_F;
+        ws[(my_head + j) * Pl::MS + D + 1] = sum;
       }
     }
+    float zg[NG][NCOL];  // of this thread's heads
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+#pragma unroll
+      for (int j = 0; j < NCOL; ++j) zg[g][j] = __shfl_sync(0xffffffffu, z[j], (4 * my_layer + g) * 4 + tig);
+#pragma unroll
+    for (int mt = 0; mt < KS; mt += 2 / NCOL) {
+      uint32_t a[8];  // WIDE: hi and lo sums of a row tile; else the sums of two
+      tmem_ld<8>(t_acc + mt * 4 * NCOL, a);
+      tc_wait_ld();
+      auto sum_of = [&](int i, int k) { return __uint_as_float(a[i]) + __uint_as_float(a[k]); };
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {  // WIDE: columns; else row tiles, which the threads of the tile's slot hold
+          const int tile = WIDE ? mt : mt + t;
+          const float v = WIDE ? sum_of(2 * h + t, 4 + 2 * h + t) : sum_of(4 * t + 2 * h, 4 * t + 2 * h + 1);
+          if (GC == 1 || my_slot == (tile / (KS / CP)) % GC)
+            ws[(my_head + (WIDE ? t : 0)) * Pl::MS + 16 * tile + gid + 8 * h] = fmaf(v, ua, zg[tile * 16 / GS][WIDE ? t % NCOL : 0]);
+        }
+    }
   }
+  tc_fence_before();
   __syncthreads();
+  tc_fence_after();
+  if (warp == W - 1) tmem_dealloc(tmem_base_sm, Pl::TMEM);
   if (p.late_wait) grid_dependency_wait();  // the preceding launch still reads and writes the scratch and its result
   if (dead_sm != 0) {
     // leaving early: no copy of this CTA may still be in flight when its shared memory is released
-    if (lane == 0 && warp < nb) {
+    if (lane == 0 && rounds > 0) {
+      if (Pl::P_OVER && last_v < last_k) mbar_arrive(bar_k);  // (in place of the copies that did not follow the codes)
       for (int it = 0; it < WAIT_LIMIT && !mbar_try_wait(bar_k, last_k & 1); ++it) {}
       for (int it = 0; it < WAIT_LIMIT && !mbar_try_wait(bar_v, last_v & 1); ++it) {}
     }
@@ -1072,58 +1265,64 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NT>::WARPS * 32, Plan<
     return;
   }
   // ---- the CTA's state: all warps; then the partial and the merge, or the result itself ----
-  const size_t slot = (size_t)blockIdx.y * ((size_t)dm.B * dm.Hq) * p.ns_q;  // this layer's partials in the scratch
+  const size_t slot = (size_t)blockIdx.y * NL * ((size_t)dm.B * dm.Hq) * p.ns_q;  // the first layer's partials in the scratch
   float* const part_acc = p.part_acc + slot * D;
   float* const part_ml = p.part_ml + slot * 2;
-  for (int item = tid; item < G * (D / 4); item += W * 32) {
-    const int h = item / (D / 4), d = item % (D / 4) * 4;
-    auto row = [&](int w) { return reinterpret_cast<const float*>(smem + w * Pl::WARP) + h * Pl::MS; };
+  const int wrows = wtiles < W ? wtiles : W;  // warps with a window row
+  for (int item = tid; item < NL * G * (D / 4); item += W * 32) {
+    const int i = item / (D / 4), d = item % (D / 4) * 4;
+    const int layer = NL == 1 || i < G ? 0 : 1, h = i - layer * G;
+    auto row = [&](int w, bool window) { return reinterpret_cast<const float*>(smem + w * Pl::WARP) + ((window ? VH : 0) + layer * HP + h) * Pl::MS; };
     float M = -CUDART_INF_F;
 #pragma unroll
-    for (int w = 0; w < W; ++w) M = fmaxf(M, row(w)[D]);
+    for (int w = 0; w < W; ++w) M = fmaxf(M, row(w, false)[D]);
+    for (int t = 0; t < wrows; ++t) M = fmaxf(M, row((t + halves) % W, true)[D]);
     float4 A = make_float4(0.f, 0.f, 0.f, 0.f);
     float Ls = 0.f;
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-      const float4 v = *reinterpret_cast<const float4*>(row(w) + d);
-      const float mw = row(w)[D];
+    auto add = [&](const float* r) {
+      const float4 v = *reinterpret_cast<const float4*>(r + d);
+      const float mw = r[D];
       const float f = mw == -CUDART_INF_F ? 0.f : ex2(mw - M);  // a warp without tokens
       A.x = fmaf(v.x, f, A.x);
       A.y = fmaf(v.y, f, A.y);
       A.z = fmaf(v.z, f, A.z);
       A.w = fmaf(v.w, f, A.w);
-      Ls = fmaf(row(w)[D + 1], f, Ls);
-    }
+      Ls = fmaf(r[D + 1], f, Ls);
+    };
+#pragma unroll
+    for (int w = 0; w < W; ++w) add(row(w, false));
+    for (int t = 0; t < wrows; ++t) add(row((t + halves) % W, true));
     const size_t hq = (size_t)b * dm.Hq + hk * G + h;
     if (ns == 1) {
-      store_out<D>(p, L, hq, d, make_float4(A.x / Ls, A.y / Ls, A.z / Ls, A.w / Ls));
+      store_out<D>(p, LL[layer], hq, d, make_float4(A.x / Ls, A.y / Ls, A.z / Ls, A.w / Ls));
     } else {
-      *reinterpret_cast<float4*>(part_acc + (hq * p.ns_q + split) * D + d) = A;
-      if (d == 0) *reinterpret_cast<float2*>(part_ml + (hq * p.ns_q + split) * 2) = make_float2(M, Ls);
+      const size_t at = ((size_t)layer * dm.B * dm.Hq + hq) * p.ns_q + split;
+      *reinterpret_cast<float4*>(part_acc + at * D + d) = A;
+      if (d == 0) *reinterpret_cast<float2*>(part_ml + at * 2) = make_float2(M, Ls);
     }
   }
   if (ns > 1)
-    ticket_merge<D>(p, L, ns, hk, b, part_acc, part_ml, p.tickets + (size_t)blockIdx.y * (dm.B * dm.Hkv) + bh, &s_flag,
-                    reinterpret_cast<float*>(smem));
+    ticket_merge<D, NL>(p, LL, ns, hk, b, part_acc, part_ml, p.tickets + (size_t)blockIdx.y * (dm.B * dm.Hkv) + bh, &s_flag,
+                        reinterpret_cast<float*>(smem));
 }
 
-template <int D, int BK, int BV, int GS, int HP, int NT>
+template <int D, int BK, int BV, int GS, int HP, int NL>
 cudaError_t launch_one(const DecodeParams& p, cudaStream_t st) {
-  using Pl = Plan<D, BK, BV, GS, HP, NT>;
-  return launch_dependent(decode_mma_kernel<D, BK, BV, GS, HP, NT>, dim3((unsigned)(p.ns_q * p.dm.B * p.dm.Hkv), p.n_layers), dim3(Pl::WARPS * 32),
+  using Pl = Plan<D, BK, BV, GS, HP, NL>;
+  return launch_dependent(decode_mma_kernel<D, BK, BV, GS, HP, NL>, dim3((unsigned)(p.ns_q * p.dm.B * p.dm.Hkv), p.n_layers / NL), dim3(Pl::WARPS * 32),
                           (size_t)Pl::TOTAL, st, p);
 }
 
 // Prepares the kernel for the current device and says how many of its CTAs share an SM and how many warps each has.
-template <int D, int BK, int BV, int GS, int HP, int NT>
+// (The occupancy calculator has no say on how many: it answers one for any kernel that allocates tensor memory.)
+template <int D, int BK, int BV, int GS, int HP, int NL>
 MmaShape shape_one() {
-  using Pl = Plan<D, BK, BV, GS, HP, NT>;
-  auto kernel = decode_mma_kernel<D, BK, BV, GS, HP, NT>;
-  MmaShape r{0, Pl::WARPS};
-  // the largest shared-memory carve-out: two CTAs of this size are to share an SM
+  using Pl = Plan<D, BK, BV, GS, HP, NL>;
+  auto kernel = decode_mma_kernel<D, BK, BV, GS, HP, NL>;
+  MmaShape r{Pl::CTAS, Pl::WARPS};
+  // the largest shared-memory carve-out: three CTAs of this size are to share an SM
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Pl::TOTAL) != cudaSuccess ||
-      cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.ctas_per_sm, kernel, Pl::WARPS * 32, Pl::TOTAL) != cudaSuccess) {
+      cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess) {
     cudaGetLastError();
     r.ctas_per_sm = 0;
   }
@@ -1132,25 +1331,25 @@ MmaShape shape_one() {
 
 #define XQ_DISPATCH(FN, ...)                               \
   switch (bk * 100 + bv * 10 + (g == 64)) {                \
-    case 220: return FN<D, 2, 2, 32, HP, NT>(__VA_ARGS__); \
-    case 221: return FN<D, 2, 2, 64, HP, NT>(__VA_ARGS__); \
-    case 210: return FN<D, 2, 1, 32, HP, NT>(__VA_ARGS__); \
-    case 211: return FN<D, 2, 1, 64, HP, NT>(__VA_ARGS__); \
-    case 120: return FN<D, 1, 2, 32, HP, NT>(__VA_ARGS__); \
-    case 121: return FN<D, 1, 2, 64, HP, NT>(__VA_ARGS__); \
-    case 110: return FN<D, 1, 1, 32, HP, NT>(__VA_ARGS__); \
-    case 111: return FN<D, 1, 1, 64, HP, NT>(__VA_ARGS__); \
+    case 220: return FN<D, 2, 2, 32, HP, NL>(__VA_ARGS__); \
+    case 221: return FN<D, 2, 2, 64, HP, NL>(__VA_ARGS__); \
+    case 210: return FN<D, 2, 1, 32, HP, NL>(__VA_ARGS__); \
+    case 211: return FN<D, 2, 1, 64, HP, NL>(__VA_ARGS__); \
+    case 120: return FN<D, 1, 2, 32, HP, NL>(__VA_ARGS__); \
+    case 121: return FN<D, 1, 2, 64, HP, NL>(__VA_ARGS__); \
+    case 110: return FN<D, 1, 1, 32, HP, NL>(__VA_ARGS__); \
+    case 111: return FN<D, 1, 1, 64, HP, NL>(__VA_ARGS__); \
   }
 
 }  // namespace
 
-template <int D, int HP, int NT>
+template <int D, int HP, int NL>
 cudaError_t launch_decode_mma_t(const DecodeParams& p, cudaStream_t st) {
   const int bk = p.layer[0].L.bk, bv = p.layer[0].L.bv, g = p.dm.g;
   XQ_DISPATCH(launch_one, p, st)
   return cudaErrorInvalidValue;
 }
-template <int D, int HP, int NT>
+template <int D, int HP, int NL>
 MmaShape decode_mma_shape_t(int g, int bk, int bv) {
   XQ_DISPATCH(shape_one)
   return MmaShape{0, 1};

@@ -1,0 +1,7 @@
+// Tensor-core decode kernels for head_dim 128, two query heads per kv head, for two layers that share their codes.
+#include "xq_decode_mma.cuh"
+
+namespace xq {
+template cudaError_t launch_decode_mma_t<128, 2, 2>(const DecodeParams&, cudaStream_t);
+template MmaShape decode_mma_shape_t<128, 2, 2>(int, int, int);
+}  // namespace xq

@@ -204,17 +204,26 @@ bool uses_mma(const xq_cache* c) {
   return dm.D == 128 || c->cfg.kernel == XQ_KERNEL_AUTO;  // XQ_KERNEL_MMA names the head_dim 128 kernel
 }
 
-// FN<D, HP, NT> of the tensor-core kernel that serves these dimensions
+// FN<D, HP, 1> of the tensor-core kernel that serves these dimensions, and FN<128, HP, 2> of the one that takes two layers
 #define XQ_MMA_BY_HEADS(FN, D, ...)                   \
   (dm.G == 1   ? FN<D, 1, 1>(__VA_ARGS__)             \
    : dm.G == 2 ? FN<D, 2, 1>(__VA_ARGS__)             \
    : dm.G <= 4 ? FN<D, 4, 1>(__VA_ARGS__)             \
-               : FN<D, 4, 2>(__VA_ARGS__))
+               : FN<D, 8, 1>(__VA_ARGS__))
+#define XQ_MMA_OF_PAIRS(FN, ...)                      \
+  (dm.G == 1   ? FN<128, 1, 2>(__VA_ARGS__)           \
+   : dm.G == 2 ? FN<128, 2, 2>(__VA_ARGS__)           \
+               : FN<128, 4, 2>(__VA_ARGS__))
 
 cudaError_t launch_decode_mma(const DecodeParams& p, cudaStream_t st) {
   const Dims& dm = p.dm;
+  if (p.paired) return XQ_MMA_OF_PAIRS(launch_decode_mma_t, p, st);
   return dm.D == 128 ? XQ_MMA_BY_HEADS(launch_decode_mma_t, 128, p, st) : XQ_MMA_BY_HEADS(launch_decode_mma_t, 64, p, st);
 }
+
+// Whether the tensor-core kernel can take two layers of a step that read the same codes in one go: the heads of both fit
+// its eight operand columns.
+bool takes_pairs(const Dims& dm) { return dm.D == 128 && dm.G <= 4; }
 
 // The tensor-core kernel that serves layer l, prepared for the handle's device on first use.
 MmaShape mma_shape(const xq_cache* c, int l) {
@@ -223,7 +232,8 @@ MmaShape mma_shape(const xq_cache* c, int l) {
   MmaShape& s = const_cast<xq_cache*>(c)->mma_shape[bk - 1][bv - 1];
   if (s.warps == 0) {
     s = dm.D == 128 ? XQ_MMA_BY_HEADS(decode_mma_shape_t, 128, dm.g, bk, bv) : XQ_MMA_BY_HEADS(decode_mma_shape_t, 64, dm.g, bk, bv);
-    if (s.ctas_per_sm <= 0) s.ctas_per_sm = 2;  // no device to ask
+    if (takes_pairs(dm)) XQ_MMA_OF_PAIRS(decode_mma_shape_t, dm.g, bk, bv);
+    s.ctas_per_sm = 2;  // of one wave of a launch alone: the third place is the next launch's
   }
   return s;
 }
@@ -449,6 +459,7 @@ int prepare_decode(const xq_cache* c, int layer, const void* q, void* out, int o
   const Dims& dm = c->plan.dm;
   p.dm = dm;
   p.n_layers = 1;
+  p.paired = 0;
   p.layer[0] = {layer_ptrs(c, layer), (const uint16_t*)q, out, (const uint16_t*)K_new, (const uint16_t*)V_new};
   p.n_q = nq;
   p.r = r;
@@ -619,32 +630,62 @@ int decode_impl(xq_cache* c, int layer, const void* q, void* out, int out_f32, c
 }
 
 
-// Tensor-core decode of the layers order[0 .. n) in one launch, or few: consecutive layers of equal length and
-// bit-widths share one.  Layer l's q and out are slice l of q and out; with K_new / V_new the launch appends slice l
-// of them to layer l (no layer's window is full).  Nothing in a launch reads what another layer of it writes: a layer
-// writes its own window row, its own part of the scratch and its own result.
+// Tensor-core decode of the layers order[0 .. n) in few launches: layers of equal length and bit-widths share one, and
+// two that read the same codes go in pairs, for which the kernel reads and expands those once.  Layer l's q and out are
+// slice l of q and out; with K_new / V_new the launch appends slice l of them to layer l (no layer's window is full).
+// Nothing in a launch reads what another layer of it writes: a layer writes its own window row, its own part of the
+// scratch and its own result.
 int decode_layers(xq_cache* c, const int* order, int n, const uint8_t* q, uint8_t* out, const uint8_t* K_new,
                   const uint8_t* V_new, cudaStream_t st) {
   const Dims& dm = c->plan.dm;
   const size_t kv_layer = (size_t)dm.B * dm.Hkv * dm.D * 2, q_layer = (size_t)dm.B * dm.Hq * dm.D * 2;
   int rc = ensure_clean_scratch(c, st);
   if (rc != XQ_OK) return rc;
+  const bool joint = n >= MIN_JOINT_LAYERS;
+  // the layers as they go to the launches: two that share their codes side by side, in the place of the first
+  std::vector<int> run;
+  std::vector<char> paired;  // of run[i]: it is one of two
+  run.reserve(n);
+  paired.reserve(n);
+  {
+    std::vector<char> taken(n, 0);
+    for (int i = 0; i < n; ++i) {
+      if (taken[i]) continue;
+      const int a = order[i];
+      int with = -1;
+      if (joint && takes_pairs(dm))
+        for (int j = i + 1; j < n && with < 0; ++j) {
+          const int b = order[j];
+          if (!taken[j] && c->seq[b] == c->seq[a] && k_owner(&c->cfg, a) == k_owner(&c->cfg, b) && v_owner(&c->cfg, a) == v_owner(&c->cfg, b)) with = j;
+        }
+      run.push_back(a);
+      paired.push_back(with >= 0);
+      if (with >= 0) {
+        taken[with] = 1;
+        run.push_back(order[with]);
+        paired.push_back(1);
+      }
+    }
+  }
   for (int i = 0; i < n;) {
     DecodeParams p;
     bool use_mma;
-    const int l0 = order[i], S = c->seq[l0] + (K_new ? 1 : 0);
+    const int l0 = run[i], S = c->seq[l0] + (K_new ? 1 : 0);
     rc = prepare_decode(c, l0, q + l0 * q_layer, out + l0 * q_layer, 0, K_new ? K_new + l0 * kv_layer : nullptr,
                         V_new ? V_new + l0 * kv_layer : nullptr, S, p, use_mma);
     if (rc != XQ_OK) return rc;
     // the layers of a launch share the scratch: XQ_MAX_SPLITS partials per query head
     int most = XQ_MAX_SPLITS / p.ns_q < DECODE_MAX_LAYERS ? XQ_MAX_SPLITS / p.ns_q : DECODE_MAX_LAYERS;
-    if (n < MIN_JOINT_LAYERS) most = 1;
+    if (!joint) most = 1;
+    p.paired = paired[i] && most >= 2;
+    if (p.paired) most -= most % 2;
     bool packed = c->repacked[l0] != 0;
     int j = i + 1;
-    for (; j < n && j - i < most && c->seq[order[j]] == c->seq[l0]; ++j) {
-      const int l = order[j];
+    for (; j < n && j - i < most && c->seq[run[j]] == c->seq[l0] && (!p.paired || paired[j]); ++j) {
+      const int l = run[j];
       const LayerPtrs L = layer_ptrs(c, l);
       if (L.bk != p.layer[0].L.bk || L.bv != p.layer[0].L.bv) break;
+      if (!p.paired && paired[j] && !paired[i]) break;
       p.layer[j - i] = {L, (const uint16_t*)(q + l * q_layer), out + l * q_layer,
                         K_new ? (const uint16_t*)(K_new + l * kv_layer) : nullptr,
                         V_new ? (const uint16_t*)(V_new + l * kv_layer) : nullptr};
@@ -663,8 +704,8 @@ int decode_layers(xq_cache* c, const int* order, int n, const uint8_t* q, uint8_
       return rc;
     }
     for (; i < j; ++i) {
-      c->repacked[order[i]] = 0;
-      if (K_new) c->seq[order[i]] += 1;
+      c->repacked[run[i]] = 0;
+      if (K_new) c->seq[run[i]] += 1;
     }
   }
   return XQ_OK;

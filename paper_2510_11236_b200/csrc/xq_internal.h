@@ -90,6 +90,7 @@ constexpr int DECODE_MAX_LAYERS = 32;  // layers one launch can take (of equal l
 struct DecodeParams {
   Dims dm;
   int n_layers;       // the scalar kernel takes one
+  int paired;         // tensor-core kernel: a CTA takes layers 2 y and 2 y + 1, which read the same codes
   int n_q;            // quantized tokens
   int r;              // window tokens
   int ns_q, ns_w;     // splits over the quantized region (most of any stream) / over the window
@@ -178,15 +179,16 @@ cudaError_t launch_dependent(void (*kernel)(P), dim3 grid, dim3 block, size_t sm
 cudaError_t launch_pack(const PackParams& p, cudaStream_t st);
 cudaError_t launch_window_append(const WindowParams& p, cudaStream_t st);
 cudaError_t launch_decode_generic(const DecodeParams& p, cudaStream_t st);
-// Tensor-core decode kernels for HP (1, 2, 4) query heads per kv head, or NT = 2 sets of four.  decode_mma_shape_t
-// also prepares the kernel for the current device: it comes before the first launch of a handle.
+// Tensor-core decode kernels for HP (1, 2, 4, 8) query heads per kv head, of one layer or of NL = 2 that read the same
+// codes (head_dim 128, up to four heads).  decode_mma_shape_t also prepares the kernel for the current device: it comes
+// before the first launch of a handle.
 struct MmaShape {
   int ctas_per_sm;  // 0: no device to ask
   int warps;        // warps of a CTA
 };
-template <int D, int HP, int NT>
+template <int D, int HP, int NL>
 cudaError_t launch_decode_mma_t(const DecodeParams& p, cudaStream_t st);
-template <int D, int HP, int NT>
+template <int D, int HP, int NL>
 MmaShape decode_mma_shape_t(int g, int bk, int bv);
 template <int D>
 cudaError_t launch_chunk_t(const ChunkParams& p, cudaStream_t st);
