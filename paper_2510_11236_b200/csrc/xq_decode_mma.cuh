@@ -112,12 +112,13 @@ struct Plan {
   static constexpr bool Q_SHARED = D == 128;
   static constexpr int QF = Q_SHARED ? KS * 32 * 8 : 0;
   static constexpr int room(int w) { return w * WARP + QB + QS + QF; }
-  // Three CTAs per SM, each of eight warps of 80 registers.
-  static constexpr int CTAS = 3, WARPS = 8;
-  // Tensor memory: the value sums of a warp between its rounds, 4 columns a row tile (WIDE: 4 more, of the lo products)
-  static constexpr int TCOLS = KS * 4 * NCOL, TUSED = (WARPS + 3) / 4 * TCOLS;
-  static constexpr int TMEM = TUSED <= 32 ? 32 : TUSED <= 64 ? 64 : TUSED <= 128 ? 128 : 256;
-  static_assert(TUSED <= TMEM && CTAS * TMEM <= 512, "tensor memory");
+  // PARK: the value sums of a warp (64 registers a thread) wait in tensor memory between its rounds, 8 columns a row tile
+  // (four sums of the hi products, four of the lo products): three CTAs per SM, each of eight warps of 80 registers.
+  // Else two CTAs, of eight warps of 128 registers.
+  static constexpr bool PARK = WIDE && D == 128;
+  static constexpr int CTAS = PARK ? 3 : 2, WARPS = 8;
+  static constexpr int TCOLS = KS * 8, TMEM = WARPS / 4 * TCOLS;
+  static_assert(!PARK || (CTAS * TMEM <= 512 && TMEM == 128), "tensor memory");
   static constexpr int TOTAL = room(WARPS);
   static_assert(TOTAL <= 228 * 1024 / CTAS - 1024 - 512, "shared memory");
   static_assert(WARPS * WARP >= VH * (256 + 1) * 4, "the merge's weights");
@@ -477,13 +478,16 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
     }
   }
   __syncwarp();
+  // The next kernel in the stream may be scheduled at once when all work before this kernel's own predecessor is
+  // known to be complete (a chained launch); otherwise only after this kernel's own wait, so that a chained
+  // successor never starts before the work this kernel waited for has completed.
   if (!p.late_wait) grid_dependency_wait();  // q may come from the preceding kernel
   // Tensor memory is asked for after the wait (a chained launch: its predecessor, a launch of this kernel, waited, and
   // the tensor memory of an SM serves all of their CTAs that fit it): a CTA of the preceding kernel that shares the SM may
   // still have to get its own, and this CTA, which waits for it, would be in its way.  For the same reason the next kernel
-  // in the stream may be scheduled only from here on: whatever this kernel waited for is complete for it too.
+  // comes after it.
   if (warp == W - 1) {
-    tmem_alloc((uint32_t)__cvta_generic_to_shared(&tmem_base_sm), Pl::TMEM);
+    if constexpr (Pl::PARK) tmem_alloc((uint32_t)__cvta_generic_to_shared(&tmem_base_sm), Pl::TMEM);
     grid_dependents_go();
   }
 
@@ -525,9 +529,9 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
             pack_io2<true>(io_to_f(v.x >> 16, p.f16) * e2, io_to_f(v.y >> 16, p.f16) * e2));
     }
   }
-  tc_fence_before();
+  if constexpr (Pl::PARK) tc_fence_before();
   __syncthreads();
-  tc_fence_after();
+  if constexpr (Pl::PARK) tc_fence_after();
   float cq[NCOL];  // of the heads of this thread's columns; of the head whose zero-point products it adds up
 #pragma unroll
   for (int j = 0; j < NCOL; ++j) cq[j] = p.scale * 1.4426950408889634f * pow2i(-eq_sm[my_head + j]);
@@ -565,11 +569,12 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
   };
 
   // Softmax state of the heads of this thread's columns: reference mr (log2 units, an integer; 0 until the first round
-  // sets it).  Value sums, in tensor memory between the rounds: of row tile mt the products' four (WIDE: of hi, then of
-  // lo).  zacc[part]: rows gid: the zero-point products of layer gid / 4, channel group gid % 4 (one layer: gid % NG), rows
+  // sets it).  Value sums acc (PARK: in tensor memory between the rounds): of row tile mt the products' four (WIDE: of hi,
+  // then of lo).  zacc[part]: rows gid: the zero-point products of layer gid / 4, channel group gid % 4 (one layer: gid % NG), rows
   // 8 and up: the sum of the numerators (with centered codes lsum, of this thread's tokens); columns hi and lo (WIDE:
   // columns heads, hi and lo apart).
-  const uint32_t t_acc = tmem_base_sm + ((uint32_t)(warp & 3) << 21) + (warp >> 2) * Pl::TCOLS;
+  const uint32_t t_acc = Pl::PARK ? tmem_base_sm + ((uint32_t)(warp & 3) << 21) + (warp >> 2) * Pl::TCOLS : 0u;
+  float acc[Pl::PARK ? 1 : KS * NCOL][4];
   constexpr int MT = GC * KS / CP;                          // row tiles of a channel part of the value products
   constexpr int MTS = MT < 2 ? MT : 2, TV = MTS * 4 * NCOL;  // that are taken at a time; their columns
   float mr[NCOL], zacc[NCOL][4], lsum[NCOL];
@@ -585,24 +590,34 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
   }
   // all value sums of columns j times f[j] (rare)
   auto scale_sums = [&](const float (&f)[NCOL]) {
-    tc_wait_st();
+    if constexpr (Pl::PARK) {
+      tc_wait_st();
 #pragma unroll 1
-    for (int c = 0; c < Pl::TCOLS; c += 8) {
-      uint32_t a[8];
-      tmem_ld<8>(t_acc + c, a);
-      tc_wait_ld();
+      for (int c = 0; c < Pl::TCOLS; c += 8) {
+        uint32_t a[8];
+        tmem_ld<8>(t_acc + c, a);
+        tc_wait_ld();
 #pragma unroll
-      for (int i = 0; i < 8; ++i) a[i] = __float_as_uint(__uint_as_float(a[i]) * f[WIDE ? i & 1 : 0]);
-      tmem_st<8>(t_acc + c, a);
+        for (int i = 0; i < 8; ++i) a[i] = __float_as_uint(__uint_as_float(a[i]) * f[WIDE ? i & 1 : 0]);
+        tmem_st<8>(t_acc + c, a);
+      }
+      tc_wait_st();
+    } else {
+#pragma unroll
+      for (int i = 0; i < KS * NCOL; ++i)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[i][k] *= f[WIDE ? k & 1 : 0];
     }
-    tc_wait_st();
   };
-  {
+  if constexpr (Pl::PARK) {
     uint32_t zero[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) zero[i] = 0u;
 #pragma unroll
     for (int c = 0; c < Pl::TCOLS; c += 8) tmem_st<8>(t_acc + c, zero);
+  } else {
+#pragma unroll
+    for (int i = 0; i < KS * NCOL; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
   }
   const unsigned layer0 = NL == 2 ? __ballot_sync(0xffffffffu, my_layer == 0) : 0xffffffffu;
   const unsigned my_lanes = my_layer == 0 ? layer0 : ~layer0;  // lanes with heads of this thread's layer
@@ -1078,11 +1093,11 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
     }
     // ---- values: p . c, one channel part after the other ----
     auto value_pair = [](uint32_t w, int e) { return Cd::template pair<BV, VBASE>(w, e); };
-    tc_wait_st();
+    if constexpr (Pl::PARK) tc_wait_st();
 #pragma unroll
     for (int vb = 0; vb < CP / GC; ++vb) {
       uint32_t sums[TV];
-      tmem_ld<TV>(t_acc + vb * (MT * 4 * NCOL), sums);
+      if constexpr (Pl::PARK) tmem_ld<TV>(t_acc + vb * (MT * 4 * NCOL), sums);
       const uint32_t sa = vs_lane + (GC * vb + col_slot) * NG / CP * (TT / 2 * 4);
       const uint4 s01 = lds128(sa), s23 = lds128(sa + 16);
       const uint32_t sc[4][2] = {{s01.x, s01.y}, {s01.z, s01.w}, {s23.x, s23.y}, {s23.z, s23.w}};
@@ -1101,7 +1116,9 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
         }
 #pragma unroll
       for (int m0 = vb * MT; m0 < (vb + 1) * MT; m0 += MTS) {
-        if (m0 > vb * MT) tmem_ld<TV>(t_acc + m0 * (4 * NCOL), sums);
+        if constexpr (Pl::PARK) {
+          if (m0 > vb * MT) tmem_ld<TV>(t_acc + m0 * (4 * NCOL), sums);
+        }
         uint32_t w[MTS][2], w8[MTS][2];  // even and odd bytes of rows (channels) 16 mt + gid, + 8
 #pragma unroll
         for (int i = 0; i < MTS; ++i)
@@ -1111,21 +1128,29 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
             w[i][h] = byte_pair_up(raw, shift_up);
             w8[i][h] = byte_pair_down(raw, shift_down);
           }
-        tc_wait_ld();
-        float acc[MTS * NCOL][4];
+        float part[MTS * NCOL][4];
+        if constexpr (Pl::PARK) {
+          tc_wait_ld();
 #pragma unroll
-        for (int i = 0; i < TV; ++i) acc[i / 4][i % 4] = __uint_as_float(sums[i]);
+          for (int i = 0; i < TV; ++i) part[i / 4][i % 4] = __uint_as_float(sums[i]);
+        }
+        auto sum_of = [&](int i) -> float (&)[4] {
+          if constexpr (Pl::PARK) return part[i];
+          else return acc[m0 * NCOL + i];
+        };
 #pragma unroll
         for (int e = 0; e < 4; ++e)
 #pragma unroll
           for (int i = 0; i < MTS; ++i) {
             const uint32_t a0 = value_pair(w[i][0], e), a1 = value_pair(w[i][1], e), a2 = value_pair(w8[i][0], e), a3 = value_pair(w8[i][1], e);
-            mma_f16(acc[NCOL * i], a0, a1, a2, a3, ps[e][0], ps[e][1]);
-            if constexpr (WIDE) mma_f16(acc[NCOL * i + 1], a0, a1, a2, a3, pr[e][0], pr[e][1]);
+            mma_f16(sum_of(NCOL * i), a0, a1, a2, a3, ps[e][0], ps[e][1]);
+            if constexpr (WIDE) mma_f16(sum_of(NCOL * i + 1), a0, a1, a2, a3, pr[e][0], pr[e][1]);
           }
+        if constexpr (Pl::PARK) {
 #pragma unroll
-        for (int i = 0; i < TV; ++i) sums[i] = __float_as_uint(acc[i / 4][i % 4]);
-        tmem_st<TV>(t_acc + m0 * (4 * NCOL), sums);
+          for (int i = 0; i < TV; ++i) sums[i] = __float_as_uint(part[i / 4][i % 4]);
+          tmem_st<TV>(t_acc + m0 * (4 * NCOL), sums);
+        }
       }
     }
     // the value half of the stage and the numerators are free
@@ -1211,7 +1236,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
     const float uz = pow2i(-P_EXP);
     const float ua = pow2i(Cd::exp(VBASE) - P_EXP - exponent_of(f16_to_f((NL == 2 && my_layer == 1 ? ev2[NL - 1] : ev2[0]) & 0xffffu)));
     float z[NCOL];  // row gid < 4 NL: channel group of a layer
-    tc_wait_st();
+    if constexpr (Pl::PARK) tc_wait_st();
 #pragma unroll
     for (int j = 0; j < NCOL; ++j) {
       z[j] = (WIDE ? zacc[0][j] + zacc[1 % NCOL][j] : zacc[0][0] + zacc[0][1]) * uz;
@@ -1234,8 +1259,13 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
 #pragma unroll
     for (int mt = 0; mt < KS; mt += 2 / NCOL) {
       uint32_t a[8];  // WIDE: hi and lo sums of a row tile; else the sums of two
-      tmem_ld<8>(t_acc + mt * 4 * NCOL, a);
-      tc_wait_ld();
+      if constexpr (Pl::PARK) {
+        tmem_ld<8>(t_acc + mt * 4 * NCOL, a);
+        tc_wait_ld();
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) a[i] = __float_as_uint(acc[mt * NCOL + i / 4][i % 4]);
+      }
       auto sum_of = [&](int i, int k) { return __uint_as_float(a[i]) + __uint_as_float(a[k]); };
 #pragma unroll
       for (int h = 0; h < 2; ++h)
@@ -1248,10 +1278,12 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
         }
     }
   }
-  tc_fence_before();
+  if constexpr (Pl::PARK) tc_fence_before();
   __syncthreads();
-  tc_fence_after();
-  if (warp == W - 1) tmem_dealloc(tmem_base_sm, Pl::TMEM);
+  if constexpr (Pl::PARK) {
+    tc_fence_after();
+    if (warp == W - 1) tmem_dealloc(tmem_base_sm, Pl::TMEM);
+  }
   if (p.late_wait) grid_dependency_wait();  // the preceding launch still reads and writes the scratch and its result
   if (dead_sm != 0) {
     // leaving early: no copy of this CTA may still be in flight when its shared memory is released
@@ -1314,7 +1346,7 @@ cudaError_t launch_one(const DecodeParams& p, cudaStream_t st) {
 }
 
 // Prepares the kernel for the current device and says how many of its CTAs share an SM and how many warps each has.
-// (The occupancy calculator has no say on how many: it answers one for any kernel that allocates tensor memory.)
+// (The occupancy calculator has no say on how many: it answers one for a kernel that allocates tensor memory.)
 template <int D, int BK, int BV, int GS, int HP, int NL>
 MmaShape shape_one() {
   using Pl = Plan<D, BK, BV, GS, HP, NL>;
