@@ -402,6 +402,11 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
   const int col_layer = NL == 1 ? 0 : col_head / HP, my_layer = NL == 1 ? 0 : my_head / HP;
   const int G = dm.G;
 
+  // The next kernel in the stream may be scheduled at once when all work before this kernel's own predecessor is
+  // known to be complete (a chained launch); otherwise only after this kernel's own wait (below), so that a chained
+  // successor never starts before the work this kernel waited for has completed.
+  if (!Pl::PARK && p.late_wait) grid_dependents_go();
+
   const uint32_t sm_base = (uint32_t)__cvta_generic_to_shared(smem);
   const uint32_t st = sm_base + warp * Pl::WARP;                     // this warp's stage
   const uint32_t pbuf = st + Pl::OFF_P;
@@ -478,17 +483,18 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
     }
   }
   __syncwarp();
-  // The next kernel in the stream may be scheduled at once when all work before this kernel's own predecessor is
-  // known to be complete (a chained launch); otherwise only after this kernel's own wait, so that a chained
-  // successor never starts before the work this kernel waited for has completed.
   if (!p.late_wait) grid_dependency_wait();  // q may come from the preceding kernel
   // Tensor memory is asked for after the wait (a chained launch: its predecessor, a launch of this kernel, waited, and
   // the tensor memory of an SM serves all of their CTAs that fit it): a CTA of the preceding kernel that shares the SM may
   // still have to get its own, and this CTA, which waits for it, would be in its way.  For the same reason the next kernel
   // comes after it.
-  if (warp == W - 1) {
-    if constexpr (Pl::PARK) tmem_alloc((uint32_t)__cvta_generic_to_shared(&tmem_base_sm), Pl::TMEM);
-    grid_dependents_go();
+  if constexpr (Pl::PARK) {
+    if (warp == W - 1) {
+      tmem_alloc((uint32_t)__cvta_generic_to_shared(&tmem_base_sm), Pl::TMEM);
+      grid_dependents_go();
+    }
+  } else {
+    if (!p.late_wait) grid_dependents_go();
   }
 
   // ---- q, and the exponents that put a head's largest |q| into [1, 2) ----
@@ -1308,22 +1314,24 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
     float M = -CUDART_INF_F;
 #pragma unroll
     for (int w = 0; w < W; ++w) M = fmaxf(M, row(w, false)[D]);
-    for (int t = 0; t < wrows; ++t) M = fmaxf(M, row((t + halves) % W, true)[D]);
+#pragma unroll
+    for (int t = 0; t < W; ++t) M = fmaxf(M, t < wrows ? row((t + halves) % W, true)[D] : -CUDART_INF_F);
     float4 A = make_float4(0.f, 0.f, 0.f, 0.f);
     float Ls = 0.f;
-    auto add = [&](const float* r) {
-      const float4 v = *reinterpret_cast<const float4*>(r + d);
-      const float mw = r[D];
+    auto add = [&](const float* r, bool there) {
+      const float4 v = there ? *reinterpret_cast<const float4*>(r + d) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float mw = there ? r[D] : -CUDART_INF_F;
       const float f = mw == -CUDART_INF_F ? 0.f : ex2(mw - M);  // a warp without tokens
       A.x = fmaf(v.x, f, A.x);
       A.y = fmaf(v.y, f, A.y);
       A.z = fmaf(v.z, f, A.z);
       A.w = fmaf(v.w, f, A.w);
-      Ls = fmaf(r[D + 1], f, Ls);
+      Ls = fmaf(there ? r[D + 1] : 0.f, f, Ls);
     };
 #pragma unroll
-    for (int w = 0; w < W; ++w) add(row(w, false));
-    for (int t = 0; t < wrows; ++t) add(row((t + halves) % W, true));
+    for (int w = 0; w < W; ++w) add(row(w, false), true);
+#pragma unroll
+    for (int t = 0; t < W; ++t) add(row((t + halves) % W, true), t < wrows);
     const size_t hq = (size_t)b * dm.Hq + hk * G + h;
     if (ns == 1) {
       store_out<D>(p, LL[layer], hq, d, make_float4(A.x / Ls, A.y / Ls, A.z / Ls, A.w / Ls));
