@@ -112,13 +112,15 @@ struct Plan {
   static constexpr bool Q_SHARED = D == 128;
   static constexpr int QF = Q_SHARED ? KS * 32 * 8 : 0;
   static constexpr int room(int w) { return w * WARP + QB + QS + QF; }
-  // PARK: the value sums of a warp (64 registers a thread) wait in tensor memory between its rounds, 8 columns a row tile
-  // (four sums of the hi products, four of the lo products): three CTAs per SM, each of eight warps of 80 registers.
-  // Else two CTAs, of eight warps of 128 registers.
-  static constexpr bool PARK = WIDE && D == 128;
+  // PARK: the value sums of a warp wait in tensor memory between its rounds, 4 columns a row tile (WIDE: 4 more, of the lo
+  // products): three CTAs per SM, each of eight warps of 80 registers.  Else two CTAs, of eight warps of 128 registers.
+  // With eight heads the sums (64 registers) would not fit otherwise; two layers of one head, 4k, batch 8: 640 us a step
+  // without, 622 with.  One layer alone, up to four heads: tensor memory costs a CTA 1.2 us at its start and end (a call
+  // at 32k 37.0 us with, 35.2 without).
+  static constexpr bool PARK = (WIDE || NL == 2) && D == 128;
   static constexpr int CTAS = PARK ? 3 : 2, WARPS = 8;
-  static constexpr int TCOLS = KS * 8, TMEM = WARPS / 4 * TCOLS;
-  static_assert(!PARK || (CTAS * TMEM <= 512 && TMEM == 128), "tensor memory");
+  static constexpr int TCOLS = KS * 4 * NCOL, TMEM = WARPS / 4 * TCOLS;
+  static_assert(!PARK || (CTAS * TMEM <= 512 && (TMEM & (TMEM - 1)) == 0), "tensor memory");
   static constexpr int TOTAL = room(WARPS);
   static_assert(TOTAL <= 228 * 1024 / CTAS - 1024 - 512, "shared memory");
   static_assert(WARPS * WARP >= VH * (256 + 1) * 4, "the merge's weights");

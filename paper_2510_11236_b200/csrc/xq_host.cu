@@ -257,7 +257,7 @@ DecodeTimes decode_times(const Dims& dm) {
   if (dm.G == 1) return {7.3, 0.48, 0.34, 10.0, 3.8, 0.37};
   if (dm.G == 2) return {7.0, 0.71, 0.36, 10.0, 4.1, 0.40};
   if (dm.G <= 4) return {7.2, 0.91, 0.37, 10.0, 4.0, 0.44};
-  return {8.3, 2.4, 0.63, 10.0, 5.0, 0.86};
+  return {8.3, 1.9, 0.50, 10.0, 5.0, 0.68};  // (13 shapes: 32k, batch 4, eight heads 47.9 alone, 16k, five heads 29.8)
 }
 
 // Number of splits of a stream's batches, and the runs in which they are dealt, for the tensor-core kernel; splits > 0:

@@ -1079,3 +1079,37 @@ def test_chunk_rows_do_not_see_later_tokens_that_are_not_finite(D, Hq, Hkv, R, S
     for o in outs[1:]:
         assert torch.equal(o[:before], outs[0][:before])
     assert torch.isnan(outs[2][at - (S - T):, ..., 5]).all() or (packed and value != value)
+
+
+@pytest.mark.parametrize("G,bits,g,f16,S", [(1, (2, 2), 32, False, 481), (1, (0, 2), 64, True, 1100), (2, (2, 0), 32, True, 290),
+                                            (2, (0, 0), 64, False, 610), (3, (2, 0), 32, False, 700), (4, (2, 2), 64, True, 130),
+                                            (4, (0, 2), 32, False, 2210), (4, (2, 0), 32, False, 64)])
+@pytest.mark.parametrize("group", [2, 4])
+def test_decode_step_pairs_of_layers(G, bits, g, f16, S, group):
+    """Two layers that read the same codes share a pass over them.  Last batches of one, two and three quarters and of less
+    than half, no batch at all, owners first or in order, groups of four layers (two pairs each): results equal
+    xq_append_kv and xq_decode_attention bit for bit."""
+    L, B, Hkv, D, R = 8, 2, 2, 128, 64 if g == 64 else 32
+    kw = dict(n_layers=L, batch=B, n_q_heads=G * Hkv, n_kv_heads=Hkv, head_dim=D, max_seq=S + 40, group_size=g, residual_len=R,
+              kq=L if bits[0] else 0, vq=L if bits[1] else 0, eta1=1 / 6, eta2=0.045, share_group=group if group > 2 else 0,
+              io_dtype=xq.XQ_F16 if f16 else xq.XQ_BF16, n_splits=3)
+    a, b = xq.Cache(xq.make_config(**kw), DEV), xq.Cache(xq.make_config(**kw), DEV)
+    dt = torch.float16 if f16 else torch.bfloat16
+    gen = torch.Generator(device=DEV).manual_seed(S)
+    for l in range(L):
+        k, v = (torch.randn(B, Hkv, S, D, generator=gen, device=DEV).to(dt) for _ in range(2))
+        for cache in (a, b):
+            cache.append_kv(l, k, v)
+    owners_first = torch.tensor(sorted(range(L), key=lambda l: (l % group, l)), dtype=torch.int32)
+    for step in range(4):
+        kn, vn = (torch.randn(L, B, Hkv, 1, D, generator=gen, device=DEV).to(dt) for _ in range(2))
+        q = torch.randn(L, B, G * Hkv, D, generator=gen, device=DEV).to(dt) * (4.0 if step == 2 else 1.0)
+        n0 = xq.xq_launch_count(a.handle)
+        out = a.decode_step(kn, vn, q, torch.empty_like(q), layer_order=owners_first if step % 2 else None)
+        assert xq.xq_launch_count(a.handle) - n0 <= 2  # (a pack before the decode launch)
+        for l in range(L):
+            b.append_kv(l, kn[l], vn[l])
+        for l in range(L):
+            assert torch.equal(b.decode_attention(l, q[l]), out[l]), (step, l)
+    a.check_device()
+    a.close(); b.close()
