@@ -381,7 +381,11 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
   constexpr int KS = Pl::KS, NG = Pl::NG, NGT = Pl::NGT, W = Pl::WARPS, WROW = Pl::WROW, GC = Pl::GC, CP = Pl::CP;
   constexpr int VH = Pl::VH, SH = Pl::SH, NSET = Pl::NSET, NCOL = Pl::NCOL, NE = Pl::NE;
   constexpr int KWORDS = (BK == 2 && D == 128) ? 2 : 1;  // packed words of a token row that a thread expands
-  constexpr int KBASE = 2, VBASE = BV == 2 ? 2 : 4;      // where the codes of an operand begin in its halves
+  // Where the codes of an operand begin in its halves.  VWIN: quads of tokens (k-steps e) whose value codes one shift of a
+  // word puts in place, with weights 2^(BV * (e % VWIN)); 2-bit codes, as far as their sums are limited by the zeros ahead
+  // of them, in two shifts.
+  constexpr int VWIN = BV == 2 && !Code<D>::CENTERED ? 2 : 4;
+  constexpr int KBASE = 2, VBASE = BV == 2 ? (VWIN == 2 ? 6 : 2) : 4;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) unsigned long long bar_mem[2 * W];
   // the CTA's packed data: key codes, value codes, and of each layer key parameters, value parameters
@@ -630,7 +634,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
   const unsigned layer0 = NL == 2 ? __ballot_sync(0xffffffffu, my_layer == 0) : 0xffffffffu;
   const unsigned my_lanes = my_layer == 0 ? layer0 : ~layer0;  // lanes with heads of this thread's layer
   // weight of the codes of this lane's tokens in the value words (the token of row gid is in quad (gid >> 1) of its tile)
-  const int wt = BV == 1 ? gid >> 1 : 2 * (gid >> 1);
+  const int wt = BV * ((gid >> 1) % VWIN);
   const float off = (float)(P_EXP - wt), weight = pow2i(wt);
   const int tok0 = 4 * (gid >> 1) + (gid & 1);                       // token of row gid, tile 0; the other rows: + 2, + 16
   const uint32_t kz_lane = st + Pl::OFF_KM + (gid & (NGT - 1)) * 4 * D + 2 * D + (gid >> 2) * D + tig * 16;  // zero-points of its row
@@ -642,7 +646,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
   // in 1 bit a half of word tig / 2 (of the two that this half of the batch has), shifted so that its codes begin at bit
   // VBASE.
   const uint32_t vc_lane = st + Pl::OFF_V + gid * 16 + (BV == 2 ? tig : 2 * (warp & 1) + (tig >> 1)) * 4;
-  const int shift_up = BV == 2 ? 2 : (tig & 1 ? 0 : 4), shift_down = BV == 2 ? 6 : (tig & 1 ? 8 : 4);
+  const int shift_up = BV == 2 ? VBASE : (tig & 1 ? 0 : 4), shift_down = BV == 2 ? 8 - VBASE : (tig & 1 ? 8 : 4);
   const uint32_t vm_read = st + Pl::OFF_VM + (4 * (lane >> 1) + (lane & 1)) * (4 * NG), vm_write = st + Pl::OFF_VM + 4 * lane;
   const uint32_t vs_lane = st + Pl::OFF_VM + (NL == 2 ? col_layer * Pl::VROOM : 0) + tig * 32;  // the scales of its pairs
   const uint32_t vz_lane = st + Pl::OFF_VM + (NL == 2 ? (gid >> 2) * Pl::VROOM : 0) + Pl::VZ + (NL == 2 ? (gid & 3) % NG : gid % NG) * Pl::VZROW + tig * 32;
@@ -1070,7 +1074,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       constexpr uint32_t STEP = BV == 2 ? 0x0800u : 0x0400u;
-      const uint32_t we = (0x3C00u + e * STEP) * 0x10001u;  // the weight of this step's codes as a pair of fp16
+      const uint32_t we = (0x3C00u + e % VWIN * STEP) * 0x10001u;  // the weight of this step's codes as a pair of fp16
       uint4 hp;
       if constexpr (WIDE) hp = lds128((p_ld ^ ((e & 1) << 4)) + (e << 7));
       else hp = lds128(p_ld + e * 16);
@@ -1100,7 +1104,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
       }
     }
     // ---- values: p . c, one channel part after the other ----
-    auto value_pair = [](uint32_t w, int e) { return Cd::template pair<BV, VBASE>(w, e); };
+    auto value_pair = [](uint32_t w, int e) { return Cd::template pair<BV, VBASE>(w, e % VWIN); };
     if constexpr (Pl::PARK) tc_wait_st();
 #pragma unroll
     for (int vb = 0; vb < CP / GC; ++vb) {
@@ -1127,14 +1131,18 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
         if constexpr (Pl::PARK) {
           if (m0 > vb * MT) tmem_ld<TV>(t_acc + m0 * (4 * NCOL), sums);
         }
-        uint32_t w[MTS][2], w8[MTS][2];  // even and odd bytes of rows (channels) 16 mt + gid, + 8
+        // even and odd bytes of rows (channels) 16 mt + gid, + 8; second shifts for the quads from VWIN on
+        uint32_t w[4 / VWIN][MTS][2], w8[4 / VWIN][MTS][2];
 #pragma unroll
         for (int i = 0; i < MTS; ++i)
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const uint32_t raw = lds32(vc_lane + (m0 + i) * 256 + h * 128);
-            w[i][h] = byte_pair_up(raw, shift_up);
-            w8[i][h] = byte_pair_down(raw, shift_down);
+#pragma unroll
+            for (int k = 0; k < 4 / VWIN; ++k) {
+              w[k][i][h] = byte_pair_up(raw, shift_up - k * BV * VWIN);
+              w8[k][i][h] = byte_pair_down(raw, shift_down + k * BV * VWIN);
+            }
           }
         float part[MTS * NCOL][4];
         if constexpr (Pl::PARK) {
@@ -1150,7 +1158,8 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
         for (int e = 0; e < 4; ++e)
 #pragma unroll
           for (int i = 0; i < MTS; ++i) {
-            const uint32_t a0 = value_pair(w[i][0], e), a1 = value_pair(w[i][1], e), a2 = value_pair(w8[i][0], e), a3 = value_pair(w8[i][1], e);
+            const int k = e / VWIN;
+            const uint32_t a0 = value_pair(w[k][i][0], e), a1 = value_pair(w[k][i][1], e), a2 = value_pair(w8[k][i][0], e), a3 = value_pair(w8[k][i][1], e);
             mma_f16(sum_of(NCOL * i), a0, a1, a2, a3, ps[e][0], ps[e][1]);
             if constexpr (WIDE) mma_f16(sum_of(NCOL * i + 1), a0, a1, a2, a3, pr[e][0], pr[e][1]);
           }
