@@ -588,7 +588,8 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
   const uint32_t t_acc = Pl::PARK ? tmem_base_sm + ((uint32_t)(warp & 3) << 21) + (warp >> 2) * Pl::TCOLS : 0u;
   float acc[Pl::PARK ? 1 : KS * NCOL][4];
   constexpr int MT = GC * KS / CP;                          // row tiles of a channel part of the value products
-  constexpr int MTS = MT < 2 ? MT : 2, TV = MTS * 4 * NCOL;  // that are taken at a time; their columns
+  // that are taken at a time (eight heads: one; with two, 80 bytes more of spills at groups of 64, 724 us a step for 705 at 8k); their columns
+  constexpr int MTS = MT < 2 || WIDE ? 1 : 2, TV = MTS * 4 * NCOL;
   float mr[NCOL], zacc[NCOL][4], lsum[NCOL];
   uint32_t ev2[NL];  // value scales are taken times 2^Ev: a pair of fp16 (0: not set)
 #pragma unroll
