@@ -708,9 +708,13 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
       if constexpr (Pl::Q_SHARED) {
         // The largest scale of the round times 2^Ek in [2^-4, 1): |q s| below 2^15, and a scale keeps its 11 bits down to
         // 2^-10 of the largest.  Ek moves only outside that, and no further than 15.
-        scale();
-        if (largest() - 0x2c00u >= 0x1000u) {
-          read();
+        bool moved = r == 0;
+        if (r > 0) {
+          scale();
+          moved = largest() - 0x2c00u >= 0x1000u;
+          if (moved) read();
+        }
+        if (moved) {
           const float smax = f16_to_f(largest());
           const int es = smax > 0.f ? exponent_of(smax) : -24, e = min(15, -1 - es);
           const float f = pow2i(e);
@@ -1043,9 +1047,13 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
         for (int g = 0; g < NG; ++g) mx = __vmaxu2(mx, v[g]);
         return redux_max_u32(max(mx & 0xffffu, mx >> 16));
       };
-      scale();
       // the largest scale times 2^Ev in [2^-6, 1): the exponent moves only outside that, and no further than 15
-      if (largest(se) - 0x2400u >= 0x1800u) {
+      bool moved = r == 0;
+      if (r > 0) {
+        scale();
+        moved = largest(se) - 0x2400u >= 0x1800u;
+      }
+      if (moved) {
         const float smax = f16_to_f(largest(sp));
         const int es = smax > 0.f ? exponent_of(smax) : -24, e = min(15, -1 - es), before = exponent_of(f16_to_f(ev2[l] & 0xffffu));
         float f[NCOL];
@@ -1185,7 +1193,8 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
 
   // ---- state rows, over the stage: acc, m, l of each head from the packed tokens, then from the window ----
   const int wt0 = place.z, wt1 = place.w, hk = place2.y, b = place2.x, split = place2.z, bh = b * dm.Hkv + hk;
-  // The CTA's share of the 16-bit window goes tile by tile to its warps, first to those with the fewest rounds.
+  // The CTA's share of the 16-bit window goes tile by tile to its warps, first to those with the fewest rounds; a warp
+  // without rounds has the window's state in place of the packed tokens'.
   const int wtiles = (wt1 - wt0 + 15) / 16;
   auto window_turn = [&](int w) { const int t = w - halves % W; return t < 0 ? t + W : t; };
   if (dead_sm == 0) {  // (else a wait gave up somewhere: copies may be in flight, the stage is not reused)
@@ -1235,7 +1244,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
       }
 #pragma unroll
       for (int s = 0; s < NSET; ++s) {
-        float* const row = ws + (VH + SH * s + tig % SH) * Pl::MS;
+        float* const row = ws + ((rounds > 0 ? VH : 0) + SH * s + tig % SH) * Pl::MS;
         if (tig / SH == 0) {
 #pragma unroll
           for (int mt = 0; mt < KS; ++mt) {
@@ -1250,50 +1259,54 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
       }
     }
     __syncwarp();
-    // the packed tokens, in true units
-    const float uz = pow2i(-P_EXP);
-    const float ua = pow2i(Cd::exp(VBASE) - P_EXP - exponent_of(f16_to_f((NL == 2 && my_layer == 1 ? ev2[NL - 1] : ev2[0]) & 0xffffu)));
-    float z[NCOL];  // row gid < 4 NL: channel group of a layer
     if constexpr (Pl::PARK) tc_wait_st();
+    // the packed tokens, in true units
+    if (rounds > 0) {
+      const float uz = pow2i(-P_EXP);
+      const float ua = pow2i(Cd::exp(VBASE) - P_EXP - exponent_of(f16_to_f((NL == 2 && my_layer == 1 ? ev2[NL - 1] : ev2[0]) & 0xffffu)));
+      float z[NCOL];  // row gid < 4 NL: channel group of a layer
 #pragma unroll
-    for (int j = 0; j < NCOL; ++j) {
-      z[j] = (WIDE ? zacc[0][j] + zacc[1 % NCOL][j] : zacc[0][0] + zacc[0][1]) * uz;
-      float sum = (WIDE ? zacc[0][2 + j] + zacc[1 % NCOL][2 + j] : zacc[0][2] + zacc[0][3]) * uz;
-      if constexpr (Cd::CENTERED) {
+      for (int j = 0; j < NCOL; ++j) {
+        z[j] = (WIDE ? zacc[0][j] + zacc[1 % NCOL][j] : zacc[0][0] + zacc[0][1]) * uz;
+        float sum = (WIDE ? zacc[0][2 + j] + zacc[1 % NCOL][2 + j] : zacc[0][2] + zacc[0][3]) * uz;
+        if constexpr (Cd::CENTERED) {
 #pragma unroll
-        for (int k = WIDE ? 4 : VH; k < 32; k <<= 1) lsum[j] += __shfl_xor_sync(0xffffffffu, lsum[j], k);
-        sum = lsum[j] * uz;
-      }
-      if (gid == 0 && my_slot == 0) {
-        ws[(my_head + j) * Pl::MS + D] = rounds > 0 ? mr[j] : -CUDART_INF_F;
-        ws[(my_head + j) * Pl::MS + D + 1] = sum;
-      }
-    }
-    float zg[NG][NCOL];  // of this thread's heads
-#pragma unroll
-    for (int g = 0; g < NG; ++g)
-#pragma unroll
-      for (int j = 0; j < NCOL; ++j) zg[g][j] = __shfl_sync(0xffffffffu, z[j], (4 * my_layer + g) * 4 + tig);
-#pragma unroll
-    for (int mt = 0; mt < KS; mt += 2 / NCOL) {
-      uint32_t a[8];  // WIDE: hi and lo sums of a row tile; else the sums of two
-      if constexpr (Pl::PARK) {
-        tmem_ld<8>(t_acc + mt * 4 * NCOL, a);
-        tc_wait_ld();
-      } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) a[i] = __float_as_uint(acc[mt * NCOL + i / 4][i % 4]);
-      }
-      auto sum_of = [&](int i, int k) { return __uint_as_float(a[i]) + __uint_as_float(a[k]); };
-#pragma unroll
-      for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {  // WIDE: columns; else row tiles, which the threads of the tile's slot hold
-          const int tile = WIDE ? mt : mt + t;
-          const float v = WIDE ? sum_of(2 * h + t, 4 + 2 * h + t) : sum_of(4 * t + 2 * h, 4 * t + 2 * h + 1);
-          if (GC == 1 || my_slot == (tile / (KS / CP)) % GC)
-            ws[(my_head + (WIDE ? t : 0)) * Pl::MS + 16 * tile + gid + 8 * h] = fmaf(v, ua, zg[tile * 16 / GS][WIDE ? t % NCOL : 0]);
+          for (int k = WIDE ? 4 : VH; k < 32; k <<= 1) lsum[j] += __shfl_xor_sync(0xffffffffu, lsum[j], k);
+          sum = lsum[j] * uz;
         }
+        if (gid == 0 && my_slot == 0) {
+          ws[(my_head + j) * Pl::MS + D] = mr[j];
+          ws[(my_head + j) * Pl::MS + D + 1] = sum;
+        }
+      }
+      float zg[NG][NCOL];  // of this thread's heads
+#pragma unroll
+      for (int g = 0; g < NG; ++g)
+#pragma unroll
+        for (int j = 0; j < NCOL; ++j) zg[g][j] = __shfl_sync(0xffffffffu, z[j], (4 * my_layer + g) * 4 + tig);
+#pragma unroll
+      for (int mt = 0; mt < KS; mt += 2 / NCOL) {
+        uint32_t a[8];  // WIDE: hi and lo sums of a row tile; else the sums of two
+        if constexpr (Pl::PARK) {
+          tmem_ld<8>(t_acc + mt * 4 * NCOL, a);
+          tc_wait_ld();
+        } else {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) a[i] = __float_as_uint(acc[mt * NCOL + i / 4][i % 4]);
+        }
+        auto sum_of = [&](int i, int k) { return __uint_as_float(a[i]) + __uint_as_float(a[k]); };
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int t = 0; t < 2; ++t) {  // WIDE: columns; else row tiles, which the threads of the tile's slot hold
+            const int tile = WIDE ? mt : mt + t;
+            const float v = WIDE ? sum_of(2 * h + t, 4 + 2 * h + t) : sum_of(4 * t + 2 * h, 4 * t + 2 * h + 1);
+            if (GC == 1 || my_slot == (tile / (KS / CP)) % GC)
+              ws[(my_head + (WIDE ? t : 0)) * Pl::MS + 16 * tile + gid + 8 * h] = fmaf(v, ua, zg[tile * 16 / GS][WIDE ? t % NCOL : 0]);
+          }
+      }
+    } else if (window_turn(warp) >= wtiles) {  // neither: nothing to add
+      for (int i = lane; i < VH * Pl::MS; i += 32) ws[i] = i % Pl::MS == D ? -CUDART_INF_F : 0.f;
     }
   }
   if constexpr (Pl::PARK) tc_fence_before();
@@ -1318,7 +1331,8 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
   const size_t slot = (size_t)blockIdx.y * NL * ((size_t)dm.B * dm.Hq) * p.ns_q;  // the first layer's partials in the scratch
   float* const part_acc = p.part_acc + slot * D;
   float* const part_ml = p.part_ml + slot * 2;
-  const int wrows = wtiles < W ? wtiles : W;  // warps with a window row
+  // turns of the warps with a row of their own for the window
+  const int wrow0 = halves < W ? W - halves : 0, wrow1 = wtiles < W ? wtiles : W;
   for (int item = tid; item < NL * G * (D / 4); item += W * 32) {
     const int i = item / (D / 4), d = item % (D / 4) * 4;
     const int layer = NL == 1 || i < G ? 0 : 1, h = i - layer * G;
@@ -1326,24 +1340,22 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
     float M = -CUDART_INF_F;
 #pragma unroll
     for (int w = 0; w < W; ++w) M = fmaxf(M, row(w, false)[D]);
-#pragma unroll
-    for (int t = 0; t < W; ++t) M = fmaxf(M, t < wrows ? row((t + halves) % W, true)[D] : -CUDART_INF_F);
+    for (int t = wrow0; t < wrow1; ++t) M = fmaxf(M, row((t + halves) % W, true)[D]);
     float4 A = make_float4(0.f, 0.f, 0.f, 0.f);
     float Ls = 0.f;
-    auto add = [&](const float* r, bool there) {
-      const float4 v = there ? *reinterpret_cast<const float4*>(r + d) : make_float4(0.f, 0.f, 0.f, 0.f);
-      const float mw = there ? r[D] : -CUDART_INF_F;
+    auto add = [&](const float* r) {
+      const float4 v = *reinterpret_cast<const float4*>(r + d);
+      const float mw = r[D];
       const float f = mw == -CUDART_INF_F ? 0.f : ex2(mw - M);  // a warp without tokens
       A.x = fmaf(v.x, f, A.x);
       A.y = fmaf(v.y, f, A.y);
       A.z = fmaf(v.z, f, A.z);
       A.w = fmaf(v.w, f, A.w);
-      Ls = fmaf(there ? r[D + 1] : 0.f, f, Ls);
+      Ls = fmaf(r[D + 1], f, Ls);
     };
 #pragma unroll
-    for (int w = 0; w < W; ++w) add(row(w, false), true);
-#pragma unroll
-    for (int t = 0; t < W; ++t) add(row((t + halves) % W, true), t < wrows);
+    for (int w = 0; w < W; ++w) add(row(w, false));
+    for (int t = wrow0; t < wrow1; ++t) add(row((t + halves) % W, true));
     const size_t hq = (size_t)b * dm.Hq + hk * G + h;
     if (ns == 1) {
       store_out<D>(p, LL[layer], hq, d, make_float4(A.x / Ls, A.y / Ls, A.z / Ls, A.w / Ls));

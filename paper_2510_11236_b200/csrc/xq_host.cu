@@ -642,6 +642,15 @@ int decode_layers(xq_cache* c, const int* order, int n, const uint8_t* q, uint8_
   int rc = ensure_clean_scratch(c, st);
   if (rc != XQ_OK) return rc;
   const bool joint = n >= MIN_JOINT_LAYERS;
+  // Pairs make half as many CTAs that take longer: where all layers one by one fit a wave they would only idle SMs (one
+  // user at 1000 tokens, 8 layers, 256 CTAs: 10.0 us a step one by one, 13.3 in pairs).
+  bool pairs = false;
+  if (joint && takes_pairs(dm)) {
+    const int S = c->seq[order[0]] + (K_new ? 1 : 0), r = residual_count(S, dm.R);
+    int ns_q = 1, ns_w = 0;
+    plan_splits(c, order[0], S - r, r, ns_q, ns_w);
+    pairs = (long long)ns_q * dm.B * dm.Hkv * n > 2LL * c->sm_count;
+  }
   // the layers as they go to the launches: two that share their codes side by side, in the place of the first
   std::vector<int> run;
   std::vector<char> paired;  // of run[i]: it is one of two
@@ -653,7 +662,7 @@ int decode_layers(xq_cache* c, const int* order, int n, const uint8_t* q, uint8_
       if (taken[i]) continue;
       const int a = order[i];
       int with = -1;
-      if (joint && takes_pairs(dm))
+      if (pairs)
         for (int j = i + 1; j < n && with < 0; ++j) {
           const int b = order[j];
           if (!taken[j] && c->seq[b] == c->seq[a] && k_owner(&c->cfg, a) == k_owner(&c->cfg, b) && v_owner(&c->cfg, a) == v_owner(&c->cfg, b)) with = j;
