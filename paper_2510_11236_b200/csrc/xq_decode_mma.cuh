@@ -49,6 +49,7 @@
 namespace xq {
 namespace {
 
+constexpr int D = 128;             // head dim
 constexpr int BT = 128;            // tokens per batch
 constexpr int TT = 64;             // tokens of a round: half a batch
 constexpr float TAU = 3.f;         // log2 units a logit may exceed the softmax reference before it is raised
@@ -56,13 +57,13 @@ constexpr int P_EXP = 11;          // numerators are carried times 2^P_EXP (at m
 constexpr int Q_BIAS_EXP = 8;      // exponent of the largest |q| in the zero-point products
 constexpr uint32_t ONES = 0x3C003C00u;
 
-// Shared-memory plan.  D: head dim, GS: quantization group, BK / BV: bits, HP: query heads per kv head and layer (1, 2,
+// Shared-memory plan.  GS: quantization group, BK / BV: bits, HP: query heads per kv head and layer (1, 2,
 // 4, 8; a G in between is padded), NL: layers that share their codes (1 or 2).  A CTA's "heads" are the VH = HP * NL
 // heads of its layers.  Up to four of them: the eight operand columns are four column pairs (hi, lo) of VH heads times
 // GC = 4 / VH slots: with fewer heads, one operand serves GC token units of the keys (or GC channel parts of the values)
 // at once, each row tile reading the columns of its own slot.  Eight (WIDE): a column is a head, hi and lo are operands
 // of two products.
-template <int D, int BK, int BV, int GS, int HP, int NL>
+template <int BK, int BV, int GS, int HP, int NL>
 struct Plan {
   static constexpr int VH = HP * NL;
   static_assert(VH == 1 || VH == 2 || VH == 4 || VH == 8, "heads of a CTA");
@@ -79,14 +80,10 @@ struct Plan {
   static constexpr int KCODES = TT * D * BK / 8;  // codes of a round; values in 1 bit: of its whole batch
   static constexpr int VCODES = 16 * D;
   static constexpr int KM = NGT * 4 * D, VM = TT * 4 * NG;  // scales and zero-points of a round and layer: keys, values
-  static constexpr bool CENTERED = D == 64;
-  static_assert(!CENTERED || NL == 1, "layers share codes only with head_dim 128");
   // value scales, then zero-points, as they are reordered over the copy: [channel group][pair of tokens] half2, a
-  // group's zero-points 8 bytes longer (bank conflicts); centered codes: second halves of the zero-points, of the
-  // values (as the first), of the keys (as the zero-points of the copy)
+  // group's zero-points 8 bytes longer (bank conflicts)
   static constexpr int VZROW = TT / 2 * 4 + 8, VZ = NG * (TT / 2) * 4;
-  static constexpr int VL = VZ + NG * VZROW;
-  static constexpr int VROOM = ((CENTERED ? VL + NG * VZROW : VL) + 15) / 16 * 16;
+  static constexpr int VROOM = (VZ + NG * VZROW + 15) / 16 * 16;
   static_assert(VROOM >= VM, "the copy fits");
   // numerators: [head][tile of 16 tokens][pair of tokens (t, t + 2)] of (hi pair, lo pair), 16 bytes more after every
   // tile and 32 more after every head against bank conflicts (WIDE: 16-byte cells in an order without any).  Two layers:
@@ -96,28 +93,24 @@ struct Plan {
   static constexpr bool P_OVER = NL == 2;
   static constexpr int OFF_V = 16 * D, OFF_KM = 2 * 16 * D;
   static constexpr int OFF_VM = OFF_KM + (P_OVER && NL * KM < PBUF ? PBUF : NL * KM);
-  static constexpr int OFF_KL = OFF_VM + NL * VROOM, KL = CENTERED ? NGT * 2 * D : 0;
-  static constexpr int OFF_P = P_OVER ? OFF_KM : (OFF_KL + KL + 127) / 128 * 128;
+  static constexpr int OFF_P = P_OVER ? OFF_KM : (OFF_VM + NL * VROOM + 127) / 128 * 128;
   static_assert(OFF_P % 128 == 0, "cells are found by exclusive or");
   static constexpr int WROW = 2 * D + 16;        // a staged window row
   static constexpr int WIN = 32 * WROW;          // 16 key rows, then 16 value rows (over the stage of the warp)
-  static constexpr int BODY = P_OVER ? OFF_KL + KL : OFF_P + PBUF;
+  static constexpr int BODY = P_OVER ? OFF_VM + NL * VROOM : OFF_P + PBUF;
   static constexpr int WARP = ((BODY > WIN ? BODY : WIN) + 127) / 128 * 128;
   static constexpr int MS = D + 4;               // state row: acc[D], m, l
   static_assert(2 * VH * MS * 4 <= WARP, "a warp's state rows, of the packed tokens and of the window, fit its own memory");
   static_assert(MS % 4 == 0, "state rows are read as vectors");
-  // after the warps' parts: B fragments of the zero-point products; q as it came; with head_dim 128 q as operand
-  // fragments, for all warps (else each keeps them in registers)
-  static constexpr int QB = NSET * KS * 32 * 4, QS = VH * D * 2;
-  static constexpr bool Q_SHARED = D == 128;
-  static constexpr int QF = Q_SHARED ? KS * 32 * 8 : 0;
+  // after the warps' parts: B fragments of the zero-point products; q as it came; q as operand fragments
+  static constexpr int QB = NSET * KS * 32 * 4, QS = VH * D * 2, QF = KS * 32 * 8;
   static constexpr int room(int w) { return w * WARP + QB + QS + QF; }
   // PARK: the value sums of a warp wait in tensor memory between its rounds, 4 columns a row tile (WIDE: 4 more, of the lo
   // products): three CTAs per SM, each of eight warps of 80 registers.  Else two CTAs, of eight warps of 128 registers.
   // With eight heads the sums (64 registers) would not fit otherwise; two layers of one head, 4k, batch 8: 640 us a step
   // without, 622 with.  One layer alone, up to four heads: tensor memory costs a CTA 1.2 us at its start and end (a call
   // at 32k 37.0 us with, 35.2 without).
-  static constexpr bool PARK = (WIDE || NL == 2) && D == 128;
+  static constexpr bool PARK = WIDE || NL == 2;
   static constexpr int CTAS = PARK ? 3 : 2, WARPS = 8;
   static constexpr int TCOLS = KS * 4 * NCOL, TMEM = WARPS / 4 * TCOLS;
   static_assert(!PARK || (CTAS * TMEM <= 512 && (TMEM & (TMEM - 1)) == 0), "tensor memory");
@@ -126,67 +119,40 @@ struct Plan {
   static_assert(WARPS * WARP >= VH * (256 + 1) * 4, "the merge's weights");
 };
 
-// Code operands.  head_dim 128: the masked code bits as they are, fp16 subnormals code * weight * 2^-22.  head_dim 64:
-// (code - center) * weight * 2^-9, normal numbers, center = (2^BITS - 1) / 2, and zero-points plus center scales, as
-// pairs of fp16, in place of the zero-points: both sums are then as small as the result, and no digit of it is lost where
-// they cancel.  That makes the kernel as exact as the scalar one, which served head_dim 64 before it (fp32 result against
-// fp64, of its norm: scalar 3.6-5.5e-7, this one 4.7-5.6e-7, with operands as for head_dim 128 1.0-2.5e-5) and costs a
-// layer of a step 0.4 us (2.8 to 3.3 us at 2048 tokens, 32 streams, four heads; scalar 500).
-template <int D>
-struct Code {
-  static constexpr bool CENTERED = D == 64;
-  template <int BITS>
-  static __device__ __forceinline__ float center() { return 0.5f * (float)((1 << BITS) - 1); }
-  // the operand pair of the code bits at BASE + BITS * i of both halves of w; their weight is 2^(BITS * i)
-  template <int BITS, int BASE>
-  static __device__ __forceinline__ uint32_t pair(uint32_t w, int i) {
-    const uint32_t m = w & (((BITS == 2 ? 0x00030003u : 0x00010001u) << BASE) << (BITS * i));
-    if constexpr (CENTERED) {
-      // times 2^(15 - BASE), less center * weight * 2^-9: 1.5 or 0.5 at exponent field 15 - 9 + BITS * i
-      const uint32_t c = BITS == 2 ? 0x8200u + ((uint32_t)(6 + 2 * i) << 10) : 0x8000u + ((uint32_t)(5 + i) << 10);
-      return hfma2(m, ((uint32_t)(30 - BASE) << 10) * 0x10001u, c * 0x10001u);
-    } else {
-      return m;
-    }
-  }
-  // exponent of the operand of a code with weight 1
-  static __host__ __device__ constexpr int exp(int base) { return CENTERED ? 9 : 24 - base; }
-};
-// z + center s of a pair of groups as an unevaluated sum of two fp16
-template <int D, int BITS>
-__device__ __forceinline__ void centered_zero(uint32_t s, uint32_t z, uint32_t& hi, uint32_t& lo) {
-  const float a = fmaf(Code<D>::template center<BITS>(), io2_lo<true>(s), io2_lo<true>(z));
-  const float b = fmaf(Code<D>::template center<BITS>(), io2_hi<true>(s), io2_hi<true>(z));
-  hi = pack_io2<true>(a, b);
-  lo = pack_io2<true>(a - io2_lo<true>(hi), b - io2_hi<true>(hi));
+// The code operand pair: the code bits at BASE + BITS * i of both halves of w as they are, fp16 subnormals; their weight is
+// 2^(BITS * i), a code of weight 1 stands for 2^-code_exp(BASE)
+template <int BITS, int BASE>
+__device__ __forceinline__ uint32_t code_pair(uint32_t w, int i) {
+  return w & (((BITS == 2 ? 0x00030003u : 0x00010001u) << BASE) << (BITS * i));
 }
+__host__ __device__ constexpr int code_exp(int base) { return 24 - base; }
 
 // log2 of the weight that the code of k-slot (step ks, any tig, any pair) carries in its operand
-template <int D, int BK>
-__device__ __forceinline__ constexpr int k_weight(int ks) { return BK == 2 ? 2 * (ks % 4) : (D == 128 ? ks : ks % 4); }
+template <int BK>
+__device__ __forceinline__ constexpr int k_weight(int ks) { return BK == 2 ? 2 * (ks % 4) : ks; }
 // channel of k-slot c (pairs (0, 2) and (1, 3)) of step ks for lane column tig
-template <int D, int BK>
+template <int BK>
 __device__ __forceinline__ int k_channel(int ks, int tig, int c) {
-  if constexpr (BK == 1 && D == 128) return 32 * tig + 4 * ks + c;
+  if constexpr (BK == 1) return 32 * tig + 4 * ks + c;
   else return 16 * (tig + 4 * (ks / 4)) + 4 * (ks % 4) + c;
 }
 // Halfword index, inside a key group's D reordered scales, of channel d: per lane column and two k-steps one 16-byte
 // vector [step][pair (c, c + 2), pair (c + 1, c + 3)].
-template <int D, int BK>
+template <int BK>
 __device__ __forceinline__ int k_slot(int d) {
   int tig, ks;
   const int c = d & 3;
-  if constexpr (BK == 1 && D == 128) { tig = d >> 5; ks = (d >> 2) & 7; }
+  if constexpr (BK == 1) { tig = d >> 5; ks = (d >> 2) & 7; }
   else { tig = (d >> 4) & 3; ks = 4 * (d >> 6) + ((d >> 2) & 3); }
   return ((ks >> 1) * 4 + tig) * 8 + (ks & 1) * 4 + (c & 1) * 2 + (c >> 1);
 }
 // k_slot of channel d + 32 j less that of channel d < 32
-template <int D, int BK>
-__device__ __forceinline__ constexpr int k_slot_step(int j) { return BK == 1 && D == 128 ? 8 * j : 16 * (j & 1) + 64 * (j >> 1); }
+template <int BK>
+__device__ __forceinline__ constexpr int k_slot_step(int j) { return BK == 1 ? 8 * j : 16 * (j & 1) + 64 * (j >> 1); }
 
 // One warp stages window tokens [tb, tb + 16) (rows at or beyond t1 are zero-filled); no commit.  With a fused
 // append the newest row (index r - 1) is not in the window yet: it comes from the step's input.
-template <int D, int WROW>
+template <int WROW>
 __device__ __forceinline__ void window_stage(const DecodeParams& p, const DecodeLayer& L, int tb, int t1, int bh,
                                              uint32_t wbuf, int lane) {
   const size_t row0 = (size_t)bh * p.dm.R;
@@ -216,7 +182,7 @@ __device__ __forceinline__ void window_stage(const DecodeParams& p, const Decode
 
 // Fused append: the staged tile [tb, tb + 16) holds the token of this step (row r - 1); the warp stores it into the
 // window, keys by lanes 0..15, values by lanes 16..31.
-template <int D, int WROW>
+template <int WROW>
 __device__ __forceinline__ void window_store_new(const DecodeParams& p, const DecodeLayer& L, int tb, int bh,
                                                  uint32_t wbuf, int lane) {
   const int row = p.r - 1 - tb, c = lane & 15;
@@ -230,7 +196,7 @@ __device__ __forceinline__ void window_store_new(const DecodeParams& p, const De
 // One warp folds the staged tile (n_valid of its 16 tokens exist) into the softmax state of four heads (head of a
 // thread: tig; the operand's odd columns are zero): S^T = K q^T with tokens as rows, O^T += V^T P.
 // o: this thread's channels 16 mt + gid and + 8 of its head; m, l: its head's reference and sum.
-template <int D, int WROW, bool F16>
+template <int WROW, bool F16>
 __device__ __forceinline__ void window_tile(uint32_t wbuf, int n_valid, const uint16_t* qrow, bool real, float scale2,
                                             float (&o)[D / 16][2], float& m, float& l, int lane) {
   constexpr int KS = D / 16;
@@ -280,7 +246,6 @@ __device__ __forceinline__ void window_tile(uint32_t wbuf, int n_valid, const ui
 }
 
 // four channels c .. c + 3 of query head hq's result
-template <int D>
 __device__ __forceinline__ void store_out(const DecodeParams& p, const DecodeLayer& L, size_t hq, int c, float4 v) {
   if (p.out_f32) {
     *reinterpret_cast<float4*>(reinterpret_cast<float*>(L.out) + hq * D + c) = v;
@@ -298,7 +263,7 @@ __device__ __forceinline__ void store_out(const DecodeParams& p, const DecodeLay
 // What it takes is two trips to L2, one for all (m, l) and one for the partials: a warp that went through its share of
 // the heads one after the other, both trips for each, made it 2.3 us with four heads and 5.1 us with eight.
 // L, part_acc, part_ml: of the first of the CTA's NL layers; weights: NL * G * (ns + 1) floats of shared memory.
-template <int D, int NL>
+template <int NL>
 __device__ __forceinline__ void ticket_merge(const DecodeParams& p, const DecodeLayer* L, int ns, int hk, int b,
                                              const float* part_acc, const float* part_ml, unsigned* ticket, int* s_flag,
                                              float* weights) {
@@ -367,24 +332,23 @@ __device__ __forceinline__ void ticket_merge(const DecodeParams& p, const Decode
     }
     const float inv = w[ns];
     const int l = NL == 1 || v < dm.G ? 0 : 1;
-    store_out<D>(p, L[l], hq0 + (v - l * dm.G), c, make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv));
+    store_out(p, L[l], hq0 + (v - l * dm.G), c, make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv));
   }
   if (threadIdx.x == 0) *ticket = 0u;  // ready for the next launch on this stream
 }
 
-template <int D, int BK, int BV, int GS, int HP, int NL>
-__global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<D, BK, BV, GS, HP, NL>::CTAS)
+template <int BK, int BV, int GS, int HP, int NL>
+__global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK, BV, GS, HP, NL>::CTAS)
     decode_mma_kernel(const __grid_constant__ DecodeParams p) {
-  using Pl = Plan<D, BK, BV, GS, HP, NL>;
-  using Cd = Code<D>;
+  using Pl = Plan<BK, BV, GS, HP, NL>;
   constexpr bool WIDE = Pl::WIDE;
   constexpr int KS = Pl::KS, NG = Pl::NG, NGT = Pl::NGT, W = Pl::WARPS, WROW = Pl::WROW, GC = Pl::GC, CP = Pl::CP;
   constexpr int VH = Pl::VH, SH = Pl::SH, NSET = Pl::NSET, NCOL = Pl::NCOL, NE = Pl::NE;
-  constexpr int KWORDS = (BK == 2 && D == 128) ? 2 : 1;  // packed words of a token row that a thread expands
+  constexpr int KWORDS = BK == 2 ? 2 : 1;  // packed words of a token row that a thread expands
   // Where the codes of an operand begin in its halves.  VWIN: quads of tokens (k-steps e) whose value codes one shift of a
   // word puts in place, with weights 2^(BV * (e % VWIN)); 2-bit codes, as far as their sums are limited by the zeros ahead
   // of them, in two shifts.
-  constexpr int VWIN = BV == 2 && !Code<D>::CENTERED ? 2 : 4;
+  constexpr int VWIN = BV == 2 ? 2 : 4;
   constexpr int KBASE = 2, VBASE = BV == 2 ? (VWIN == 2 ? 6 : 2) : 4;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) unsigned long long bar_mem[2 * W];
@@ -533,10 +497,10 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
     }
     sts64(qb + ((i >> 1) * 32 + lane) * 16 + (i & 1) * 8, pack_io2<true>(v[0], v[1]), pack_io2<true>(v[2], v[3]));
   }
-  if constexpr (Pl::Q_SHARED) {  // largest |q| in [2^14, 2^15); the key scales carry the rest of the exponent
+  {  // largest |q| in [2^14, 2^15); the key scales carry the rest of the exponent
     for (int ks = warp; ks < KS; ks += W) {
-      const float e2 = pow2i(eq_sm[col_head] + 14 - k_weight<D, BK>(ks));
-      const uint2 v = *reinterpret_cast<const uint2*>(q_sm + col_head * D + k_channel<D, BK>(ks, tig, 0));
+      const float e2 = pow2i(eq_sm[col_head] + 14 - k_weight<BK>(ks));
+      const uint2 v = *reinterpret_cast<const uint2*>(q_sm + col_head * D + k_channel<BK>(ks, tig, 0));
       sts64(qf + ks * 256, pack_io2<true>(io_to_f(v.x & 0xffffu, p.f16) * e2, io_to_f(v.y & 0xffffu, p.f16) * e2),
             pack_io2<true>(io_to_f(v.x >> 16, p.f16) * e2, io_to_f(v.y >> 16, p.f16) * e2));
     }
@@ -550,54 +514,34 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
   const float cz = WIDE ? p.scale * 1.4426950408889634f * pow2i(-eq_sm[4 * (lane >> 4) + tig]) : cq[0];
 
   const uint32_t low_mask = low ? 0xffffffffu : 0u;
-  // q of this lane's operand column as fp16 pairs, times 2^Ek and divided by the weights of the codes (head_dim 64)
-  uint32_t qk[Pl::Q_SHARED ? 1 : KS][2];
-  int Ek = -100;  // not set
-  // With Q_SHARED the scales are taken times 2^Ek of their layer instead: ek2, a pair of fp16 (0: not set).
+  // key scales are taken times 2^Ek of their layer: ek2, a pair of fp16 (0: not set)
   uint32_t ek2[NL];
   float ck[NCOL];
 #pragma unroll
   for (int j = 0; j < NCOL; ++j) ck[j] = 0.f;
   auto set_unit = [&](int l, int e) {
-    const float unit = pow2i(Cd::exp(KBASE) - e);
+    const float unit = pow2i(code_exp(KBASE) - 14 - e);
 #pragma unroll
     for (int j = 0; j < NCOL; ++j) ck[j] = NL == 1 || my_layer == l ? cq[j] * unit : ck[j];
   };
-  auto set_ek = [&](int e) {
-    Ek = e;
-    set_unit(0, e);
-    const int eh = e + eq_sm[col_head];
-#pragma unroll
-    for (int ks = 0; ks < (Pl::Q_SHARED ? 0 : KS); ++ks) {
-      const float e2 = pow2i(eh - k_weight<D, BK>(ks));
-      const uint2 v = *reinterpret_cast<const uint2*>(q_sm + col_head * D + k_channel<D, BK>(ks, tig, 0));
-      qk[ks][0] = pack_io2<true>(io_to_f(v.x & 0xffffu, p.f16) * e2, io_to_f(v.y & 0xffffu, p.f16) * e2);
-      qk[ks][1] = pack_io2<true>(io_to_f(v.x >> 16, p.f16) * e2, io_to_f(v.y >> 16, p.f16) * e2);
-    }
-  };
-  auto q_pair = [&](int ks) {
-    if constexpr (Pl::Q_SHARED) return lds64(qf + ks * 256);
-    else return make_uint2(qk[ks][0], qk[ks][1]);
-  };
+  auto q_pair = [&](int ks) { return lds64(qf + ks * 256); };
 
   // Softmax state of the heads of this thread's columns: reference mr (log2 units, an integer; 0 until the first round
   // sets it).  Value sums acc (PARK: in tensor memory between the rounds): of row tile mt the products' four (WIDE: of hi,
   // then of lo).  zacc[part]: rows gid: the zero-point products of layer gid / 4, channel group gid % 4 (one layer: gid % NG), rows
-  // 8 and up: the sum of the numerators (with centered codes lsum, of this thread's tokens); columns hi and lo (WIDE:
-  // columns heads, hi and lo apart).
+  // 8 and up: the sum of the numerators; columns hi and lo (WIDE: columns heads, hi and lo apart).
   const uint32_t t_acc = Pl::PARK ? tmem_base_sm + ((uint32_t)(warp & 3) << 21) + (warp >> 2) * Pl::TCOLS : 0u;
   float acc[Pl::PARK ? 1 : KS * NCOL][4];
   constexpr int MT = GC * KS / CP;                          // row tiles of a channel part of the value products
   // that are taken at a time (eight heads: one; with two, 80 bytes more of spills at groups of 64, 724 us a step for 705 at 8k); their columns
   constexpr int MTS = MT < 2 || WIDE ? 1 : 2, TV = MTS * 4 * NCOL;
-  float mr[NCOL], zacc[NCOL][4], lsum[NCOL];
+  float mr[NCOL], zacc[NCOL][4];
   uint32_t ev2[NL];  // value scales are taken times 2^Ev: a pair of fp16 (0: not set)
 #pragma unroll
   for (int l = 0; l < NL; ++l) ek2[l] = ev2[l] = 0u;
 #pragma unroll
   for (int j = 0; j < NCOL; ++j) {
     mr[j] = 0.f;
-    lsum[j] = 0.f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) zacc[j][i] = 0.f;
   }
@@ -636,12 +580,12 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
   const unsigned my_lanes = my_layer == 0 ? layer0 : ~layer0;  // lanes with heads of this thread's layer
   // weight of the codes of this lane's tokens in the value words (the token of row gid is in quad (gid >> 1) of its tile)
   const int wt = BV * ((gid >> 1) % VWIN);
-  const float off = (float)(P_EXP - wt), weight = pow2i(wt);
+  const float off = (float)(P_EXP - wt);
   const int tok0 = 4 * (gid >> 1) + (gid & 1);                       // token of row gid, tile 0; the other rows: + 2, + 16
   const uint32_t kz_lane = st + Pl::OFF_KM + (gid & (NGT - 1)) * 4 * D + 2 * D + (gid >> 2) * D + tig * 16;  // zero-points of its row
   const uint32_t qb_lane = qb + lane * 16;
-  const uint32_t kc_lane = st + tok0 * (BK == 1 && D == 64 ? 8 : 16) + (BK == 1 && D == 64 ? (tig >> 1) : tig) * 4;
-  const uint32_t km_read = st + Pl::OFF_KM + lane * (D / 16), km_write = st + Pl::OFF_KM + 2 * k_slot<D, BK>(lane);
+  const uint32_t kc_lane = st + tok0 * 16 + tig * 4;
+  const uint32_t km_read = st + Pl::OFF_KM + lane * (D / 16), km_write = st + Pl::OFF_KM + 2 * k_slot<BK>(lane);
   const uint32_t km_lane = st + Pl::OFF_KM + (NL == 2 ? col_layer * Pl::KM : 0) + tig * 16;
   // Lane column tig owns the tokens 16 tig ... of a round in the value products: in 2 bits word tig of a channel's chunk,
   // in 1 bit a half of word tig / 2 (of the two that this half of the batch has), shifted so that its codes begin at bit
@@ -682,12 +626,8 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
       auto read = [&]() {
 #pragma unroll
         for (int g = 0; g < NGT; ++g) {
-          if constexpr (V == 4) {
-            const uint2 x = lds64(km_read + l * Pl::KM + g * 4 * D);
-            s[g][0] = x.x; s[g][1] = x.y;
-          } else {
-            s[g][0] = lds32(km_read + l * Pl::KM + g * 4 * D);
-          }
+          const uint2 x = lds64(km_read + l * Pl::KM + g * 4 * D);
+          s[g][0] = x.x; s[g][1] = x.y;
         }
       };
       auto scale = [&]() {
@@ -705,45 +645,28 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
         return redux_max_u32(max(mx & 0xffffu, mx >> 16));
       };
       read();
-      if constexpr (Pl::Q_SHARED) {
-        // The largest scale of the round times 2^Ek in [2^-4, 1): |q s| below 2^15, and a scale keeps its 11 bits down to
-        // 2^-10 of the largest.  Ek moves only outside that, and no further than 15.
-        bool moved = r == 0;
-        if (r > 0) {
-          scale();
-          moved = largest() - 0x2c00u >= 0x1000u;
-          if (moved) read();
-        }
-        if (moved) {
-          const float smax = f16_to_f(largest());
-          const int es = smax > 0.f ? exponent_of(smax) : -24, e = min(15, -1 - es);
-          const float f = pow2i(e);
-          ek2[l] = pack_io2<true>(f, f);
-          set_unit(l, 14 + e);
-          scale();
-        }
-      } else {
-        // |q s| below 2^15 and its largest at least 2^8 (where 2^14 |q| allows): exponents of q move only outside that
-        const float smax = f16_to_f(largest());
-        const int es = smax > 0.f ? exponent_of(smax) : -24;
-        if (es > 13 - Ek || (es < 7 - Ek && Ek < 14) || Ek == -100) set_ek(min(14, 13 - es));
+      // The largest scale of the round times 2^Ek in [2^-4, 1): |q s| below 2^15, and a scale keeps its 11 bits down to
+      // 2^-10 of the largest.  Ek moves only outside that, and no further than 15.
+      bool moved = r == 0;
+      if (r > 0) {
+        scale();
+        moved = largest() - 0x2c00u >= 0x1000u;
+        if (moved) read();
       }
-      if constexpr (Cd::CENTERED) {
-#pragma unroll
-        for (int g = 0; g < NGT; ++g) {
-          const uint32_t a = km_read + g * 4 * D + 2 * D;
-          uint32_t hi, lo;
-          centered_zero<D, BK>(s[g][0], lds32(a), hi, lo);
-          sts32(a, hi);
-          sts32(st + Pl::OFF_KL + g * 2 * D + lane * 4, lo);
-        }
+      if (moved) {
+        const float smax = f16_to_f(largest());
+        const int es = smax > 0.f ? exponent_of(smax) : -24, e = min(15, -1 - es);
+        const float f = pow2i(e);
+        ek2[l] = pack_io2<true>(f, f);
+        set_unit(l, e);
+        scale();
       }
       __syncwarp();
 #pragma unroll
       for (int g = 0; g < NGT; ++g)
 #pragma unroll
         for (int j = 0; j < V; ++j)
-          sts16(km_write + l * Pl::KM + g * 4 * D + 2 * k_slot_step<D, BK>(j), j & 1 ? s[g][j / 2] >> 16 : s[g][j / 2]);
+          sts16(km_write + l * Pl::KM + g * 4 * D + 2 * k_slot_step<BK>(j), j & 1 ? s[g][j / 2] >> 16 : s[g][j / 2]);
     }
     __syncwarp();
     // Logits x[n][r][j] of row gid + 8 r (tokens 2 r further) of tile tile_of(n), head my_head + j; less the reference and
@@ -762,16 +685,11 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
 #pragma unroll
       for (int n = 0; n < (WIDE ? NSET : NL); ++n) {
         const int l = NL == 2 ? n : 0, set = WIDE ? n : 0;
-        const uint32_t za = kz_lane + l * Pl::KM, zl = st + Pl::OFF_KL + (gid & (NGT - 1)) * 2 * D + (gid >> 2) * D + tig * 16;
+        const uint32_t za = kz_lane + l * Pl::KM;
 #pragma unroll
         for (int kp = 0; kp < KS / 4; ++kp) {
           const uint4 a = lds128(za + kp * 64);
           const uint4 q = lds128(qb_lane + (set * KS / 4 + kp) * 512);
-          if constexpr (Cd::CENTERED) {
-            const uint4 c = lds128(zl + kp * 64);
-            mma_f16(zc[n], c.x, c.y, c.z, c.w, q.x, q.z);
-            mma_f16(zd[n], c.x, c.y, c.z, c.w, q.y, q.w);
-          }
           mma_f16(zc[n], a.x, a.y, a.z, a.w, q.x, q.z);
           mma_f16(zd[n], a.x, a.y, a.z, a.w, q.y, q.w);
         }
@@ -794,14 +712,12 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int tk = 16 * t + 2 * h;
-          uint32_t raw;
-          if constexpr (BK == 1 && D == 64) raw = lds32(kc_lane + u * 256 + tk * 8) >> (4 * (tig & 1));
-          else raw = lds32(kc_lane + u * (32 * D * BK / 8) + kw * 512 + tk * 16);
+          const uint32_t raw = lds32(kc_lane + u * (32 * D * BK / 8) + kw * 512 + tk * 16);
           w[t][h] = byte_pair_up(raw, 2);
           w8[t][h] = byte_pair_down(raw, 6);
         }
     };
-    auto key_pair = [](uint32_t w, int k) { return Cd::template pair<BK, KBASE>(w, BK == 2 ? k & 3 : k); };
+    auto key_pair = [](uint32_t w, int k) { return code_pair<BK, KBASE>(w, BK == 2 ? k & 3 : k); };
     constexpr int KPW = KS / KWORDS;  // k-steps a word serves
     if constexpr (WIDE) {
 #pragma unroll
@@ -980,7 +896,6 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
       if (r > 0) {  // (else nothing has been accumulated yet)
 #pragma unroll
         for (int j = 0; j < NCOL; ++j) {
-          lsum[j] *= f[j];
 #pragma unroll
           for (int k = 0; k < 4; ++k)
             if constexpr (WIDE) zacc[k & 1][2 * (k >> 1) + j] *= f[j];
@@ -995,7 +910,6 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
 #pragma unroll
       for (int n = 0; n < NE; ++n) {
         const float pa = ex2(x[n][0][j]), pb = ex2(x[n][1][j]);
-        if constexpr (Cd::CENTERED) lsum[j] = fmaf(pa + pb, weight, lsum[j]);
         const uint32_t h = pack_io2<true>(pa, pb);
         const uint32_t lo = pack_io2<true>(pa - io2_lo<true>(h), pb - io2_hi<true>(h));
         if constexpr (WIDE) sts64(p_st ^ ((n << 1 | j) << 4), h, lo);
@@ -1014,26 +928,20 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
       uint32_t sp[NG], zp[NG];
       {  // raw rows of the two tokens: NG scales, NG zero-points
         const uint32_t a = vm_read + l * Pl::VROOM;
-        if constexpr (NG == 1) {
-          const uint32_t ra = lds32(a), rb = lds32(a + 8);
-          sp[0] = __byte_perm(ra, rb, 0x5410);
-          zp[0] = __byte_perm(ra, rb, 0x7632);
+        uint32_t ra[NG], rb[NG];
+        if constexpr (NG == 4) {
+          const uint4 x4 = lds128(a), y4 = lds128(a + 32);
+          ra[0] = x4.x; ra[1] = x4.y; ra[2] = x4.z; ra[3] = x4.w;
+          rb[0] = y4.x; rb[1] = y4.y; rb[2] = y4.z; rb[3] = y4.w;
         } else {
-          uint32_t ra[NG], rb[NG];
-          if constexpr (NG == 4) {
-            const uint4 x4 = lds128(a), y4 = lds128(a + 32);
-            ra[0] = x4.x; ra[1] = x4.y; ra[2] = x4.z; ra[3] = x4.w;
-            rb[0] = y4.x; rb[1] = y4.y; rb[2] = y4.z; rb[3] = y4.w;
-          } else {
-            const uint2 x2 = lds64(a), y2 = lds64(a + 16);
-            ra[0] = x2.x; ra[1] = x2.y; rb[0] = y2.x; rb[1] = y2.y;
-          }
+          const uint2 x2 = lds64(a), y2 = lds64(a + 16);
+          ra[0] = x2.x; ra[1] = x2.y; rb[0] = y2.x; rb[1] = y2.y;
+        }
 #pragma unroll
-          for (int g = 0; g < NG; ++g) {
-            const uint32_t sel = g & 1 ? 0x7632 : 0x5410;
-            sp[g] = __byte_perm(ra[g / 2], rb[g / 2], sel);
-            zp[g] = __byte_perm(ra[NG / 2 + g / 2], rb[NG / 2 + g / 2], sel);
-          }
+        for (int g = 0; g < NG; ++g) {
+          const uint32_t sel = g & 1 ? 0x7632 : 0x5410;
+          sp[g] = __byte_perm(ra[g / 2], rb[g / 2], sel);
+          zp[g] = __byte_perm(ra[NG / 2 + g / 2], rb[NG / 2 + g / 2], sel);
         }
       }
       uint32_t se[NG];
@@ -1067,11 +975,6 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
       __syncwarp();
 #pragma unroll
       for (int g = 0; g < NG; ++g) {
-        if constexpr (Cd::CENTERED) {
-          uint32_t lo;
-          centered_zero<D, BV>(sp[g], zp[g], zp[g], lo);
-          sts32(vm_write + Pl::VL + g * Pl::VZROW, lo);
-        }
         sts32(vm_write + l * Pl::VROOM + g * (TT / 2 * 4), se[g]);
         sts32(vm_write + l * Pl::VROOM + Pl::VZ + g * Pl::VZROW, zp[g]);
       }
@@ -1093,11 +996,6 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
       if constexpr (WIDE) {
         pl[e][0] = hp.y; pl[e][1] = hp.w;
         const uint32_t h0 = hmul2(hp.x, we), h1 = hmul2(hp.z, we), l0 = hmul2(hp.y, we), l1 = hmul2(hp.w, we);
-        if constexpr (Cd::CENTERED) {
-          const uint2 y = lds64(zo + Pl::VL - Pl::VZ);
-          mma_f16(zacc[0], y.x, 0u, y.y, 0u, h0, h1);
-          mma_f16(zacc[1], y.x, 0u, y.y, 0u, l0, l1);
-        }
         mma_f16(zacc[0], z.x, ONES, z.y, ONES, h0, h1);
         mma_f16(zacc[1], z.x, ONES, z.y, ONES, l0, l1);
       } else {
@@ -1105,15 +1003,11 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
         pn[e][0] = (hp.x ^ 0x80008000u) & low_mask; pn[e][1] = (hp.z ^ 0x80008000u) & low_mask;
         pl[e][0] = hp.y & low_mask; pl[e][1] = hp.w & low_mask;
         const uint32_t pz0 = hmul2(low ? hp.y : hp.x, we), pz1 = hmul2(low ? hp.w : hp.z, we);
-        if constexpr (Cd::CENTERED) {
-          const uint2 y = lds64(zo + Pl::VL - Pl::VZ);
-          mma_f16(zacc[0], y.x, 0u, y.y, 0u, pz0, pz1);
-        }
         mma_f16(zacc[0], z.x, ONES, z.y, ONES, pz0, pz1);
       }
     }
     // ---- values: p . c, one channel part after the other ----
-    auto value_pair = [](uint32_t w, int e) { return Cd::template pair<BV, VBASE>(w, e % VWIN); };
+    auto value_pair = [](uint32_t w, int e) { return code_pair<BV, VBASE>(w, e % VWIN); };
     if constexpr (Pl::PARK) tc_wait_st();
 #pragma unroll
     for (int vb = 0; vb < CP / GC; ++vb) {
@@ -1214,11 +1108,11 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
         const DecodeLayer& L = LL[layer];
 #pragma unroll 1
         for (int tb = wt0 + 16 * window_turn(warp); tb < wt1; tb += 16 * W) {
-          window_stage<D, WROW>(p, L, tb, wt1, bh, st, lane);
+          window_stage<WROW>(p, L, tb, wt1, bh, st, lane);
           cp_async_commit();
           cp_async_wait_all();
           __syncwarp();
-          if (L.K_new != nullptr && tb + 16 > p.r - 1 && wt1 == p.r) window_store_new<D, WROW>(p, L, tb, bh, st, lane);
+          if (L.K_new != nullptr && tb + 16 > p.r - 1 && wt1 == p.r) window_store_new<WROW>(p, L, tb, bh, st, lane);
 #pragma unroll
           for (int s = 0; s < NSET; ++s) {
             if (WIDE && NL == 2 && s != layer) continue;
@@ -1230,8 +1124,8 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
             float o2[KS][2], m2 = ms[s], l2 = l[s];
 #pragma unroll
             for (int mt = 0; mt < KS; ++mt) o2[mt][0] = o[s][mt][0], o2[mt][1] = o[s][mt][1];
-            if (p.f16) window_tile<D, WROW, true>(st, wt1 - tb, qrow, real, scale2, o2, m2, l2, lane);
-            else window_tile<D, WROW, false>(st, wt1 - tb, qrow, real, scale2, o2, m2, l2, lane);
+            if (p.f16) window_tile<WROW, true>(st, wt1 - tb, qrow, real, scale2, o2, m2, l2, lane);
+            else window_tile<WROW, false>(st, wt1 - tb, qrow, real, scale2, o2, m2, l2, lane);
             if (mine) {
               ms[s] = m2;
               l[s] = l2;
@@ -1263,17 +1157,12 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
     // the packed tokens, in true units
     if (rounds > 0) {
       const float uz = pow2i(-P_EXP);
-      const float ua = pow2i(Cd::exp(VBASE) - P_EXP - exponent_of(f16_to_f((NL == 2 && my_layer == 1 ? ev2[NL - 1] : ev2[0]) & 0xffffu)));
+      const float ua = pow2i(code_exp(VBASE) - P_EXP - exponent_of(f16_to_f((NL == 2 && my_layer == 1 ? ev2[NL - 1] : ev2[0]) & 0xffffu)));
       float z[NCOL];  // row gid < 4 NL: channel group of a layer
 #pragma unroll
       for (int j = 0; j < NCOL; ++j) {
         z[j] = (WIDE ? zacc[0][j] + zacc[1 % NCOL][j] : zacc[0][0] + zacc[0][1]) * uz;
-        float sum = (WIDE ? zacc[0][2 + j] + zacc[1 % NCOL][2 + j] : zacc[0][2] + zacc[0][3]) * uz;
-        if constexpr (Cd::CENTERED) {
-#pragma unroll
-          for (int k = WIDE ? 4 : VH; k < 32; k <<= 1) lsum[j] += __shfl_xor_sync(0xffffffffu, lsum[j], k);
-          sum = lsum[j] * uz;
-        }
+        const float sum = (WIDE ? zacc[0][2 + j] + zacc[1 % NCOL][2 + j] : zacc[0][2] + zacc[0][3]) * uz;
         if (gid == 0 && my_slot == 0) {
           ws[(my_head + j) * Pl::MS + D] = mr[j];
           ws[(my_head + j) * Pl::MS + D + 1] = sum;
@@ -1358,7 +1247,7 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
     for (int t = wrow0; t < wrow1; ++t) add(row((t + halves) % W, true));
     const size_t hq = (size_t)b * dm.Hq + hk * G + h;
     if (ns == 1) {
-      store_out<D>(p, LL[layer], hq, d, make_float4(A.x / Ls, A.y / Ls, A.z / Ls, A.w / Ls));
+      store_out(p, LL[layer], hq, d, make_float4(A.x / Ls, A.y / Ls, A.z / Ls, A.w / Ls));
     } else {
       const size_t at = ((size_t)layer * dm.B * dm.Hq + hq) * p.ns_q + split;
       *reinterpret_cast<float4*>(part_acc + at * D + d) = A;
@@ -1366,23 +1255,23 @@ __global__ void __launch_bounds__(Plan<D, BK, BV, GS, HP, NL>::WARPS * 32, Plan<
     }
   }
   if (ns > 1)
-    ticket_merge<D, NL>(p, LL, ns, hk, b, part_acc, part_ml, p.tickets + (size_t)blockIdx.y * (dm.B * dm.Hkv) + bh, &s_flag,
+    ticket_merge<NL>(p, LL, ns, hk, b, part_acc, part_ml, p.tickets + (size_t)blockIdx.y * (dm.B * dm.Hkv) + bh, &s_flag,
                         reinterpret_cast<float*>(smem));
 }
 
-template <int D, int BK, int BV, int GS, int HP, int NL>
+template <int BK, int BV, int GS, int HP, int NL>
 cudaError_t launch_one(const DecodeParams& p, cudaStream_t st) {
-  using Pl = Plan<D, BK, BV, GS, HP, NL>;
-  return launch_dependent(decode_mma_kernel<D, BK, BV, GS, HP, NL>, dim3((unsigned)(p.ns_q * p.dm.B * p.dm.Hkv), p.n_layers / NL), dim3(Pl::WARPS * 32),
+  using Pl = Plan<BK, BV, GS, HP, NL>;
+  return launch_dependent(decode_mma_kernel<BK, BV, GS, HP, NL>, dim3((unsigned)(p.ns_q * p.dm.B * p.dm.Hkv), p.n_layers / NL), dim3(Pl::WARPS * 32),
                           (size_t)Pl::TOTAL, st, p);
 }
 
 // Prepares the kernel for the current device and says how many of its CTAs share an SM and how many warps each has.
 // (The occupancy calculator has no say on how many: it answers one for a kernel that allocates tensor memory.)
-template <int D, int BK, int BV, int GS, int HP, int NL>
+template <int BK, int BV, int GS, int HP, int NL>
 MmaShape shape_one() {
-  using Pl = Plan<D, BK, BV, GS, HP, NL>;
-  auto kernel = decode_mma_kernel<D, BK, BV, GS, HP, NL>;
+  using Pl = Plan<BK, BV, GS, HP, NL>;
+  auto kernel = decode_mma_kernel<BK, BV, GS, HP, NL>;
   MmaShape r{Pl::CTAS, Pl::WARPS};
   // the largest shared-memory carve-out: three CTAs of this size are to share an SM
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Pl::TOTAL) != cudaSuccess ||
@@ -1395,25 +1284,25 @@ MmaShape shape_one() {
 
 #define XQ_DISPATCH(FN, ...)                               \
   switch (bk * 100 + bv * 10 + (g == 64)) {                \
-    case 220: return FN<D, 2, 2, 32, HP, NL>(__VA_ARGS__); \
-    case 221: return FN<D, 2, 2, 64, HP, NL>(__VA_ARGS__); \
-    case 210: return FN<D, 2, 1, 32, HP, NL>(__VA_ARGS__); \
-    case 211: return FN<D, 2, 1, 64, HP, NL>(__VA_ARGS__); \
-    case 120: return FN<D, 1, 2, 32, HP, NL>(__VA_ARGS__); \
-    case 121: return FN<D, 1, 2, 64, HP, NL>(__VA_ARGS__); \
-    case 110: return FN<D, 1, 1, 32, HP, NL>(__VA_ARGS__); \
-    case 111: return FN<D, 1, 1, 64, HP, NL>(__VA_ARGS__); \
+    case 220: return FN<2, 2, 32, HP, NL>(__VA_ARGS__); \
+    case 221: return FN<2, 2, 64, HP, NL>(__VA_ARGS__); \
+    case 210: return FN<2, 1, 32, HP, NL>(__VA_ARGS__); \
+    case 211: return FN<2, 1, 64, HP, NL>(__VA_ARGS__); \
+    case 120: return FN<1, 2, 32, HP, NL>(__VA_ARGS__); \
+    case 121: return FN<1, 2, 64, HP, NL>(__VA_ARGS__); \
+    case 110: return FN<1, 1, 32, HP, NL>(__VA_ARGS__); \
+    case 111: return FN<1, 1, 64, HP, NL>(__VA_ARGS__); \
   }
 
 }  // namespace
 
-template <int D, int HP, int NL>
+template <int HP, int NL>
 cudaError_t launch_decode_mma_t(const DecodeParams& p, cudaStream_t st) {
   const int bk = p.layer[0].L.bk, bv = p.layer[0].L.bv, g = p.dm.g;
   XQ_DISPATCH(launch_one, p, st)
   return cudaErrorInvalidValue;
 }
-template <int D, int HP, int NL>
+template <int HP, int NL>
 MmaShape decode_mma_shape_t(int g, int bk, int bv) {
   XQ_DISPATCH(shape_one)
   return MmaShape{0, 1};

@@ -1,7 +1,7 @@
 // Tensor-core decode kernels for head_dim 64, one query head per kv head.
-#include "xq_decode_mma.cuh"
+#include "xq_decode_mma64.cuh"
 
 namespace xq {
-template cudaError_t launch_decode_mma_t<64, 1, 1>(const DecodeParams&, cudaStream_t);
-template MmaShape decode_mma_shape_t<64, 1, 1>(int, int, int);
+template cudaError_t launch_decode_mma64_t<1, 1>(const DecodeParams&, cudaStream_t);
+template MmaShape decode_mma64_shape_t<1, 1>(int, int, int);
 }  // namespace xq

@@ -204,21 +204,16 @@ bool uses_mma(const xq_cache* c) {
   return dm.D == 128 || c->cfg.kernel == XQ_KERNEL_AUTO;  // XQ_KERNEL_MMA names the head_dim 128 kernel
 }
 
-// FN<D, HP, 1> of the tensor-core kernel that serves these dimensions, and FN<128, HP, 2> of the one that takes two layers
-#define XQ_MMA_BY_HEADS(FN, D, ...)                   \
-  (dm.G == 1   ? FN<D, 1, 1>(__VA_ARGS__)             \
-   : dm.G == 2 ? FN<D, 2, 1>(__VA_ARGS__)             \
-   : dm.G <= 4 ? FN<D, 4, 1>(__VA_ARGS__)             \
-               : FN<D, 8, 1>(__VA_ARGS__))
-#define XQ_MMA_OF_PAIRS(FN, ...)                      \
-  (dm.G == 1   ? FN<128, 1, 2>(__VA_ARGS__)           \
-   : dm.G == 2 ? FN<128, 2, 2>(__VA_ARGS__)           \
-               : FN<128, 4, 2>(__VA_ARGS__))
+// FN<HP, 1> of the head_dim 128 kernel that serves these dimensions, FN<HP, 2> of the one that takes two layers, FN<HP, NT>
+// of the head_dim 64 kernel
+#define XQ_MMA128(FN, ...) (dm.G == 1 ? FN<1, 1>(__VA_ARGS__) : dm.G == 2 ? FN<2, 1>(__VA_ARGS__) : dm.G <= 4 ? FN<4, 1>(__VA_ARGS__) : FN<8, 1>(__VA_ARGS__))
+#define XQ_MMA_PAIRS(FN, ...) (dm.G == 1 ? FN<1, 2>(__VA_ARGS__) : dm.G == 2 ? FN<2, 2>(__VA_ARGS__) : FN<4, 2>(__VA_ARGS__))
+#define XQ_MMA64(FN, ...) (dm.G == 1 ? FN<1, 1>(__VA_ARGS__) : dm.G == 2 ? FN<2, 1>(__VA_ARGS__) : dm.G <= 4 ? FN<4, 1>(__VA_ARGS__) : FN<4, 2>(__VA_ARGS__))
 
 cudaError_t launch_decode_mma(const DecodeParams& p, cudaStream_t st) {
   const Dims& dm = p.dm;
-  if (p.paired) return XQ_MMA_OF_PAIRS(launch_decode_mma_t, p, st);
-  return dm.D == 128 ? XQ_MMA_BY_HEADS(launch_decode_mma_t, 128, p, st) : XQ_MMA_BY_HEADS(launch_decode_mma_t, 64, p, st);
+  if (p.paired) return XQ_MMA_PAIRS(launch_decode_mma_t, p, st);
+  return dm.D == 128 ? XQ_MMA128(launch_decode_mma_t, p, st) : XQ_MMA64(launch_decode_mma64_t, p, st);
 }
 
 // Whether the tensor-core kernel can take two layers of a step that read the same codes in one go: the heads of both fit
@@ -231,8 +226,8 @@ MmaShape mma_shape(const xq_cache* c, int l) {
   const int bk = layer_bits(l, c->cfg.kq), bv = layer_bits(l, c->cfg.vq);
   MmaShape& s = const_cast<xq_cache*>(c)->mma_shape[bk - 1][bv - 1];
   if (s.warps == 0) {
-    s = dm.D == 128 ? XQ_MMA_BY_HEADS(decode_mma_shape_t, 128, dm.g, bk, bv) : XQ_MMA_BY_HEADS(decode_mma_shape_t, 64, dm.g, bk, bv);
-    if (takes_pairs(dm)) XQ_MMA_OF_PAIRS(decode_mma_shape_t, dm.g, bk, bv);
+    s = dm.D == 128 ? XQ_MMA128(decode_mma_shape_t, dm.g, bk, bv) : XQ_MMA64(decode_mma64_shape_t, dm.g, bk, bv);
+    if (takes_pairs(dm)) XQ_MMA_PAIRS(decode_mma_shape_t, dm.g, bk, bv);
     s.ctas_per_sm = 2;  // of one wave of a launch alone: the third place is the next launch's
   }
   return s;

@@ -179,17 +179,21 @@ cudaError_t launch_dependent(void (*kernel)(P), dim3 grid, dim3 block, size_t sm
 cudaError_t launch_pack(const PackParams& p, cudaStream_t st);
 cudaError_t launch_window_append(const WindowParams& p, cudaStream_t st);
 cudaError_t launch_decode_generic(const DecodeParams& p, cudaStream_t st);
-// Tensor-core decode kernels for HP (1, 2, 4, 8) query heads per kv head, of one layer or of NL = 2 that read the same
-// codes (head_dim 128, up to four heads).  decode_mma_shape_t also prepares the kernel for the current device: it comes
-// before the first launch of a handle.
+// Tensor-core decode kernels.  head_dim 128: for HP (1, 2, 4, 8) query heads per kv head, of one layer or of NL = 2 that
+// read the same codes (up to four heads); head_dim 64: HP (1, 2, 4) heads, or NT = 2 sets of four.  decode_mma_shape_t
+// also prepares the kernel for the current device: it comes before the first launch of a handle.
 struct MmaShape {
   int ctas_per_sm;  // 0: no device to ask
   int warps;        // warps of a CTA
 };
-template <int D, int HP, int NL>
+template <int HP, int NL>
 cudaError_t launch_decode_mma_t(const DecodeParams& p, cudaStream_t st);
-template <int D, int HP, int NL>
+template <int HP, int NL>
 MmaShape decode_mma_shape_t(int g, int bk, int bv);
+template <int HP, int NT>
+cudaError_t launch_decode_mma64_t(const DecodeParams& p, cudaStream_t st);
+template <int HP, int NT>
+MmaShape decode_mma64_shape_t(int g, int bk, int bv);
 template <int D>
 cudaError_t launch_chunk_t(const ChunkParams& p, cudaStream_t st);
 cudaError_t launch_merge(const MergeParams& p, cudaStream_t st);
