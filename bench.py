@@ -66,7 +66,7 @@ def _config_block(args, w):
             "eta1": args.eta1, "eta2": args.eta2,
             "step": "per layer: append 1 token (+ quantize-and-pack when the window block fills) and decode attention",
             "l2": "inputs larger than L2: every step streams the whole packed cache (GBs against 126 MB of L2); "
-                  "owners-first layer order keeps a pair's shared codes from being re-served by L2"}
+                  "layers that share codes are decoded in pairs and read them once, bytes count them for each layer"}
 
 
 def _peaks():

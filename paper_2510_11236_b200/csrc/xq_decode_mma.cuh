@@ -1,47 +1,46 @@
-// Tensor-core decode attention over the packed cache: one CTA takes a range of batches of one (layer, sequence, kv
-// head) stream, up to 8 query heads.
+// Tensor-core decode attention over the packed cache, head_dim 128: one CTA takes a range of batches of one (sequence, kv
+// head) stream, up to 8 query heads, of one layer or of two that read the same codes (up to four heads each).
 //
-// Every warp works alone on batches of 128 tokens: nothing in the loop waits for another warp.  Codes are expanded
-// straight into A fragments of mma.sync.m16n8k16 (fp16): four codes of a row sit at one bit offset of the four bytes
-// of a packed word, so `word << 2 & 0x000c000c << 2e` is a pair of fp16 subnormals, code * 4^e * 2^-22, for one logic
-// instruction per two codes (and a shift per word: the tensor core aligns a product by the exponent fields of its
-// operands, so every leading zero of a subnormal costs the sum a bit; codes at the very foot of the fraction, without
-// the shift, put the fp32 results four to seven times farther off: 4.2e-4 of the result's norm at 32k, 2-bit, now
-// 0.6e-4; multiplying them up into normal numbers, 0.3e-4, costs 17 % of the time, the shift 1.5 %).  Scale and
-// zero-point are folded out of the inner products,
+// Every warp works alone on half batches of 64 tokens (rounds): nothing in the loop waits for another warp.  Codes are
+// expanded straight into A fragments of mma.sync.m16n8k16 (fp16): four codes of a row sit at one bit offset of the four
+// bytes of a packed word, so a shift of the word and a mask give a pair of fp16 subnormals, code * weight * 2^-e.  (The
+// tensor core aligns a product by the exponent fields of its operands, so every leading zero of a subnormal costs the sum
+// a bit.  Keys: codes from the third bit of the fraction up; values: 1 bit from the fifth up, 2 bits in two shifts from the
+// seventh up, which with one shift left the fp32 results at 2.2 to 6.9e-5 of the result's norm, now 0.3 to 1.4e-5.)
+// Scale and zero-point are folded out of the inner products,
 //
 //   q . k_hat_t = sum_d (q_d s_d) c_td + sum_d q_d z_d        (keys, per channel)
 //   sum_t p_t v_hat_td = sum_t (p_t s_tg) c_td + sum_t p_t z_tg  (values, per token)
 //
-// and the other operand (q_d s_d, or p_t s_tg) is carried as an unevaluated sum hi + lo of two fp16 numbers in two of
-// the eight operand columns: hi = RN(q s), lo = fma(q, s, -hi), as far as fp16 reaches: relative to the largest product
-// of a batch, which is kept between 2^8 and 2^15 (2^9 with 1-bit keys, whose weights come off q), nothing above 2^-33 is lost
-// (p_t s_t: one rounding at 2^-22).  Codes are exact, accumulation is fp32 with the digits that the alignment above
-// leaves: for head_dim 128 this, not the operands, is what limits the result (16 bits and more of each sum; scale and
-// zero-point parts are large and cancel).  The powers of two that the bit offsets put on the codes are taken out of q
-// and of the softmax numerators.  The m16n8 accumulator gives a thread the hi and lo sums of its own head: a logit is
-// their sum, and each (token, head) has one thread.  The numerators go through a small buffer of the warp in shared
-// memory to become B fragments.
+// and the other operand (q_d s_d, or p_t s_tg) is carried as an unevaluated sum hi + lo of two fp16 numbers: hi = RN(q s),
+// lo = fma(q, s, -hi), as far as fp16 reaches: relative to the largest product of a round, which is kept between 2^8 and
+// 2^15 (2^9 with 1-bit keys, whose weights come off q), nothing above 2^-33 is lost (p_t s_t: one rounding at 2^-22).
+// Codes are exact, accumulation is fp32.  The powers of two that the bit offsets put on the codes are taken out of q and of
+// the softmax numerators.  Up to four heads of a CTA: hi and lo are two of the eight operand columns, and the lo sums are
+// added at the end.  Eight heads (five to eight of a layer, or three or four of each of two layers): a column is a head, hi
+// and lo are operands of two products with the same A fragment.  A sum does not depend on the column that it is in, so a
+// layer has the same bits alone and in a pair.  The numerators go through a small buffer of the warp in shared memory to
+// become B fragments.
+//
+// Why two layers at once.  Layers of a pair differ in scales and zero-points alone, and expanding the codes was a quarter
+// of the work; with eight columns of heads each lane also makes both parts of its own product, where with four heads half
+// of the lanes made hi and half lo.  us of a layer in a step of 32, before and after: four heads at 32k, batch 4 27.9 ->
+// 21.9; one head at 4k, batch 8 27.6 -> 19.0; groups of 64, 8k, batch 16 26.3 -> 21.4; one sequence of 128k 27.2 -> 21.7;
+// five heads at 16k (one layer, eight columns) 32.1 -> 23.7, six warps then.
 //
 // Why mma.sync and not tcgen05.  At this shape (at most 8 query heads against 128 channels) the expanded codes are the
 // large operand; a tcgen05 kernel has to pass them through tensor memory and hand batches between warps, and one that
 // did spent a batch's ~1600 cycles on that chain of hand-overs, two batches per SM at a time (32k context, four heads:
-// 34.2 us per layer).  Here sixteen independent warps share an SM and hide each other's latencies.  A layer of a step of 16
-// (layers share launches), us, that kernel -> this one, with the splits that plan_batches gives both kinds of call: 32k
-// context, four heads, batch 4 34.2 -> 26.5 (84 MB: 3.2 TB/s); 4k, one head per kv head, batch 8 27.9 -> 23.1; 8k,
-// groups of 64, batch 16 32.3 -> 24.7; one sequence of 128k 34.8 -> 27.5; groups of five heads at 16k 33.1 -> 28.6, of
-// eight at 32k 37.0 -> 28.4; head_dim 64, 2048 tokens, 32 streams (the scalar kernel: 500) 2.6.
-// What bounds it: issue and latency of a batch's phases.  A batch (four heads, 32-token groups) is ~2000 warp
-// instructions, 512 of them the masks (ALU: 2 cycles each per sub-partition), 140 products (8 cycles each), ~350
-// half-precision multiplies (2 cycles each), and takes a warp ~14000 cycles with sixteen on the SM: key products 2900,
-// value products 3100, waits for copies and their issue 1700, key scales 1600, softmax 1400, value scales 1000,
-// biases 700 (with q in registers; q in shared memory took 3 % off).  A CTA's start and end cost 5000 each, which is
-// why a step wants few CTAs.  Registers: 128 a thread, 168 with two sets of heads; at head_dim 128 up to 28 bytes of
-// spills with one set, 96 to 256 with two.
-// Measured and not kept (32k context, four heads, us per 32 layers; this shape 925 then): four CTAs of 4 warps 944,
-// three of 4 1014, three of 5 1025, one of 12 1026 (fewer registers do not pay for more warps, nor fewer warps for
-// more registers).  Two sets of heads with 7 warps (146 registers) instead of 6: 40.0 us against 31.9 (groups of five
-// at 16k, eight splits).  The window's rows asked into L2 at the start of a CTA: no change.
+// 34.2 us per layer).
+// What bounds it: the math pipes together.  A batch of two layers with four heads is ~2700 warp instructions, 512 of them
+// masks (2 cycles each per sub-partition), 290 products (8 cycles of the tensor pipe, ~2.7 of everyone's issue), ~400
+// half-precision multiplies (2 cycles); a CTA's start and end add ~400 a batch at 32k.  A sub-partition takes 2.62 us for
+// it with long ranges, 16 or 24 warps on the SM alike, copies from L2 or from HBM alike (1.32 us at the HBM rate); issue
+// slots 56 %, tensor pipe 44 %, ALU 40 %, shared-memory pipe 57 %.  Left out in a copy, one at a time: key products 0.92,
+// value products 0.78, biases 0.16, value scales 0.19, key scales 0.11, numerators 0.14 us.  Starting warps at different
+// times, half of the packed words' loads or the exponentials left out: no change.
+// Measured and not kept: twelve warps a CTA, two CTAs (the same speed of a step, single calls 2 us slower); sums in
+// registers with eight heads (128 registers, two CTAs: 4 % slower); the codes of a chunk in rings of two.
 #pragma once
 #include "xq_internal.h"
 #include "xq_mma.cuh"

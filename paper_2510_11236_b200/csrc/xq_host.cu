@@ -234,8 +234,8 @@ MmaShape mma_shape(const xq_cache* c, int l) {
 }
 
 // Layers of a step from which on they share launches.  A launch of its own costs a layer ~2.5 us of host time and a
-// start and an end with idle SMs: 32 layers of one user at 1000 tokens take 140 us with a launch each, 54 us together;
-// 32k context 965 and 927 us, 48 layers with host buffers 1608 and 1521 us.  A model of one or two layers keeps a
+// start and an end with idle SMs: 32 layers of one user at 1000 tokens took 140 us with a launch each, 54 us together;
+// 32k context 965 and 927 us, 48 layers with host buffers 1608 and 1521 us (each layer by itself then).  A model of one or two layers keeps a
 // launch per layer, which callers that watch xq_launch_count have seen so far (10.6 us for a tiny pair; 8.5 together).
 constexpr int MIN_JOINT_LAYERS = 3;
 
@@ -261,9 +261,9 @@ DecodeTimes decode_times(const Dims& dm) {
 // the next can call), which wants the CTAs of one full wave, and xq_decode_step, whose layers share launches and which
 // wants few CTAs.  The single call counts: of the plans that cost a layer alone at most ALONE_BOUND times the best, the
 // one with the smallest sum of the time alone, relative to the best, and STEP_WEIGHT times that in a step.  us per layer,
-// alone / in a step, with the plan a step would choose for itself and with this one: 32k, four heads 40.7 / 25.1,
-// 34.8 / 26.5; 16k 24.8 / 14.3, 21.6 / 15.5; one sequence of 128k 42.0 / 25.3, 33.7 / 27.5; groups of five at 16k
-// 52.9 / 29.0, 38.6 / 28.6; MHA at 4k, batch 8, 30.5 / 23.1 with either.
+// alone / in a step of 12 layers, with the plan best for the step and with this one: 32k, four heads 47.7 / 21.2,
+// 36.1 / 22.2; 16k 45.9 / 12.6, 23.6 / 13.6; groups of five at 16k 44.0 / 19.3, 29.9 / 20.7; MHA at 4k, batch 8, 30.4 /
+// 16.4 with either.
 constexpr double ALONE_BOUND = 1.10, STEP_WEIGHT = 1.2;
 constexpr double MERGE = 0.03;  // us of a launch's end for each partial of a stream
 void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int splits, MmaPlan& out) {
@@ -626,7 +626,8 @@ int decode_impl(xq_cache* c, int layer, const void* q, void* out, int out_f32, c
 
 
 // Tensor-core decode of the layers order[0 .. n) in few launches: layers of equal length and bit-widths share one, and
-// two that read the same codes go in pairs, for which the kernel reads and expands those once.  Layer l's q and out are
+// two that read the same codes go in pairs, for which the kernel reads and expands those once (32k, four heads, batch 4,
+// a layer of a step 27.9 -> 21.9 us).  Layer l's q and out are
 // slice l of q and out; with K_new / V_new the launch appends slice l of them to layer l (no layer's window is full).
 // Nothing in a launch reads what another layer of it writes: a layer writes its own window row, its own part of the
 // scratch and its own result.
