@@ -36,8 +36,8 @@ BULK_MIN, BULK_MAX = 16, 64  # between 16 and 64 window blocks per call
 # dram__bytes_read.sum + dram__bytes_write.sum of one layer call of the decode kernel (ncu, a launch of four layers;
 # see profiles/), with the SHA-256 of the kernel's sources at the time the counters were taken: the
 # figure is reported only while the sources still hash to that.
-NCU_TRAFFIC = {"c2": {"bytes": 334.2e6 / 4 + 4.9e6 / 4,
-                      "sources_sha256": "1722a858a7671b55c5eb1ab7ac1ae34f53edb0b60b349a2ae7cfb0bbf5634296"}}
+NCU_TRAFFIC = {"c2": {"bytes": 235.9e6 / 4 + 7.2e6 / 4,
+                      "sources_sha256": "9f0f68e6f95d4b9eb933821d90a6a12336bf994889f6e781c8cea98e58b1fb42"}}
 KERNEL_SOURCES = ("xq_decode_mma.cuh", "xq_mma.cuh", "xq_layout.cuh", "xq_internal.h")
 
 
@@ -331,6 +331,20 @@ def main():
                 tot += W.algorithmic_bytes(w, first_seq + i, l)
         return tot
 
+    def moved_bytes(first_seq, n_steps):
+        """What the launches of these steps must move: with up to four heads per kv head the layers of a pair are decoded
+        together and their shared codes are read once (step_bytes counts them for each layer)."""
+        tot = step_bytes(first_seq, n_steps)
+        if w["head_dim"] != 128 or w["n_q_heads"] > 4 * w["n_kv_heads"]:
+            return tot
+        for i in range(n_steps):
+            S = first_seq + i
+            nq = S - ((S - 1) % w["residual_len"] + 1)
+            for l in range(1, L, 2):
+                bits = (2 if l < w["kq"] else 1) * (l >= w["km"]) + (2 if l < w["vq"] else 1) * (l >= w["vm"])
+                tot -= w["batch"] * w["n_kv_heads"] * nq * w["head_dim"] * bits // 8
+        return tot
+
     import datetime
     sampler = ClockSampler(local) if rank == 0 else None  # runs from before the warm-up to the end of pass 3
     for _ in range(Wm):
@@ -369,15 +383,15 @@ def main():
         kinds[name] = {"launches": n, "total_ms": tot, "avg_us": (tot / n * 1e3) if n else None}
     xq.xq_timing_enable(cache.handle, 0)
     dec = kinds["decode_split"]
-    bytes_pass2 = step_bytes(seq_before2 + 1, K)
     peak, peak_kind = _peaks()
-    isolated = bytes_pass2 / (dec["total_ms"] * 1e-3) / 1e9 if dec["launches"] else 0.0
+    isolated = moved_bytes(seq_before2 + 1, K) / (dec["total_ms"] * 1e-3) / 1e9 if dec["launches"] else 0.0
     # The layers of a step share decode launches, which run back to back, so a layer call's duration is the timed
     # region's time over the number of layer calls; the few other kernels of the region (the steps that quantize a
     # window block) are charged to them.
     layer_calls_pass1 = K * L
     avg_launch_us = ms / layer_calls_pass1 * 1e3
-    achieved = bytes_pass1 / (ms * 1e-3) / 1e9
+    moved_pass1 = moved_bytes(seq_before + 1, K)
+    achieved = moved_pass1 / (ms * 1e-3) / 1e9
 
     # ---- pass 3: end to end through the C ABI with host buffers
     seq_before3 = cache.seq_len(0)
@@ -469,7 +483,7 @@ def main():
             "data": "synthetic",
             "config": _config_block(args, w),
             "run": {"equiv_bits": xq.xq_equiv_bits(cfg), "layer_order": args.layer_order,
-                    "bytes_streamed_per_step_gb": bytes_pass1 / K / 1e9,
+                    "bytes_streamed_per_step_gb": moved_pass1 / K / 1e9,
                     "splits_quantized": nsq, "splits_window": nsw,
                     "algorithmic_bytes_per_layer_call": W.algorithmic_bytes(w, S, 0)},
             "frac_of_8TBps": value / world / 8000.0,
@@ -483,7 +497,7 @@ def main():
                          "peak_source": peak_kind, "unit": "GB/s", "frac": achieved / peak,
                          "frac_of_8TBps": achieved / 8000.0,
                          "traffic": _ncu_traffic(args.config) if not (args.layers or args.seq or args.splits) else None,
-                         "algorithmic_bytes_per_launch": bytes_pass1 / layer_calls_pass1,
+                         "algorithmic_bytes_per_launch": moved_pass1 / layer_calls_pass1,
                          "avg_launch_us": avg_launch_us, "launches": layer_calls_pass1,
                          "timing": "CUDA events around the timed region of back-to-back launches, per layer call (a launch serves up to 32 layers)",
                          "isolated": {"avg_launch_us": dec["avg_us"], "achieved": isolated, "frac": isolated / peak,
