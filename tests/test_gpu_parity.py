@@ -1089,7 +1089,7 @@ def test_decode_step_pairs_of_layers(G, bits, g, f16, S, group):
     """Two layers that read the same codes share a pass over them.  Last batches of one, two and three quarters and of less
     than half, no batch at all, owners first or in order, groups of four layers (two pairs each): results equal
     xq_append_kv and xq_decode_attention bit for bit."""
-    L, B, Hkv, D, R = 8, 2, 2, 128, 64 if g == 64 else 32
+    L, B, Hkv, D, R = 8, 4, 10, 128, 64 if g == 64 else 32  # (more CTAs than a wave: else layers go one by one)
     kw = dict(n_layers=L, batch=B, n_q_heads=G * Hkv, n_kv_heads=Hkv, head_dim=D, max_seq=S + 40, group_size=g, residual_len=R,
               kq=L if bits[0] else 0, vq=L if bits[1] else 0, eta1=1 / 6, eta2=0.045, share_group=group if group > 2 else 0,
               io_dtype=xq.XQ_F16 if f16 else xq.XQ_BF16, n_splits=3)
