@@ -37,7 +37,7 @@ BULK_MIN, BULK_MAX = 16, 64  # between 16 and 64 window blocks per call
 # see profiles/), with the SHA-256 of the kernel's sources at the time the counters were taken: the
 # figure is reported only while the sources still hash to that.
 NCU_TRAFFIC = {"c2": {"bytes": 235.9e6 / 4 + 7.2e6 / 4,
-                      "sources_sha256": "9f0f68e6f95d4b9eb933821d90a6a12336bf994889f6e781c8cea98e58b1fb42"}}
+                      "sources_sha256": "a7a564592a316a409bf618ab632ee9dfbb29f5ac18b4ea83cf308c13e9e68c27"}}
 KERNEL_SOURCES = ("xq_decode_mma.cuh", "xq_mma.cuh", "xq_layout.cuh", "xq_internal.h")
 
 

@@ -40,7 +40,7 @@
 // value products 0.78, biases 0.16, value scales 0.19, key scales 0.11, numerators 0.14 us.  Starting warps at different
 // times, half of the packed words' loads or the exponentials left out: no change.
 // Measured and not kept: twelve warps a CTA, two CTAs (the same speed of a step, single calls 2 us slower); sums in
-// registers with eight heads (128 registers, two CTAs: 4 % slower); the codes of a chunk in rings of two.
+// registers with eight heads (128 registers, two CTAs: 4 % slower).
 #pragma once
 #include "xq_internal.h"
 #include "xq_mma.cuh"
