@@ -496,12 +496,7 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NT>::WARPS * 32, Plan<BK,
 #pragma unroll
       for (int g = 0; g < NGT; ++g) {
         const uint32_t a = st + Pl::OFF_KM + g * 4 * D + lane * 2 * V;
-        if constexpr (V == 4) {
-          const uint2 x = lds64(a);
-          s[g][0] = x.x; s[g][1] = x.y;
-        } else {
-          s[g][0] = lds32(a);
-        }
+        s[g][0] = lds32(a);
       }
       if (valid < BT) {
 #pragma unroll
@@ -569,7 +564,7 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NT>::WARPS * 32, Plan<BK,
     }
     // ---- keys: q . c ----
     // packed words of rows gid, gid + 8: even bytes, odd bytes
-    auto load_rows = [&](int u, int kw, uint32_t (&w)[2][2], uint32_t (&w8)[2][2]) {
+    auto load_rows = [&](int u, uint32_t (&w)[2][2], uint32_t (&w8)[2][2]) {
 #pragma unroll
       for (int t = 0; t < 2; ++t)
 #pragma unroll
@@ -577,13 +572,12 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NT>::WARPS * 32, Plan<BK,
           const int tk = 16 * t + 2 * r;
           uint32_t raw;
           if constexpr (BK == 1) raw = lds32(kc_lane + u * 256 + tk * 8) >> (4 * (tig & 1));
-          else raw = lds32(kc_lane + u * (32 * D * BK / 8) + kw * 512 + tk * 16);
+          else raw = lds32(kc_lane + u * (32 * D * BK / 8) + tk * 16);
           w[t][r] = byte_pair_up(raw, 2);
           w8[t][r] = byte_pair_down(raw, 6);
         }
     };
     auto key_pair = [](uint32_t w, int k) { return code_pair<BK>(w, BK == 2 ? k & 3 : k); };
-    constexpr int KPW = KS;  // k-steps a word serves
     if constexpr (GC == 1) {
       constexpr int UG = GS / 32;  // units of a group
       // fma(q, s, qn * s) is hi where qn = 0 and lo where qn = -q
@@ -598,38 +592,34 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NT>::WARPS * 32, Plan<BK,
 #pragma unroll
       for (int g = 0; g < NGT; ++g) {
         float c[NT][2 * UG][4];
+        uint32_t w[UG][2][2], w8[UG][2][2];
 #pragma unroll
-        for (int kw = 0; kw < 1; ++kw) {
-          uint32_t w[UG][2][2], w8[UG][2][2];
+        for (int u = 0; u < UG; ++u) load_rows(g * UG + u, w[u], w8[u]);
+        const uint32_t sa = st + Pl::OFF_KM + g * 4 * D + tig * 16;
+        uint4 sv;
 #pragma unroll
-          for (int u = 0; u < UG; ++u) load_rows(g * UG + u, kw, w[u], w8[u]);
-          const uint32_t sa = st + Pl::OFF_KM + g * 4 * D + tig * 16 + kw * (KPW / 2) * 64;
-          uint4 sv;
+        for (int k = 0; k < KS; ++k) {
+          if ((k & 1) == 0) sv = lds128(sa + (k / 2) * 64);
+          const uint32_t s0 = k & 1 ? sv.z : sv.x, s1 = k & 1 ? sv.w : sv.y;
 #pragma unroll
-          for (int k = 0; k < KPW; ++k) {
-            if ((k & 1) == 0) sv = lds128(sa + (k / 2) * 64);
-            const uint32_t s0 = k & 1 ? sv.z : sv.x, s1 = k & 1 ? sv.w : sv.y;
-            const int ks = kw * KPW + k;
-#pragma unroll
-            for (int n = 0; n < NT; ++n) {
-              uint32_t p0, p1;
-              if constexpr (NT == 1) {
-                p0 = hfma2(qk[n][ks][0], s0, hmul2(qn[ks][0], s0));
-                p1 = hfma2(qk[n][ks][1], s1, hmul2(qn[ks][1], s1));
-              } else {
-                p0 = product_part(qk[n][ks][0], s0, low);
-                p1 = product_part(qk[n][ks][1], s1, low);
-              }
-#pragma unroll
-              for (int u = 0; u < UG; ++u)
-#pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                  const uint32_t a0 = key_pair(w[u][t][0], k), a1 = key_pair(w[u][t][1], k);
-                  const uint32_t a2 = key_pair(w8[u][t][0], k), a3 = key_pair(w8[u][t][1], k);
-                  if (ks == 0) mma_f16_first(c[n][2 * u + t], a0, a1, a2, a3, p0, p1);
-                  else mma_f16(c[n][2 * u + t], a0, a1, a2, a3, p0, p1);
-                }
+          for (int n = 0; n < NT; ++n) {
+            uint32_t p0, p1;
+            if constexpr (NT == 1) {
+              p0 = hfma2(qk[n][k][0], s0, hmul2(qn[k][0], s0));
+              p1 = hfma2(qk[n][k][1], s1, hmul2(qn[k][1], s1));
+            } else {
+              p0 = product_part(qk[n][k][0], s0, low);
+              p1 = product_part(qk[n][k][1], s1, low);
             }
+#pragma unroll
+            for (int u = 0; u < UG; ++u)
+#pragma unroll
+              for (int t = 0; t < 2; ++t) {
+                const uint32_t a0 = key_pair(w[u][t][0], k), a1 = key_pair(w[u][t][1], k);
+                const uint32_t a2 = key_pair(w8[u][t][0], k), a3 = key_pair(w8[u][t][1], k);
+                if (k == 0) mma_f16_first(c[n][2 * u + t], a0, a1, a2, a3, p0, p1);
+                else mma_f16(c[n][2 * u + t], a0, a1, a2, a3, p0, p1);
+              }
           }
         }
 #pragma unroll
@@ -661,20 +651,17 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NT>::WARPS * 32, Plan<BK,
 #pragma unroll
         for (int j = 0; j < GC; ++j) {
           float c[2][4];
+          uint32_t w[2][2], w8[2][2];
+          load_rows(GC * ux + j, w, w8);
 #pragma unroll
-          for (int kw = 0; kw < 1; ++kw) {
-            uint32_t w[2][2], w8[2][2];
-            load_rows(GC * ux + j, kw, w, w8);
+          for (int k = 0; k < KS; ++k)
 #pragma unroll
-            for (int k = 0; k < KPW; ++k)
-#pragma unroll
-              for (int t = 0; t < 2; ++t) {
-                const uint32_t a0 = key_pair(w[t][0], k), a1 = key_pair(w[t][1], k);
-                const uint32_t a2 = key_pair(w8[t][0], k), a3 = key_pair(w8[t][1], k);
-                if (kw + k == 0) mma_f16_first(c[t], a0, a1, a2, a3, pp[0][0], pp[0][1]);
-                else mma_f16(c[t], a0, a1, a2, a3, pp[kw * KPW + k][0], pp[kw * KPW + k][1]);
-              }
-          }
+            for (int t = 0; t < 2; ++t) {
+              const uint32_t a0 = key_pair(w[t][0], k), a1 = key_pair(w[t][1], k);
+              const uint32_t a2 = key_pair(w8[t][0], k), a3 = key_pair(w8[t][1], k);
+              if (k == 0) mma_f16_first(c[t], a0, a1, a2, a3, pp[0][0], pp[0][1]);
+              else mma_f16(c[t], a0, a1, a2, a3, pp[k][0], pp[k][1]);
+            }
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const float v = fmaf(c[k / 2][2 * (k & 1)] + c[k / 2][2 * (k & 1) + 1], ck[0], bias[k >> 1]);
