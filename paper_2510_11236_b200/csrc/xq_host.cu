@@ -647,22 +647,21 @@ int decode_layers(xq_cache* c, const int* order, int n, const uint8_t* q, uint8_
     plan_splits(c, order[0], S - r, r, ns_q, ns_w);
     pairs = (long long)ns_q * dm.B * dm.Hkv * n > 2LL * c->sm_count;
   }
-  // the layers as they go to the launches: two that share their codes side by side, in the place of the first
+  // in pairs, the layers as they go to the launches: two that share their codes side by side, in the place of the first
   std::vector<int> run;
   std::vector<char> paired;  // of run[i]: it is one of two
-  run.reserve(n);
-  paired.reserve(n);
-  {
+  if (pairs) {
+    run.reserve(n);
+    paired.reserve(n);
     std::vector<char> taken(n, 0);
     for (int i = 0; i < n; ++i) {
       if (taken[i]) continue;
       const int a = order[i];
       int with = -1;
-      if (pairs)
-        for (int j = i + 1; j < n && with < 0; ++j) {
-          const int b = order[j];
-          if (!taken[j] && c->seq[b] == c->seq[a] && k_owner(&c->cfg, a) == k_owner(&c->cfg, b) && v_owner(&c->cfg, a) == v_owner(&c->cfg, b)) with = j;
-        }
+      for (int j = i + 1; j < n && with < 0; ++j) {
+        const int b = order[j];
+        if (!taken[j] && c->seq[b] == c->seq[a] && k_owner(&c->cfg, a) == k_owner(&c->cfg, b) && v_owner(&c->cfg, a) == v_owner(&c->cfg, b)) with = j;
+      }
       run.push_back(a);
       paired.push_back(with >= 0);
       if (with >= 0) {
@@ -671,26 +670,28 @@ int decode_layers(xq_cache* c, const int* order, int n, const uint8_t* q, uint8_
         paired.push_back(1);
       }
     }
+    order = run.data();
   }
+  auto in_pair = [&](int i) { return pairs && paired[i]; };
   for (int i = 0; i < n;) {
     DecodeParams p;
     bool use_mma;
-    const int l0 = run[i], S = c->seq[l0] + (K_new ? 1 : 0);
+    const int l0 = order[i], S = c->seq[l0] + (K_new ? 1 : 0);
     rc = prepare_decode(c, l0, q + l0 * q_layer, out + l0 * q_layer, 0, K_new ? K_new + l0 * kv_layer : nullptr,
                         V_new ? V_new + l0 * kv_layer : nullptr, S, p, use_mma);
     if (rc != XQ_OK) return rc;
     // the layers of a launch share the scratch: XQ_MAX_SPLITS partials per query head
     int most = XQ_MAX_SPLITS / p.ns_q < DECODE_MAX_LAYERS ? XQ_MAX_SPLITS / p.ns_q : DECODE_MAX_LAYERS;
     if (!joint) most = 1;
-    p.paired = paired[i] && most >= 2;
+    p.paired = in_pair(i) && most >= 2;
     if (p.paired) most -= most % 2;
     bool packed = c->repacked[l0] != 0;
     int j = i + 1;
-    for (; j < n && j - i < most && c->seq[run[j]] == c->seq[l0] && (!p.paired || paired[j]); ++j) {
-      const int l = run[j];
+    for (; j < n && j - i < most && c->seq[order[j]] == c->seq[l0] && (!p.paired || in_pair(j)); ++j) {
+      const int l = order[j];
       const LayerPtrs L = layer_ptrs(c, l);
       if (L.bk != p.layer[0].L.bk || L.bv != p.layer[0].L.bv) break;
-      if (!p.paired && paired[j] && !paired[i]) break;
+      if (!p.paired && in_pair(j) && !in_pair(i)) break;
       p.layer[j - i] = {L, (const uint16_t*)(q + l * q_layer), out + l * q_layer,
                         K_new ? (const uint16_t*)(K_new + l * kv_layer) : nullptr,
                         V_new ? (const uint16_t*)(V_new + l * kv_layer) : nullptr};
@@ -709,8 +710,8 @@ int decode_layers(xq_cache* c, const int* order, int n, const uint8_t* q, uint8_
       return rc;
     }
     for (; i < j; ++i) {
-      c->repacked[run[i]] = 0;
-      if (K_new) c->seq[run[i]] += 1;
+      c->repacked[order[i]] = 0;
+      if (K_new) c->seq[order[i]] += 1;
     }
   }
   return XQ_OK;
