@@ -70,7 +70,8 @@ extern "C" {
  * 128 (XQ_KERNEL_AUTO takes it for head_dim 64 too).  The products q_d * s_d (query times
  * key scale) and p_t * s_t (softmax numerator times value scale) enter the matrix products
  * as unevaluated sums of two halves (22 bits of every product down to 2^-10 of the largest
- * of its 128 tokens), codes are exact.  The fp32 sums of the matrix products keep 16 bits or
+ * of its 64 tokens, with head_dim 64 of its 128; with head_dim 128 and three to eight heads in
+ * the group, key scales below 2^-10 of the largest lose bits), codes are exact.  The fp32 sums of the matrix products keep 16 bits or
  * more; with head_dim 128 they set the error: 1e-5 to 1e-4 of the result's norm (2-norm), in
  * xq_attention_chunk's own kernel 1e-6 to 1e-5.  With head_dim 64, and over the window alone,
  * the result is as exact as the scalar kernel's (below 1e-6). */

@@ -14,7 +14,10 @@
 //
 // and the other operand (q_d s_d, or p_t s_tg) is carried as an unevaluated sum hi + lo of two fp16 numbers: hi = RN(q s),
 // lo = fma(q, s, -hi), as far as fp16 reaches: relative to the largest product of a round, which is kept between 2^8 and
-// 2^15 (2^9 with 1-bit keys, whose weights come off q), nothing above 2^-33 is lost (p_t s_t: one rounding at 2^-22).
+// 2^15 (2^9 with 1-bit keys, whose weights come off q), nothing above 2^-33 is lost (p_t s_t: one rounding at 2^-22).  The
+// power of two that keeps it there: with one or two heads on q (a multiplication at each product, for which no time was
+// measured: 32 layers of one head at 4k, batch 8 618.7 us without, 618.0 with), so that key scales keep the bits that they
+// are stored with; with three to eight on the scales, which lose bits below 2^-10 of the round's largest.
 // Codes are exact, accumulation is fp32.  The powers of two that the bit offsets put on the codes are taken out of q and of
 // the softmax numerators.  Up to four heads of a CTA: hi and lo are two of the eight operand columns, and the lo sums are
 // added at the end.  Eight heads (five to eight of a layer, or three or four of each of two layers): a column is a head, hi
@@ -98,6 +101,7 @@ struct Plan {
   static constexpr int WIN = 32 * WROW;          // 16 key rows, then 16 value rows (over the stage of the warp)
   static constexpr int BODY = P_OVER ? OFF_VM + NL * VROOM : OFF_P + PBUF;
   static constexpr int WARP = ((BODY > WIN ? BODY : WIN) + 127) / 128 * 128;
+  static constexpr bool Q_FACTOR = HP <= 2;      // the factor that keeps q s in fp16's range is taken on q
   static constexpr int MS = D + 4;               // state row: acc[D], m, l
   static_assert(2 * VH * MS * 4 <= WARP, "a warp's state rows, of the packed tokens and of the window, fit its own memory");
   static_assert(MS % 4 == 0, "state rows are read as vectors");
@@ -513,8 +517,10 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK,
   const float cz = WIDE ? p.scale * 1.4426950408889634f * pow2i(-eq_sm[4 * (lane >> 4) + tig]) : cq[0];
 
   const uint32_t low_mask = low ? 0xffffffffu : 0u;
-  // key scales are taken times 2^Ek of their layer: ek2, a pair of fp16 (0: not set)
-  uint32_t ek2[NL];
+  // The products q s are taken times 2^Ek of their layer: up to two heads a layer, the factor (at most 1) is q's, at the
+  // product, else the scales'.  ek2: that factor as a pair of fp16; k_in: for which bits of the round's largest scale (low
+  // half: from, high half: how many) the exponent stays.
+  uint32_t ek2[NL], k_in[NL], eq2 = 0u;  // eq2: ek2 of this thread's operand column
   float ck[NCOL];
 #pragma unroll
   for (int j = 0; j < NCOL; ++j) ck[j] = 0.f;
@@ -523,7 +529,14 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK,
 #pragma unroll
     for (int j = 0; j < NCOL; ++j) ck[j] = NL == 1 || my_layer == l ? cq[j] * unit : ck[j];
   };
-  auto q_pair = [&](int ks) { return lds64(qf + ks * 256); };
+  auto q_pair = [&](int ks) {
+    uint2 q = lds64(qf + ks * 256);
+    if constexpr (Pl::Q_FACTOR) {
+      q.x = hmul2(q.x, eq2);
+      q.y = hmul2(q.y, eq2);
+    }
+    return q;
+  };
 
   // Softmax state of the heads of this thread's columns: reference mr (log2 units, an integer; 0 until the first round
   // sets it).  Value sums acc (PARK: in tensor memory between the rounds): of row tile mt the products' four (WIDE: of hi,
@@ -537,7 +550,7 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK,
   float mr[NCOL], zacc[NCOL][4];
   uint32_t ev2[NL];  // value scales are taken times 2^Ev: a pair of fp16 (0: not set)
 #pragma unroll
-  for (int l = 0; l < NL; ++l) ek2[l] = ev2[l] = 0u;
+  for (int l = 0; l < NL; ++l) ek2[l] = ev2[l] = k_in[l] = 0u;
 #pragma unroll
   for (int j = 0; j < NCOL; ++j) {
     mr[j] = 0.f;
@@ -617,7 +630,7 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK,
       }
       __syncwarp();
     }
-    // ---- keys: scales into the order of the operand slots (in place), times 2^Ek ----
+    // ---- keys: scales into the order of the operand slots (in place) ----
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
       constexpr int V = D / 32;
@@ -644,21 +657,36 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK,
         return redux_max_u32(max(mx & 0xffffu, mx >> 16));
       };
       read();
-      // The largest scale of the round times 2^Ek in [2^-4, 1): |q s| below 2^15, and a scale keeps its 11 bits down to
-      // 2^-10 of the largest.  Ek moves only outside that, and no further than 15.
-      bool moved = r == 0;
-      if (r > 0) {
-        scale();
-        moved = largest() - 0x2c00u >= 0x1000u;
-        if (moved) read();
-      }
-      if (moved) {
-        const float smax = f16_to_f(largest());
-        const int es = smax > 0.f ? exponent_of(smax) : -24, e = min(15, -1 - es);
-        const float f = pow2i(e);
-        ek2[l] = pack_io2<true>(f, f);
-        set_unit(l, e);
-        scale();
+      if constexpr (Pl::Q_FACTOR) {
+        // The largest scale of the round times 2^Ek in [2^-7, 1), Ek at most 0: |q s| below 2^15, scales as they are
+        // stored.  Ek moves only outside that.
+        const uint32_t mx = largest();
+        if (mx - (k_in[l] & 0xffffu) >= k_in[l] >> 16) {
+          const float smax = f16_to_f(mx);
+          const int e = smax >= 0.5f ? max(-16, -1 - exponent_of(smax)) : 0;
+          const float f = pow2i(e);
+          ek2[l] = pack_io2<true>(f, f);
+          k_in[l] = e < 0 ? (uint32_t)(8 - e) << 10 | 0x1c000000u : 0x3c000000u;
+          if (NL == 1 || col_layer == l) eq2 = ek2[l];
+          set_unit(l, e);
+        }
+      } else {
+        // The largest scale of the round times 2^Ek in [2^-4, 1): |q s| below 2^15, and a scale keeps its 11 bits down to
+        // 2^-10 of the largest.  Ek moves only outside that, and no further than 15.
+        bool moved = r == 0;
+        if (r > 0) {
+          scale();
+          moved = largest() - 0x2c00u >= 0x1000u;
+          if (moved) read();
+        }
+        if (moved) {
+          const float smax = f16_to_f(largest());
+          const int es = smax > 0.f ? exponent_of(smax) : -24, e = min(15, -1 - es);
+          const float f = pow2i(e);
+          ek2[l] = pack_io2<true>(f, f);
+          set_unit(l, e);
+          scale();
+        }
       }
       __syncwarp();
 #pragma unroll

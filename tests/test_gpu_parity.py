@@ -973,6 +973,36 @@ def test_key_scales_far_from_one(G, kq, f16, kind):
     assert _relative_error(cache, cfg, {0: (K, V)}, 0, q) <= 1.2e-4
 
 
+@pytest.mark.parametrize("G,kq", [(1, 0), (1, 2), (2, 0), (2, 2)])
+@pytest.mark.parametrize("octaves", [11, 12, 13])
+def test_key_scales_of_one_and_two_heads_are_used_as_stored(G, kq, octaves):
+    # Channels up to 2^13 apart: an fp16 scale has its 11 bits down to 2^-14, and with one or two heads the factor that
+    # keeps products q s in range is q's, 2^-7 at most here, where q is at least 2^(14 - 13 - 7 - 7) before the codes'
+    # weights: nothing is lost but the sums' 16 bits, as in test_two_bit_values_keep_sixteen_bits_of_the_sums, of which
+    # 1 / 4 shows on this data; an operand with fewer bits shows 2^-14 and more.  In a step the layers go in pairs.
+    S, D, B, Hkv, L = 300, 128, 4, 20, 4
+    w = dict(n_layers=L, batch=B, n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=D, seq=S, residual_len=32, group_size=32,
+             kq=kq and L, vq=0, km=0, vm=0, n_outliers=3, outlier_scale=4.0, seed=25, n_splits=1)
+    cfg = W.make_xq_config(w, max_seq=S + 8)
+    f = torch.exp2(-float(octaves) * (torch.arange(D) % 2)).to(DEV)
+    a, b = xq.Cache(cfg, DEV), xq.Cache(cfg, DEV)
+    kv = {}
+    for pair in range(L // 2):
+        k0, v0, k1, v1 = W.pair_tokens(w, pair, 0, S, DEV)
+        for l, k, v in ((2 * pair, k0, v0), (2 * pair + 1, k1, v1)):
+            kv[l] = ((k.float() * f).to(torch.bfloat16), v)
+            for cache in (a, b):
+                cache.append_kv(l, *kv[l])
+    q = torch.stack([(W.queries(w, l, 0, DEV).float() / f).to(torch.bfloat16) for l in range(L)])
+    assert _relative_error(b, cfg, kv, 0, q[0]) <= 3e-5
+    kn, vn = (torch.stack([kv[l][i][:, :, :1] for l in range(L)]).contiguous() for i in (0, 1))
+    out = a.decode_step(kn, vn, q, torch.empty_like(q))
+    for l in range(L):
+        b.append_kv(l, kn[l], vn[l])
+        assert torch.equal(b.decode_attention(l, q[l]), out[l]), l
+    a.close(); b.close()
+
+
 @pytest.mark.parametrize("B,Hkv,G,S", [(4, 8, 4, 32768), (1, 8, 4, 131072), (4, 8, 5, 16384), (16, 2, 1, 20000)])
 def test_splits_of_many_layers_fill_one_wave(B, Hkv, G, S):
     # A layer alone (xq_decode_attention) is fastest with the CTAs of one wave, two an SM, however many layers the model
