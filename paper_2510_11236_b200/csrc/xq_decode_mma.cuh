@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK,
     }
   }
   if (lane == 0) {
-    mbar_init(bar_k, 2);  // codes; scales and zero-points
+    mbar_init(bar_k, Pl::P_OVER ? 2 : 1);  // two: codes; scales and zero-points
     mbar_init(bar_v, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
@@ -427,14 +427,20 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK,
   const int rounds = warp < halves ? (halves - 1 - warp) / W + 1 : 0;
   static_assert(W % 2 == 0, "a warp's rounds are all first, or all second halves");
 
-  // Copies of round r into this warp's stage (one lane; the stage is free)
+  // Copies of round r into this warp's stage (one lane; the stage is free).  A copy costs a warp its issue, ~33 cycles with a
+  // branch on the lane's index (all of them left out of a layer at 32k, four heads: 33.5 of 35.7 us), and half batches have
+  // twice as many as batches: calls of one layer had become slower by 5 to 13 % with them.  Behind elect_one, and with one
+  // arrival for codes and parameters where they go together: 36.4 -> 35.0 us, MHA at 4k, batch 8 30.8 -> 30.1, a layer of a
+  // step of 32 that shares no codes 29.4 -> 28.6 and 25.6 -> 24.7, in pairs 21.4 -> 21.1 and 18.4 -> 17.9.  Measured and
+  // not kept: two stages a warp (the waits were not it: 35.8), whole batches a round with one copy each (36.1; one head
+  // 3 % faster, pairs slower), products of more row tiles at a time, q kept in registers (no change).
   auto half_of = [&](int r) { return (unsigned)(warp + W * r); };
   auto load_key_codes = [&](int r) {
-    mbar_expect_tx(bar_k, Pl::KCODES);
+    mbar_expect_tx(bar_k, Pl::KCODES + (Pl::P_OVER ? 0 : NL * Pl::KM));
     bulk_load(st, src_sm[0] + (size_t)half_of(r) * Pl::KCODES, Pl::KCODES, bar_k);
   };
   auto load_key_params = [&](int r) {
-    mbar_expect_tx(bar_k, NL * Pl::KM);
+    if (Pl::P_OVER) mbar_expect_tx(bar_k, NL * Pl::KM);
 #pragma unroll
     for (int l = 0; l < NL; ++l) bulk_load(st + Pl::OFF_KM + l * Pl::KM, src_sm[2 + 2 * l] + (size_t)half_of(r) * Pl::KM, Pl::KM, bar_k);
   };
@@ -874,7 +880,7 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK,
     proxy_fence();
     __syncwarp();
     if (r + 1 < rounds) {
-      if (lane == 0) {
+      if (elect_one()) {
         load_key_codes(r + 1);
         if (!Pl::P_OVER) load_key_params(r + 1);
       }
@@ -1104,7 +1110,7 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK,
     proxy_fence();
     __syncwarp();
     if (r + 1 < rounds) {
-      if (lane == 0) {
+      if (elect_one()) {
         if (Pl::P_OVER) load_key_params(r + 1);
         load_values(r + 1);
       }

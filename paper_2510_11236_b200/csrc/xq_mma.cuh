@@ -81,6 +81,13 @@ __device__ __forceinline__ float4 ld_cg4(const float* p) {
   return v;
 }
 
+// True for one lane of a whole warp.  Bulk copies behind it are issued without the code that a branch on the lane's index
+// needs because more than one lane might take it.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t one;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(one) : : "memory");
+  return one != 0;
+}
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
 }
