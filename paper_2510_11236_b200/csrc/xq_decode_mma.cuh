@@ -435,20 +435,28 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK,
   // not kept: two stages a warp (the waits were not it: 35.8), whole batches a round with one copy each (36.1; one head
   // 3 % faster, pairs slower), products of more row tiles at a time, q kept in registers (no change).
   auto half_of = [&](int r) { return (unsigned)(warp + W * r); };
-  auto load_key_codes = [&](int r) {
-    mbar_expect_tx(bar_k, Pl::KCODES + (Pl::P_OVER ? 0 : NL * Pl::KM));
-    bulk_load(st, src_sm[0] + (size_t)half_of(r) * Pl::KCODES, Pl::KCODES, bar_k);
+  struct Sources { const uint8_t *codes, *params[NL]; };
+  auto sources = [&](int kind) {  // read before the copies, which are not reordered
+    Sources s;
+    s.codes = src_sm[kind];
+#pragma unroll
+    for (int l = 0; l < NL; ++l) s.params[l] = src_sm[2 + 2 * l + kind];
+    return s;
   };
-  auto load_key_params = [&](int r) {
+  auto load_key_codes = [&](int r, const Sources& s) {
+    mbar_expect_tx(bar_k, Pl::KCODES + (Pl::P_OVER ? 0 : NL * Pl::KM));
+    bulk_load(st, s.codes + (size_t)half_of(r) * Pl::KCODES, Pl::KCODES, bar_k);
+  };
+  auto load_key_params = [&](int r, const Sources& s) {
     if (Pl::P_OVER) mbar_expect_tx(bar_k, NL * Pl::KM);
 #pragma unroll
-    for (int l = 0; l < NL; ++l) bulk_load(st + Pl::OFF_KM + l * Pl::KM, src_sm[2 + 2 * l] + (size_t)half_of(r) * Pl::KM, Pl::KM, bar_k);
+    for (int l = 0; l < NL; ++l) bulk_load(st + Pl::OFF_KM + l * Pl::KM, s.params[l] + (size_t)half_of(r) * Pl::KM, Pl::KM, bar_k);
   };
-  auto load_values = [&](int r) {
+  auto load_values = [&](int r, const Sources& s) {
     mbar_expect_tx(bar_v, NL * Pl::VM + Pl::VCODES);
-    bulk_load(st + Pl::OFF_V, src_sm[1] + (size_t)(BV == 2 ? half_of(r) : half_of(r) >> 1) * Pl::VCODES, Pl::VCODES, bar_v);
+    bulk_load(st + Pl::OFF_V, s.codes + (size_t)(BV == 2 ? half_of(r) : half_of(r) >> 1) * Pl::VCODES, Pl::VCODES, bar_v);
 #pragma unroll
-    for (int l = 0; l < NL; ++l) bulk_load(st + Pl::OFF_VM + l * Pl::VROOM, src_sm[3 + 2 * l] + (size_t)half_of(r) * Pl::VM, Pl::VM, bar_v);
+    for (int l = 0; l < NL; ++l) bulk_load(st + Pl::OFF_VM + l * Pl::VROOM, s.params[l] + (size_t)half_of(r) * Pl::VM, Pl::VM, bar_v);
   };
 
   if (lane == 0) {
@@ -456,9 +464,10 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK,
     // kernel may have written it since this layer's last decode, the first copies wait for that kernel.
     if (!p.early_fetch) grid_dependency_wait();
     if (rounds > 0) {
-      load_key_codes(0);
-      load_key_params(0);
-      load_values(0);
+      const Sources sk = sources(0), sv = sources(1);
+      load_key_codes(0, sk);
+      load_key_params(0, sk);
+      load_values(0, sv);
     }
   }
   __syncwarp();
@@ -881,8 +890,9 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK,
     __syncwarp();
     if (r + 1 < rounds) {
       if (elect_one()) {
-        load_key_codes(r + 1);
-        if (!Pl::P_OVER) load_key_params(r + 1);
+        const Sources sk = sources(0);
+        load_key_codes(r + 1, sk);
+        if (!Pl::P_OVER) load_key_params(r + 1, sk);
       }
       last_k = r + 1;
     }
@@ -1111,8 +1121,9 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK,
     __syncwarp();
     if (r + 1 < rounds) {
       if (elect_one()) {
-        if (Pl::P_OVER) load_key_params(r + 1);
-        load_values(r + 1);
+        const Sources sk = sources(0), sv = sources(1);
+        if (Pl::P_OVER) load_key_params(r + 1, sk);
+        load_values(r + 1, sv);
       }
       last_v = r + 1;
     }
