@@ -65,7 +65,7 @@ constexpr uint32_t ONES = 0x3C003C00u;
 // GC = 4 / VH slots: with fewer heads, one operand serves GC token units of the keys (or GC channel parts of the values)
 // at once, each row tile reading the columns of its own slot.  Eight (WIDE): a column is a head, hi and lo are operands
 // of two products.
-template <int BK, int BV, int GS, int HP, int NL>
+template <int BK, int BV, int GS, int HP, int NL, bool MANY>
 struct Plan {
   static constexpr int VH = HP * NL;
   static_assert(VH == 1 || VH == 2 || VH == 4 || VH == 8, "heads of a CTA");
@@ -113,7 +113,8 @@ struct Plan {
   // With eight heads the sums (64 registers) would not fit otherwise; two layers of one head, 4k, batch 8: 640 us a step
   // without, 622 with.  One layer alone, up to four heads: tensor memory costs a CTA 1.2 us at its start and end (a call
   // at 32k 37.0 us with, 35.2 without).
-  static constexpr bool PARK = WIDE || NL == 2;
+  // MANY: one layer of up to four heads for launches of many CTAs, where a CTA's start and end overlap with others' work.
+  static constexpr bool PARK = WIDE || NL == 2 || MANY;
   static constexpr int CTAS = PARK ? 3 : 2, WARPS = 8;
   static constexpr int TCOLS = KS * 4 * NCOL, TMEM = WARPS / 4 * TCOLS;
   static_assert(!PARK || (CTAS * TMEM <= 512 && (TMEM & (TMEM - 1)) == 0), "tensor memory");
@@ -340,10 +341,10 @@ __device__ __forceinline__ void ticket_merge(const DecodeParams& p, const Decode
   if (threadIdx.x == 0) *ticket = 0u;  // ready for the next launch on this stream
 }
 
-template <int BK, int BV, int GS, int HP, int NL>
-__global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK, BV, GS, HP, NL>::CTAS)
+template <int BK, int BV, int GS, int HP, int NL, bool MANY>
+__global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL, MANY>::WARPS * 32, Plan<BK, BV, GS, HP, NL, MANY>::CTAS)
     decode_mma_kernel(const __grid_constant__ DecodeParams p) {
-  using Pl = Plan<BK, BV, GS, HP, NL>;
+  using Pl = Plan<BK, BV, GS, HP, NL, MANY>;
   constexpr bool WIDE = Pl::WIDE;
   constexpr int KS = Pl::KS, NG = Pl::NG, NGT = Pl::NGT, W = Pl::WARPS, WROW = Pl::WROW, GC = Pl::GC, CP = Pl::CP;
   constexpr int VH = Pl::VH, SH = Pl::SH, NSET = Pl::NSET, NCOL = Pl::NCOL, NE = Pl::NE;
@@ -1303,19 +1304,19 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL>::WARPS * 32, Plan<BK,
                         reinterpret_cast<float*>(smem));
 }
 
-template <int BK, int BV, int GS, int HP, int NL>
+template <int BK, int BV, int GS, int HP, int NL, bool MANY>
 cudaError_t launch_one(const DecodeParams& p, cudaStream_t st) {
-  using Pl = Plan<BK, BV, GS, HP, NL>;
-  return launch_dependent(decode_mma_kernel<BK, BV, GS, HP, NL>, dim3((unsigned)(p.ns_q * p.dm.B * p.dm.Hkv), p.n_layers / NL), dim3(Pl::WARPS * 32),
+  using Pl = Plan<BK, BV, GS, HP, NL, MANY>;
+  return launch_dependent(decode_mma_kernel<BK, BV, GS, HP, NL, MANY>, dim3((unsigned)(p.ns_q * p.dm.B * p.dm.Hkv), p.n_layers / NL), dim3(Pl::WARPS * 32),
                           (size_t)Pl::TOTAL, st, p);
 }
 
 // Prepares the kernel for the current device and says how many of its CTAs share an SM and how many warps each has.
 // (The occupancy calculator has no say on how many: it answers one for a kernel that allocates tensor memory.)
-template <int BK, int BV, int GS, int HP, int NL>
+template <int BK, int BV, int GS, int HP, int NL, bool MANY>
 MmaShape shape_one() {
-  using Pl = Plan<BK, BV, GS, HP, NL>;
-  auto kernel = decode_mma_kernel<BK, BV, GS, HP, NL>;
+  using Pl = Plan<BK, BV, GS, HP, NL, MANY>;
+  auto kernel = decode_mma_kernel<BK, BV, GS, HP, NL, MANY>;
   MmaShape r{Pl::CTAS, Pl::WARPS};
   // the largest shared-memory carve-out: three CTAs of this size are to share an SM
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Pl::TOTAL) != cudaSuccess ||
@@ -1328,25 +1329,25 @@ MmaShape shape_one() {
 
 #define XQ_DISPATCH(FN, ...)                               \
   switch (bk * 100 + bv * 10 + (g == 64)) {                \
-    case 220: return FN<2, 2, 32, HP, NL>(__VA_ARGS__); \
-    case 221: return FN<2, 2, 64, HP, NL>(__VA_ARGS__); \
-    case 210: return FN<2, 1, 32, HP, NL>(__VA_ARGS__); \
-    case 211: return FN<2, 1, 64, HP, NL>(__VA_ARGS__); \
-    case 120: return FN<1, 2, 32, HP, NL>(__VA_ARGS__); \
-    case 121: return FN<1, 2, 64, HP, NL>(__VA_ARGS__); \
-    case 110: return FN<1, 1, 32, HP, NL>(__VA_ARGS__); \
-    case 111: return FN<1, 1, 64, HP, NL>(__VA_ARGS__); \
+    case 220: return FN<2, 2, 32, HP, NL, MANY>(__VA_ARGS__); \
+    case 221: return FN<2, 2, 64, HP, NL, MANY>(__VA_ARGS__); \
+    case 210: return FN<2, 1, 32, HP, NL, MANY>(__VA_ARGS__); \
+    case 211: return FN<2, 1, 64, HP, NL, MANY>(__VA_ARGS__); \
+    case 120: return FN<1, 2, 32, HP, NL, MANY>(__VA_ARGS__); \
+    case 121: return FN<1, 2, 64, HP, NL, MANY>(__VA_ARGS__); \
+    case 110: return FN<1, 1, 32, HP, NL, MANY>(__VA_ARGS__); \
+    case 111: return FN<1, 1, 64, HP, NL, MANY>(__VA_ARGS__); \
   }
 
 }  // namespace
 
-template <int HP, int NL>
+template <int HP, int NL, bool MANY>
 cudaError_t launch_decode_mma_t(const DecodeParams& p, cudaStream_t st) {
   const int bk = p.layer[0].L.bk, bv = p.layer[0].L.bv, g = p.dm.g;
   XQ_DISPATCH(launch_one, p, st)
   return cudaErrorInvalidValue;
 }
-template <int HP, int NL>
+template <int HP, int NL, bool MANY>
 MmaShape decode_mma_shape_t(int g, int bk, int bv) {
   XQ_DISPATCH(shape_one)
   return MmaShape{0, 1};

@@ -2,6 +2,6 @@
 #include "xq_decode_mma.cuh"
 
 namespace xq {
-template cudaError_t launch_decode_mma_t<2, 2>(const DecodeParams&, cudaStream_t);
-template MmaShape decode_mma_shape_t<2, 2>(int, int, int);
+template cudaError_t launch_decode_mma_t<2, 2, false>(const DecodeParams&, cudaStream_t);
+template MmaShape decode_mma_shape_t<2, 2, false>(int, int, int);
 }  // namespace xq

@@ -1,0 +1,7 @@
+// Tensor-core decode kernels for head_dim 128, three or four query heads per kv head, for launches of many CTAs.
+#include "xq_decode_mma.cuh"
+
+namespace xq {
+template cudaError_t launch_decode_mma_t<4, 1, true>(const DecodeParams&, cudaStream_t);
+template MmaShape decode_mma_shape_t<4, 1, true>(int, int, int);
+}  // namespace xq

@@ -2,6 +2,6 @@
 #include "xq_decode_mma.cuh"
 
 namespace xq {
-template cudaError_t launch_decode_mma_t<8, 1>(const DecodeParams&, cudaStream_t);
-template MmaShape decode_mma_shape_t<8, 1>(int, int, int);
+template cudaError_t launch_decode_mma_t<8, 1, false>(const DecodeParams&, cudaStream_t);
+template MmaShape decode_mma_shape_t<8, 1, false>(int, int, int);
 }  // namespace xq

@@ -204,15 +204,17 @@ bool uses_mma(const xq_cache* c) {
   return dm.D == 128 || c->cfg.kernel == XQ_KERNEL_AUTO;  // XQ_KERNEL_MMA names the head_dim 128 kernel
 }
 
-// FN<HP, 1> of the head_dim 128 kernel that serves these dimensions, FN<HP, 2> of the one that takes two layers, FN<HP, NT>
-// of the head_dim 64 kernel
-#define XQ_MMA128(FN, ...) (dm.G == 1 ? FN<1, 1>(__VA_ARGS__) : dm.G == 2 ? FN<2, 1>(__VA_ARGS__) : dm.G <= 4 ? FN<4, 1>(__VA_ARGS__) : FN<8, 1>(__VA_ARGS__))
-#define XQ_MMA_PAIRS(FN, ...) (dm.G == 1 ? FN<1, 2>(__VA_ARGS__) : dm.G == 2 ? FN<2, 2>(__VA_ARGS__) : FN<4, 2>(__VA_ARGS__))
+// FN<HP, NL, MANY> of the head_dim 128 kernel that serves these dimensions: a layer, a layer in a launch of many CTAs, two
+// layers; FN<HP, NT> of the head_dim 64 kernel
+#define XQ_MMA128(FN, ...) (dm.G == 1 ? FN<1, 1, false>(__VA_ARGS__) : dm.G == 2 ? FN<2, 1, false>(__VA_ARGS__) : dm.G <= 4 ? FN<4, 1, false>(__VA_ARGS__) : FN<8, 1, false>(__VA_ARGS__))
+#define XQ_MMA_MANY(FN, ...) (dm.G == 1 ? FN<1, 1, true>(__VA_ARGS__) : dm.G == 2 ? FN<2, 1, true>(__VA_ARGS__) : FN<4, 1, true>(__VA_ARGS__))
+#define XQ_MMA_PAIRS(FN, ...) (dm.G == 1 ? FN<1, 2, false>(__VA_ARGS__) : dm.G == 2 ? FN<2, 2, false>(__VA_ARGS__) : FN<4, 2, false>(__VA_ARGS__))
 #define XQ_MMA64(FN, ...) (dm.G == 1 ? FN<1, 1>(__VA_ARGS__) : dm.G == 2 ? FN<2, 1>(__VA_ARGS__) : dm.G <= 4 ? FN<4, 1>(__VA_ARGS__) : FN<4, 2>(__VA_ARGS__))
 
 cudaError_t launch_decode_mma(const DecodeParams& p, cudaStream_t st) {
   const Dims& dm = p.dm;
   if (p.paired) return XQ_MMA_PAIRS(launch_decode_mma_t, p, st);
+  if (p.many) return XQ_MMA_MANY(launch_decode_mma_t, p, st);
   return dm.D == 128 ? XQ_MMA128(launch_decode_mma_t, p, st) : XQ_MMA64(launch_decode_mma64_t, p, st);
 }
 
@@ -227,7 +229,10 @@ MmaShape mma_shape(const xq_cache* c, int l) {
   MmaShape& s = const_cast<xq_cache*>(c)->mma_shape[bk - 1][bv - 1];
   if (s.warps == 0) {
     s = dm.D == 128 ? XQ_MMA128(decode_mma_shape_t, dm.g, bk, bv) : XQ_MMA64(decode_mma64_shape_t, dm.g, bk, bv);
-    if (takes_pairs(dm)) XQ_MMA_PAIRS(decode_mma_shape_t, dm.g, bk, bv);
+    if (takes_pairs(dm)) {
+      XQ_MMA_PAIRS(decode_mma_shape_t, dm.g, bk, bv);
+      XQ_MMA_MANY(decode_mma_shape_t, dm.g, bk, bv);
+    }
     s.ctas_per_sm = 2;  // of one wave of a launch alone: the third place is the next launch's
   }
   return s;
@@ -238,6 +243,7 @@ MmaShape mma_shape(const xq_cache* c, int l) {
 // 32k context 965 and 927 us, 48 layers with host buffers 1608 and 1521 us (each layer by itself then).  A model of one or two layers keeps a
 // launch per layer, which callers that watch xq_launch_count have seen so far (10.6 us for a tiny pair; 8.5 together).
 constexpr int MIN_JOINT_LAYERS = 3;
+constexpr int MANY_BATCHES = 12;  // batches of a CTA from which on a launch of many takes the kernel for that
 
 // Times of the tensor-core kernel, us, as plan_batches adds them up: fitted to 75 shapes (one to eight heads, 6 to 256
 // streams of 1500 to 131072 tokens; head_dim 64 by two), each with up to 29 numbers of splits; rms error 6 %.
@@ -455,6 +461,7 @@ int prepare_decode(const xq_cache* c, int layer, const void* q, void* out, int o
   p.dm = dm;
   p.n_layers = 1;
   p.paired = 0;
+  p.many = 0;
   p.layer[0] = {layer_ptrs(c, layer), (const uint16_t*)q, out, (const uint16_t*)K_new, (const uint16_t*)V_new};
   p.n_q = nq;
   p.r = r;
@@ -698,6 +705,12 @@ int decode_layers(xq_cache* c, const int* order, int n, const uint8_t* q, uint8_
       packed = packed || c->repacked[l] != 0;
     }
     p.n_layers = j - i;
+    // One by one, with many CTAs of some length, the kernel with three CTAs an SM: its tensor memory costs a CTA ~1 us, which
+    // short CTAs and launches of a few waves do not get back.  us of a layer of 12, without / with: 32k, four heads, batch 4,
+    // 28 batches a CTA 30.1 / 27.8, batch 1, 14 batches 9.1 / 8.5; one head at 8k, batch 4, 16 batches 8.5 / 8.0, batch 1, 7
+    // batches 3.0 / 3.2; two heads at 8k, batch 4, 8 batches 10.9 / 11.4; four at 2000 tokens, 5 batches 4.0 / 4.4.
+    const long long ctas = (long long)p.n_layers * p.ns_q * dm.B * dm.Hkv;
+    p.many = takes_pairs(dm) && !p.paired && p.n_q / (p.ns_q * XQ_BATCH) >= MANY_BATCHES && ctas >= 6LL * c->sm_count;
     // The packed streams may be fetched ahead of the preceding kernel unless a pack kernel wrote them since the
     // layers' last decode (then that kernel may be the writer, or only just behind it).  The launches after the first
     // are chained: nothing they read (q, the new token, the window, the packed streams) can still be written when

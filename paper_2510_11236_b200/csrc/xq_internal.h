@@ -91,6 +91,7 @@ struct DecodeParams {
   Dims dm;
   int n_layers;       // the scalar kernel takes one
   int paired;         // tensor-core kernel: a CTA takes layers 2 y and 2 y + 1, which read the same codes
+  int many;           // tensor-core kernel, head_dim 128, up to four heads, not paired: the variant for many CTAs
   int n_q;            // quantized tokens
   int r;              // window tokens
   int ns_q, ns_w;     // splits over the quantized region (most of any stream) / over the window
@@ -180,15 +181,15 @@ cudaError_t launch_pack(const PackParams& p, cudaStream_t st);
 cudaError_t launch_window_append(const WindowParams& p, cudaStream_t st);
 cudaError_t launch_decode_generic(const DecodeParams& p, cudaStream_t st);
 // Tensor-core decode kernels.  head_dim 128: for HP (1, 2, 4, 8) query heads per kv head, of one layer or of NL = 2 that
-// read the same codes (up to four heads); head_dim 64: HP (1, 2, 4) heads, or NT = 2 sets of four.  decode_mma_shape_t
+// read the same codes (up to four heads), MANY: of one layer of up to four, for launches of many CTAs; head_dim 64: HP (1, 2, 4) heads, or NT = 2 sets of four.  decode_mma_shape_t
 // also prepares the kernel for the current device: it comes before the first launch of a handle.
 struct MmaShape {
   int ctas_per_sm;  // 0: no device to ask
   int warps;        // warps of a CTA
 };
-template <int HP, int NL>
+template <int HP, int NL, bool MANY>
 cudaError_t launch_decode_mma_t(const DecodeParams& p, cudaStream_t st);
-template <int HP, int NL>
+template <int HP, int NL, bool MANY>
 MmaShape decode_mma_shape_t(int g, int bk, int bv);
 template <int HP, int NT>
 cudaError_t launch_decode_mma64_t(const DecodeParams& p, cudaStream_t st);

@@ -1143,3 +1143,30 @@ def test_decode_step_pairs_of_layers(G, bits, g, f16, S, group):
             assert torch.equal(b.decode_attention(l, q[l]), out[l]), (step, l)
     a.check_device()
     a.close(); b.close()
+
+
+@pytest.mark.parametrize("G,kq,vq,g,f16,S", [(1, 2, 2, 32, False, 1601), (1, 0, 2, 64, True, 1700), (2, 2, 0, 64, False, 1680),
+                                             (2, 0, 0, 32, True, 1601), (3, 2, 2, 32, False, 1650), (4, 2, 0, 32, True, 1601),
+                                             (4, 0, 2, 64, False, 1780)])
+def test_decode_step_of_many_ctas_one_layer_each(G, kq, vq, g, f16, S):
+    """Layers that share no codes, in launches of many CTAs of 12 or 13 batches: the kernel with its sums in tensor memory
+    between rounds, last batches of less and of more than half; bit for bit as xq_append_kv and xq_decode_attention."""
+    L, B, Hkv, D = 12, 4, 20, 128
+    kw = dict(n_layers=L, batch=B, n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=D, max_seq=S + 40, group_size=g, residual_len=64,
+              kq=kq and L, vq=vq and L, km=L, vm=L, eta1=1 / 6, eta2=0.045, io_dtype=xq.XQ_F16 if f16 else xq.XQ_BF16, n_splits=1)
+    a, b = xq.Cache(xq.make_config(**kw), DEV), xq.Cache(xq.make_config(**kw), DEV)
+    dt = torch.float16 if f16 else torch.bfloat16
+    gen = torch.Generator(device=DEV).manual_seed(S)
+    for l in range(L):
+        k, v = (torch.randn(B, Hkv, S, D, generator=gen, device=DEV).to(dt) for _ in range(2))
+        for cache in (a, b):
+            cache.append_kv(l, k, v)
+    for step in range(2):
+        kn, vn = (torch.randn(L, B, Hkv, 1, D, generator=gen, device=DEV).to(dt) for _ in range(2))
+        q = torch.randn(L, B, Hkv * G, D, generator=gen, device=DEV).to(dt) * (3.0 if step else 1.0)
+        out = a.decode_step(kn, vn, q, torch.empty_like(q))
+        for l in range(L):
+            b.append_kv(l, kn[l], vn[l])
+            assert torch.equal(b.decode_attention(l, q[l]), out[l]), (step, l)
+    a.check_device()
+    a.close(); b.close()
