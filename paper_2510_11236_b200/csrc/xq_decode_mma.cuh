@@ -1311,20 +1311,16 @@ cudaError_t launch_one(const DecodeParams& p, cudaStream_t st) {
                           (size_t)Pl::TOTAL, st, p);
 }
 
-// Prepares the kernel for the current device and says how many of its CTAs share an SM and how many warps each has.
-// (The occupancy calculator has no say on how many: it answers one for a kernel that allocates tensor memory.)
+// Prepares the kernel for the current device.
 template <int BK, int BV, int GS, int HP, int NL, bool MANY>
 MmaShape shape_one() {
   using Pl = Plan<BK, BV, GS, HP, NL, MANY>;
   auto kernel = decode_mma_kernel<BK, BV, GS, HP, NL, MANY>;
-  MmaShape r{Pl::CTAS, Pl::WARPS};
-  // the largest shared-memory carve-out: three CTAs of this size are to share an SM
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Pl::TOTAL) != cudaSuccess ||
-      cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess) {
-    cudaGetLastError();
-    r.ctas_per_sm = 0;
-  }
-  return r;
+  // the largest shared-memory carve-out: two or three CTAs of this size are to share an SM
+  const bool ready = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Pl::TOTAL) == cudaSuccess &&
+                     cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100) == cudaSuccess;
+  if (!ready) cudaGetLastError();
+  return {Pl::WARPS, ready};
 }
 
 #define XQ_DISPATCH(FN, ...)                               \
@@ -1350,7 +1346,7 @@ cudaError_t launch_decode_mma_t(const DecodeParams& p, cudaStream_t st) {
 template <int HP, int NL, bool MANY>
 MmaShape decode_mma_shape_t(int g, int bk, int bv) {
   XQ_DISPATCH(shape_one)
-  return MmaShape{0, 1};
+  return MmaShape{1, false};
 }
 
 }  // namespace xq

@@ -1003,20 +1003,16 @@ cudaError_t launch_one(const DecodeParams& p, cudaStream_t st) {
                           (size_t)Pl::TOTAL, st, p);
 }
 
-// Prepares the kernel for the current device and says how many of its CTAs share an SM and how many warps each has.
+// Prepares the kernel for the current device.
 template <int BK, int BV, int GS, int HP, int NT>
 MmaShape shape_one() {
   using Pl = Plan<BK, BV, GS, HP, NT>;
   auto kernel = decode_mma64_kernel<BK, BV, GS, HP, NT>;
-  MmaShape r{0, Pl::WARPS};
   // the largest shared-memory carve-out: two CTAs of this size are to share an SM
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Pl::TOTAL) != cudaSuccess ||
-      cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.ctas_per_sm, kernel, Pl::WARPS * 32, Pl::TOTAL) != cudaSuccess) {
-    cudaGetLastError();
-    r.ctas_per_sm = 0;
-  }
-  return r;
+  const bool ready = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Pl::TOTAL) == cudaSuccess &&
+                     cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100) == cudaSuccess;
+  if (!ready) cudaGetLastError();
+  return {Pl::WARPS, ready};
 }
 
 #define XQ_DISPATCH(FN, ...)                               \
@@ -1042,7 +1038,7 @@ cudaError_t launch_decode_mma64_t(const DecodeParams& p, cudaStream_t st) {
 template <int HP, int NT>
 MmaShape decode_mma64_shape_t(int g, int bk, int bv) {
   XQ_DISPATCH(shape_one)
-  return MmaShape{0, 1};
+  return MmaShape{1, false};
 }
 
 }  // namespace xq

@@ -124,6 +124,10 @@ constexpr int TIMING_POOL = 1 << 15;
 
 struct EventPair { cudaEvent_t a, b; int kind; };
 
+// The tensor-core kernels of a layer's bit-widths, prepared for the handle's device: warps of a CTA (0: not asked yet), and
+// whether the variants for pairs of layers and for many CTAs can be launched there.
+struct MmaKernels { int warps; bool pairs, many; };
+
 // modelled times, us: of a launch alone, and of one more in a row of launches that overlap
 struct MmaPlan { int batches, ns, deal; double alone, next; };
 
@@ -164,7 +168,7 @@ struct xq_cache {
   bool tickets_clean;  // the ticket counters have been zeroed on a stream
   bool delta_clean;    // the code-difference counters have been zeroed on a stream
   std::vector<uint8_t> repacked;  // per layer: codes or parameters it reads were written since its last decode
-  MmaShape mma_shape[2][2];  // the tensor-core kernel by (key bits - 1, value bits - 1); warps 0 = not asked yet
+  MmaKernels mma_kernels[2][2];  // by (key bits - 1, value bits - 1)
   MmaPlan mma_plan[2][2];    // and the splits of the latest number of batches asked for; batches 0 = none yet
   // timing
   bool timing;
@@ -213,6 +217,7 @@ bool uses_mma(const xq_cache* c) {
 
 cudaError_t launch_decode_mma(const DecodeParams& p, cudaStream_t st) {
   const Dims& dm = p.dm;
+  if (p.paired && p.n_layers % 2) return cudaErrorInvalidValue;  // (the last one would have no CTA)
   if (p.paired) return XQ_MMA_PAIRS(launch_decode_mma_t, p, st);
   if (p.many) return XQ_MMA_MANY(launch_decode_mma_t, p, st);
   return dm.D == 128 ? XQ_MMA128(launch_decode_mma_t, p, st) : XQ_MMA64(launch_decode_mma64_t, p, st);
@@ -222,20 +227,20 @@ cudaError_t launch_decode_mma(const DecodeParams& p, cudaStream_t st) {
 // its eight operand columns.
 bool takes_pairs(const Dims& dm) { return dm.D == 128 && dm.G <= 4; }
 
-// The tensor-core kernel that serves layer l, prepared for the handle's device on first use.
-MmaShape mma_shape(const xq_cache* c, int l) {
+// The tensor-core kernels that serve layer l, prepared for the handle's device on first use.  (One that is not ready fails
+// at its launch, but the variants of a step are then left out.)
+const MmaKernels& mma_kernels(const xq_cache* c, int l) {
   const Dims& dm = c->plan.dm;
   const int bk = layer_bits(l, c->cfg.kq), bv = layer_bits(l, c->cfg.vq);
-  MmaShape& s = const_cast<xq_cache*>(c)->mma_shape[bk - 1][bv - 1];
-  if (s.warps == 0) {
-    s = dm.D == 128 ? XQ_MMA128(decode_mma_shape_t, dm.g, bk, bv) : XQ_MMA64(decode_mma64_shape_t, dm.g, bk, bv);
+  MmaKernels& k = const_cast<xq_cache*>(c)->mma_kernels[bk - 1][bv - 1];
+  if (k.warps == 0) {
+    k.warps = (dm.D == 128 ? XQ_MMA128(decode_mma_shape_t, dm.g, bk, bv) : XQ_MMA64(decode_mma64_shape_t, dm.g, bk, bv)).warps;
     if (takes_pairs(dm)) {
-      XQ_MMA_PAIRS(decode_mma_shape_t, dm.g, bk, bv);
-      XQ_MMA_MANY(decode_mma_shape_t, dm.g, bk, bv);
+      k.pairs = XQ_MMA_PAIRS(decode_mma_shape_t, dm.g, bk, bv).ready;
+      k.many = XQ_MMA_MANY(decode_mma_shape_t, dm.g, bk, bv).ready;
     }
-    s.ctas_per_sm = 2;  // of one wave of a launch alone: the third place is the next launch's
   }
-  return s;
+  return k;
 }
 
 // Layers of a step from which on they share launches.  A launch of its own costs a layer ~2.5 us of host time and a
@@ -270,11 +275,12 @@ DecodeTimes decode_times(const Dims& dm) {
 // alone / in a step of 12 layers, with the plan best for the step and with this one: 32k, four heads 47.7 / 21.2,
 // 36.1 / 22.2; 16k 45.9 / 12.6, 23.6 / 13.6; groups of five at 16k 44.0 / 19.3, 29.9 / 20.7; MHA at 4k, batch 8, 30.4 /
 // 16.4 with either.
+constexpr int WAVE_CTAS = 2;  // CTAs of a layer's own launch on an SM: the third place, where there is one, is the next launch's
 constexpr double ALONE_BOUND = 1.10, STEP_WEIGHT = 1.2;
 constexpr double MERGE = 0.03;  // us of a launch's end for each partial of a stream
-void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int splits, MmaPlan& out) {
+void plan_batches(const xq_cache* c, int warps, int batches, int splits, MmaPlan& out) {
   const Dims& dm = c->plan.dm;
-  const long long streams = (long long)dm.B * dm.Hkv, slots = (long long)c->sm_count * shape.ctas_per_sm;
+  const long long streams = (long long)dm.B * dm.Hkv, slots = (long long)c->sm_count * WAVE_CTAS;
   const DecodeTimes t = decode_times(dm);
   const bool joint = c->cfg.n_layers >= MIN_JOINT_LAYERS;
   struct Candidate { int ns, deal; double alone, step, next; };
@@ -283,7 +289,7 @@ void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int spl
   double alone_min = 0.0, step_min = 0.0;
   // batches are dealt to the splits one by one, or in runs of one per warp: no warp of a CTA then waits for another's
   // last batch
-  for (int deal : {1, shape.warps}) {
+  for (int deal : {1, warps}) {
     const int runs = (batches + deal - 1) / deal;
     const int limit = runs < XQ_MAX_SPLITS ? runs : XQ_MAX_SPLITS;
     for (int ns = splits > 0 ? splits : 1; ns <= (splits > 0 ? splits : limit); ++ns) {
@@ -295,15 +301,15 @@ void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int spl
       // the last wave: a start and an end, and the rounds of a CTA, whose last one may leave warps without a batch
       auto wave = [&](long long ctas) {
         long long resident = (ctas + c->sm_count - 1) / c->sm_count;
-        if (resident > shape.ctas_per_sm) resident = shape.ctas_per_sm;
-        const int rounds = per / shape.warps;
-        double left = (double)batches / ns - rounds * shape.warps;  // on average: the SM's CTAs share its rate
-        if (left < 0.0 || per % shape.warps == 0) left = 0.0;
-        return t.launch + MERGE * ns + rounds * (t.round + t.warp * resident * shape.warps) + (left > 0.0 ? t.round + t.warp * resident * left : 0.0);
+        if (resident > WAVE_CTAS) resident = WAVE_CTAS;
+        const int rounds = per / warps;
+        double left = (double)batches / ns - rounds * warps;  // on average: the SM's CTAs share its rate
+        if (left < 0.0 || per % warps == 0) left = 0.0;
+        return t.launch + MERGE * ns + rounds * (t.round + t.warp * resident * warps) + (left > 0.0 ? t.round + t.warp * resident * left : 0.0);
       };
       // earlier waves: a CTA follows the one before it in its slot; the warps that have no batch in its last round idle
-      const int idle = deal == 1 ? (shape.warps - per % shape.warps) % shape.warps : 0;
-      const double each = t.cta + ((double)batches / ns * shape.ctas_per_sm + idle) * t.batch;
+      const int idle = deal == 1 ? (warps - per % warps) % warps : 0;
+      const double each = t.cta + ((double)batches / ns * WAVE_CTAS + idle) * t.batch;
       auto launch = [&](long long ctas) {
         const long long last_wave = (ctas - 1) % slots + 1;
         return (double)((ctas - last_wave) / slots) * each + wave(last_wave);
@@ -332,7 +338,7 @@ void plan_batches(const xq_cache* c, const MmaShape& shape, int batches, int spl
 // The plan of a number of batches is kept: making it costs the host about 10 us at 32k.
 const MmaPlan& batches_plan(const xq_cache* c, int l, int batches) {
   MmaPlan& plan = const_cast<xq_cache*>(c)->mma_plan[layer_bits(l, c->cfg.kq) - 1][layer_bits(l, c->cfg.vq) - 1];
-  if (plan.batches != batches) plan_batches(c, mma_shape(c, l), batches, c->cfg.n_splits < batches ? c->cfg.n_splits : batches, plan);
+  if (plan.batches != batches) plan_batches(c, mma_kernels(c, l).warps, batches, c->cfg.n_splits < batches ? c->cfg.n_splits : batches, plan);
   return plan;
 }
 
@@ -345,14 +351,14 @@ void plan_splits(const xq_cache* c, int l, int nq, int r, int& ns_q, int& ns_w, 
   int units = (nq + 31) / 32, tiles = (r + 15) / 16;
   const int streams = dm.B * dm.Hkv;
   if (uses_mma(c)) {
-    const MmaShape shape = mma_shape(c, l);
+    const int warps = mma_kernels(c, l).warps;
     const int batches = (nq + XQ_BATCH - 1) / XQ_BATCH;
     ns_w = 0;
     int deal = 1;
     if (batches == 0) {
       // the window alone: a round of a CTA's warps takes a tile each; more splits while that leaves the wave one wave
-      ns_q = c->cfg.n_splits > 0 ? c->cfg.n_splits : (tiles + shape.warps - 1) / shape.warps;
-      const int most = c->sm_count * shape.ctas_per_sm / streams;
+      ns_q = c->cfg.n_splits > 0 ? c->cfg.n_splits : (tiles + warps - 1) / warps;
+      const int most = c->sm_count * WAVE_CTAS / streams;
       if (c->cfg.n_splits == 0 && ns_q > most) ns_q = most > 1 ? most : 1;
       if (ns_q > tiles) ns_q = tiles;
       if (ns_q > XQ_MAX_SPLITS) ns_q = XQ_MAX_SPLITS;
@@ -690,7 +696,7 @@ int decode_layers(xq_cache* c, const int* order, int n, const uint8_t* q, uint8_
     // the layers of a launch share the scratch: XQ_MAX_SPLITS partials per query head
     int most = XQ_MAX_SPLITS / p.ns_q < DECODE_MAX_LAYERS ? XQ_MAX_SPLITS / p.ns_q : DECODE_MAX_LAYERS;
     if (!joint) most = 1;
-    p.paired = in_pair(i) && most >= 2;
+    p.paired = in_pair(i) && most >= 2 && mma_kernels(c, l0).pairs;
     if (p.paired) most -= most % 2;
     bool packed = c->repacked[l0] != 0;
     int j = i + 1;
@@ -710,7 +716,7 @@ int decode_layers(xq_cache* c, const int* order, int n, const uint8_t* q, uint8_
     // 28 batches a CTA 30.1 / 27.8, batch 1, 14 batches 9.1 / 8.5; one head at 8k, batch 4, 16 batches 8.5 / 8.0, batch 1, 7
     // batches 3.0 / 3.2; two heads at 8k, batch 4, 8 batches 10.9 / 11.4; four at 2000 tokens, 5 batches 4.0 / 4.4.
     const long long ctas = (long long)p.n_layers * p.ns_q * dm.B * dm.Hkv;
-    p.many = takes_pairs(dm) && !p.paired && p.n_q / (p.ns_q * XQ_BATCH) >= MANY_BATCHES && ctas >= 6LL * c->sm_count;
+    p.many = mma_kernels(c, l0).many && !p.paired && p.n_q / (p.ns_q * XQ_BATCH) >= MANY_BATCHES && ctas >= 6LL * c->sm_count;
     // The packed streams may be fetched ahead of the preceding kernel unless a pack kernel wrote them since the
     // layers' last decode (then that kernel may be the writer, or only just behind it).  The launches after the first
     // are chained: nothing they read (q, the new token, the window, the packed streams) can still be written when
@@ -766,7 +772,7 @@ int xq_create(const xq_config* cfg, void* dev_workspace, size_t bytes, xq_cache*
   c->delta_clean = false;
   c->device = -1;
   c->static_base = nullptr;
-  memset(c->mma_shape, 0, sizeof(c->mma_shape));
+  memset(c->mma_kernels, 0, sizeof(c->mma_kernels));
   memset(c->mma_plan, 0, sizeof(c->mma_plan));
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) == cudaSuccess &&

@@ -184,8 +184,8 @@ cudaError_t launch_decode_generic(const DecodeParams& p, cudaStream_t st);
 // read the same codes (up to four heads), MANY: of one layer of up to four, for launches of many CTAs; head_dim 64: HP (1, 2, 4) heads, or NT = 2 sets of four.  decode_mma_shape_t
 // also prepares the kernel for the current device: it comes before the first launch of a handle.
 struct MmaShape {
-  int ctas_per_sm;  // 0: no device to ask
-  int warps;        // warps of a CTA
+  int warps;   // warps of a CTA
+  bool ready;  // the kernel can be launched with its shared memory on this device
 };
 template <int HP, int NL, bool MANY>
 cudaError_t launch_decode_mma_t(const DecodeParams& p, cudaStream_t st);
