@@ -5,6 +5,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -170,6 +171,10 @@ struct xq_cache {
   std::vector<uint8_t> repacked;  // per layer: codes or parameters it reads were written since its last decode
   MmaKernels mma_kernels[2][2];  // by (key bits - 1, value bits - 1)
   MmaPlan mma_plan[2][2];    // and the splits of the latest number of batches asked for; batches 0 = none yet
+  // lists of xq_decode_step, n_layers long from the start: a step allocates nothing, and so cannot run out of host memory
+  // (an exception) when some of its launches are under way
+  std::vector<int> step_len, step_order, step_run;
+  std::vector<char> step_seen, step_paired, step_taken;
   // timing
   bool timing;
   std::vector<EventPair> pool;
@@ -661,12 +666,11 @@ int decode_layers(xq_cache* c, const int* order, int n, const uint8_t* q, uint8_
     pairs = (long long)ns_q * dm.B * dm.Hkv * n > 2LL * c->sm_count;
   }
   // in pairs, the layers as they go to the launches: two that share their codes side by side, in the place of the first
-  std::vector<int> run;
-  std::vector<char> paired;  // of run[i]: it is one of two
+  std::vector<int>& run = c->step_run;
+  std::vector<char>&paired = c->step_paired, &taken = c->step_taken;  // paired: of run[i], it is one of two
   if (pairs) {
-    run.reserve(n);
-    paired.reserve(n);
-    std::vector<char> taken(n, 0);
+    std::fill(taken.begin(), taken.begin() + n, 0);
+    int at = 0;
     for (int i = 0; i < n; ++i) {
       if (taken[i]) continue;
       const int a = order[i];
@@ -675,12 +679,12 @@ int decode_layers(xq_cache* c, const int* order, int n, const uint8_t* q, uint8_
         const int b = order[j];
         if (!taken[j] && c->seq[b] == c->seq[a] && k_owner(&c->cfg, a) == k_owner(&c->cfg, b) && v_owner(&c->cfg, a) == v_owner(&c->cfg, b)) with = j;
       }
-      run.push_back(a);
-      paired.push_back(with >= 0);
+      run[at] = a;
+      paired[at++] = with >= 0;
       if (with >= 0) {
         taken[with] = 1;
-        run.push_back(order[with]);
-        paired.push_back(1);
+        run[at] = order[with];
+        paired[at++] = 1;
       }
     }
     order = run.data();
@@ -744,9 +748,13 @@ int xq_config_check(const xq_config* cfg) { return check(cfg) ? XQ_OK : XQ_ERR_C
 
 size_t xq_workspace_bytes(const xq_config* cfg) {
   if (!check(cfg)) return 0;
-  Plan pl;
-  make_plan(cfg, pl);
-  return pl.total;
+  try {
+    Plan pl;
+    make_plan(cfg, pl);
+    return pl.total;
+  } catch (const std::bad_alloc&) {
+    return 0;
+  }
 }
 
 int xq_create(const xq_config* cfg, void* dev_workspace, size_t bytes, xq_cache** out) {
@@ -757,11 +765,18 @@ int xq_create(const xq_config* cfg, void* dev_workspace, size_t bytes, xq_cache*
   xq_cache* c = new (std::nothrow) xq_cache();
   if (!c) return XQ_ERR_NOMEM;
   c->cfg = *cfg;
-  make_plan(cfg, c->plan);
+  try {
+    make_plan(cfg, c->plan);
+    c->seq.assign(cfg->n_layers, 0);
+    c->repacked.assign(cfg->n_layers, 1);
+    for (auto* v : {&c->step_len, &c->step_order, &c->step_run}) v->assign(cfg->n_layers, 0);
+    for (auto* v : {&c->step_seen, &c->step_paired, &c->step_taken}) v->assign(cfg->n_layers, 0);
+  } catch (const std::bad_alloc&) {
+    delete c;
+    return XQ_ERR_NOMEM;
+  }
   if (bytes < c->plan.total) { delete c; return XQ_ERR_CAPACITY; }
   c->ws = (uint8_t*)dev_workspace;
-  c->seq.assign(cfg->n_layers, 0);
-  c->repacked.assign(cfg->n_layers, 1);
   c->launches = 0;
   c->last_cuda = 0;
   c->scale = cfg->sm_scale > 0.f ? cfg->sm_scale : 1.0f / sqrtf((float)cfg->head_dim);
@@ -1018,8 +1033,10 @@ int xq_decode_step(xq_cache* c, const void* K_new, const void* V_new, const void
   // Everything that can be refused is checked before the first copy or launch, on a copy of the layer lengths
   // advanced in processing order, so that a refused call leaves the cache as it was.
   {
-    std::vector<char> seen(L, 0);
-    std::vector<int> len(c->seq);
+    std::vector<char>& seen = c->step_seen;
+    std::vector<int>& len = c->step_len;
+    std::fill(seen.begin(), seen.end(), 0);
+    std::copy(c->seq.begin(), c->seq.end(), len.begin());
     for (int i = 0; i < L; ++i) {
       const int l = layer_order ? layer_order[i] : i;
       if (l < 0 || l >= L || seen[l]) return XQ_ERR_ARG;
@@ -1071,7 +1088,7 @@ int xq_decode_step(xq_cache* c, const void* K_new, const void* V_new, const void
       appended = true;
     }
   }
-  std::vector<int> order(L);
+  std::vector<int>& order = c->step_order;
   for (int i = 0; i < L; ++i) order[i] = layer_order ? layer_order[i] : i;
   for (int i = 0; i < L;) {
     const int l = order[i];
@@ -1168,7 +1185,11 @@ long long xq_launch_count(const xq_cache* c) { return c ? c->launches : 0; }
 int xq_timing_enable(xq_cache* c, int on) {
   if (!c) return XQ_ERR_ARG;
   if (on && c->pool.empty()) {
-    c->pool.reserve(TIMING_POOL);
+    try {
+      c->pool.reserve(TIMING_POOL);
+    } catch (const std::bad_alloc&) {
+      return XQ_ERR_NOMEM;
+    }
     for (int i = 0; i < TIMING_POOL; ++i) {
       EventPair e;
       if (cudaEventCreate(&e.a) != cudaSuccess || cudaEventCreate(&e.b) != cudaSuccess)

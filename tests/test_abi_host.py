@@ -3,6 +3,8 @@ declared symbol, validates configurations and evaluates the equivalent bit-width
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -159,3 +161,59 @@ def test_decode_step_refuses_before_it_touches_anything():
     assert xq.xq_decode_step(h, a, a, a, a) == xq.XQ_ERR_CONFIG
     assert xq.xq_seq_len(h, 0) == 0 and xq.xq_reset(h) == 0
     assert xq.xq_destroy(h) == 0
+
+
+FAILING_NEW = r"""
+#include <cstdlib>
+#include <new>
+extern "C" long new_left = -1;  // calls until one fails (-1: none does)
+static void* get(std::size_t n) { return new_left >= 0 && new_left-- == 0 ? nullptr : std::malloc(n ? n : 1); }
+void* operator new(std::size_t n) { void* p = get(n); if (!p) throw std::bad_alloc(); return p; }
+void* operator new[](std::size_t n) { return operator new(n); }
+void* operator new(std::size_t n, const std::nothrow_t&) noexcept { return get(n); }
+void operator delete(void* p) noexcept { std::free(p); }
+void operator delete(void* p, std::size_t) noexcept { std::free(p); }
+void operator delete[](void* p) noexcept { std::free(p); }
+void operator delete[](void* p, std::size_t) noexcept { std::free(p); }
+"""
+
+OUT_OF_MEMORY = r"""
+import ctypes, sys
+left = ctypes.c_long.in_dll(ctypes.CDLL(sys.argv[1]), "new_left")
+import paper_2510_11236_b200 as xq
+lib = xq.binding.lib()
+cfg = xq.make_config(n_layers=6, batch=1, n_q_heads=8, n_kv_heads=2, head_dim=128, max_seq=512)
+handle, results = ctypes.c_void_p(), []
+
+def call(f, *args):
+    for n in range(40):  # the first, the second ... allocation of the call fails, then none does
+        left.value = n
+        rc = f(*args)
+        spent, left.value = left.value < 0, -1
+        results.append((f.__name__, n, rc))
+        if not spent:
+            return rc
+
+whole = call(lib.xq_workspace_bytes, ctypes.byref(cfg))
+assert whole > 0 and all(rc == 0 for _, _, rc in results[:-1]) and len(results) > 1, results
+created = len(results)
+assert call(lib.xq_create, ctypes.byref(cfg), 256, 1 << 40, ctypes.byref(handle)) == xq.XQ_OK
+assert all(rc == xq.XQ_ERR_NOMEM for _, _, rc in results[created:-1]) and len(results) > created + 2, results
+a, order = 1 << 20, (ctypes.c_int32 * 6)(1, 0, 2, 3, 4, 5)  # refused: layer 1 reads layer 0's codes
+left.value = 0
+assert lib.xq_decode_step(handle, a, a, a, a, order, 0, 0) == xq.XQ_ERR_ORDER and left.value == 0  # allocates nothing
+left.value = -1
+print("done")
+"""
+
+
+def test_out_of_host_memory_is_an_error_code(tmp_path):
+    """An allocation that fails inside a C entry comes back as XQ_ERR_NOMEM (xq_workspace_bytes: 0), never as a C++
+    exception, and xq_decode_step allocates nothing.  A child process whose operator new fails on request, no device."""
+    source, preload = tmp_path / "new.cpp", tmp_path / "libnew.so"
+    source.write_text(FAILING_NEW)
+    subprocess.run(["g++", "-shared", "-fPIC", "-O1", str(source), "-o", str(preload)], check=True)
+    env = dict(os.environ, LD_PRELOAD=str(preload), CUDA_VISIBLE_DEVICES="", PYTHONPATH=ROOT)
+    child = subprocess.run([sys.executable, "-c", OUT_OF_MEMORY, str(preload)], env=env, cwd=ROOT, capture_output=True,
+                           text=True, timeout=300)
+    assert child.returncode == 0 and child.stdout.strip().endswith("done"), (child.returncode, child.stdout, child.stderr[-2000:])
