@@ -331,19 +331,20 @@ def main():
                 tot += W.algorithmic_bytes(w, first_seq + i, l)
         return tot
 
-    def moved_bytes(first_seq, n_steps):
-        """What the launches of these steps must move: with up to four heads per kv head the layers of a pair are decoded
-        together and their shared codes are read once (step_bytes counts them for each layer)."""
-        tot = step_bytes(first_seq, n_steps)
-        if w["head_dim"] != 128 or w["n_q_heads"] > 4 * w["n_kv_heads"]:
-            return tot
+    def moved_bytes(first_seq, n_steps, paired):
+        """What the launches of these steps must move: step_bytes counts the codes for each layer, but layers that the library
+        decoded in pairs (`paired` of them in these steps, xq_pair_count) read them once.  Only layers that share both keys
+        and values go in pairs."""
+        shared = 0
+        could = range(max(w["km"], w["vm"]) | 1, L, 2)
         for i in range(n_steps):
             S = first_seq + i
             nq = S - ((S - 1) % w["residual_len"] + 1)
-            for l in range(1, L, 2):
-                bits = (2 if l < w["kq"] else 1) * (l >= w["km"]) + (2 if l < w["vq"] else 1) * (l >= w["vm"])
-                tot -= w["batch"] * w["n_kv_heads"] * nq * w["head_dim"] * bits // 8
-        return tot
+            for l in could:
+                bits = (2 if l < w["kq"] else 1) + (2 if l < w["vq"] else 1)
+                shared += w["batch"] * w["n_kv_heads"] * nq * w["head_dim"] * bits // 8
+        share = paired / (2 * n_steps * len(could)) if len(could) else 0.0
+        return step_bytes(first_seq, n_steps) - shared * share
 
     import datetime
     sampler = ClockSampler(local) if rank == 0 else None  # runs from before the warm-up to the end of pass 3
@@ -354,6 +355,7 @@ def main():
     # ---- pass 1: whole steps, inputs resident in HBM
     seq_before = cache.seq_len(0)
     launches_before = xq.xq_launch_count(cache.handle)
+    paired_before = xq.xq_pair_count(cache.handle)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     barrier()
     t_lo = datetime.datetime.now()
@@ -373,6 +375,7 @@ def main():
     # ---- pass 2: the same steps with CUDA events around every kernel (roofline of the dominant kernel)
     xq.xq_timing_enable(cache.handle, 1)
     seq_before2 = cache.seq_len(0)
+    paired_pass1 = xq.xq_pair_count(cache.handle) - paired_before
     barrier()
     for _ in range(K):
         device_step()
@@ -384,13 +387,14 @@ def main():
     xq.xq_timing_enable(cache.handle, 0)
     dec = kinds["decode_split"]
     peak, peak_kind = _peaks()
-    isolated = moved_bytes(seq_before2 + 1, K) / (dec["total_ms"] * 1e-3) / 1e9 if dec["launches"] else 0.0
+    paired_pass2 = xq.xq_pair_count(cache.handle) - paired_before - paired_pass1
+    isolated = moved_bytes(seq_before2 + 1, K, paired_pass2) / (dec["total_ms"] * 1e-3) / 1e9 if dec["launches"] else 0.0
     # The layers of a step share decode launches, which run back to back, so a layer call's duration is the timed
     # region's time over the number of layer calls; the few other kernels of the region (the steps that quantize a
     # window block) are charged to them.
     layer_calls_pass1 = K * L
     avg_launch_us = ms / layer_calls_pass1 * 1e3
-    moved_pass1 = moved_bytes(seq_before + 1, K)
+    moved_pass1 = moved_bytes(seq_before + 1, K, paired_pass1)
     achieved = moved_pass1 / (ms * 1e-3) / 1e9
 
     # ---- pass 3: end to end through the C ABI with host buffers

@@ -311,6 +311,9 @@ int xq_region(const xq_cache* c, int layer, int which, size_t* offset, size_t* s
 
 /* Kernel launches issued through this handle since creation (all kinds). */
 long long xq_launch_count(const xq_cache* c);
+/* Layers that decode steps of this handle have taken two at a time since creation, one
+ * pass over the codes that the two share (tests, counting of bytes). */
+long long xq_pair_count(const xq_cache* c);
 
 /* Optional per-kernel timing with CUDA events recorded on the launching stream
  * around each kernel.  xq_timing_enable(c, 1) allocates an event pool (host

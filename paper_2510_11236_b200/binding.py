@@ -68,6 +68,7 @@ _SIGNATURES = {
     "xq_region": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_size_t),
                                  ctypes.POINTER(ctypes.c_size_t)]),
     "xq_launch_count": (ctypes.c_longlong, [ctypes.c_void_p]),
+    "xq_pair_count": (ctypes.c_longlong, [ctypes.c_void_p]),
     "xq_timing_enable": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]),
     "xq_timing_read": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.POINTER(ctypes.c_int),
                                       ctypes.POINTER(ctypes.c_double)]),
@@ -203,6 +204,10 @@ def xq_region(handle, layer: int, which: int):
 
 def xq_launch_count(handle) -> int:
     return lib().xq_launch_count(handle)
+
+
+def xq_pair_count(handle) -> int:
+    return lib().xq_pair_count(handle)
 
 
 def xq_timing_enable(handle, on: int) -> int:

@@ -160,7 +160,7 @@ struct xq_cache {
   Plan plan;
   uint8_t* ws;
   std::vector<int> seq;  // tokens cached per layer
-  long long launches;
+  long long launches, pair_layers;
   int last_cuda;
   float scale;
   int sm_count;
@@ -732,6 +732,7 @@ int decode_layers(xq_cache* c, const int* order, int n, const uint8_t* q, uint8_
       c->tickets_clean = false;
       return rc;
     }
+    if (p.paired) c->pair_layers += p.n_layers;
     for (; i < j; ++i) {
       c->repacked[order[i]] = 0;
       if (K_new) c->seq[order[i]] += 1;
@@ -777,7 +778,7 @@ int xq_create(const xq_config* cfg, void* dev_workspace, size_t bytes, xq_cache*
   }
   if (bytes < c->plan.total) { delete c; return XQ_ERR_CAPACITY; }
   c->ws = (uint8_t*)dev_workspace;
-  c->launches = 0;
+  c->launches = c->pair_layers = 0;
   c->last_cuda = 0;
   c->scale = cfg->sm_scale > 0.f ? cfg->sm_scale : 1.0f / sqrtf((float)cfg->head_dim);
   c->timing = false;
@@ -1181,6 +1182,7 @@ int xq_region(const xq_cache* c, int layer, int which, size_t* offset, size_t* s
 }
 
 long long xq_launch_count(const xq_cache* c) { return c ? c->launches : 0; }
+long long xq_pair_count(const xq_cache* c) { return c ? c->pair_layers : 0; }
 
 int xq_timing_enable(xq_cache* c, int on) {
   if (!c) return XQ_ERR_ARG;

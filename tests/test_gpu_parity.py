@@ -973,6 +973,62 @@ def test_key_scales_far_from_one(G, kq, f16, kind):
     assert _relative_error(cache, cfg, {0: (K, V)}, 0, q) <= 1.2e-4
 
 
+def _step_equals_single_calls(kw, lengths, steps, f16=False):
+    """Decode steps against xq_append_kv and xq_decode_attention layer by layer, bit for bit; returns how many layers each
+    step took in pairs."""
+    a, b = xq.Cache(xq.make_config(**kw), DEV), xq.Cache(xq.make_config(**kw), DEV)
+    dt = torch.float16 if f16 else torch.bfloat16
+    L, B, Hkv, Hq, D = len(lengths), kw["batch"], kw["n_kv_heads"], kw["n_q_heads"], kw["head_dim"]
+    gen = torch.Generator(device=DEV).manual_seed(sum(lengths))
+    for l, S in enumerate(lengths):
+        k, v = (torch.randn(B, Hkv, S, D, generator=gen, device=DEV).to(dt) for _ in range(2))
+        for cache in (a, b):
+            cache.append_kv(l, k, v)
+    paired = []
+    for step in range(steps):
+        kn, vn = (torch.randn(L, B, Hkv, 1, D, generator=gen, device=DEV).to(dt) for _ in range(2))
+        q = torch.randn(L, B, Hq, D, generator=gen, device=DEV).to(dt)
+        before = xq.xq_pair_count(a.handle)
+        out = a.decode_step(kn, vn, q, torch.empty_like(q))
+        paired.append(xq.xq_pair_count(a.handle) - before)
+        for l in range(L):
+            b.append_kv(l, kn[l], vn[l])
+        for l in range(L):
+            assert torch.equal(b.decode_attention(l, q[l]), out[l]), (step, l)
+    a.check_device()
+    a.close(); b.close()
+    return paired
+
+
+@pytest.mark.parametrize("G,L,group,kq,vq,km,vm,ahead,S,want", [
+    (4, 9, 3, 9, 9, 0, 0, 0, 300, [6, 6]),           # groups of three: a pair and a layer by itself
+    (1, 8, 0, 8, 0, 4, 2, 0, 300, [4, 4]),           # from layer 4 on both kinds are shared
+    (2, 8, 0, 8, 0, 2, 8, 0, 300, [0, 0]),           # keys alone: nothing goes in pairs
+    (3, 8, 0, 4, 2, 0, 0, 0, 300, [8, 8]),           # three combinations of bit-widths
+    (4, 8, 0, 4, 2, 0, 2, 5, 300, [6, 6]),           # and a last pair of another length
+    (1, 8, 0, 0, 8, 0, 0, 5, 315, [8, 8, 8, 8, 8, 8, 8]),  # the last pair, then the others fill a window block meanwhile
+])
+def test_decode_step_mixed_layers_in_pairs(G, L, group, kq, vq, km, vm, ahead, S, want):
+    """Steps of more than one wave of CTAs in which only some layers go in pairs, or pairs in several launches."""
+    kw = dict(n_layers=L, batch=4, n_q_heads=14 * G, n_kv_heads=14, head_dim=128, max_seq=S + 40, residual_len=32, kq=kq,
+              vq=vq, km=km, vm=vm, eta1=1 / 6, eta2=0.045, share_group=group, n_splits=2)
+    lengths = [S + (ahead if l >= L - 2 else 0) for l in range(L)]
+    paired = _step_equals_single_calls(kw, lengths, len(want))
+    fills = [any((n + i) % 32 == 0 for n in lengths) and len(set(lengths)) > 1 for i in range(len(want))]
+    for got, expected, fill in zip(paired, want, fills):  # (a layer whose block fills appends on its own first)
+        assert got == expected or (fill and got < expected), (paired, fills)
+    assert not all(fills)
+
+
+@pytest.mark.parametrize("n_splits,want", [(64, 4), (85, 4), (100, 4), (128, 4), (129, 0), (200, 0)])
+def test_decode_step_pairs_within_the_scratch(n_splits, want):
+    """The partials of a launch's layers share XQ_MAX_SPLITS a query head: launches of four layers, of three (a pair), of two,
+    of one."""
+    kw = dict(n_layers=4, batch=1, n_q_heads=4, n_kv_heads=2, head_dim=128, max_seq=26100, residual_len=32, eta1=1 / 6,
+              eta2=0.045, n_splits=n_splits)
+    assert _step_equals_single_calls(kw, [26000] * 4, 2) == [want, want]
+
+
 @pytest.mark.parametrize("G,kq", [(1, 0), (1, 2), (2, 0), (2, 2)])
 @pytest.mark.parametrize("octaves", [11, 12, 13])
 def test_key_scales_of_one_and_two_heads_are_used_as_stored(G, kq, octaves):
