@@ -142,7 +142,8 @@ typedef struct xq_cache xq_cache; /* opaque; owns host memory only */
 int xq_config_check(const xq_config* cfg);
 
 /* Device bytes xq_create needs for `cfg`: windows, scale / zero-point, codes of
- * code-owning layers, split-K partials and the host-staging area.  0 if invalid. */
+ * code-owning layers, split-K partials and the host-staging area.  0 if invalid, or
+ * out of host memory. */
 size_t xq_workspace_bytes(const xq_config* cfg);
 
 /* Creates a cache over the caller's device buffer `dev_workspace` (256-byte

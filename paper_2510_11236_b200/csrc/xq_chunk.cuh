@@ -96,7 +96,7 @@ struct ChunkPlan {
   // of its norm off.  With head_dim 64, where the scalar kernel is the measure (4.1, 5.3, 7.8e-7 at 512, 2000, 8000
   // tokens), sums of 8 tiles leave 15.6e-7 at 8000, of 4 10.8e-7, of 2 8.5e-7, and those with the small products first
   // 4.4, 5.8, 7.6e-7.  300 query tokens at 2048: 49 us without, 50, 52, 56 us.  (head_dim 128 has no columns left; its
-  // measure, one decode call per token, is 1.0-1.7e-4.)
+  // measure, one decode call per token, is 0.2-1.4e-5.)
   static constexpr int FLUSH = D == 64 ? 2 : 0;
   static_assert(TOTAL <= 226 * 1024, "shared memory");
 };

@@ -35,13 +35,16 @@
 // large operand; a tcgen05 kernel has to pass them through tensor memory and hand batches between warps, and one that
 // did spent a batch's ~1600 cycles on that chain of hand-overs, two batches per SM at a time (32k context, four heads:
 // 34.2 us per layer).
-// What bounds it: the math pipes together.  A batch of two layers with four heads is ~2700 warp instructions, 512 of them
-// masks (2 cycles each per sub-partition), 290 products (8 cycles of the tensor pipe, ~2.7 of everyone's issue), ~400
-// half-precision multiplies (2 cycles); a CTA's start and end add ~400 a batch at 32k.  A sub-partition takes 2.62 us for
-// it with long ranges, 16 or 24 warps on the SM alike, copies from L2 or from HBM alike (1.32 us at the HBM rate); issue
-// slots 56 %, tensor pipe 44 %, ALU 40 %, shared-memory pipe 57 %.  Left out in a copy, one at a time: key products 0.92,
-// value products 0.78, biases 0.16, value scales 0.19, key scales 0.11, numerators 0.14 us.  Starting warps at different
-// times, half of the packed words' loads or the exponentials left out: no change.
+// What bounds it: not one pipe.  In a launch of four layers at 32k, four heads, issue slots are 52 % used, the tensor pipe
+// 38 %, ALU 37 %, the shared-memory pipe 41 %.  A batch of two layers is ~3080 warp instructions there (~2700 in long ranges,
+// where a CTA's start and end do not count), 512 of them masks (2 cycles each per sub-partition), 290 products (8 cycles of
+// the tensor pipe, ~2.7 of everyone's issue), ~400 half-precision multiplies (2 cycles).  Microbenchmarks of the instructions
+// of both product phases come to 2900 of the 5150 cycles that a sub-partition takes for the batch (2.62 us in long ranges, 16
+// or 24 warps on the SM alike, copies from L2 or HBM alike; 1.32 us at the HBM rate).  Of the rest, the issue of copies is
+// known (load_key_codes); what else the warps wait for is not.  Left out in a copy, one at a time: key products 0.92, value
+// products 0.78, biases 0.16, value scales 0.19, key scales 0.11, numerators 0.14 us.  Starting warps at different times,
+// half of the packed words' loads or the exponentials left out: no change.
+// Spills, bytes stored: pairs of four heads 56 to 116, eight heads 44 to 68, MANY 16 to 60, the others up to 20.
 // Measured and not kept: twelve warps a CTA, two CTAs (the same speed of a step, single calls 2 us slower); sums in
 // registers with eight heads (128 registers, two CTAs: 4 % slower).
 #pragma once
