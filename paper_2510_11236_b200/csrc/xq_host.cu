@@ -255,19 +255,25 @@ const MmaKernels& mma_kernels(const xq_cache* c, int l) {
 constexpr int MIN_JOINT_LAYERS = 3;
 constexpr int MANY_BATCHES = 12;  // batches of a CTA from which on a launch of many takes the kernel for that
 
-// Times of the tensor-core kernel, us, as plan_batches adds them up: fitted to 75 shapes (one to eight heads, 6 to 256
-// streams of 1500 to 131072 tokens; head_dim 64 by two), each with up to 29 numbers of splits; rms error 6 %.
+// Times of the tensor-core kernel, us, as plan_batches adds them up.  They rank plans and are not predictions: head_dim 64
+// and one to four heads were fitted (75 shapes, rms error 6 %) when a warp took whole batches and every layer of a step its
+// own CTAs, five to eight heads to the kernel with half batches.  What the picks are worth with the present kernels, 37 shapes
+// of head_dim 128 (4 to 256 streams of 1300 to 64000 tokens), each with up to 20 numbers of splits: a call alone takes 1.08
+// times the best, a layer of a step of twelve 1.09 times (geometric means); worst alone 1.3 (2000 tokens: a step wants one or
+// two splits there, a call alone eight), worst in a step 1.5 (eight heads, eight streams of 8k), because one plan serves both.
 struct DecodeTimes {
   double launch;         // start and end of a launch that runs alone
   double round, warp;    // a warp's batch, while w warps of its SM work: round + warp * w
   double floor;          // host time of a call: no plan makes a layer alone faster
-  double cta, batch;     // with other CTAs waiting for the slot: a CTA's start and end, and a batch's share of the SM
+  // with other CTAs waiting for the slot: a CTA's start and end (up to four heads, in pairs: 1 us in long ranges, 3 in short
+  // ones for a layer; a layer by itself twice that), and a batch's share of the SM
+  double cta, batch;
 };
 DecodeTimes decode_times(const Dims& dm) {
   if (dm.D == 64) return {6.5, 1.0, 0.19, 9.0, 4.0, 0.25};
-  if (dm.G == 1) return {7.3, 0.48, 0.34, 10.0, 3.8, 0.37};
-  if (dm.G == 2) return {7.0, 0.71, 0.36, 10.0, 4.1, 0.40};
-  if (dm.G <= 4) return {7.2, 0.91, 0.37, 10.0, 4.0, 0.44};
+  if (dm.G == 1) return {7.3, 0.48, 0.34, 10.0, 1.9, 0.37};
+  if (dm.G == 2) return {7.0, 0.71, 0.36, 10.0, 2.05, 0.40};
+  if (dm.G <= 4) return {7.2, 0.91, 0.37, 10.0, 2.0, 0.44};
   return {8.3, 1.9, 0.50, 10.0, 5.0, 0.68};  // (13 shapes: 32k, batch 4, eight heads 47.9 alone, 16k, five heads 29.8)
 }
 
@@ -277,11 +283,11 @@ DecodeTimes decode_times(const Dims& dm) {
 // the next can call), which wants the CTAs of one full wave, and xq_decode_step, whose layers share launches and which
 // wants few CTAs.  The single call counts: of the plans that cost a layer alone at most ALONE_BOUND times the best, the
 // one with the smallest sum of the time alone, relative to the best, and STEP_WEIGHT times that in a step.  us per layer,
-// alone / in a step of 12 layers, with the plan best for the step and with this one: 32k, four heads 47.7 / 21.2,
-// 36.1 / 22.2; 16k 45.9 / 12.6, 23.6 / 13.6; groups of five at 16k 44.0 / 19.3, 29.9 / 20.7; MHA at 4k, batch 8, 30.4 /
-// 16.4 with either.
-constexpr int WAVE_CTAS = 2;  // CTAs of a layer's own launch on an SM: the third place, where there is one, is the next launch's
+// alone / in a step of 12 layers, with the plan best for the step and with this one: 32k, four heads 46.9 / 21.0,
+// 35.6 / 21.8; 16k 27.7 / 12.5, 21.6 / 13.1; groups of five at 16k 34.0 / 19.3, 30.2 / 20.5; MHA at 4k, batch 8, 30.3 /
+// 15.5 with either.
 constexpr double ALONE_BOUND = 1.10, STEP_WEIGHT = 1.2;
+constexpr int WAVE_CTAS = 2;    // CTAs of a layer's own launch on an SM: the third place, where there is one, is the next launch's
 constexpr double MERGE = 0.03;  // us of a launch's end for each partial of a stream
 void plan_batches(const xq_cache* c, int warps, int batches, int splits, MmaPlan& out) {
   const Dims& dm = c->plan.dm;
@@ -292,8 +298,8 @@ void plan_batches(const xq_cache* c, int warps, int batches, int splits, MmaPlan
   Candidate all[2 * XQ_MAX_SPLITS];
   int n = 0;
   double alone_min = 0.0, step_min = 0.0;
-  // batches are dealt to the splits one by one, or in runs of one per warp: no warp of a CTA then waits for another's
-  // last batch
+  // batches are dealt to the splits one by one, or in runs of one per warp (head_dim 128: of two rounds a warp): no warp of
+  // a CTA then waits for another's last batch
   for (int deal : {1, warps}) {
     const int runs = (batches + deal - 1) / deal;
     const int limit = runs < XQ_MAX_SPLITS ? runs : XQ_MAX_SPLITS;
@@ -320,7 +326,7 @@ void plan_batches(const xq_cache* c, int warps, int batches, int splits, MmaPlan
         return (double)((ctas - last_wave) / slots) * each + wave(last_wave);
       };
       Candidate k{ns, deal, launch(streams * ns), joint ? launch(streams * ns * c->cfg.n_layers) / c->cfg.n_layers : 1.0,
-                  (dm.G > 4 ? 5.5 : 2.5) + (double)(streams * ns) / slots * each};
+                  (dm.G > 4 ? 5.5 : 2.5) + (double)(streams * ns) / slots * (each + (takes_pairs(dm) ? t.cta : 0.0))};
       if (k.alone < t.floor) k.alone = t.floor;
       if (n == 0 || k.alone < alone_min) alone_min = k.alone;
       if (n == 0 || k.step < step_min) step_min = k.step;
@@ -898,9 +904,9 @@ int plan_chunk(const xq_cache* c, int S, int T, int row_tiles) {
 // which expands every tile of 64 tokens whatever T is.  Modelled times in us, fitted to T = 2 .. 16 on 19 shapes:
 // decode, as plan_batches has them; chunk, 14 for a wave (head_dim 64: 9), 1.47 (1.1) for a tile, 4 and 0.02 for each
 // partial of a row where splits merge.
-// Tokens from which on the chunk kernel is chosen / was measured to be the faster: four heads, 32k, batch 4 7 / 8; one
-// sequence of 1000 6 / 8, of 8000 6 / 7, of 128k 13 / 14; MHA at 4k, batch 8 9 / 11; groups of five at 16k 3 / 4, of
-// eight at 8k 3 / 4.  Two tokens at 32k, batch 4: 64 us a layer, in the chunk kernel 217.
+// Tokens from which on the chunk kernel is chosen / was measured to be the faster: four heads, 32k, batch 4 7 / 7; one
+// sequence of 1000 7 / 7, of 8000 7 / 7, of 128k 13 / 12; MHA at 4k, batch 8 9 / 10; groups of five at 16k 4 / 5, of
+// eight at 8k 4 / 4.  Two tokens at 32k, batch 4: 70 us a layer, in the chunk kernel 194.
 bool tokens_one_by_one(const xq_cache* c, int layer, int T) {
   if (T > 16) return false;  // (and the host's 2 us a launch)
   const Dims& dm = c->plan.dm;
