@@ -44,7 +44,7 @@
 // known (load_key_codes); what else the warps wait for is not.  Left out in a copy, one at a time: key products 0.92, value
 // products 0.78, biases 0.16, value scales 0.19, key scales 0.11, numerators 0.14 us.  Starting warps at different times,
 // half of the packed words' loads or the exponentials left out: no change.
-// Spills, bytes stored: pairs of four heads 56 to 116, eight heads 44 to 68, MANY 16 to 60, the others up to 20.
+// Spills, bytes stored: pairs of four heads 56 to 76, eight heads 44 to 60, MANY 16 to 60, the others up to 20.
 // Measured and not kept: twelve warps a CTA, two CTAs (the same speed of a step, single calls 2 us slower); sums in
 // registers with eight heads (128 registers, two CTAs: 4 % slower).
 #pragma once
@@ -440,7 +440,9 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL, MANY>::WARPS * 32, Pl
   // 3 % faster, pairs slower), products of more row tiles at a time, q kept in registers (no change).
   auto half_of = [&](int r) { return (unsigned)(warp + W * r); };
   struct Sources { const uint8_t *codes, *params[NL]; };
-  auto sources = [&](int kind) {  // read before the copies, which are not reordered
+  // read before the copies, which are not reordered (eight heads: by all lanes, before the branch, with less to spill: pairs of
+  // three heads, groups of 64, 263.5 -> 261.8 us; five heads, groups of 64, 153.5 -> 150.2)
+  auto sources = [&](int kind) {
     Sources s;
     s.codes = src_sm[kind];
 #pragma unroll
@@ -890,11 +892,13 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL, MANY>::WARPS * 32, Pl
       }
     }
     // the key half of the stage is free: fetch the keys of this warp's next round
+    Sources sk;
+    if constexpr (WIDE) sk = sources(0);
     proxy_fence();
     __syncwarp();
     if (r + 1 < rounds) {
       if (elect_one()) {
-        const Sources sk = sources(0);
+        if constexpr (!WIDE) sk = sources(0);
         load_key_codes(r + 1, sk);
         if (!Pl::P_OVER) load_key_params(r + 1, sk);
       }
@@ -1121,11 +1125,19 @@ __global__ void __launch_bounds__(Plan<BK, BV, GS, HP, NL, MANY>::WARPS * 32, Pl
       }
     }
     // the value half of the stage and the numerators are free
+    Sources sv;
+    if constexpr (WIDE) {
+      sk = sources(0);
+      sv = sources(1);
+    }
     proxy_fence();
     __syncwarp();
     if (r + 1 < rounds) {
       if (elect_one()) {
-        const Sources sk = sources(0), sv = sources(1);
+        if constexpr (!WIDE) {
+          sk = sources(0);
+          sv = sources(1);
+        }
         if (Pl::P_OVER) load_key_params(r + 1, sk);
         load_values(r + 1, sv);
       }
