@@ -36,8 +36,8 @@ BULK_MIN, BULK_MAX = 16, 64  # between 16 and 64 window blocks per call
 # dram__bytes_read.sum + dram__bytes_write.sum of one layer call of the decode kernel (ncu, a launch of four layers;
 # see profiles/), with the SHA-256 of the kernel's sources at the time the counters were taken: the
 # figure is reported only while the sources still hash to that.
-NCU_TRAFFIC = {"c2": {"bytes": 235.9e6 / 4 + 7.2e6 / 4,
-                      "sources_sha256": "a7a564592a316a409bf618ab632ee9dfbb29f5ac18b4ea83cf308c13e9e68c27"}}
+NCU_TRAFFIC = {"c2": {"bytes": 236.0e6 / 4 + 7.1e6 / 4,
+                      "sources_sha256": "73bb9dc5fd37c2fc1d8d89cd3d49d1307901694650c745c234e4de8e17169484"}}
 KERNEL_SOURCES = ("xq_decode_mma.cuh", "xq_mma.cuh", "xq_layout.cuh", "xq_internal.h")
 
 
