@@ -37,7 +37,7 @@ BULK_MIN, BULK_MAX = 16, 64  # between 16 and 64 window blocks per call
 # see profiles/), with the SHA-256 of the kernel's sources at the time the counters were taken: the
 # figure is reported only while the sources still hash to that.
 NCU_TRAFFIC = {"c2": {"bytes": 236.0e6 / 4 + 7.1e6 / 4,
-                      "sources_sha256": "73bb9dc5fd37c2fc1d8d89cd3d49d1307901694650c745c234e4de8e17169484"}}
+                      "sources_sha256": "3bdd52607fe94cd6fa41e2ef0ec552835e2fd8c1d60ddb8bc31f5300bab65ebc"}}
 KERNEL_SOURCES = ("xq_decode_mma.cuh", "xq_mma.cuh", "xq_layout.cuh", "xq_internal.h")
 
 

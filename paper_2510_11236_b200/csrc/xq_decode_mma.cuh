@@ -36,7 +36,7 @@
 // did spent a batch's ~1600 cycles on that chain of hand-overs, two batches per SM at a time (32k context, four heads:
 // 34.2 us per layer).
 // What bounds it: not one pipe.  In a launch of four layers at 32k, four heads, issue slots are 52 % used, the tensor pipe
-// 38 %, ALU 37 %, the shared-memory pipe 41 %.  A batch of two layers is ~3080 warp instructions there (~2700 in long ranges,
+// 38 %, ALU 35 %, the shared-memory pipe 51 %.  A batch of two layers is ~3010 warp instructions there (~2700 in long ranges,
 // where a CTA's start and end do not count), 512 of them masks (2 cycles each per sub-partition), 290 products (8 cycles of
 // the tensor pipe, ~2.7 of everyone's issue), ~400 half-precision multiplies (2 cycles).  Microbenchmarks of the instructions
 // of both product phases come to 2900 of the 5150 cycles that a sub-partition takes for the batch (2.62 us in long ranges, 16
